@@ -9,6 +9,7 @@
 #include <algorithm>
 
 #include "likelihood.cuh"
+#include "tcgen05.cuh"
 
 namespace gpuns {
 
@@ -107,11 +108,26 @@ __device__ __forceinline__ T act_apply(const ActDev<T>& a, int n, T x) {
     return (g + (T(1) - g) / (T(1) + ex_acc<T>(-a.beta[n] * x))) * x;
 }
 
-template <typename TO, typename T> __device__ inline TO cvt_out(T v) { return (TO)v; }
-template <> __device__ inline __nv_bfloat16 cvt_out<__nv_bfloat16, float>(float v) { return __float2bfloat16_rn(v); }
-
-template <typename T> __device__ inline T cvt_in(T v) { return v; }
-__device__ inline float cvt_in(__nv_bfloat16 v) { return __bfloat162float(v); }
+// Where the input layer puts h[row][n]: a plain matrix in the next layer's
+// type, or the three bf16 planes that hold an FP32 value (gemm_planes.cu).
+struct OutF64 {
+    double* p;
+    __device__ __forceinline__ void put(int row, int n, int N, double v) const { p[(size_t)row * N + n] = v; }
+};
+struct OutBf16 {
+    __nv_bfloat16* p;
+    __device__ __forceinline__ void put(int row, int n, int N, float v) const {
+        p[(size_t)row * N + n] = __float2bfloat16_rn(v);
+    }
+};
+struct OutPlanes {
+    __nv_bfloat16* p;
+    long long stride;
+    int pitch;
+    __device__ __forceinline__ void put(int row, int n, int, float v) const {
+        tc::plane_store<3>(v, p + (size_t)row * pitch + n, stride);
+    }
+};
 
 // Input layer: h = act(W0 x + b0), x = (theta[inputs] - center) / scale.  A
 // CTA takes kInRows consecutive rows; thread t owns units t, t + blockDim, ...
@@ -119,13 +135,13 @@ __device__ inline float cvt_in(__nv_bfloat16 v) { return __bfloat162float(v); }
 // rows, so the weights are read once per CTA and the launch has
 // ceil(rows / kInRows) CTAs rather than one per (row, 256 units).
 constexpr int kInRows = 2;
-template <typename T, typename TO, int KMAX>
+template <typename T, typename OUT, int KMAX>
 __global__ void __launch_bounds__(256)
 k_emu_input(const double* __restrict__ theta_full, int P, const int* __restrict__ inputs,
             const double* __restrict__ center, const double* __restrict__ scale,
             const double* __restrict__ inv_scale, int K0,
             const T* __restrict__ W0, const T* __restrict__ b0, ActDev<T> act, int N,
-            TO* __restrict__ out, const int* __restrict__ nrows) {
+            const OUT out, const int* __restrict__ nrows) {
     // the weights of a thread's first UP units are problem constants: in
     // registers before the dependency wait
     constexpr int UP = KMAX <= 8 ? 4 : 1;
@@ -157,7 +173,7 @@ k_emu_input(const double* __restrict__ theta_full, int P, const int* __restrict_
 #pragma unroll
             for (int j = 0; j < KMAX; ++j)
                 if (j < K0) acc = fma(w[j], x[r][j], acc);
-            out[(size_t)(r0 + r) * N + n] = cvt_out<TO, T>(act_apply<T>(act, n, acc));
+            out.put(r0 + r, n, N, act_apply<T>(act, n, acc));
         }
     };
 #pragma unroll
@@ -175,14 +191,14 @@ k_emu_input(const double* __restrict__ theta_full, int P, const int* __restrict_
 
 // C[M x N] = epi(A[M x K] W[N x K]^T + b).  Threads own an interleaved
 // TM x TN sub-tile (rows ty + i*BM/TM, cols tx + j*BN/TN) so shared-memory
-// reads and global stores are conflict-free / coalesced.  A may be stored in
-// a narrower type (bf16 activations) and is widened on load.
+// reads and global stores are conflict-free / coalesced.  FP64 problems and
+// set-up work (FP32 layers run on the tensor cores, gemm_planes.cu).
 //   EPI_ACT: act(acc + b);  EPI_OUT: mu + s (acc + b), s = sig_vec[n] or sigma.
 enum { EPI_ACT = 0, EPI_OUT = 1 };
 
-template <typename T, typename TA, int BM, int BN, int BK, int TM, int TN, int EPI>
+template <typename T, int BM, int BN, int BK, int TM, int TN, int EPI>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN))
-k_gemm_simt(const TA* __restrict__ A, const T* __restrict__ W, const T* __restrict__ bias, ActDev<T> act,
+k_gemm_simt(const T* __restrict__ A, const T* __restrict__ W, const T* __restrict__ bias, ActDev<T> act,
             const T* __restrict__ out_mu, const T* __restrict__ sig_vec, T out_sigma, T* __restrict__ C,
             const int* __restrict__ nrows, int N, int K) {
     constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
@@ -201,7 +217,7 @@ k_gemm_simt(const TA* __restrict__ A, const T* __restrict__ W, const T* __restri
         for (int i = tid; i < BM * BK; i += NT) {
             const int r = i / BK, c = i % BK;
             const int gm = m0 + r, gk = k0 + c;
-            As[c][r] = (gm < M && gk < K) ? (T)cvt_in(A[(size_t)gm * K + gk]) : T(0);
+            As[c][r] = (gm < M && gk < K) ? A[(size_t)gm * K + gk] : T(0);
         }
         for (int i = tid; i < BN * BK; i += NT) {
             const int r = i / BK, c = i % BK;
@@ -258,23 +274,14 @@ __global__ void k_zinterp(const T* __restrict__ coarse, int nzc, const int* __re
     }
 }
 
-template <typename T, typename TA>
-struct SimtTile;
-template <typename TA> struct SimtTile<double, TA> { static constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4; };
-template <typename TA> struct SimtTile<float, TA> { static constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8; };
-
-template <typename T, typename TA>
-int launch_gemm_simt(const TA* A, const T* W, const T* bias, ActDev<T> act, const T* mu, const T* sig_vec, T sigma,
-                     T* C, const int* nrows, int grid_rows, int N, int K, int epi, cudaStream_t st) {
-    using S = SimtTile<T, TA>;
-    constexpr int NT = (S::BM / S::TM) * (S::BN / S::TN);
-    dim3 grid((N + S::BN - 1) / S::BN, (grid_rows + S::BM - 1) / S::BM);
-    if (epi == EPI_ACT)
-        k_gemm_simt<T, TA, S::BM, S::BN, S::BK, S::TM, S::TN, EPI_ACT><<<grid, NT, 0, st>>>(
-            A, W, bias, act, mu, sig_vec, sigma, C, nrows, N, K);
-    else
-        k_gemm_simt<T, TA, S::BM, S::BN, S::BK, S::TM, S::TN, EPI_OUT><<<grid, NT, 0, st>>>(
-            A, W, bias, act, mu, sig_vec, sigma, C, nrows, N, K);
+static int launch_gemm_simt(const double* A, const double* W, const double* bias, ActDev<double> act, const double* mu,
+                            const double* sig_vec, double sigma, double* C, const int* nrows, int grid_rows, int N,
+                            int K, int epi, cudaStream_t st) {
+    constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4, NT = (BM / TM) * (BN / TN);
+    const dim3 grid((N + BN - 1) / BN, (grid_rows + BM - 1) / BM);
+    auto kern = epi == EPI_ACT ? k_gemm_simt<double, BM, BN, BK, TM, TN, EPI_ACT>
+                               : k_gemm_simt<double, BM, BN, BK, TM, TN, EPI_OUT>;
+    kern<<<grid, NT, 0, st>>>(A, W, bias, act, mu, sig_vec, sigma, C, nrows, N, K);
     NS_CUDA_TRY(cudaGetLastError());
     return NS_OK;
 }
@@ -283,7 +290,7 @@ int launch_gemm_simt(const TA* A, const T* W, const T* bias, ActDev<T> act, cons
 // (the CMB whitening fold); nrows_dev holds M.
 int gemm_f64_plain(const double* A, const double* W, double* C, const int* nrows_dev, int M, int N, int K,
                    const double* zeros_n, cudaStream_t st) {
-    return launch_gemm_simt<double, double>(A, W, zeros_n, ActDev<double>{0, nullptr, nullptr}, zeros_n, nullptr,
+    return launch_gemm_simt(A, W, zeros_n, ActDev<double>{0, nullptr, nullptr}, zeros_n, nullptr,
                                             1.0, C, nrows_dev, M, N, K, EPI_OUT, st);
 }
 
@@ -306,12 +313,12 @@ static ActDev<T> layer_act(const ns_problem* p, int l) {
     return a;
 }
 
-template <typename T, typename TO>
-static int launch_emu_input(const ns_problem* p, const Workspace* ws, int grid_rows, TO* out, bool pdl,
+template <typename T, typename OUT>
+static int launch_emu_input(const ns_problem* p, const Workspace* ws, int grid_rows, const OUT& out, bool pdl,
                             cudaStream_t st) {
     const int K0 = p->dims[0], H1 = p->dims[1];
     const dim3 g((grid_rows + kInRows - 1) / kInRows);
-    auto kern = K0 <= 8 ? k_emu_input<T, TO, 8> : k_emu_input<T, TO, 32>;
+    auto kern = K0 <= 8 ? k_emu_input<T, OUT, 8> : k_emu_input<T, OUT, 32>;
     if (pdl) {
         NS_CUDA_TRY(launch_pdl(kern, g, dim3(256), 0, st, (const double*)ws->theta_full, p->P,
                                (const int*)p->d_inputs, (const double*)p->d_in_center, (const double*)p->d_in_scale,
@@ -328,7 +335,8 @@ static int launch_emu_input(const ns_problem* p, const Workspace* ws, int grid_r
 
 // The emulator's last layer: W h + b, de-standardised as mu + s * (.), written to out.
 struct Head {
-    const void* W;
+    const void* W;           // FP64 problems
+    const CUtensorMap* tmW;  // FP32 heads: three bf16 planes
     const void* bias;
     const void* mu;
     const void* sig_vec;
@@ -339,28 +347,68 @@ struct Head {
 
 static Head model_head(const ns_problem* p, void* out) {
     const int L = p->n_layers;
-    return Head{p->d_W[L - 1], p->d_b[L - 1], p->d_out_mu, p->d_out_sig, p->out_sigma, out};
+    return Head{p->d_W[L - 1], p->tmWp.empty() ? nullptr : &p->tmWp[L - 1], p->d_b[L - 1], p->d_out_mu, p->d_out_sig,
+                p->out_sigma, out};
 }
 
-template <typename T>
-static int run_emulator_simt(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, const Head& hd) {
+static int run_emulator_f64(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, const Head& hd) {
     const int L = p->n_layers;
-    NS_TRY((launch_emu_input<T, T>(p, ws, grid_rows, (T*)ws->act[0], false, st)));
+    NS_TRY((launch_emu_input<double>(p, ws, grid_rows, OutF64{(double*)ws->act[0]}, false, st)));
     int cur = 0;
     for (int l = 1; l < L; ++l) {
         const int K = p->dims[l], N = p->dims[l + 1];
+        const double* x = (const double*)ws->act[cur];
         if (l == L - 1) {
-            NS_TRY((launch_gemm_simt<T, T>((const T*)ws->act[cur], (const T*)hd.W, (const T*)hd.bias, ActDev<T>{0, nullptr, nullptr},
-                                           (const T*)hd.mu, (const T*)hd.sig_vec, (T)hd.sigma, (T*)hd.out,
-                                           ws->d_nrows, grid_rows, hd.n_out ? hd.n_out : N, K, EPI_OUT, st)));
+            NS_TRY(launch_gemm_simt(x, (const double*)hd.W, (const double*)hd.bias, ActDev<double>{0, nullptr, nullptr},
+                                    (const double*)hd.mu, (const double*)hd.sig_vec, hd.sigma, (double*)hd.out,
+                                    ws->d_nrows, grid_rows, hd.n_out ? hd.n_out : N, K, EPI_OUT, st));
         } else {
-            NS_TRY((launch_gemm_simt<T, T>((const T*)ws->act[cur], (const T*)p->d_W[l], (const T*)p->d_b[l],
-                                           layer_act<T>(p, l), nullptr, nullptr, T(0), (T*)ws->act[cur ^ 1],
-                                           ws->d_nrows, grid_rows, N, K, EPI_ACT, st)));
+            NS_TRY(launch_gemm_simt(x, (const double*)p->d_W[l], (const double*)p->d_b[l], layer_act<double>(p, l),
+                                    nullptr, nullptr, 0.0, (double*)ws->act[cur ^ 1], ws->d_nrows, grid_rows, N, K,
+                                    EPI_ACT, st));
         }
         cur ^= 1;
     }
     return NS_OK;
+}
+
+// An FP32 head (FP32 problems: px = 3 planes of activations; BF16 CMB: px = 1).
+static int launch_head_f32(const ns_problem* p, Workspace* ws, int grid_rows, int px, const Head& hd, cudaStream_t st) {
+    const int L = p->n_layers;
+    PlaneEpi e;
+    e.mode = PLN_OUT;
+    e.bias = (const float*)hd.bias;
+    e.mu = (const float*)hd.mu;
+    e.sig_vec = (const float*)hd.sig_vec;
+    e.sigma = (float)hd.sigma;
+    e.out = (float*)hd.out;
+    return launch_gemm_planes(px, 3, hd.tmW, &ws->tmXp[L - 1], e, ws->d_nrows, grid_rows,
+                              hd.n_out ? hd.n_out : p->dims[L], p->dims[L - 1], ws->d_err, st);
+}
+
+// FP32: the input layer on CUDA cores, every further layer as an FP32-accurate
+// GEMM on the tensor cores; activations travel as three bf16 planes.
+static int run_emulator_f32(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, const Head& hd) {
+    const int L = p->n_layers;
+    NS_TRY((launch_emu_input<float>(p, ws, grid_rows,
+                                    OutPlanes{(__nv_bfloat16*)ws->act[0], ws->plane_stride, plane_pitch(p->dims[1])},
+                                    true, st)));
+    int cur = 0;
+    for (int l = 1; l + 1 < L; ++l) {
+        const ActDev<float> a = layer_act<float>(p, l);
+        PlaneEpi e;
+        e.mode = p->act == NS_ACT_SIGMOID_LINEAR ? PLN_SIGLIN : PLN_TANH;
+        e.bias = (const float*)p->d_b[l];
+        e.g = a.g;
+        e.beta = a.beta;
+        e.planes = (__nv_bfloat16*)ws->act[cur ^ 1];
+        e.plane_stride = ws->plane_stride;
+        e.pitch = plane_pitch(p->dims[l + 1]);
+        NS_TRY(launch_gemm_planes(3, 3, &p->tmWp[l], &ws->tmXp[l], e, ws->d_nrows, grid_rows, p->dims[l + 1],
+                                  p->dims[l], ws->d_err, st));
+        cur ^= 1;
+    }
+    return launch_head_f32(p, ws, grid_rows, 3, hd, st);
 }
 
 static int probe_begin(const StageProbe* pr, int stage, Workspace* ws, cudaStream_t st) {
@@ -392,7 +440,7 @@ static int run_emulator_bf16(const ns_problem* p, Workspace* ws, int grid_rows, 
         cur = (L - 2) & 1;
         l1 = L - 1;
     } else {
-        NS_TRY((launch_emu_input<float, __nv_bfloat16>(p, ws, grid_rows, (__nv_bfloat16*)ws->act[0], true, st)));
+        NS_TRY((launch_emu_input<float>(p, ws, grid_rows, OutBf16{(__nv_bfloat16*)ws->act[0]}, true, st)));
     }
     for (int l = l1; l < L; ++l) {
         const int K = p->dims[l], N = p->dims[l + 1];
@@ -400,11 +448,7 @@ static int run_emulator_bf16(const ns_problem* p, Workspace* ws, int grid_rows, 
         const int stage = last ? PROBE_EMU_OUT : (l == 1 ? PROBE_EMU_HIDDEN : PROBE_NONE);
         NS_TRY(probe_begin(probe, stage, ws, st));
         if (last && hd) {
-            NS_TRY((launch_gemm_simt<float, __nv_bfloat16>(
-                (const __nv_bfloat16*)ws->act[cur], (const float*)hd->W, (const float*)hd->bias,
-                ActDev<float>{0, nullptr, nullptr}, (const float*)hd->mu, (const float*)hd->sig_vec,
-                (float)hd->sigma, (float*)hd->out, ws->d_nrows, grid_rows, hd->n_out ? hd->n_out : N, K, EPI_OUT,
-                st)));
+            NS_TRY(launch_head_f32(p, ws, grid_rows, 1, *hd, st));
         } else if (last && p->tile_n[l] == 128) {
             // the output layer with few rows: features as the MMA's M (one wave of CTAs)
             NS_TRY(launch_gemm_tc_out_swap(&p->tmB[l], &ws->tmX_out, (const float*)p->d_b[l],
@@ -484,10 +528,10 @@ int run_emulator_only(const ns_problem* p, Workspace* ws, int grid_rows, double*
     dim3 g((n_out + 255) / 256, grid_rows);
     const Head hd = model_head(p, ws->table);
     if (p->precision == NS_PREC_FP64) {
-        NS_TRY(run_emulator_simt<double>(p, ws, grid_rows, st, hd));
+        NS_TRY(run_emulator_f64(p, ws, grid_rows, st, hd));
         k_to_double<double><<<g, 256, 0, st>>>((const double*)ws->table, out, n_out, ws->d_nrows);
     } else {
-        if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_simt<float>(p, ws, grid_rows, st, hd));
+        if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_f32(p, ws, grid_rows, st, hd));
         else NS_TRY(run_emulator_bf16(p, ws, grid_rows, st, nullptr, p->kind == NS_KIND_CMB ? &hd : nullptr));
         k_to_double<float><<<g, 256, 0, st>>>((const float*)ws->table, out, n_out, ws->d_nrows);
     }
@@ -508,8 +552,8 @@ static int run_cmb(const ns_problem* p, Workspace* ws, int grid_rows, double* lo
         // the TT block of the head only (the first n_tt outputs), then the sums
         Head hd = model_head(p, ws->table);
         hd.n_out = p->n_tt;
-        if (f64) NS_TRY(run_emulator_simt<double>(p, ws, grid_rows, st, hd));
-        else if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_simt<float>(p, ws, grid_rows, st, hd));
+        if (f64) NS_TRY(run_emulator_f64(p, ws, grid_rows, st, hd));
+        else if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_f32(p, ws, grid_rows, st, hd));
         else NS_TRY(run_emulator_bf16(p, ws, grid_rows, st, probe, &hd));
         NS_TRY(probe_begin(probe, PROBE_CHI2, ws, st));
         if (f64)
@@ -525,16 +569,16 @@ static int run_cmb(const ns_problem* p, Workspace* ws, int grid_rows, double* lo
     }
     if (p->cmb_solve == NS_SOLVE_LITERAL) {
         const int L = p->n_layers;
-        const Head hd{p->d_W[L - 1], p->d_b[L - 1], p->d_lit_mu, p->d_lit_sig, 0.0, ws->resid};
-        NS_TRY(run_emulator_simt<double>(p, ws, grid_rows, st, hd));
+        const Head hd{p->d_W[L - 1], nullptr, p->d_b[L - 1], p->d_lit_mu, p->d_lit_sig, 0.0, ws->resid};
+        NS_TRY(run_emulator_f64(p, ws, grid_rows, st, hd));
         NS_TRY(probe_begin(probe, PROBE_CHI2, ws, st));
         NS_TRY((launch_chi2<double, double>((const double*)ws->resid, D, p->d_LinvT64, p->c0, logL_out,
                                             ws->d_nrows, grid_rows, st)));
         return probe_end(probe, PROBE_CHI2, st);
     }
-    const Head hd{p->d_Wfold, p->d_zeroD, p->d_cfold, nullptr, -1.0, ws->table};
-    if (f64) NS_TRY(run_emulator_simt<double>(p, ws, grid_rows, st, hd));
-    else if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_simt<float>(p, ws, grid_rows, st, hd));
+    const Head hd{p->d_Wfold, &p->tmWfold, p->d_zeroD, p->d_cfold, nullptr, -1.0, ws->table};
+    if (f64) NS_TRY(run_emulator_f64(p, ws, grid_rows, st, hd));
+    else if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_f32(p, ws, grid_rows, st, hd));
     else NS_TRY(run_emulator_bf16(p, ws, grid_rows, st, probe, &hd));
     NS_TRY(probe_begin(probe, PROBE_CHI2, ws, st));
     if (f64) k_rowsq<double><<<grid_rows, 256, 0, st>>>((const double*)ws->table, D, p->c0, logL_out, ws->d_nrows);
@@ -568,7 +612,7 @@ int run_likelihood(const ns_problem* p, Workspace* ws, int grid_rows, double* lo
     NS_TRY(probe_end(probe, PROBE_WINDOWS, ws->side));
     NS_CUDA_TRY(cudaEventRecord(ws->ev_join, ws->side));
     if (f64) {
-        NS_TRY(run_emulator_simt<double>(p, ws, grid_rows, st, model_head(p, ws->table)));
+        NS_TRY(run_emulator_f64(p, ws, grid_rows, st, model_head(p, ws->table)));
         const double* tab = (const double*)ws->table;
         if (coarse) {
             dim3 g((sp.n_z * sp.n_k + 255) / 256, grid_rows);
@@ -585,7 +629,7 @@ int run_likelihood(const ns_problem* p, Workspace* ws, int grid_rows, double* lo
                                            ws->d_nrows, grid_rows, st, true);
     }
     // FP32 stages (FP32 / BF16 / BF16_F64CHI2)
-    if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_simt<float>(p, ws, grid_rows, st, model_head(p, ws->table)));
+    if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_f32(p, ws, grid_rows, st, model_head(p, ws->table)));
     else NS_TRY(run_emulator_bf16(p, ws, grid_rows, st, probe, nullptr));
     const float* tab = (const float*)ws->table;
     if (coarse) {

@@ -44,6 +44,11 @@ struct ShearParams {
     const float* tmpl_f;
 };
 
+// Tensor maps of an activation operand of k_gemm_planes, one per row tile (32, 64, 128).
+struct PlaneMapX {
+    CUtensorMap m[3];
+};
+
 struct Workspace {
     int cap = 0;
     int* d_nrows = nullptr;       // device row count used by every stage
@@ -58,6 +63,9 @@ struct Workspace {
     double* logL = nullptr;       // cap
     // tcgen05 tensor maps (BF16 precision): A operand of layer l >= 1 and its output
     std::vector<CUtensorMap> tmA;
+    // k_gemm_planes: layer l's input planes (FP32: three; the FP32 head of a BF16 CMB problem: one)
+    std::vector<PlaneMapX> tmXp;
+    long long plane_stride = 0;   // FP32: elements between the planes of an activation buffer
     CUtensorMap tmX_out{};        // the last layer's activations in kSwapRows-row boxes
     CUtensorMap tmF_out{};        // fused emulator stack: its output activations in 64-row boxes of two k-blocks
     std::vector<void*> owned;
@@ -82,6 +90,7 @@ struct ns_problem {
     std::vector<int> dims;
     std::vector<void*> d_W;          // per layer, compute dtype (layer 0: FP64 or FP32)
     std::vector<void*> d_b;          // per layer, FP64 (FP64 mode) else FP32
+    std::vector<CUtensorMap> tmWp;   // FP32 layers >= 1 (and a BF16 CMB head): the weights as three bf16 planes
     std::vector<CUtensorMap> tmB;    // BF16: weight tensor maps for layers >= 1
     std::vector<int> tile_n;         // BF16: N tile per layer (hidden layers autotuned at creation)
     std::vector<float> tile_ms;      // BF16: measured time per launch of the chosen hidden tiles
@@ -111,7 +120,8 @@ struct ns_problem {
     void* d_out_sig = nullptr;       // per-output scales (compute dtype) or null: scalar out_sigma
     // CMB
     int cmb_solve = 0;
-    void* d_Wfold = nullptr;         // D x H: W' = L^-1 diag(sigma) W_out (compute dtype)
+    void* d_Wfold = nullptr;         // D x H: W' = L^-1 diag(sigma) W_out (FP64 problems)
+    CUtensorMap tmWfold{};           // the same as three bf16 planes (FP32, BF16 problems)
     void* d_cfold = nullptr;         // D: c' = L^-1 (d - mu - sigma b_out)
     void* d_zeroD = nullptr;         // D zeros: bias of the folded head
     double* d_lit_mu = nullptr;      // LITERAL: d - mu
@@ -229,6 +239,39 @@ int launch_emu_fused(const ns_problem* p, const Workspace* ws, int grid_rows, cu
 int launch_gemm_tc_out_swap(const CUtensorMap* tmW, const CUtensorMap* tmX, const float* bias, const float* out_mu,
                             float out_sigma, float* C, const int* d_nrows, int grid_rows, int N, int K, int* d_err,
                             cudaStream_t st);
+// GEMMs of FP32 accuracy on the bf16 tensor path (gemm_planes.cu): out[r][f] =
+// epi(sum_k X[r][k] W[f][k]) with X in px and W in pw bf16 planes.
+enum { PLN_TANH = 0, PLN_SIGLIN = 1, PLN_OUT = 2, PLN_DTANH = 3, PLN_DTANH32 = 4 };
+struct PlaneEpi {
+    int mode = PLN_OUT;
+    const float* bias = nullptr;      // TANH, SIGLIN, OUT
+    const float* mu = nullptr;        // OUT: mu + s (acc + bias), s = sig_vec[f] or sigma
+    const float* sig_vec = nullptr;
+    float sigma = 0.f;
+    const float* g = nullptr;         // SIGLIN
+    const float* beta = nullptr;
+    float* out = nullptr;             // OUT, DTANH32: FP32, rows x N
+    __nv_bfloat16* planes = nullptr;  // TANH, SIGLIN, DTANH: px planes of row pitch `pitch`
+    long long plane_stride = 0;
+    int pitch = 0;
+    const __nv_bfloat16* aux = nullptr;  // DTANH: acc (1 - h^2), h in px planes
+    long long aux_stride = 0;
+    int aux_pitch = 0;
+};
+struct PlaneTiling {
+    int br, split;                    // rows per tile; CTAs of a cluster sharing the k-blocks
+};
+PlaneTiling plane_tiling(int rows, int N, int K, int px, int pw);
+int launch_gemm_planes(int px, int pw, const CUtensorMap* tmW, const PlaneMapX* tmX, const PlaneEpi& e,
+                       const int* nrows, int grid_rows, int N, int K, int* err, cudaStream_t st);
+// planes of s * in (rows x cols, packed); nrows: device row count or null
+int launch_split_planes(int planes, const float* in, float s, int rows, int cols, __nv_bfloat16* out, long long stride,
+                        int pitch, const int* nrows, cudaStream_t st);
+inline int plane_pitch(int K) { return (K + 7) & ~7; }   // rows of 16-byte multiples
+// tensor map over `planes` matrices rows x K (row pitch plane_pitch(K)), box = every plane's box_rows x 64
+int make_tensor_map_planes(CUtensorMap* tm, const void* base, int rows, int K, long long stride, int planes,
+                           int box_rows);
+int make_plane_maps_x(PlaneMapX* m, const void* base, int rows, int K, long long stride, int planes);
 // Dense FP64 set-up kernels (dense_linalg.cu): C (device, overwritten by L) ->
 // L^-1 (new device buffer) and sum ln L_aa; NS_EINVAL if C is not SPD.
 int device_cholesky_inverse(double* dC, int D, double** Xout, double* sum_log_diag, cudaStream_t st);

@@ -109,15 +109,23 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
     NS_TRY(dalloc(sizeof(double) * (size_t)cap, &v, ws->owned));
     ws->logL = (double*)v;
     if (p->kind == NS_KIND_GAUSS) return NS_OK;
-    const int elt = (p->precision == NS_PREC_FP64) ? 8 : (p->precision == NS_PREC_FP32 ? 4 : 2);
+    // activations: FP64, bf16, or FP32 as three bf16 planes
+    const int elt = (p->precision == NS_PREC_FP64) ? 8 : (p->precision == NS_PREC_FP32 ? 6 : 2);
+    const int rows_pad = ((cap + 127) / 128) * 128;
+    const size_t act_bytes = (size_t)elt * rows_pad * plane_pitch(p->hidden_max);
+    for (int i = 0; i < 2; ++i) {
+        NS_TRY(dalloc(act_bytes, &v, ws->owned));
+        ws->act[i] = v;
+        NS_CUDA_TRY(cudaMemset(v, 0, act_bytes));
+    }
+    if (p->precision == NS_PREC_FP32) {
+        ws->plane_stride = (long long)rows_pad * plane_pitch(p->hidden_max);
+        ws->tmXp.resize(p->n_layers);
+        for (int l = 1; l < p->n_layers; ++l)
+            NS_TRY(make_plane_maps_x(&ws->tmXp[l], ws->act[(l - 1) & 1], rows_pad, p->dims[l], ws->plane_stride, 3));
+    }
     if (p->kind == NS_KIND_CMB) {
         const int tab_elt = (p->precision == NS_PREC_FP64) ? 8 : 4;
-        const int rows_pad = ((cap + 127) / 128) * 128;
-        for (int i = 0; i < 2; ++i) {
-            NS_TRY(dalloc((size_t)elt * rows_pad * p->hidden_max, &v, ws->owned));
-            ws->act[i] = v;
-            NS_CUDA_TRY(cudaMemset(v, 0, (size_t)elt * rows_pad * p->hidden_max));
-        }
         NS_TRY(dalloc((size_t)tab_elt * cap * std::max(p->D, p->dims.back()), &v, ws->owned));
         ws->table = v;
         if (p->cmb_solve == NS_SOLVE_LITERAL && p->cmb_form == NS_CMB_GAUSS) {
@@ -132,16 +140,15 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
                                             gemm_tc_kps(p->dims[l])));
                 cur ^= 1;
             }
+            // the FP32 head reads the last hidden layer's bf16 activations as one plane
+            const int Kh = p->dims[p->n_layers - 1];
+            ws->tmXp.resize(p->n_layers);
+            NS_TRY(make_plane_maps_x(&ws->tmXp[p->n_layers - 1], ws->act[cur], rows_pad, Kh,
+                                     (long long)rows_pad * plane_pitch(Kh), 1));
         }
         return NS_OK;
     }
     const int tab_elt = (p->precision == NS_PREC_FP64) ? 8 : 4;
-    const int rows_pad = ((cap + 127) / 128) * 128;
-    for (int i = 0; i < 2; ++i) {
-        NS_TRY(dalloc((size_t)elt * rows_pad * p->hidden_max, &v, ws->owned));
-        ws->act[i] = v;
-        NS_CUDA_TRY(cudaMemset(v, 0, (size_t)elt * rows_pad * p->hidden_max));
-    }
     const int n_out = p->dims.back();
     NS_TRY(dalloc((size_t)tab_elt * cap * n_out, &v, ws->owned));
     ws->table = v;
@@ -203,6 +210,29 @@ static int upload_compute(const ns_problem* p, const double* h, size_t n, void**
         *out = v;
     }
     return NS_OK;
+}
+
+// An FP32 matrix (rows x K) on the device as three bf16 planes and their
+// tensor map (the weights of k_gemm_planes).
+static int make_planes(const float* d, int rows, int K, CUtensorMap* tm, std::vector<void*>& owned) {
+    const int pitch = plane_pitch(K);
+    const long long stride = (long long)rows * pitch;
+    void* v = nullptr;
+    NS_TRY(dalloc(sizeof(uint16_t) * 3 * (size_t)stride, &v, owned));
+    NS_TRY(launch_split_planes(3, d, 1.f, rows, K, (__nv_bfloat16*)v, stride, pitch, nullptr, nullptr));
+    NS_CUDA_TRY(cudaStreamSynchronize(nullptr));   // calls may come on any stream
+    return make_tensor_map_planes(tm, v, rows, K, stride, 3, 128);
+}
+
+// FP32 copy of a host FP64 matrix as planes only; the copy is freed again.
+static int upload_planes(const double* h, int rows, int K, CUtensorMap* tm, std::vector<void*>& owned) {
+    std::vector<float> f(h, h + (size_t)rows * K);
+    std::vector<void*> tmp;
+    float* d = nullptr;
+    int s = upload(f.data(), f.size(), &d, tmp);
+    if (!s) s = make_planes(d, rows, K, tm, owned);
+    for (void* q : tmp) cudaFree(q);
+    return s;
 }
 
 // CMB set-up: FP64 factorisation of the covariance (host for D <= 256, else
@@ -319,7 +349,8 @@ static int cmb_setup(ns_problem* p, const ns_problem_desc* desc) {
             return done(NS_ECUDA);
         done(NS_OK);
     }
-    NS_TRY(upload_compute(p, Wf.data(), Wf.size(), &p->d_Wfold, p->owned));
+    if (p->precision == NS_PREC_FP64) NS_TRY(upload_compute(p, Wf.data(), Wf.size(), &p->d_Wfold, p->owned));
+    else NS_TRY(upload_planes(Wf.data(), D, H, &p->tmWfold, p->owned));
     NS_TRY(upload_compute(p, cf.data(), cf.size(), &p->d_cfold, p->owned));
     return NS_OK;
 }
@@ -520,6 +551,7 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
     }
     p->d_W.assign(e.n_layers, nullptr);
     p->d_b.assign(e.n_layers, nullptr);
+    if (!f64) p->tmWp.resize(e.n_layers);
     for (int l = 0; l < e.n_layers; ++l) {
         const size_t nw = (size_t)p->dims[l + 1] * p->dims[l];
         const size_t nb = p->dims[l + 1];
@@ -541,12 +573,16 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
                 uint16_t* w;
                 if ((s = upload(wb.data(), nw, &w, p->owned))) return fail(s);
                 p->d_W[l] = w;
+            } else if (l >= 1 && cmb) {
+                if ((s = upload_planes(e.W[l], p->dims[l + 1], p->dims[l], &p->tmWp[l], p->owned))) return fail(s);
             } else {
+                // FP32 weights: the input layer, and the shear gradient's layers
                 std::vector<float> wf(nw);
                 for (size_t i = 0; i < nw; ++i) wf[i] = (float)e.W[l][i];
                 float* w;
                 if ((s = upload(wf.data(), nw, &w, p->owned))) return fail(s);
                 p->d_W[l] = w;
+                if (l >= 1 && (s = make_planes(w, p->dims[l + 1], p->dims[l], &p->tmWp[l], p->owned))) return fail(s);
             }
         }
     }
