@@ -675,19 +675,50 @@ __global__ void k_emu_in_store(const double* __restrict__ theta_full, int P, con
     out[(size_t)row * N + n] = tanh(acc);
 }
 
-// g_pre_1 (rows x N1) -> g_x (rows x K0) = g_pre_1 W0; then add to the full gradient.
-template <typename T>
-__global__ void k_emu_in_back(const T* __restrict__ gpre, const T* __restrict__ W0, int N1, int K0,
-                              const int* __restrict__ inputs, const double* __restrict__ scale, double* __restrict__ gfull,
-                              int P, const int* __restrict__ nrows) {
+// The emulator inputs' share g_x = g_pre_1 W0 (rows x K0, K0 <= KMAX) added to
+// the projection's parameter gradient, free parameters only.  One block per
+// row; the K0 sums are formed in one pass over the row and reduced together
+// (a block reduction per input took 42 us at 4096 rows of 7 inputs).
+template <typename T, int KMAX>
+__global__ void __launch_bounds__(256)
+k_finish_grad(const T* __restrict__ gpre, const T* __restrict__ W0, int N1, int K0, const int* __restrict__ inputs,
+              const double* __restrict__ scale, const double* __restrict__ gfull, int P,
+              const int* __restrict__ free_of_full, double* __restrict__ grad, int d,
+              const int* __restrict__ nrows) {
+    pdl_begin();
     const int row = blockIdx.x;
     if (row >= *nrows) return;
-    __shared__ T red[32];
-    for (int j = 0; j < K0; ++j) {
-        T s = T(0);
-        for (int n = threadIdx.x; n < N1; n += blockDim.x) s += gpre[(size_t)row * N1 + n] * W0[(size_t)n * K0 + j];
-        s = block_sum(s, red);
-        if (threadIdx.x == 0) gfull[(size_t)row * P + inputs[j]] += (double)s / scale[j];
+    __shared__ T part[8][KMAX];
+    __shared__ double gx[KMAX];
+    T s[KMAX];
+#pragma unroll
+    for (int j = 0; j < KMAX; ++j) s[j] = T(0);
+    for (int n = threadIdx.x; n < N1; n += 256) {
+        const T g = gpre[(size_t)row * N1 + n];
+#pragma unroll
+        for (int j = 0; j < KMAX; ++j)
+            if (j < K0) s[j] = fma(g, W0[(size_t)n * K0 + j], s[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < KMAX; ++j) {
+        if (j >= K0) break;
+        const T t = warp_sum(s[j]);
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5][j] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x < K0) {
+        T t = T(0);
+        for (int w = 0; w < 8; ++w) t += part[w][threadIdx.x];
+        gx[threadIdx.x] = (double)t / scale[threadIdx.x];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < P; i += 256) {
+        const int f = free_of_full[i];
+        if (f < 0) continue;
+        double v = gfull[(size_t)row * P + i];
+        for (int j = 0; j < K0; ++j)
+            if (inputs[j] == i) v += gx[j];
+        grad[(size_t)row * d + f] = v;
     }
 }
 
@@ -717,53 +748,18 @@ __global__ void k_zinterp_adj(const T* __restrict__ gfine, int nz, const int* __
     }
 }
 
-__global__ void k_gather_grad(const double* __restrict__ gfull, int P, const int* __restrict__ free_of_full,
-                              double* __restrict__ grad, int d, int B) {
-    const int row = blockIdx.x;
-    if (row >= B) return;
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const int f = free_of_full[i];
-        if (f >= 0) grad[(size_t)row * d + f] = gfull[(size_t)row * P + i];
-    }
-}
-
-// BF16 problems, split path.  Input layer: h = tanh(W0 x + b0) in FP32 with
-// x standardised once per row (reciprocal scale), written as a bf16 (hi, lo)
-// pair: layer 1's A operand and the stored activation for the backward pass.
-__global__ void k_emu_in_split(const double* __restrict__ theta_full, int P, const int* __restrict__ inputs,
-                               const double* __restrict__ center, const double* __restrict__ inv_scale, int K0,
-                               const float* __restrict__ W0, const float* __restrict__ b0, int N,
-                               __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
-                               const int* __restrict__ nrows) {
-    const int row = blockIdx.y;
-    if (row >= *nrows) return;
-    __shared__ float x[32];
-    if (threadIdx.x < K0) {
-        const int j = threadIdx.x;
-        x[j] = (float)((theta_full[(size_t)row * P + inputs[j]] - center[j]) * inv_scale[j]);
-    }
+// T[p][k][n] = W[p][n][k] for bf16 planes: W N rows of pitch wp, T K rows of pitch tp.
+__global__ void __launch_bounds__(256) k_transpose_planes(const __nv_bfloat16* __restrict__ W, int N, int K, int wp,
+                                                          __nv_bfloat16* __restrict__ T, int tp) {
+    __shared__ __nv_bfloat16 t[32][33];
+    const __nv_bfloat16* w = W + (size_t)blockIdx.z * N * wp;
+    __nv_bfloat16* o = T + (size_t)blockIdx.z * K * tp;
+    const int n0 = blockIdx.y * 32, k0 = blockIdx.x * 32, x = threadIdx.x & 31;
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (n0 + y < N && k0 + x < K) t[y][x] = w[(size_t)(n0 + y) * wp + k0 + x];
     __syncthreads();
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
-    float acc = b0[n];
-    for (int j = 0; j < K0; ++j) acc = fmaf(W0[(size_t)n * K0 + j], x[j], acc);
-    const float h = tanhf(acc);
-    const __nv_bfloat16 hh = __float2bfloat16_rn(h);
-    hi[(size_t)row * N + n] = hh;
-    lo[(size_t)row * N + n] = __float2bfloat16_rn(h - __bfloat162float(hh));
-}
-
-// g = s * in (rows x n) written as a bf16 (hi, lo) pair.
-__global__ void k_scale_split(const float* __restrict__ in, float s, int n, __nv_bfloat16* __restrict__ hi,
-                              __nv_bfloat16* __restrict__ lo, const int* __restrict__ nrows) {
-    const int row = blockIdx.y;
-    if (row >= *nrows) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const float g = s * in[(size_t)row * n + i];
-        const __nv_bfloat16 gh = __float2bfloat16_rn(g);
-        hi[(size_t)row * n + i] = gh;
-        lo[(size_t)row * n + i] = __float2bfloat16_rn(g - __bfloat162float(gh));
-    }
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (k0 + y < K && n0 + x < N) o[(size_t)(k0 + y) * tp + n0 + x] = t[x][y];
 }
 
 template <typename T>
@@ -778,249 +774,214 @@ static int dense(const T* A, const T* W, const T* bias, const T* mu, T sigma, T*
 
 }  // namespace adj
 
-struct GradWorkspace {
-    int cap = 0;
-    std::vector<void*> H;      // stored activations per hidden layer (index 1..L-1)
-    void* gA = nullptr;        // ping-pong adjoint buffers (cap x max(hidden, n_out))
-    void* gB = nullptr;
-    void* gtab = nullptr;      // cap x n_z n_k
+// One problem's gradient state.
+struct GradState {
+    const ns_problem* p = nullptr;
+    int* d_nrows = nullptr;
+    int* d_err = nullptr;
+    double* theta_full = nullptr;
     void* table = nullptr;     // cap x n_out (emulator output)
     void* table_fine = nullptr;
+    void* gtab = nullptr;      // cap x n_z n_k
+    void* gcoarse = nullptr;   // cap x n_out, coarse-z emulators
     void* scratch = nullptr;   // cap x adjoint_scratch_elems
     double* gfull = nullptr;   // cap x P
+    // FP64: stored activations per hidden layer and ping-pong adjoints
+    std::vector<double*> H;
+    double* g64[2] = {nullptr, nullptr};
+    // FP32 and BF16: activations and adjoints in px bf16 planes (3: FP32; 2: the
+    // leading 16 bits beside exact bf16 weights), weights in pw planes.  Layer l
+    // (1 .. L-1) maps dims[l] -> dims[l+1].
+    int px = 0, pw = 0;
+    long long rows_pad = 0;
+    std::vector<__nv_bfloat16*> Hp;          // input activations of layer l: px x rows_pad x pitch
+    __nv_bfloat16* Gp[2] = {nullptr, nullptr};
+    float* G1 = nullptr;                     // gradient of layer 1's input pre-activations (rows x dims[1])
+    std::vector<CUtensorMap> tmW, tmWT;      // W_l and its transpose
+    std::vector<PlaneMapX> tmH, tmG;         // layer l's forward and backward operands
     std::vector<void*> owned;
 };
 
 static std::mutex g_grad_mu;
 
-template <typename T>
-static int grad_ws_create(const ns_problem* p, int cap, GradWorkspace* g) {
-    g->cap = cap;
-    auto alloc = [&](size_t bytes, void** out) -> int {
-        if (cudaMalloc(out, bytes) != cudaSuccess) return NS_ENOMEM;
-        g->owned.push_back(*out);
-        return NS_OK;
-    };
-    const int L = p->n_layers;
-    const int n_out = p->dims.back();
-    const int nzk = p->sp.n_z * p->sp.n_k;
-    g->H.assign(L, nullptr);
-    for (int l = 1; l < L; ++l) NS_TRY(alloc(sizeof(T) * (size_t)cap * p->dims[l], &g->H[l]));
-    const size_t wmax = std::max(p->hidden_max, std::max(n_out, nzk));
-    NS_TRY(alloc(sizeof(T) * (size_t)cap * wmax, &g->gA));
-    NS_TRY(alloc(sizeof(T) * (size_t)cap * wmax, &g->gB));
-    NS_TRY(alloc(sizeof(T) * (size_t)cap * nzk, &g->gtab));
-    NS_TRY(alloc(sizeof(T) * (size_t)cap * n_out, &g->table));
-    if (p->n_z_emu != p->sp.n_z) NS_TRY(alloc(sizeof(T) * (size_t)cap * nzk, &g->table_fine));
-    NS_TRY(alloc(sizeof(T) * (size_t)cap * adjoint_scratch_elems(p->sp), &g->scratch));
-    void* gf;
-    NS_TRY(alloc(sizeof(double) * (size_t)cap * p->P, &gf));
-    g->gfull = (double*)gf;
+static int grad_alloc(GradState* g, size_t bytes, void** out) {
+    if (cudaMalloc(out, bytes) != cudaSuccess) return NS_ENOMEM;
+    g->owned.push_back(*out);
     return NS_OK;
 }
 
-// Weights of the gradient path in its arithmetic type (FP64 problems: as
-// stored; FP32 / BF16 problems: FP32 copies made here from the FP64 master).
-struct GradWeights {
-    std::vector<void*> W, b;
-    void* mu = nullptr;
-    std::vector<void*> owned;
-};
-
-template <typename T>
-static int run_grad(const ns_problem* p, GradWorkspace* g, const GradWeights* gw, const double* theta_full,
-                    const int* d_nrows, int B, double* logL, double* grad, cudaStream_t st) {
-    const int L = p->n_layers;
-    const ShearParams& sp = p->sp;
-    const int n_out = p->dims.back();
-    const int nzk = sp.n_z * sp.n_k;
-    // forward emulator with stored activations
-    {
-        dim3 g0((p->dims[1] + 255) / 256, B);
-        adj::k_emu_in_store<T><<<g0, 256, 0, st>>>(theta_full, p->P, p->d_inputs, p->d_in_center, p->d_in_scale,
-                                                   p->dims[0], (const T*)gw->W[0], (const T*)gw->b[0], p->dims[1],
-                                                   (T*)g->H[1], d_nrows);
-        NS_CUDA_TRY(cudaGetLastError());
-        for (int l = 1; l < L; ++l) {
-            const bool last = (l == L - 1);
-            T* out = last ? (T*)g->table : (T*)g->H[l + 1];
-            NS_TRY(adj::dense<T>((const T*)g->H[l], (const T*)gw->W[l], (const T*)gw->b[l], (const T*)gw->mu,
-                                 (T)p->out_sigma, out, d_nrows, B, p->dims[l + 1], p->dims[l], last ? 1 : 0, nullptr,
-                                 st));
-        }
-    }
-    const T* tab = (const T*)g->table;
-    if (p->n_z_emu != sp.n_z) {
-        // forward coarse -> fine interpolation
-        NS_TRY(launch_zinterp_generic(p, g->table, g->table_fine, d_nrows, B, (int)sizeof(T), st));
-        tab = (const T*)g->table_fine;
-    }
-    const T* LT = (sizeof(T) == 8) ? (const T*)(const void*)p->d_LinvT64 : (const T*)(const void*)p->d_LinvT32;
-    NS_TRY(launch_projection_adj<T>(sp, theta_full, tab, LT, p->c0, (T*)g->scratch, (T*)g->gtab, g->gfull, logL,
-                                    d_nrows, B, st));
-    // table adjoint -> emulator output adjoint (transpose of the z interpolation) -> g_pre_L
-    T* gcur = (T*)g->gA;
-    T* gnext = (T*)g->gB;
-    if (p->n_z_emu != sp.n_z) {
-        dim3 gz((p->n_z_emu * sp.n_k + 255) / 256, B);
-        adj::k_zinterp_adj<T><<<gz, 256, 0, st>>>((const T*)g->gtab, sp.n_z, p->d_zi_row, p->d_zi_w, gnext,
-                                                  p->n_z_emu, sp.n_k, d_nrows);
-        dim3 gs((n_out + 255) / 256, B);
-        adj::k_scale<T><<<gs, 256, 0, st>>>(gnext, gcur, (T)p->out_sigma, n_out, d_nrows);
-    } else {
-        dim3 gs((n_out + 255) / 256, B);
-        adj::k_scale<T><<<gs, 256, 0, st>>>((const T*)g->gtab, gcur, (T)p->out_sigma, n_out, d_nrows);
-    }
-    NS_CUDA_TRY(cudaGetLastError());
-    // g_pre_{l} = (g_pre_{l+1} W_l) * (1 - h_l^2), l = L-1 .. 1
-    for (int l = L - 1; l >= 1; --l) {
-        NS_TRY(adj::dense<T>(gcur, (const T*)gw->W[l], nullptr, nullptr, T(0), gnext, d_nrows, B, p->dims[l],
-                             p->dims[l + 1], 2, (const T*)g->H[l], st));
-        std::swap(gcur, gnext);
-    }
-    adj::k_emu_in_back<T><<<B, 256, 0, st>>>(gcur, (const T*)gw->W[0], p->dims[1], p->dims[0], p->d_inputs,
-                                             p->d_in_scale, g->gfull, p->P, d_nrows);
-    adj::k_gather_grad<<<B, 64, 0, st>>>(g->gfull, p->P, p->d_free_of_full, grad, p->d, B);
-    NS_CUDA_TRY(cudaGetLastError());
-    return NS_OK;
-}
-
-// BF16 problems: the emulator forward and backward on the tensor cores
-// (split-BF16 activations and gradients, exact bf16 weights, FP32 accumulate),
-// the projection adjoint in FP32.  Layer l (1 .. L-1) maps dims[l] -> dims[l+1].
-struct SplitGrad {
-    int rows_pad = 0;
-    std::vector<__nv_bfloat16*> Hhi, Hlo;   // input activations of layer l (rows_pad x dims[l])
-    __nv_bfloat16* Ghi[2] = {nullptr, nullptr};
-    __nv_bfloat16* Glo[2] = {nullptr, nullptr};  // backward ping-pong (rows_pad x wmax)
-    float* G1 = nullptr;                     // gradient of layer 1's pre-activations (rows_pad x dims[1])
-    std::vector<__nv_bfloat16*> WT;          // W_l^T (dims[l] x dims[l+1])
-    std::vector<CUtensorMap> tmHhi, tmHlo, tmW, tmGhi, tmGlo, tmWT;
-    std::vector<void*> owned;
-};
-
-constexpr int kSplitHiddenTile = 128;        // forward hidden layers and every backward layer
-constexpr int kSplitOutTile = 256;           // forward output layer
-
-static bool split_supported(const ns_problem* p) {
-    if (p->kind != NS_KIND_SHEAR || (p->precision != NS_PREC_BF16 && p->precision != NS_PREC_BF16_F64CHI2)) return false;
-    if (p->act != NS_ACT_TANH || p->d_out_sig || p->n_layers < 2 || p->dims[0] > 32) return false;
-    for (int l = 1; l <= p->n_layers; ++l)
-        if (p->dims[l] % 8) return false;
-    return true;
-}
-
-static int split_grad_create(const ns_problem* p, int cap, SplitGrad* g) {
-    const int L = p->n_layers;
-    const int rows_pad = ((cap + 127) / 128) * 128;
-    g->rows_pad = rows_pad;
-    auto alloc = [&](size_t bytes, void** out) -> int {
-        if (cudaMalloc(out, bytes) != cudaSuccess) return NS_ENOMEM;
-        g->owned.push_back(*out);
-        return cudaMemset(*out, 0, bytes) == cudaSuccess ? NS_OK : NS_ECUDA;
-    };
+static int grad_state_create(const ns_problem* p, GradState* g) {
+    const int L = p->n_layers, cap = p->max_batch, n_out = p->dims.back(), nzk = p->sp.n_z * p->sp.n_k;
+    const bool f64 = p->precision == NS_PREC_FP64, coarse = p->n_z_emu != p->sp.n_z;
+    const size_t T = f64 ? 8 : 4;
     void* v;
-    g->Hhi.assign(L, nullptr);
-    g->Hlo.assign(L, nullptr);
-    for (int l = 1; l < L; ++l) {
-        NS_TRY(alloc(sizeof(__nv_bfloat16) * (size_t)rows_pad * p->dims[l], &v)); g->Hhi[l] = (__nv_bfloat16*)v;
-        NS_TRY(alloc(sizeof(__nv_bfloat16) * (size_t)rows_pad * p->dims[l], &v)); g->Hlo[l] = (__nv_bfloat16*)v;
+    g->p = p;
+    NS_TRY(grad_alloc(g, sizeof(int), (void**)&g->d_nrows));
+    NS_TRY(grad_alloc(g, sizeof(int), (void**)&g->d_err));
+    NS_CUDA_TRY(cudaMemset(g->d_err, 0, sizeof(int)));
+    NS_TRY(grad_alloc(g, sizeof(double) * (size_t)cap * p->P, (void**)&g->theta_full));
+    NS_TRY(grad_alloc(g, sizeof(double) * (size_t)cap * p->P, (void**)&g->gfull));
+    NS_TRY(grad_alloc(g, T * (size_t)cap * n_out, &g->table));
+    NS_TRY(grad_alloc(g, T * (size_t)cap * nzk, &g->gtab));
+    if (coarse) {
+        NS_TRY(grad_alloc(g, T * (size_t)cap * nzk, &g->table_fine));
+        NS_TRY(grad_alloc(g, T * (size_t)cap * n_out, &g->gcoarse));
     }
+    NS_TRY(grad_alloc(g, T * (size_t)cap * adjoint_scratch_elems(p->sp), &g->scratch));
     int wmax = 0;
     for (int l = 1; l <= L; ++l) wmax = std::max(wmax, p->dims[l]);
+    if (f64) {
+        g->H.assign(L, nullptr);
+        for (int l = 1; l < L; ++l) NS_TRY(grad_alloc(g, 8 * (size_t)cap * p->dims[l], (void**)&g->H[l]));
+        for (int i = 0; i < 2; ++i) NS_TRY(grad_alloc(g, 8 * (size_t)cap * wmax, (void**)&g->g64[i]));
+        return NS_OK;
+    }
+    const bool f32 = p->precision == NS_PREC_FP32;
+    g->px = f32 ? 3 : 2;
+    g->pw = f32 ? 3 : 1;
+    g->rows_pad = ((cap + 127) / 128) * 128;
+    g->Hp.assign(L, nullptr);
+    g->tmH.resize(L); g->tmG.resize(L); g->tmW.resize(L); g->tmWT.resize(L);
     for (int i = 0; i < 2; ++i) {
-        NS_TRY(alloc(sizeof(__nv_bfloat16) * (size_t)rows_pad * wmax, &v)); g->Ghi[i] = (__nv_bfloat16*)v;
-        NS_TRY(alloc(sizeof(__nv_bfloat16) * (size_t)rows_pad * wmax, &v)); g->Glo[i] = (__nv_bfloat16*)v;
+        // the first holds the widest operand (the output layer's), the second hidden layers only
+        const size_t n = (size_t)g->px * g->rows_pad * plane_pitch(i == 0 ? wmax : p->hidden_max);
+        NS_TRY(grad_alloc(g, 2 * n, &v));
+        g->Gp[i] = (__nv_bfloat16*)v;
+        NS_CUDA_TRY(cudaMemset(v, 0, 2 * n));
     }
-    NS_TRY(alloc(sizeof(float) * (size_t)rows_pad * p->dims[1], &v)); g->G1 = (float*)v;
-    // W_l^T in bf16 (the problem's tensor-core weights are bf16 already)
-    g->WT.assign(L, nullptr);
+    NS_TRY(grad_alloc(g, 4 * (size_t)g->rows_pad * p->dims[1], (void**)&g->G1));
     for (int l = 1; l < L; ++l) {
-        const int No = p->dims[l + 1], Ki = p->dims[l];
-        std::vector<uint16_t> w((size_t)No * Ki), wt((size_t)No * Ki);
-        NS_CUDA_TRY(cudaMemcpy(w.data(), p->d_W[l], w.size() * 2, cudaMemcpyDeviceToHost));
-        for (int n = 0; n < No; ++n)
-            for (int k = 0; k < Ki; ++k) wt[(size_t)k * No + n] = w[(size_t)n * Ki + k];
-        if (cudaMalloc(&v, wt.size() * 2) != cudaSuccess) return NS_ENOMEM;
-        g->owned.push_back(v);
-        NS_CUDA_TRY(cudaMemcpy(v, wt.data(), wt.size() * 2, cudaMemcpyHostToDevice));
-        g->WT[l] = (__nv_bfloat16*)v;
+        const int K = p->dims[l], N = p->dims[l + 1], kp = plane_pitch(K), np = plane_pitch(N);
+        const long long hs = g->rows_pad * kp;
+        NS_TRY(grad_alloc(g, 2 * (size_t)g->px * hs, &v));
+        NS_CUDA_TRY(cudaMemset(v, 0, 2 * (size_t)g->px * hs));
+        g->Hp[l] = (__nv_bfloat16*)v;
+        NS_TRY(make_plane_maps_x(&g->tmH[l], v, (int)g->rows_pad, K, hs, g->px));
+        // backward step l reads G_{l+1} from buffer (L - l - 1) % 2
+        NS_TRY(make_plane_maps_x(&g->tmG[l], g->Gp[(L - l - 1) & 1], (int)g->rows_pad, N, g->rows_pad * np, g->px));
+        const __nv_bfloat16* W = f32 ? p->d_Wp[l] : (const __nv_bfloat16*)p->d_W[l];
+        NS_TRY(make_tensor_map_planes(&g->tmW[l], W, N, K, (long long)N * kp, g->pw, 128));
+        NS_TRY(grad_alloc(g, 2 * (size_t)g->pw * K * np, &v));
+        adj::k_transpose_planes<<<dim3((K + 31) / 32, (N + 31) / 32, g->pw), 256>>>(W, N, K, kp, (__nv_bfloat16*)v, np);
+        NS_CUDA_TRY(cudaGetLastError());
+        NS_TRY(make_tensor_map_planes(&g->tmWT[l], v, K, N, (long long)K * np, g->pw, 128));
     }
-    g->tmHhi.resize(L); g->tmHlo.resize(L); g->tmW.resize(L); g->tmGhi.resize(L); g->tmGlo.resize(L); g->tmWT.resize(L);
-    for (int l = 1; l < L; ++l) {
-        const bool last = (l == L - 1);
-        NS_TRY(make_tensor_map_bf16(&g->tmHhi[l], g->Hhi[l], rows_pad, p->dims[l], 128));
-        NS_TRY(make_tensor_map_bf16(&g->tmHlo[l], g->Hlo[l], rows_pad, p->dims[l], 128));
-        NS_TRY(make_tensor_map_bf16(&g->tmW[l], p->d_W[l], p->dims[l + 1], p->dims[l],
-                                    last ? kSplitOutTile : kSplitHiddenTile));
-        // backward step l reads G_{l+1} (K = dims[l+1]) from buffer (L - l - 1) % 2
-        const int b = (L - l - 1) % 2;
-        NS_TRY(make_tensor_map_bf16(&g->tmGhi[l], g->Ghi[b], rows_pad, p->dims[l + 1], 128));
-        NS_TRY(make_tensor_map_bf16(&g->tmGlo[l], g->Glo[b], rows_pad, p->dims[l + 1], 128));
-        NS_TRY(make_tensor_map_bf16(&g->tmWT[l], g->WT[l], p->dims[l], p->dims[l + 1], kSplitHiddenTile));
-    }
+    NS_CUDA_TRY(cudaStreamSynchronize(nullptr));   // calls may come on any stream
     return NS_OK;
 }
 
-static int run_grad_split(const ns_problem* p, GradWorkspace* gw_, SplitGrad* g, const double* theta_full,
-                          const int* d_nrows, int B, double* logL, double* grad, int* d_err, cudaStream_t st) {
-    const int L = p->n_layers;
+template <typename T>
+static int launch_finish_grad(const ns_problem* p, GradState* g, const T* gpre, int B, double* grad, cudaStream_t st) {
+    auto kern = p->dims[0] <= 8 ? adj::k_finish_grad<T, 8> : adj::k_finish_grad<T, 32>;
+    NS_CUDA_TRY(launch_pdl(kern, dim3(B), dim3(256), 0, st, gpre, (const T*)p->d_W[0], p->dims[1], p->dims[0],
+                           (const int*)p->d_inputs, (const double*)p->d_in_scale, (const double*)g->gfull, p->P,
+                           (const int*)p->d_free_of_full, grad, p->d, (const int*)g->d_nrows));
+    return NS_OK;
+}
+
+// FP64 problems: the emulator forward and backward on CUDA cores.
+static int run_grad_f64(const ns_problem* p, GradState* g, int B, double* logL, double* grad, cudaStream_t st) {
+    const int L = p->n_layers, n_out = p->dims.back();
     const ShearParams& sp = p->sp;
-    const int n_out = p->dims.back();
-    // forward: input layer, hidden layers (split tanh), output layer (FP32 table)
-    {
-        dim3 g0((p->dims[1] + 255) / 256, B);
-        adj::k_emu_in_split<<<g0, 256, 0, st>>>(theta_full, p->P, p->d_inputs, p->d_in_center, p->d_in_inv_scale,
-                                                p->dims[0], (const float*)p->d_W[0], (const float*)p->d_b[0],
-                                                p->dims[1], g->Hhi[1], g->Hlo[1], d_nrows);
-        NS_CUDA_TRY(cudaGetLastError());
-        for (int l = 1; l < L; ++l) {
-            const bool last = (l == L - 1);
-            if (last)
-                NS_TRY(launch_gemm_split(&g->tmHhi[l], &g->tmHlo[l], &g->tmW[l], kSplitOutTile,
-                                         (const float*)p->d_b[l], (const float*)p->d_out_mu, (float)p->out_sigma,
-                                         gw_->table, nullptr, nullptr, nullptr, d_nrows, B, n_out, p->dims[l], SPL_OUT,
-                                         d_err, st));
-            else
-                NS_TRY(launch_gemm_split(&g->tmHhi[l], &g->tmHlo[l], &g->tmW[l], kSplitHiddenTile,
-                                         (const float*)p->d_b[l], nullptr, 0.f, g->Hhi[l + 1], g->Hlo[l + 1], nullptr,
-                                         nullptr, d_nrows, B, p->dims[l + 1], p->dims[l], SPL_TANH, d_err, st));
+    const dim3 g0((p->dims[1] + 255) / 256, B);
+    adj::k_emu_in_store<double><<<g0, 256, 0, st>>>(g->theta_full, p->P, p->d_inputs, p->d_in_center, p->d_in_scale,
+                                                    p->dims[0], (const double*)p->d_W[0], (const double*)p->d_b[0],
+                                                    p->dims[1], g->H[1], g->d_nrows);
+    NS_CUDA_TRY(cudaGetLastError());
+    for (int l = 1; l < L; ++l) {
+        const bool last = (l == L - 1);
+        NS_TRY(adj::dense<double>(g->H[l], (const double*)p->d_W[l], (const double*)p->d_b[l],
+                                  (const double*)p->d_out_mu, p->out_sigma, last ? (double*)g->table : g->H[l + 1],
+                                  g->d_nrows, B, p->dims[l + 1], p->dims[l], last ? 1 : 0, nullptr, st));
+    }
+    const double* tab = (const double*)g->table;
+    const bool coarse = p->n_z_emu != sp.n_z;
+    if (coarse) {
+        NS_TRY(launch_zinterp_generic(p, g->table, g->table_fine, g->d_nrows, B, 8, st));
+        tab = (const double*)g->table_fine;
+    }
+    NS_TRY(launch_projection_adj<double>(sp, g->theta_full, tab, p->d_LinvT64, p->c0, (double*)g->scratch,
+                                         (double*)g->gtab, g->gfull, logL, g->d_nrows, B, st));
+    // table adjoint -> emulator output adjoint (transpose of the z interpolation) -> g_pre_L
+    const double* gt = (const double*)g->gtab;
+    if (coarse) {
+        const dim3 gz((n_out + 255) / 256, B);
+        adj::k_zinterp_adj<double><<<gz, 256, 0, st>>>(gt, sp.n_z, p->d_zi_row, p->d_zi_w, (double*)g->gcoarse,
+                                                       p->n_z_emu, sp.n_k, g->d_nrows);
+        gt = (const double*)g->gcoarse;
+    }
+    const dim3 gs((n_out + 255) / 256, B);
+    adj::k_scale<double><<<gs, 256, 0, st>>>(gt, g->g64[0], p->out_sigma, n_out, g->d_nrows);
+    NS_CUDA_TRY(cudaGetLastError());
+    // g_pre_{l} = (g_pre_{l+1} W_l) * (1 - h_l^2), l = L-1 .. 1
+    int cur = 0;
+    for (int l = L - 1; l >= 1; --l) {
+        NS_TRY(adj::dense<double>(g->g64[cur], (const double*)p->d_W[l], nullptr, nullptr, 0.0, g->g64[cur ^ 1],
+                                  g->d_nrows, B, p->dims[l], p->dims[l + 1], 2, g->H[l], st));
+        cur ^= 1;
+    }
+    return launch_finish_grad<double>(p, g, g->g64[cur], B, grad, st);
+}
+
+// FP32 and BF16 problems: the emulator forward and backward as plane GEMMs
+// (gemm_planes.cu), the projection adjoint in FP32.
+static int run_grad_planes(const ns_problem* p, GradState* g, int B, double* logL, double* grad, cudaStream_t st) {
+    const int L = p->n_layers, n_out = p->dims.back(), px = g->px, pw = g->pw;
+    const ShearParams& sp = p->sp;
+    auto planes_out = [&](PlaneEpi& e, __nv_bfloat16* buf, int width) {
+        e.planes = buf;
+        e.pitch = plane_pitch(width);
+        e.plane_stride = g->rows_pad * e.pitch;
+    };
+    NS_TRY(launch_emu_input_planes(p, g->theta_full, g->d_nrows, B, px, g->Hp[1],
+                                   g->rows_pad * plane_pitch(p->dims[1]), st));
+    for (int l = 1; l < L; ++l) {
+        const bool last = (l == L - 1);
+        PlaneEpi e;
+        e.mode = last ? PLN_OUT : PLN_TANH;
+        e.bias = (const float*)p->d_b[l];
+        if (last) {
+            e.mu = (const float*)p->d_out_mu;
+            e.sigma = (float)p->out_sigma;
+            e.out = (float*)g->table;
+        } else {
+            planes_out(e, g->Hp[l + 1], p->dims[l + 1]);
         }
+        NS_TRY(launch_gemm_planes(px, pw, &g->tmW[l], &g->tmH[l], e, g->d_nrows, B, p->dims[l + 1], p->dims[l],
+                                  g->d_err, st));
     }
-    const float* tab = (const float*)gw_->table;
-    if (p->n_z_emu != sp.n_z) {
-        NS_TRY(launch_zinterp_generic(p, gw_->table, gw_->table_fine, d_nrows, B, (int)sizeof(float), st));
-        tab = (const float*)gw_->table_fine;
+    const float* tab = (const float*)g->table;
+    const bool coarse = p->n_z_emu != sp.n_z;
+    if (coarse) {
+        NS_TRY(launch_zinterp_generic(p, g->table, g->table_fine, g->d_nrows, B, 4, st));
+        tab = (const float*)g->table_fine;
     }
-    NS_TRY(launch_projection_adj<float>(sp, theta_full, tab, p->d_LinvT32, p->c0, (float*)gw_->scratch,
-                                        (float*)gw_->gtab, gw_->gfull, logL, d_nrows, B, st));
-    // d log L / d (output pre-scaling) = sigma * d log L / d table, split
-    const float* gtab = (const float*)gw_->gtab;
-    if (p->n_z_emu != sp.n_z) {
-        dim3 gz((p->n_z_emu * sp.n_k + 255) / 256, B);
-        adj::k_zinterp_adj<float><<<gz, 256, 0, st>>>((const float*)gw_->gtab, sp.n_z, p->d_zi_row, p->d_zi_w,
-                                                      (float*)gw_->gA, p->n_z_emu, sp.n_k, d_nrows);
-        gtab = (const float*)gw_->gA;
-    }
-    {
-        dim3 gs((n_out + 255) / 256, B);
-        adj::k_scale_split<<<gs, 256, 0, st>>>(gtab, (float)p->out_sigma, n_out, g->Ghi[0], g->Glo[0], d_nrows);
+    NS_TRY(launch_projection_adj<float>(sp, g->theta_full, tab, p->d_LinvT32, p->c0, (float*)g->scratch,
+                                        (float*)g->gtab, g->gfull, logL, g->d_nrows, B, st));
+    // d log L / d (output pre-scaling) = sigma * d log L / d table
+    const float* gt = (const float*)g->gtab;
+    if (coarse) {
+        const dim3 gz((n_out + 255) / 256, B);
+        adj::k_zinterp_adj<float><<<gz, 256, 0, st>>>(gt, sp.n_z, p->d_zi_row, p->d_zi_w, (float*)g->gcoarse,
+                                                      p->n_z_emu, sp.n_k, g->d_nrows);
         NS_CUDA_TRY(cudaGetLastError());
+        gt = (const float*)g->gcoarse;
     }
+    NS_TRY(launch_split_planes(px, gt, (float)p->out_sigma, B, n_out, g->Gp[0], g->rows_pad * plane_pitch(n_out),
+                               plane_pitch(n_out), g->d_nrows, st));
     // backward: G_l = (G_{l+1} W_l) (1 - h_l^2), l = L-1 .. 1 (the last in FP32)
     for (int l = L - 1; l >= 1; --l) {
-        const int out = (L - l) % 2;
-        const bool first = (l == 1);
-        NS_TRY(launch_gemm_split(&g->tmGhi[l], &g->tmGlo[l], &g->tmWT[l], kSplitHiddenTile, nullptr, nullptr, 0.f,
-                                 first ? (void*)g->G1 : (void*)g->Ghi[out], first ? nullptr : g->Glo[out], g->Hhi[l],
-                                 g->Hlo[l], d_nrows, B, p->dims[l], p->dims[l + 1],
-                                 first ? SPL_DTANH32 : SPL_DTANH, d_err, st));
+        PlaneEpi e;
+        e.mode = l == 1 ? PLN_DTANH32 : PLN_DTANH;
+        e.aux = g->Hp[l];
+        e.aux_pitch = plane_pitch(p->dims[l]);
+        e.aux_stride = g->rows_pad * e.aux_pitch;
+        if (l == 1) e.out = g->G1;
+        else planes_out(e, g->Gp[(L - l) & 1], p->dims[l]);
+        NS_TRY(launch_gemm_planes(px, pw, &g->tmWT[l], &g->tmG[l], e, g->d_nrows, B, p->dims[l], p->dims[l + 1],
+                                  g->d_err, st));
     }
-    adj::k_emu_in_back<float><<<B, 256, 0, st>>>(g->G1, (const float*)p->d_W[0], p->dims[1], p->dims[0], p->d_inputs,
-                                                 p->d_in_scale, gw_->gfull, p->P, d_nrows);
-    adj::k_gather_grad<<<B, 64, 0, st>>>(gw_->gfull, p->P, p->d_free_of_full, grad, p->d, B);
-    NS_CUDA_TRY(cudaGetLastError());
-    return NS_OK;
+    return launch_finish_grad<float>(p, g, g->G1, B, grad, st);
 }
 
 }  // namespace gpuns
@@ -1028,55 +989,7 @@ static int run_grad_split(const ns_problem* p, GradWorkspace* gw_, SplitGrad* g,
 using namespace gpuns;
 
 namespace {
-struct GradState {
-    const ns_problem* p = nullptr;
-    GradWorkspace ws;
-    GradWeights w;
-    SplitGrad split;                 // BF16 problems on the tensor cores
-    bool use_split = false;
-    int* d_nrows = nullptr;
-    int* d_err = nullptr;
-    double* theta_full = nullptr;
-};
 std::vector<GradState*> g_grad_states;
-
-template <typename T>
-int make_grad_weights(const ns_problem* p, GradWeights* gw) {
-    // FP64 problems keep FP64 master weights on the device already
-    const int L = p->n_layers;
-    gw->W.assign(L, nullptr);
-    gw->b.assign(L, nullptr);
-    if (p->precision == NS_PREC_FP64) {
-        for (int l = 0; l < L; ++l) { gw->W[l] = p->d_W[l]; gw->b[l] = p->d_b[l]; }
-        gw->mu = p->d_out_mu;
-        return NS_OK;
-    }
-    if (p->precision == NS_PREC_FP32) {
-        for (int l = 0; l < L; ++l) { gw->W[l] = p->d_W[l]; gw->b[l] = p->d_b[l]; }
-        gw->mu = p->d_out_mu;
-        return NS_OK;
-    }
-    // BF16 problems: the gradient path runs in FP32 from bf16-valued weights
-    for (int l = 0; l < L; ++l) {
-        const size_t nw = (size_t)p->dims[l + 1] * p->dims[l];
-        if (l == 0) { gw->W[l] = p->d_W[l]; }
-        else {
-            std::vector<uint16_t> hb(nw);
-            NS_CUDA_TRY(cudaMemcpy(hb.data(), p->d_W[l], nw * 2, cudaMemcpyDeviceToHost));
-            std::vector<float> hf(nw);
-            for (size_t i = 0; i < nw; ++i) { uint32_t u = (uint32_t)hb[i] << 16; std::memcpy(&hf[i], &u, 4); }
-            void* d;
-            if (cudaMalloc(&d, nw * 4) != cudaSuccess) return NS_ENOMEM;
-            gw->owned.push_back(d);
-            NS_CUDA_TRY(cudaMemcpy(d, hf.data(), nw * 4, cudaMemcpyHostToDevice));
-            gw->W[l] = d;
-        }
-        gw->b[l] = p->d_b[l];
-    }
-    gw->mu = p->d_out_mu;
-    (void)sizeof(T);
-    return NS_OK;
-}
 }  // namespace
 
 // Isotropic Gaussian test likelihood and its gradient at free parameters
@@ -1112,27 +1025,9 @@ extern "C" int loglike_grad_batch(const ns_problem* p, const double* theta_dev, 
         for (GradState* s : g_grad_states) if (s->p == p) gs = s;
         if (!gs) {
             gs = new GradState();
-            gs->p = p;
-            const bool f64 = p->precision == NS_PREC_FP64;
-            gs->use_split = split_supported(p);
-            int rc = f64 ? grad_ws_create<double>(p, p->max_batch, &gs->ws) : grad_ws_create<float>(p, p->max_batch, &gs->ws);
-            if (rc == NS_OK && gs->use_split) rc = split_grad_create(p, p->max_batch, &gs->split);
-            else if (rc == NS_OK) rc = f64 ? make_grad_weights<double>(p, &gs->w) : make_grad_weights<float>(p, &gs->w);
-            void* v = nullptr;
-            if (rc == NS_OK && cudaMalloc(&v, sizeof(int)) != cudaSuccess) rc = NS_ENOMEM;
-            gs->d_nrows = (int*)v;
-            v = nullptr;
-            if (rc == NS_OK && (cudaMalloc(&v, sizeof(int)) != cudaSuccess || cudaMemset(v, 0, sizeof(int)) != cudaSuccess))
-                rc = NS_ENOMEM;
-            gs->d_err = (int*)v;
-            v = nullptr;
-            if (rc == NS_OK && cudaMalloc(&v, sizeof(double) * (size_t)p->max_batch * p->P) != cudaSuccess) rc = NS_ENOMEM;
-            gs->theta_full = (double*)v;
+            const int rc = grad_state_create(p, gs);
             if (rc != NS_OK) {
-                for (void* q : gs->ws.owned) cudaFree(q);
-                for (void* q : gs->w.owned) cudaFree(q);
-                for (void* q : gs->split.owned) cudaFree(q);
-                cudaFree(gs->d_nrows); cudaFree(gs->d_err); cudaFree(gs->theta_full);
+                for (void* q : gs->owned) cudaFree(q);
                 delete gs;
                 return rc;
             }
@@ -1142,11 +1037,8 @@ extern "C" int loglike_grad_batch(const ns_problem* p, const double* theta_dev, 
     NS_TRY(launch_free_to_full_ext(p, theta_dev, B, gs->theta_full, st));
     k_set_int<<<1, 1, 0, st>>>(gs->d_nrows, B);
     NS_CUDA_TRY(cudaGetLastError());
-    if (p->precision == NS_PREC_FP64)
-        return run_grad<double>(p, &gs->ws, &gs->w, gs->theta_full, gs->d_nrows, B, logL_dev, grad_dev, st);
-    if (gs->use_split)
-        return run_grad_split(p, &gs->ws, &gs->split, gs->theta_full, gs->d_nrows, B, logL_dev, grad_dev, gs->d_err, st);
-    return run_grad<float>(p, &gs->ws, &gs->w, gs->theta_full, gs->d_nrows, B, logL_dev, grad_dev, st);
+    if (p->precision == NS_PREC_FP64) return run_grad_f64(p, gs, B, logL_dev, grad_dev, st);
+    return run_grad_planes(p, gs, B, logL_dev, grad_dev, st);
 }
 
 // Called by ns_problem_free: release the gradient state of a problem.
@@ -1155,12 +1047,7 @@ void gpuns_release_grad_state(const ns_problem* p) {
     for (size_t i = 0; i < g_grad_states.size(); ++i) {
         GradState* s = g_grad_states[i];
         if (s->p != p) continue;
-        for (void* q : s->ws.owned) cudaFree(q);
-        for (void* q : s->w.owned) cudaFree(q);
-        for (void* q : s->split.owned) cudaFree(q);
-        cudaFree(s->d_nrows);
-        cudaFree(s->d_err);
-        cudaFree(s->theta_full);
+        for (void* q : s->owned) cudaFree(q);
         delete s;
         g_grad_states.erase(g_grad_states.begin() + i);
         return;

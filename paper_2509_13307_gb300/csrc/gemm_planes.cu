@@ -17,7 +17,8 @@
 // second TMEM buffer.
 //
 // Tiles.  The MMA's M is 128 features (rows of W), its N is BR rows of X, so
-// few rows waste no tensor work; BR = 32, 64 or 128.  When the (feature, row)
+// few rows waste no tensor work; BR = 32, 64, 128, or 256 where two ring slots
+// of that size fit (two planes of X beside one of W: 4096-row gradients).  When the (feature, row)
 // tiles are fewer than the SMs the k-blocks are split over a cluster of S
 // CTAs; each leaves its FP32 partial tile in shared memory and rank q adds
 // the S partials of its share of the rows in rank order (deterministic) and
@@ -33,9 +34,13 @@
 // the 39-d emulator, 42 us at the measured peak) for many rows, the copies and
 // the fixed cost of a launch for few.  Against the FP32 FMA GEMM it replaced
 // (128 x 128 tiles, 32 CTAs per hidden layer at 500 rows): log-likelihoods of
-// 500 rows of the 39-d problem 2082 -> 275 us, of 250 rows of the dense CMB
-// problem 814 -> 73 us, of 333 rows of its TT form with BF16 hidden layers
-// 200 -> 52 us.  Error of the 39-d emulator's table against FP64 over 500
+// 500 rows of the 39-d problem 2082 -> 247 us, of 250 rows of the dense CMB
+// problem 814 -> 65 us, of 333 rows of its TT form with BF16 hidden layers
+// 200 -> 54 us; gradients of 129 rows in FP32 4128 -> 781 us (with the
+// projection's 540 us unchanged), and of 64 rows in BF16 775 -> 608 us against
+// one-CTA tiles that walked all of K = 10000.  Sending the tile through shared
+// memory to one rolled epilogue loop, instead of an epilogue unrolled over the
+// registers, took the 500-row call from 275 to 247 us.  Error of the 39-d emulator's table against FP64 over 500
 // rows: rms 8.90e-8 dex, largest 4.8e-7 (FMA chain: 9.01e-8 and 5.2e-7).
 #include <algorithm>
 
@@ -57,6 +62,9 @@ struct CfgP {
     static_assert(STAGES >= 2, "two slots");
     static_assert(STAGES * STAGE_BYTES >= 128 * BR * 4, "the partial tile reuses the ring");
 };
+
+// 256-row tiles where two slots of them fit
+template <int PX, int PW> constexpr bool kPlaneRows256 = 2 * 128 * (128 * PW + 256 * PX) <= 192 * 1024;
 
 constexpr int kPlaneEpiWarps = 8, kPlaneThreads = 32 * (kPlaneEpiWarps + 2);
 
@@ -219,23 +227,27 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
 #pragma unroll
         for (int j = 0; j < HC; ++j) acc[j] = NAN;
     }
-    if (S == 1) {
-        if (warp < kPlaneEpiWarps) {
+    // the (partial) tile goes through shared memory, so that one rolled loop
+    // applies the epilogue: rows of all 128 features, 256 threads to two rows
+    float* red = reinterpret_cast<float*>(gbase);
+    if (warp < kPlaneEpiWarps) {
 #pragma unroll
-            for (int j = 0; j < HC; ++j) finish((warp >> 2) * HC + j, acc[j]);
+        for (int j = 0; j < HC; ++j) red[((warp >> 2) * HC + j) * 128 + (tid & 127)] = acc[j];
+    }
+    if (S == 1) {
+        __syncthreads();
+        if (warp < kPlaneEpiWarps) {
+            const int hi = min(BR, M - r0);
+#pragma unroll 2
+            for (int rl = tid >> 7; rl < hi; rl += 2) finish(rl, red[rl * 128 + (tid & 127)]);
         }
     } else {
-        float* red = reinterpret_cast<float*>(gbase);
-        if (warp < kPlaneEpiWarps) {
-#pragma unroll
-            for (int j = 0; j < HC; ++j) red[((warp >> 2) * HC + j) * 128 + (tid & 127)] = acc[j];
-        }
         cluster_sync_all();
         if (warp < kPlaneEpiWarps) {
-            const int lo = BR * rank / S, hi = BR * (rank + 1) / S;
+            const int hi = min(BR * (rank + 1) / S, M - r0);
             const uint32_t off = base + 4u * (uint32_t)(tid & 127);
-            for (int rl = lo + (tid >> 7); rl < hi; rl += 2) {
-                if (r0 + rl >= M) break;
+#pragma unroll 1
+            for (int rl = BR * rank / S + (tid >> 7); rl < hi; rl += 2) {
                 float v = 0.f;
                 for (int q = 0; q < S; ++q) v += ld_cluster_f32(mapa_u32(off + 512u * (uint32_t)rl, (uint32_t)q));
                 finish(rl, v);
@@ -286,21 +298,43 @@ static int launch_planes_p(const CUtensorMap* tmW, const PlaneMapX* tmX, const P
         case 32: return launch_planes_t<PX, PW, 32>(tmW, &tmX->m[0], e, nrows, grid_rows, N, K, t.split, err, st);
         case 64: return launch_planes_t<PX, PW, 64>(tmW, &tmX->m[1], e, nrows, grid_rows, N, K, t.split, err, st);
         case 128: return launch_planes_t<PX, PW, 128>(tmW, &tmX->m[2], e, nrows, grid_rows, N, K, t.split, err, st);
+        case 256:
+            if constexpr (kPlaneRows256<PX, PW>)
+                return launch_planes_t<PX, PW, 256>(tmW, &tmX->m[3], e, nrows, grid_rows, N, K, t.split, err, st);
+            return NS_EINVAL;
         default: return NS_EINVAL;
     }
 }
 
-// planes[p][r][c] = plane p of s * in[r][c] (row pitch `pitch`)
-template <int P>
+// planes[p][r][c] = plane p of s * in[r][c] (row pitch `pitch`).  A thread takes
+// four columns when rows and pitch keep 16-byte loads and 8-byte stores aligned.
+template <int P, int V>
 __global__ void __launch_bounds__(256) k_split_planes(const float* __restrict__ in, float s, int rows, int cols,
                                                       __nv_bfloat16* __restrict__ planes, long long stride, int pitch,
                                                       const int* __restrict__ nrows) {
     pdl_begin();
     const int n = nrows ? min(rows, *nrows) : rows;
-    const int c = blockIdx.x * 256 + threadIdx.x;
+    const int c = (blockIdx.x * 256 + threadIdx.x) * V;
     if (c >= cols) return;
-    for (int r = blockIdx.y; r < n; r += gridDim.y)
-        plane_store<P>(s * in[(size_t)r * cols + c], planes + (size_t)r * pitch + c, stride);
+    for (int r = blockIdx.y; r < n; r += gridDim.y) {
+        __align__(16) float v[V];
+        if constexpr (V == 4) *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(in + (size_t)r * cols + c);
+        else v[0] = in[(size_t)r * cols + c];
+#pragma unroll
+        for (int j = 0; j < V; ++j) v[j] *= s;
+        __nv_bfloat16* o = planes + (size_t)r * pitch + c;
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+            __align__(8) __nv_bfloat16 q[V];
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                q[j] = __float2bfloat16_rn(v[j]);
+                v[j] -= __bfloat162float(q[j]);
+            }
+            if constexpr (V == 4) *reinterpret_cast<uint2*>(o + p * stride) = *reinterpret_cast<const uint2*>(q);
+            else o[p * stride] = q[0];
+        }
+    }
 }
 
 }  // namespace tc
@@ -323,9 +357,9 @@ PlaneTiling plane_tiling(int rows, int N, int K, int px, int pw) {
     const int nk = (K + tc::BK - 1) / tc::BK, mt = (N + 127) / 128;
     PlaneTiling best{128, 1};
     double best_t = 1e300;
-    for (int br : {32, 64, 128})
+    for (int br : {32, 64, 128, 256})
         for (int s : {1, 2, 4, 8}) {
-            if (s > nk) continue;
+            if (s > nk || (br == 256 && 256 * (128 * pw + 256 * px) > 192 * 1024)) continue;
             const double mma = prod * 4.0 * std::max(br / 2.0, (128 + br) / 4.0);
             const double load = std::max(450.0, 128.0 * (128 * pw + br * px) / 54.0);
             const int sms = s == 8 ? 96 : s == 4 ? 128 : 152;
@@ -343,6 +377,7 @@ int launch_gemm_planes(int px, int pw, const CUtensorMap* tmW, const PlaneMapX* 
     if (grid_rows <= 0) return NS_OK;
     const PlaneTiling t = plane_tiling(grid_rows, N, K, px, pw);
     if (px == 3 && pw == 3) return tc::launch_planes_p<3, 3>(tmW, tmX, e, nrows, grid_rows, N, K, t, err, st);
+    if (px == 2 && pw == 1) return tc::launch_planes_p<2, 1>(tmW, tmX, e, nrows, grid_rows, N, K, t, err, st);
     if (px == 1 && pw == 3) return tc::launch_planes_p<1, 3>(tmW, tmX, e, nrows, grid_rows, N, K, t, err, st);
     return NS_EINVAL;
 }
@@ -350,8 +385,13 @@ int launch_gemm_planes(int px, int pw, const CUtensorMap* tmW, const PlaneMapX* 
 int launch_split_planes(int planes, const float* in, float s, int rows, int cols, __nv_bfloat16* out, long long stride,
                         int pitch, const int* nrows, cudaStream_t st) {
     if (rows <= 0 || cols <= 0) return NS_OK;
-    const dim3 g((cols + 255) / 256, std::min(rows, 16384));
-    auto kern = planes == 3 ? tc::k_split_planes<3> : planes == 2 ? tc::k_split_planes<2> : tc::k_split_planes<1>;
+    const bool vec = cols % 4 == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0 &&
+                     pitch % 4 == 0 && stride % 4 == 0;
+    const int per = vec ? 1024 : 256;
+    const dim3 g((cols + per - 1) / per, std::min(rows, 16384));
+    auto kern = planes == 3 ? (vec ? tc::k_split_planes<3, 4> : tc::k_split_planes<3, 1>)
+                            : (vec ? tc::k_split_planes<2, 4> : tc::k_split_planes<2, 1>);
+    if (planes != 2 && planes != 3) return NS_EINVAL;
     NS_CUDA_TRY(launch_pdl(kern, g, dim3(256), 0, st, in, s, rows, cols, out, stride, pitch, nrows));
     return NS_OK;
 }

@@ -120,12 +120,13 @@ struct OutBf16 {
         p[(size_t)row * N + n] = __float2bfloat16_rn(v);
     }
 };
+template <int P>
 struct OutPlanes {
     __nv_bfloat16* p;
     long long stride;
     int pitch;
     __device__ __forceinline__ void put(int row, int n, int, float v) const {
-        tc::plane_store<3>(v, p + (size_t)row * pitch + n, stride);
+        tc::plane_store<P>(v, p + (size_t)row * pitch + n, stride);
     }
 };
 
@@ -314,23 +315,25 @@ static ActDev<T> layer_act(const ns_problem* p, int l) {
 }
 
 template <typename T, typename OUT>
-static int launch_emu_input(const ns_problem* p, const Workspace* ws, int grid_rows, const OUT& out, bool pdl,
-                            cudaStream_t st) {
+static int launch_emu_input(const ns_problem* p, const double* theta_full, const int* nrows, int grid_rows,
+                            const ActDev<T>& act, const OUT& out, cudaStream_t st) {
     const int K0 = p->dims[0], H1 = p->dims[1];
     const dim3 g((grid_rows + kInRows - 1) / kInRows);
     auto kern = K0 <= 8 ? k_emu_input<T, OUT, 8> : k_emu_input<T, OUT, 32>;
-    if (pdl) {
-        NS_CUDA_TRY(launch_pdl(kern, g, dim3(256), 0, st, (const double*)ws->theta_full, p->P,
-                               (const int*)p->d_inputs, (const double*)p->d_in_center, (const double*)p->d_in_scale,
-                               (const double*)p->d_in_inv_scale, K0, (const T*)p->d_W[0], (const T*)p->d_b[0],
-                               layer_act<T>(p, 0), H1, out, (const int*)ws->d_nrows));
-    } else {
-        kern<<<g, 256, 0, st>>>(ws->theta_full, p->P, p->d_inputs, p->d_in_center, p->d_in_scale,
-                                p->d_in_inv_scale, K0, (const T*)p->d_W[0], (const T*)p->d_b[0], layer_act<T>(p, 0),
-                                H1, out, ws->d_nrows);
-        NS_CUDA_TRY(cudaGetLastError());
-    }
+    NS_CUDA_TRY(launch_pdl(kern, g, dim3(256), 0, st, theta_full, p->P, (const int*)p->d_inputs,
+                           (const double*)p->d_in_center, (const double*)p->d_in_scale,
+                           (const double*)p->d_in_inv_scale, K0, (const T*)p->d_W[0], (const T*)p->d_b[0], act, H1,
+                           out, nrows));
     return NS_OK;
+}
+
+int launch_emu_input_planes(const ns_problem* p, const double* theta_full, const int* nrows, int grid_rows, int px,
+                            __nv_bfloat16* out, long long stride, cudaStream_t st) {
+    const ActDev<float> tanh_act{NS_ACT_TANH, nullptr, nullptr};
+    const int pitch = plane_pitch(p->dims[1]);
+    if (px == 3) return launch_emu_input<float>(p, theta_full, nrows, grid_rows, tanh_act, OutPlanes<3>{out, stride, pitch}, st);
+    if (px == 2) return launch_emu_input<float>(p, theta_full, nrows, grid_rows, tanh_act, OutPlanes<2>{out, stride, pitch}, st);
+    return NS_EINVAL;
 }
 
 // The emulator's last layer: W h + b, de-standardised as mu + s * (.), written to out.
@@ -353,7 +356,8 @@ static Head model_head(const ns_problem* p, void* out) {
 
 static int run_emulator_f64(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, const Head& hd) {
     const int L = p->n_layers;
-    NS_TRY((launch_emu_input<double>(p, ws, grid_rows, OutF64{(double*)ws->act[0]}, false, st)));
+    NS_TRY(launch_emu_input<double>(p, ws->theta_full, ws->d_nrows, grid_rows, layer_act<double>(p, 0),
+                                    OutF64{(double*)ws->act[0]}, st));
     int cur = 0;
     for (int l = 1; l < L; ++l) {
         const int K = p->dims[l], N = p->dims[l + 1];
@@ -390,9 +394,9 @@ static int launch_head_f32(const ns_problem* p, Workspace* ws, int grid_rows, in
 // GEMM on the tensor cores; activations travel as three bf16 planes.
 static int run_emulator_f32(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, const Head& hd) {
     const int L = p->n_layers;
-    NS_TRY((launch_emu_input<float>(p, ws, grid_rows,
-                                    OutPlanes{(__nv_bfloat16*)ws->act[0], ws->plane_stride, plane_pitch(p->dims[1])},
-                                    true, st)));
+    NS_TRY(launch_emu_input<float>(
+        p, ws->theta_full, ws->d_nrows, grid_rows, layer_act<float>(p, 0),
+        OutPlanes<3>{(__nv_bfloat16*)ws->act[0], ws->plane_stride, plane_pitch(p->dims[1])}, st));
     int cur = 0;
     for (int l = 1; l + 1 < L; ++l) {
         const ActDev<float> a = layer_act<float>(p, l);
@@ -440,7 +444,8 @@ static int run_emulator_bf16(const ns_problem* p, Workspace* ws, int grid_rows, 
         cur = (L - 2) & 1;
         l1 = L - 1;
     } else {
-        NS_TRY((launch_emu_input<float>(p, ws, grid_rows, OutBf16{(__nv_bfloat16*)ws->act[0]}, true, st)));
+        NS_TRY(launch_emu_input<float>(p, ws->theta_full, ws->d_nrows, grid_rows, layer_act<float>(p, 0),
+                                       OutBf16{(__nv_bfloat16*)ws->act[0]}, st));
     }
     for (int l = l1; l < L; ++l) {
         const int K = p->dims[l], N = p->dims[l + 1];

@@ -44,9 +44,9 @@ struct ShearParams {
     const float* tmpl_f;
 };
 
-// Tensor maps of an activation operand of k_gemm_planes, one per row tile (32, 64, 128).
+// Tensor maps of an activation operand of k_gemm_planes, one per row tile (32, 64, 128, 256).
 struct PlaneMapX {
-    CUtensorMap m[3];
+    CUtensorMap m[4];
 };
 
 struct Workspace {
@@ -90,6 +90,7 @@ struct ns_problem {
     std::vector<int> dims;
     std::vector<void*> d_W;          // per layer, compute dtype (layer 0: FP64 or FP32)
     std::vector<void*> d_b;          // per layer, FP64 (FP64 mode) else FP32
+    std::vector<__nv_bfloat16*> d_Wp;   // and the planes themselves (row pitch plane_pitch(K))
     std::vector<CUtensorMap> tmWp;   // FP32 layers >= 1 (and a BF16 CMB head): the weights as three bf16 planes
     std::vector<CUtensorMap> tmB;    // BF16: weight tensor maps for layers >= 1
     std::vector<int> tile_n;         // BF16: N tile per layer (hidden layers autotuned at creation)
@@ -215,17 +216,6 @@ int gemm_tc_kps(int K);
 // bf16 tensor map over a row-major rows x K matrix: kps = 1 a 2-D map with
 // box_rows x 64 boxes; kps > 1 a 3-D view whose box is kps such tiles.
 int make_tensor_map_bf16(CUtensorMap* tm, const void* base, int rows, int K, int box_rows, int kps = 1);
-// Split-BF16 tcgen05 GEMM (adjoint): C = epi((A_hi + A_lo) W^T + ...) with A
-// given as a bf16 (hi, lo) pair whose sum is the FP32 operand; tmAhi / tmAlo box
-// 128 rows, tmB boxes tile_n (64, 128, 256) rows of W (N x K).  Epilogues:
-// SPL_TANH (C, C_lo) = split(tanh(acc + b)); SPL_OUT C (FP32) = mu + sigma (acc + b);
-// SPL_DTANH (C, C_lo) = split(acc (1 - h^2)), h = aux_hi + aux_lo (rows x N);
-// SPL_DTANH32 the same into FP32 C.  Row pitch of every output and aux: N.
-enum { SPL_TANH = 0, SPL_OUT = 1, SPL_DTANH = 2, SPL_DTANH32 = 3 };
-int launch_gemm_split(const CUtensorMap* tmAhi, const CUtensorMap* tmAlo, const CUtensorMap* tmB, int tile_n,
-                      const float* bias, const float* out_mu, float out_sigma, void* C, __nv_bfloat16* C_lo,
-                      const __nv_bfloat16* aux_hi, const __nv_bfloat16* aux_lo, const int* d_nrows, int grid_rows,
-                      int N, int K, int epi, int* d_err, cudaStream_t st);
 // Output layer with swapped operands (rows of W as the MMA's M, activation rows
 // as its N, kSwapRows per CTA): tmW boxes 128 rows of W, tmX boxes kSwapRows
 // activation rows; FP32 out = mu + sigma (acc + b), row-major rows x N.
@@ -267,6 +257,9 @@ int launch_gemm_planes(int px, int pw, const CUtensorMap* tmW, const PlaneMapX* 
 // planes of s * in (rows x cols, packed); nrows: device row count or null
 int launch_split_planes(int planes, const float* in, float s, int rows, int cols, __nv_bfloat16* out, long long stride,
                         int pitch, const int* nrows, cudaStream_t st);
+// the input layer (tanh) of `grid_rows` full parameter vectors as px planes of row pitch plane_pitch(H1)
+int launch_emu_input_planes(const ns_problem* p, const double* theta_full, const int* nrows, int grid_rows, int px,
+                            __nv_bfloat16* out, long long stride, cudaStream_t st);
 inline int plane_pitch(int K) { return (K + 7) & ~7; }   // rows of 16-byte multiples
 // tensor map over `planes` matrices rows x K (row pitch plane_pitch(K)), box = every plane's box_rows x 64
 int make_tensor_map_planes(CUtensorMap* tm, const void* base, int rows, int K, long long stride, int planes,

@@ -214,23 +214,26 @@ static int upload_compute(const ns_problem* p, const double* h, size_t n, void**
 
 // An FP32 matrix (rows x K) on the device as three bf16 planes and their
 // tensor map (the weights of k_gemm_planes).
-static int make_planes(const float* d, int rows, int K, CUtensorMap* tm, std::vector<void*>& owned) {
+static int make_planes(const float* d, int rows, int K, CUtensorMap* tm, __nv_bfloat16** planes,
+                       std::vector<void*>& owned) {
     const int pitch = plane_pitch(K);
     const long long stride = (long long)rows * pitch;
     void* v = nullptr;
     NS_TRY(dalloc(sizeof(uint16_t) * 3 * (size_t)stride, &v, owned));
+    if (planes) *planes = (__nv_bfloat16*)v;
     NS_TRY(launch_split_planes(3, d, 1.f, rows, K, (__nv_bfloat16*)v, stride, pitch, nullptr, nullptr));
     NS_CUDA_TRY(cudaStreamSynchronize(nullptr));   // calls may come on any stream
     return make_tensor_map_planes(tm, v, rows, K, stride, 3, 128);
 }
 
 // FP32 copy of a host FP64 matrix as planes only; the copy is freed again.
-static int upload_planes(const double* h, int rows, int K, CUtensorMap* tm, std::vector<void*>& owned) {
+static int upload_planes(const double* h, int rows, int K, CUtensorMap* tm, __nv_bfloat16** planes,
+                         std::vector<void*>& owned) {
     std::vector<float> f(h, h + (size_t)rows * K);
     std::vector<void*> tmp;
     float* d = nullptr;
     int s = upload(f.data(), f.size(), &d, tmp);
-    if (!s) s = make_planes(d, rows, K, tm, owned);
+    if (!s) s = make_planes(d, rows, K, tm, planes, owned);
     for (void* q : tmp) cudaFree(q);
     return s;
 }
@@ -350,7 +353,7 @@ static int cmb_setup(ns_problem* p, const ns_problem_desc* desc) {
         done(NS_OK);
     }
     if (p->precision == NS_PREC_FP64) NS_TRY(upload_compute(p, Wf.data(), Wf.size(), &p->d_Wfold, p->owned));
-    else NS_TRY(upload_planes(Wf.data(), D, H, &p->tmWfold, p->owned));
+    else NS_TRY(upload_planes(Wf.data(), D, H, &p->tmWfold, nullptr, p->owned));
     NS_TRY(upload_compute(p, cf.data(), cf.size(), &p->d_cfold, p->owned));
     return NS_OK;
 }
@@ -551,7 +554,10 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
     }
     p->d_W.assign(e.n_layers, nullptr);
     p->d_b.assign(e.n_layers, nullptr);
-    if (!f64) p->tmWp.resize(e.n_layers);
+    if (!f64) {
+        p->tmWp.resize(e.n_layers);
+        p->d_Wp.assign(e.n_layers, nullptr);
+    }
     for (int l = 0; l < e.n_layers; ++l) {
         const size_t nw = (size_t)p->dims[l + 1] * p->dims[l];
         const size_t nb = p->dims[l + 1];
@@ -573,16 +579,15 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
                 uint16_t* w;
                 if ((s = upload(wb.data(), nw, &w, p->owned))) return fail(s);
                 p->d_W[l] = w;
-            } else if (l >= 1 && cmb) {
-                if ((s = upload_planes(e.W[l], p->dims[l + 1], p->dims[l], &p->tmWp[l], p->owned))) return fail(s);
+            } else if (l >= 1) {
+                if ((s = upload_planes(e.W[l], p->dims[l + 1], p->dims[l], &p->tmWp[l], &p->d_Wp[l], p->owned)))
+                    return fail(s);
             } else {
-                // FP32 weights: the input layer, and the shear gradient's layers
                 std::vector<float> wf(nw);
                 for (size_t i = 0; i < nw; ++i) wf[i] = (float)e.W[l][i];
                 float* w;
                 if ((s = upload(wf.data(), nw, &w, p->owned))) return fail(s);
                 p->d_W[l] = w;
-                if (l >= 1 && (s = make_planes(w, p->dims[l + 1], p->dims[l], &p->tmWp[l], p->owned))) return fail(s);
             }
         }
     }
