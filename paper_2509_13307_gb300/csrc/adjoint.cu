@@ -1,601 +1,18 @@
 // Hand-written adjoint of the shear likelihood (row A14): d log L / d theta.
 //
-// k_projection_adj (one CTA per evaluation) recomputes the forward projection
-// into per-evaluation scratch (distances, growth, windows, padded P table,
-// Limber sums, data vector, residual r, y = L^-1 r, log L) and then runs the
-// reverse pass:
-//   g_m = Sigma^-1 r = L^-T y                       (chi^2, Gaussian)
-//   g_C[p][ell] = g_m (1+m_i)(1+m_j); g_b = T^T g_m; g_m_i from the bias products
-//   Limber / lookup: per node, per multipole, g_P = sum_p g_C V_i V_j;
-//     g_V_i += g_C V_j P; g_v = ln10 P g_P scattered onto the 16 table taps;
-//     d v / d ln k (Catmull-Rom derivative) gives g_ln chi
-//   windows (Eq. 5-6): the exclusive suffix sums transpose to exclusive prefix
-//     sums of their adjoints; n(z) normalisation and the D_z shifts
-//   growth: suffix sums of g_ln D through the trapezoid segments
-//   distances: suffix sums of g_chi onto each Gauss-Legendre interval,
-//     then d E^2 / d(Omega_m, w0, wa) at every quadrature point
-//   scalars: Omega_m = (omega_b + omega_cdm)/h^2, c/H0 = c/(100 h), gamma(w0, wa)
-// The table gradient (ghost rows/columns folded back) feeds the emulator
-// backward pass (transposed GEMMs, tanh' from stored activations); the
-// emulator-input gradient is added to the parameter gradient in
-// k_finish_grad.
+// The emulator forward with stored activations, the projection and its reverse
+// (projection_adj.cu: log L, the table gradient and the gradient of the
+// parameters that enter the projection), the emulator backward (transposed
+// GEMMs, tanh' from the stored activations), and the emulator inputs' share
+// added to the parameter gradient in k_finish_grad.
 #include <cstring>
 #include <mutex>
 #include <vector>
 
 #include "likelihood.cuh"
+#include "projection_adj.cuh"
 
 namespace gpuns {
-
-namespace adj {
-
-// 4-point Gauss-Legendre nodes and weights as compile-time constants of the
-// kernel's type (no double -> float conversions at run time).
-template <typename T> __device__ __forceinline__ T glx(int g) {
-    return g == 0 ? T(-0.86113631159405257522) : g == 1 ? T(-0.33998104358485626480)
-         : g == 2 ? T(0.33998104358485626480) : T(0.86113631159405257522);
-}
-template <typename T> __device__ __forceinline__ T glw(int g) {
-    return (g == 0 || g == 3) ? T(0.34785484513745385737) : T(0.65214515486254614263);
-}
-
-template <typename T> __device__ __forceinline__ const T* pick(const double* d, const float* f);
-template <> __device__ __forceinline__ const double* pick<double>(const double* d, const float*) { return d; }
-template <> __device__ __forceinline__ const float* pick<float>(const double*, const float* f) { return f; }
-template <typename T> __device__ __forceinline__ T pick_s(double d, float f);
-template <> __device__ __forceinline__ double pick_s<double>(double d, float) { return d; }
-template <> __device__ __forceinline__ float pick_s<float>(double, float f) { return f; }
-
-template <typename T> __device__ __forceinline__ T ex(T x);
-template <> __device__ __forceinline__ double ex<double>(double x) { return exp(x); }
-template <> __device__ __forceinline__ float ex<float>(float x) { return expf(x); }
-template <typename T> __device__ __forceinline__ T lg(T x);
-template <> __device__ __forceinline__ double lg<double>(double x) { return log(x); }
-template <> __device__ __forceinline__ float lg<float>(float x) { return logf(x); }
-
-// Scalar adjoints accumulated in shared memory.
-enum { S_OM = 0, S_CHIH, S_W0, S_WA, S_GAMMA, S_PREF, S_AIA, S_ETA, S_COUNT };
-
-struct AdjArgs {
-    ShearParams sp;
-    const double* theta_full;
-    const void* table;       // rows x (n_z n_k), T
-    const void* LinvT;       // D x D, T: LinvT[b*D + a] = (L^-1)[a][b]
-    double c0;
-    void* scratch;           // rows x per_eval, T
-    long long per_eval;
-    void* gtab_out;          // rows x (n_z n_k), T: d log L / d table
-    double* gfull;           // rows x n_params: d log L / d theta_full (emulator inputs excluded)
-    double* logL;
-    const int* nrows;
-};
-
-template <typename T>
-__device__ __forceinline__ void cr_w(T t, T w[4]) {   // doubled Catmull-Rom weights
-    const T t2 = t * t;
-    w[0] = t * (t * (T(2) - t) - T(1));
-    w[1] = T(2) + t2 * (T(3) * t - T(5));
-    w[2] = t * (T(1) + t * (T(4) - T(3) * t));
-    w[3] = t2 * (t - T(1));
-}
-template <typename T>
-__device__ __forceinline__ void cr_dw(T t, T w[4]) {  // d/dt of the doubled weights
-    w[0] = T(-1) + t * (T(4) - T(3) * t);
-    w[1] = t * (T(9) * t - T(10));
-    w[2] = T(1) + t * (T(8) - T(9) * t);
-    w[3] = t * (T(3) * t - T(2));
-}
-
-template <typename T, int NB>
-__global__ void __launch_bounds__(256)
-k_projection_adj(const AdjArgs A) {
-    constexpr int NP = NB * (NB + 1) / 2;
-    const ShearParams& sp = A.sp;
-    const int row = blockIdx.x;
-    if (row >= *A.nrows) return;
-    const int N = sp.N, n_k = sp.n_k, n_z = sp.n_z, PK = n_k + 2, PT = (n_z + 2) * PK, D = sp.D;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int lane = tid & 31, wid = tid >> 5;
-    T* S = reinterpret_cast<T*>(A.scratch) + (size_t)row * A.per_eval;
-    T* chi = S;
-    T* lnchi = S + N;
-    T* Ez = S + 2 * N;
-    T* Dg = S + 3 * N;
-    T* omw = S + 4 * N;
-    T* fg = S + 5 * N;
-    T* gchi = S + 6 * N;
-    T* gE = S + 7 * N;
-    T* gomw = S + 8 * N;
-    T* gD = S + 9 * N;
-    T* t1 = S + 10 * N;
-    T* t2 = S + 11 * N;
-    T* raw = S + 12 * N;
-    T* nchi = raw + NB * N;
-    T* E0 = nchi + NB * N;
-    T* E1 = E0 + NB * N;
-    T* V = E1 + NB * N;
-    T* gV = V + NB * N;
-    T* tab = gV + NB * N;      // PT
-    T* gtab = tab + PT;        // PT
-    T* r = gtab + PT;          // D
-    T* gm = r + D;             // D
-    const T* nz_mu = pick<T>(sp.nz_mean, sp.nz_mean_f);
-    const T* nz_sg = pick<T>(sp.nz_sigma, sp.nz_sigma_f);
-    const T* lnell = pick<T>(sp.lnell, sp.lnell_f);
-    const T* tmplT = pick<T>(sp.tmpl, sp.tmpl_f);
-    const T* dataT = pick<T>(sp.data, sp.data_f);
-    const T ia_piv = pick_s<T>(sp.ia_pivot, sp.ia_pivot_f), c1rho = pick_s<T>(sp.c1rho, sp.c1rho_f);
-    const T* a_ = pick<T>(sp.a, sp.a_f);
-    const T* lna_ = pick<T>(sp.lna, sp.lna_f);
-    const T* z_ = pick<T>(sp.z, sp.z_f);
-    const T* wa_ = pick<T>(sp.wa, sp.wa_f);
-    const T* zwp = pick<T>(sp.zw4d, sp.zw4f);
-
-    __shared__ T th[128];
-    __shared__ T gth[128];
-    __shared__ T gs[S_COUNT];
-    __shared__ T red[64];
-    __shared__ T red2[8 * NP];                 // per-warp pair sums of one multipole
-    __shared__ T Cl[NP * 64];
-    __shared__ T gC[NP * 64];
-    __shared__ T norm[NB];
-    for (int i = tid; i < sp.n_params; i += nt) {
-        th[i] = (T)A.theta_full[(size_t)row * sp.n_params + i];
-        gth[i] = T(0);
-    }
-    if (tid < S_COUNT) gs[tid] = T(0);
-    __syncthreads();
-    const T h = th[2];
-    const T om = (th[0] + th[1]) / (h * h);
-    const T w0 = th[5], wa = th[6];
-    const T pde = T(3) * (T(1) + w0 + wa);
-    const T chiH = T(kCover100) / h;
-    const T gamma = T(0.55) + T(0.05) * (T(1) + w0 + T(0.5) * wa);
-    const T pref = T(1.5) * om / (chiH * chiH);
-    const T A_IA = th[9], eta = th[10];
-
-    // ===================== forward (recorded) =====================
-    for (int n = tid; n < N; n += nt) {
-        const T a = a_[n], lna = lna_[n];
-        const T de = ex<T>(-pde * lna - T(3) * wa * (T(1) - a));
-        Ez[n] = sqrt(om * ex<T>(T(-3) * lna) + (T(1) - om) * de);
-        T inc = T(0);
-        if (n < N - 1) {
-            const T a1 = a_[n + 1];
-            const T mid = T(0.5) * (a + a1), half = T(0.5) * (a - a1);
-            for (int g = 0; g < 4; ++g) {
-                const T ag = mid + half * glx<T>(g);
-                const T lgg = lg<T>(ag);
-                const T e2 = om / (ag * ag * ag) + (T(1) - om) * ex<T>(-pde * lgg - T(3) * wa * (T(1) - ag));
-                inc += glw<T>(g) / (ag * ag * sqrt(e2));
-            }
-            inc *= chiH * half;
-        }
-        t1[n] = inc;
-    }
-    __syncthreads();
-    block_exclusive_scan(t1, N, red);
-    for (int n = tid; n < N; n += nt) {
-        const T c = t1[n];
-        chi[n] = c;
-        lnchi[n] = (n >= 1) ? lg<T>(c) : T(0);
-        const T oma = om * ex<T>(T(-3) * lna_[n]) / (Ez[n] * Ez[n]);
-        fg[n] = ex<T>(gamma * lg<T>(oma));
-        omw[n] = wa_[n] * chiH / (a_[n] * a_[n] * Ez[n]);
-        gchi[n] = T(0); gE[n] = T(0); gomw[n] = T(0); gD[n] = T(0);
-    }
-    __syncthreads();
-    for (int n = tid; n < N; n += nt) t2[n] = (n < N - 1) ? T(0.5) * (fg[n] + fg[n + 1]) * (lna_[n] - lna_[n + 1]) : T(0);
-    __syncthreads();
-    block_exclusive_scan(t2, N, red);
-    for (int n = tid; n < N; n += nt) Dg[n] = ex<T>(-t2[n]);
-    __syncthreads();
-    for (int i = 0; i < NB; ++i) {
-        T part = T(0);
-        for (int n = tid; n < N; n += nt) {
-            const T u = (z_[n] - th[11 + i] - nz_mu[i]) / nz_sg[i];
-            const T rw = ex<T>(T(-0.5) * u * u);
-            raw[i * N + n] = rw;
-            part += wa_[n] * rw / (a_[n] * a_[n]);
-        }
-        const T s = block_sum(part, red);
-        if (tid == 0) norm[i] = s;
-        __syncthreads();
-        for (int n = tid; n < N; n += nt) {
-            const T nc = raw[i * N + n] * Ez[n] / (chiH * s);
-            nchi[i * N + n] = nc;
-            E0[i * N + n] = (n >= 1) ? omw[n] * nc : T(0);
-            E1[i * N + n] = (n >= 1) ? omw[n] * nc / chi[n] : T(0);
-            gV[i * N + n] = T(0);
-        }
-        __syncthreads();
-        block_exclusive_suffix_scan(E0 + i * N, N, red);
-        block_exclusive_suffix_scan(E1 + i * N, N, red);
-    }
-    for (int n = tid; n < N; n += nt) {
-        const T c = chi[n];
-        const T amp = A_IA * ex<T>(eta * lg<T>((T(1) + z_[n]) / ia_piv)) * c1rho * om / Dg[n];
-        for (int i = 0; i < NB; ++i) {
-            T v = T(0);
-            if (n >= 1) {
-                const T W = pref * c / a_[n] * (E0[i * N + n] - c * E1[i * N + n]) - amp * nchi[i * N + n];
-                v = sqrt(omw[n]) / c * W;
-            }
-            V[i * N + n] = v;
-        }
-    }
-    // padded table (ghosts by linear extrapolation) and its zeroed gradient
-    {
-        const T* src = reinterpret_cast<const T*>(A.table) + (size_t)row * n_z * n_k;
-        for (int i = tid; i < n_z * n_k; i += nt) tab[(i / n_k + 1) * PK + i % n_k + 1] = src[i];
-        for (int i = tid; i < PT; i += nt) gtab[i] = T(0);
-        __syncthreads();
-        for (int k = 1 + tid; k <= n_k; k += nt) {
-            tab[k] = T(2) * tab[PK + k] - tab[2 * PK + k];
-            tab[(n_z + 1) * PK + k] = T(2) * tab[n_z * PK + k] - tab[(n_z - 1) * PK + k];
-        }
-        __syncthreads();
-        for (int rr = tid; rr < n_z + 2; rr += nt) {
-            tab[rr * PK] = T(2) * tab[rr * PK + 1] - tab[rr * PK + 2];
-            tab[rr * PK + n_k + 1] = T(2) * tab[rr * PK + n_k] - tab[rr * PK + n_k - 1];
-        }
-    }
-    __syncthreads();
-    const T lkmin = pick_s<T>(sp.lnk_min, sp.lnk_min_f), lkmax = pick_s<T>(sp.lnk_max, sp.lnk_max_f);
-    const T inv_dk = pick_s<T>(1.0 / sp.dlnk, sp.inv_dlnk_f);
-    // Limber: C_p(ell) (block reductions, fixed order)
-    for (int l = 0; l < sp.n_ell; ++l) {
-        T acc[NP];
-        for (int p = 0; p < NP; ++p) acc[p] = T(0);
-        const T lne = lnell[l];
-        for (int n = 1 + tid; n < N; n += nt) {
-            T s = fmin(fmax(lne - lnchi[n], lkmin), lkmax);
-            const T uk = (s - lkmin) * inv_dk;
-            int ik = min(max((int)floor(uk), 0), n_k - 2);
-            T wk[4];
-            cr_w<T>(uk - (T)ik, wk);
-            const T* c = tab + sp.zrp[n] * PK + ik;
-            T v = T(0);
-            for (int pz = 0; pz < 4; ++pz)
-                v += zwp[4 * n + pz] * (wk[0] * c[pz * PK] + wk[1] * c[pz * PK + 1] + wk[2] * c[pz * PK + 2] + wk[3] * c[pz * PK + 3]);
-            const T P = ex<T>(T(0.25) * v * (T)kLn10);
-            int p = 0;
-            for (int i = 0; i < NB; ++i)
-                for (int j = i; j < NB; ++j) { acc[p] += V[i * N + n] * V[j * N + n] * P; ++p; }
-        }
-        // all NP pair sums at once: warp sums, then a fixed-order sum over warps
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            const T s = warp_sum(acc[p]);
-            if (lane == 0) red2[wid * NP + p] = s;
-        }
-        __syncthreads();
-        if (tid < NP) {
-            T s = T(0);
-            for (int w = 0; w < (nt >> 5); ++w) s += red2[w * NP + tid];
-            Cl[tid * sp.n_ell + l] = s;
-        }
-        __syncthreads();
-    }
-    __syncthreads();
-    // data vector, residual, whitening, log L
-    for (int a = tid; a < D; a += nt) {
-        const int p = a / sp.n_ell, e = a % sp.n_ell;
-        const int i = sp.pi[p], j = sp.pj[p];
-        T m = (T(1) + th[11 + NB + i]) * (T(1) + th[11 + NB + j]) * Cl[p * sp.n_ell + e];
-        for (int t = 0; t < sp.n_tmpl; ++t) m += tmplT[(size_t)a * sp.n_tmpl + t] * th[11 + 2 * NB + t];
-        r[a] = dataT[a] - m;
-    }
-    __syncthreads();
-    const T* LT = reinterpret_cast<const T*>(A.LinvT);
-    T sq = T(0);
-    for (int a = tid; a < D; a += nt) {
-        T y = T(0);
-        for (int b = 0; b <= a; ++b) y += LT[(size_t)b * D + a] * r[b];
-        gm[a] = y;                      // y stored temporarily in gm
-        sq += y * y;
-    }
-    sq = block_sum(sq, red);
-    if (tid == 0) A.logL[row] = A.c0 - 0.5 * (double)sq;
-    // ===================== reverse =====================
-    // g_m = L^-T y: (g_m)_a = sum_{b >= a} (L^-1)[b][a] y_b = sum_{b >= a} LinvT[a*D + b] y_b
-    for (int a = tid; a < D; a += nt) {
-        T g = T(0);
-        for (int b = a; b < D; ++b) g += LT[(size_t)a * D + b] * gm[b];
-        r[a] = g;                       // r now holds g_m
-    }
-    __syncthreads();
-    // bias, templates, g_C
-    for (int a = tid; a < D; a += nt) {
-        const int p = a / sp.n_ell, e = a % sp.n_ell;
-        const int i = sp.pi[p], j = sp.pj[p];
-        const T g = r[a];
-        const T fi = T(1) + th[11 + NB + i], fj = T(1) + th[11 + NB + j];
-        const T C = Cl[p * sp.n_ell + e];
-        gC[p * sp.n_ell + e] = g * fi * fj;
-        atomicAdd(&gth[11 + NB + i], g * C * fj);
-        atomicAdd(&gth[11 + NB + j], g * C * fi);
-        for (int t = 0; t < sp.n_tmpl; ++t) atomicAdd(&gth[11 + 2 * NB + t], g * tmplT[(size_t)a * sp.n_tmpl + t]);
-    }
-    __syncthreads();
-    // Limber + lookup reverse: threads own nodes, loop over multipoles
-    for (int n = 1 + tid; n < N; n += nt) {
-        T vv[NB], gv_[NB];
-        for (int i = 0; i < NB; ++i) { vv[i] = V[i * N + n]; gv_[i] = T(0); }
-        T glnc = T(0);
-        const int zr = sp.zrp[n];
-        T wz[4];
-        for (int pz = 0; pz < 4; ++pz) wz[pz] = zwp[4 * n + pz];
-        for (int l = 0; l < sp.n_ell; ++l) {
-            const T s_raw = lnell[l] - lnchi[n];
-            const bool clamped = (s_raw < lkmin) || (s_raw > lkmax);
-            const T s = fmin(fmax(s_raw, lkmin), lkmax);
-            const T uk = (s - lkmin) * inv_dk;
-            int ik = min(max((int)floor(uk), 0), n_k - 2);
-            const T t = uk - (T)ik;
-            T wk[4], dwk[4];
-            cr_w<T>(t, wk);
-            cr_dw<T>(t, dwk);
-            const T* c = tab + zr * PK + ik;
-            T v = T(0), dv = T(0);
-            for (int pz = 0; pz < 4; ++pz) {
-                const T* cr = c + pz * PK;
-                v += wz[pz] * (wk[0] * cr[0] + wk[1] * cr[1] + wk[2] * cr[2] + wk[3] * cr[3]);
-                dv += wz[pz] * (dwk[0] * cr[0] + dwk[1] * cr[1] + dwk[2] * cr[2] + dwk[3] * cr[3]);
-            }
-            const T P = ex<T>(T(0.25) * v * (T)kLn10);
-            T gP = T(0);
-            int p = 0;
-            for (int i = 0; i < NB; ++i)
-                for (int j = i; j < NB; ++j) {
-                    const T g = gC[p * sp.n_ell + l];
-                    gP += g * vv[i] * vv[j];
-                    gv_[i] += g * vv[j] * P;
-                    gv_[j] += g * vv[i] * P;
-                    ++p;
-                }
-            const T gvv = gP * P * (T)kLn10 * T(0.25);   // d log L / d (doubled-weight sum)
-            T* gc = gtab + zr * PK + ik;
-            for (int pz = 0; pz < 4; ++pz)
-                for (int q = 0; q < 4; ++q) atomicAdd(gc + pz * PK + q, gvv * wz[pz] * wk[q]);
-            if (!clamped) glnc -= gvv * dv * inv_dk;     // s = ln(ell+1/2) - ln chi
-        }
-        for (int i = 0; i < NB; ++i) gV[i * N + n] = gv_[i];
-        gchi[n] += glnc / chi[n];
-    }
-    __syncthreads();
-    // fold the ghost-cell gradients back onto the table (reverse of the padding)
-    for (int rr = tid; rr < n_z + 2; rr += nt) {
-        const T g0 = gtab[rr * PK], g1 = gtab[rr * PK + n_k + 1];
-        gtab[rr * PK + 1] += T(2) * g0; gtab[rr * PK + 2] -= g0;
-        gtab[rr * PK + n_k] += T(2) * g1; gtab[rr * PK + n_k - 1] -= g1;
-    }
-    __syncthreads();
-    for (int k = 1 + tid; k <= n_k; k += nt) {
-        const T g0 = gtab[k], g1 = gtab[(n_z + 1) * PK + k];
-        gtab[PK + k] += T(2) * g0; gtab[2 * PK + k] -= g0;
-        gtab[n_z * PK + k] += T(2) * g1; gtab[(n_z - 1) * PK + k] -= g1;
-    }
-    __syncthreads();
-    {
-        T* dst = reinterpret_cast<T*>(A.gtab_out) + (size_t)row * n_z * n_k;
-        for (int i = tid; i < n_z * n_k; i += nt) dst[i] = gtab[(i / n_k + 1) * PK + i % n_k + 1];
-    }
-    // windows reverse: V = sqrt(omw)/chi * W, W = pc (E0 - chi E1) - amp nchi
-    T l_pref = T(0), l_aia = T(0), l_eta = T(0), l_om = T(0);
-    for (int n = 1 + tid; n < N; n += nt) {
-        const T c = chi[n], an = a_[n];
-        const T so = sqrt(omw[n]);
-        const T q = ex<T>(eta * lg<T>((T(1) + z_[n]) / ia_piv));
-        const T ampc = q * c1rho * om / Dg[n];       // amp = A_IA * ampc
-        const T pc = pref * c / an;
-        T g_so = T(0), g_c = T(0), g_amp = T(0);
-        for (int i = 0; i < NB; ++i) {
-            const T e0 = E0[i * N + n], e1 = E1[i * N + n], nc = nchi[i * N + n];
-            const T W = pc * (e0 - c * e1) - A_IA * ampc * nc;
-            const T gVv = gV[i * N + n];
-            const T gW = gVv * so / c;
-            g_so += gVv * W / c;
-            g_c += -gVv * so * W / (c * c);
-            // W partials
-            const T gpc = gW * (e0 - c * e1);
-            l_pref += gpc * c / an;
-            g_c += gpc * pref / an - gW * pc * e1;
-            E0[i * N + n] = gW * pc;            // reuse E0/E1 storage as their adjoints
-            E1[i * N + n] = -gW * pc * c;
-            g_amp += -gW * nc;
-            raw[i * N + n] = -gW * A_IA * ampc; // reuse raw as g_nchi (direct term)
-        }
-        gomw[n] += g_so * T(0.5) / so;
-        gchi[n] += g_c;
-        // amp = A_IA q c1rho Om / D
-        l_aia += g_amp * ampc;
-        l_eta += g_amp * A_IA * ampc * lg<T>((T(1) + z_[n]) / ia_piv);
-        l_om += g_amp * A_IA * ampc / om;
-        gD[n] += -g_amp * A_IA * ampc / Dg[n];
-    }
-    if (true) {   // node 0 carries no window value; its direct g_nchi is zero
-        for (int i = 0; i < NB; ++i) if (tid == 0) { raw[i * N] = T(0); E0[i * N] = T(0); E1[i * N] = T(0); }
-    }
-    l_pref = block_sum(l_pref, red);
-    l_aia = block_sum(l_aia, red);
-    l_eta = block_sum(l_eta, red);
-    l_om = block_sum(l_om, red);
-    if (tid == 0) {
-        gs[S_PREF] += l_pref; gs[S_AIA] += l_aia; gs[S_ETA] += l_eta; gs[S_OM] += l_om;
-    }
-    __syncthreads();
-    // E0_i(n) = sum_{m>n} omw_m nchi_m  ->  G0(m) = sum_{n<m} gE0(n) (exclusive prefix)
-    for (int i = 0; i < NB; ++i) {
-        block_exclusive_scan(E0 + i * N, N, red);
-        block_exclusive_scan(E1 + i * N, N, red);
-        T gdz = T(0), gnorm = T(0);
-        for (int m = tid; m < N; m += nt) {
-            T gnc = raw[i * N + m];
-            if (m >= 1) {
-                const T G0 = E0[i * N + m], G1 = E1[i * N + m];
-                const T nc = nchi[i * N + m], c = chi[m];
-                gomw[m] += nc * (G0 + G1 / c);
-                gnc += omw[m] * (G0 + G1 / c);
-                gchi[m] += -omw[m] * nc * G1 / (c * c);
-            }
-            raw[i * N + m] = gnc;   // total g_nchi
-        }
-        __syncthreads();
-        // nchi = raw E / (chiH norm)
-        const T nrm = norm[i];
-        T l_chih = T(0);
-        for (int m = tid; m < N; m += nt) {
-            const T gnc = raw[i * N + m];
-            const T nc = nchi[i * N + m];
-            const T u = (z_[m] - th[11 + i] - nz_mu[i]) / nz_sg[i];
-            gE[m] += gnc * nc / Ez[m];
-            l_chih += -gnc * nc / chiH;
-            gnorm += -gnc * nc / nrm;
-            // d raw / d Dz = raw u / sigma and nchi is proportional to raw
-            gdz += gnc * nc * u / nz_sg[i];
-        }
-        gnorm = block_sum(gnorm, red);
-        // norm = sum wa raw / a^2  ->  d norm / d Dz = sum wa raw u / sigma / a^2
-        for (int m = tid; m < N; m += nt) {
-            const T u = (z_[m] - th[11 + i] - nz_mu[i]) / nz_sg[i];
-            const T rw = ex<T>(T(-0.5) * u * u);
-            gdz += gnorm * wa_[m] * rw * u / nz_sg[i] / (a_[m] * a_[m]);
-        }
-        gdz = block_sum(gdz, red);
-        l_chih = block_sum(l_chih, red);
-        if (tid == 0) { gth[11 + i] += gdz; gs[S_CHIH] += l_chih; }
-        __syncthreads();
-    }
-    // omw = wa chiH / (a^2 E)
-    {
-        T l_chih = T(0);
-        for (int n = tid; n < N; n += nt) {
-            l_chih += gomw[n] * omw[n] / chiH;
-            gE[n] += -gomw[n] * omw[n] / Ez[n];
-        }
-        l_chih = block_sum(l_chih, red);
-        if (tid == 0) gs[S_CHIH] += l_chih;
-    }
-    // growth: D_n = exp(-S_n), S_n = sum_{m<n} seg_m, seg_m = (f_m + f_{m+1}) / 2 * dlna_m
-    for (int n = tid; n < N; n += nt) t1[n] = -gD[n] * Dg[n];   // g_S
-    __syncthreads();
-    block_exclusive_suffix_scan(t1, N, red);                     // g_seg_m = sum_{n>m} g_S_n
-    {
-        T l_om = T(0), l_gam = T(0);
-        for (int m = tid; m < N; m += nt) {
-            T gf = T(0);
-            if (m < N - 1) gf += T(0.5) * t1[m] * (lna_[m] - lna_[m + 1]);
-            if (m >= 1) gf += T(0.5) * t1[m - 1] * (lna_[m - 1] - lna_[m]);
-            const T oma = om * ex<T>(T(-3) * lna_[m]) / (Ez[m] * Ez[m]);
-            l_gam += gf * fg[m] * lg<T>(oma);
-            const T goma = gf * fg[m] * gamma / oma;
-            l_om += goma * oma / om;
-            gE[m] += goma * T(-2) * oma / Ez[m];
-        }
-        l_om = block_sum(l_om, red);
-        l_gam = block_sum(l_gam, red);
-        if (tid == 0) { gs[S_OM] += l_om; gs[S_GAMMA] += l_gam; }
-    }
-    __syncthreads();
-    // distances: chi_n = sum_{m<n} dchi_m  ->  g_dchi_m = sum_{n>m} g_chi_n
-    for (int n = tid; n < N; n += nt) t2[n] = gchi[n];
-    __syncthreads();
-    block_exclusive_suffix_scan(t2, N, red);
-    {
-        T l_om = T(0), l_w0 = T(0), l_wa = T(0), l_chih = T(0);
-        for (int n = tid; n < N; n += nt) {
-            const T a = a_[n], lna = lna_[n];
-            const T de = ex<T>(-pde * lna - T(3) * wa * (T(1) - a));
-            // node E: E^2 = om a^-3 + (1 - om) de
-            const T ge2 = gE[n] / (T(2) * Ez[n]);
-            l_om += ge2 * (ex<T>(T(-3) * lna) - de);
-            l_w0 += ge2 * (T(1) - om) * de * (T(-3) * lna);
-            l_wa += ge2 * (T(1) - om) * de * (T(-3) * lna - T(3) * (T(1) - a));
-            if (n < N - 1) {
-                const T g = t2[n];
-                const T a1 = a_[n + 1];
-                const T mid = T(0.5) * (a + a1), half = T(0.5) * (a - a1);
-                T inc = T(0);
-                for (int q = 0; q < 4; ++q) {
-                    const T ag = mid + half * glx<T>(q);
-                    const T lgg = lg<T>(ag);
-                    const T deg = ex<T>(-pde * lgg - T(3) * wa * (T(1) - ag));
-                    const T e2 = om / (ag * ag * ag) + (T(1) - om) * deg;
-                    const T F = T(1) / (ag * ag * sqrt(e2));
-                    inc += glw<T>(q) * F;
-                    const T gF = g * chiH * half * glw<T>(q);
-                    const T gE2 = gF * T(-0.5) * F / e2;
-                    l_om += gE2 * (T(1) / (ag * ag * ag) - deg);
-                    l_w0 += gE2 * (T(1) - om) * deg * (T(-3) * lgg);
-                    l_wa += gE2 * (T(1) - om) * deg * (T(-3) * lgg - T(3) * (T(1) - ag));
-                }
-                l_chih += g * half * inc;
-            }
-        }
-        l_om = block_sum(l_om, red);
-        l_w0 = block_sum(l_w0, red);
-        l_wa = block_sum(l_wa, red);
-        l_chih = block_sum(l_chih, red);
-        if (tid == 0) { gs[S_OM] += l_om; gs[S_W0] += l_w0; gs[S_WA] += l_wa; gs[S_CHIH] += l_chih; }
-    }
-    __syncthreads();
-    if (tid == 0) {
-        // pref = 1.5 om / chiH^2; gamma = 0.55 + 0.05 (1 + w0 + wa/2)
-        const T g_om = gs[S_OM] + gs[S_PREF] * pref / om;
-        const T g_chih = gs[S_CHIH] - T(2) * gs[S_PREF] * pref / chiH;
-        const T g_w0 = gs[S_W0] + T(0.05) * gs[S_GAMMA];
-        const T g_wa = gs[S_WA] + T(0.025) * gs[S_GAMMA];
-        // om = (wb + wc) / h^2; chiH = c / (100 h)
-        gth[0] += g_om / (h * h);
-        gth[1] += g_om / (h * h);
-        gth[2] += -T(2) * g_om * om / h - g_chih * chiH / h;
-        gth[5] += g_w0;
-        gth[6] += g_wa;
-        gth[9] += gs[S_AIA];
-        gth[10] += gs[S_ETA];
-    }
-    __syncthreads();
-    for (int i = tid; i < sp.n_params; i += nt) A.gfull[(size_t)row * sp.n_params + i] = (double)gth[i];
-}
-
-template <typename T, int NB>
-size_t per_eval_elems(const ShearParams& sp) {
-    return (size_t)(12 + 6 * NB) * sp.N + 2 * (size_t)(sp.n_z + 2) * (sp.n_k + 2) + 2 * (size_t)sp.D;
-}
-
-}  // namespace adj
-
-int adjoint_scratch_elems(const ShearParams& sp) {
-    return (12 + 6 * sp.nb) * sp.N + 2 * (sp.n_z + 2) * (sp.n_k + 2) + 2 * sp.D;
-}
-
-template <typename T>
-int launch_projection_adj(const ShearParams& sp, const double* theta_full, const T* table, const T* LinvT, double c0,
-                          T* scratch, T* gtab, double* gfull, double* logL, const int* nrows, int grid_rows,
-                          cudaStream_t st) {
-    if (sp.n_ell > 64 || sp.n_params > 128) return NS_ENOTSUP;
-    adj::AdjArgs A{sp, theta_full, table, LinvT, c0, scratch, (long long)adjoint_scratch_elems(sp), gtab, gfull,
-                   logL, nrows};
-    auto go = [&](auto kern) -> int {
-        kern<<<grid_rows, 256, 0, st>>>(A);
-        return NS_OK;
-    };
-    switch (sp.nb) {
-        case 1: NS_TRY(go(adj::k_projection_adj<T, 1>)); break;
-        case 2: NS_TRY(go(adj::k_projection_adj<T, 2>)); break;
-        case 3: NS_TRY(go(adj::k_projection_adj<T, 3>)); break;
-        case 4: NS_TRY(go(adj::k_projection_adj<T, 4>)); break;
-        case 5: NS_TRY(go(adj::k_projection_adj<T, 5>)); break;
-        default: return NS_ENOTSUP;
-    }
-    NS_CUDA_TRY(cudaGetLastError());
-    return NS_OK;
-}
-template int launch_projection_adj<double>(const ShearParams&, const double*, const double*, const double*, double,
-                                           double*, double*, double*, double*, const int*, int, cudaStream_t);
-template int launch_projection_adj<float>(const ShearParams&, const double*, const float*, const float*, double,
-                                          float*, float*, double*, double*, const int*, int, cudaStream_t);
 
 // ------------------------------------------------------------------ emulator backward
 namespace adj {
@@ -748,6 +165,17 @@ __global__ void k_zinterp_adj(const T* __restrict__ gfine, int nz, const int* __
     }
 }
 
+template <typename T>
+__global__ void __launch_bounds__(256) k_transpose(const T* __restrict__ A, T* __restrict__ B, int D) {
+    __shared__ T t[32][33];
+    const int x0 = blockIdx.x * 32, y0 = blockIdx.y * 32, x = threadIdx.x & 31;
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (y0 + y < D && x0 + x < D) t[y][x] = A[(size_t)(y0 + y) * D + x0 + x];
+    __syncthreads();
+    for (int y = threadIdx.x >> 5; y < 32; y += 8)
+        if (x0 + y < D && y0 + x < D) B[(size_t)(x0 + y) * D + y0 + x] = t[x][y];
+}
+
 // T[p][k][n] = W[p][n][k] for bf16 planes: W N rows of pitch wp, T K rows of pitch tp.
 __global__ void __launch_bounds__(256) k_transpose_planes(const __nv_bfloat16* __restrict__ W, int N, int K, int wp,
                                                           __nv_bfloat16* __restrict__ T, int tp) {
@@ -784,7 +212,8 @@ struct GradState {
     void* table_fine = nullptr;
     void* gtab = nullptr;      // cap x n_z n_k
     void* gcoarse = nullptr;   // cap x n_out, coarse-z emulators
-    void* scratch = nullptr;   // cap x adjoint_scratch_elems
+    void* Linv = nullptr;      // D x D, L^-1 row-major in the arithmetic type
+    ProjectionAdj proj;
     double* gfull = nullptr;   // cap x P
     // FP64: stored activations per hidden layer and ping-pong adjoints
     std::vector<double*> H;
@@ -827,13 +256,21 @@ static int grad_state_create(const ns_problem* p, GradState* g) {
         NS_TRY(grad_alloc(g, T * (size_t)cap * nzk, &g->table_fine));
         NS_TRY(grad_alloc(g, T * (size_t)cap * n_out, &g->gcoarse));
     }
-    NS_TRY(grad_alloc(g, T * (size_t)cap * adjoint_scratch_elems(p->sp), &g->scratch));
+    NS_TRY(projection_adj_create(p->sp, (int)T, cap, &g->proj));
+    NS_TRY(grad_alloc(g, T * (size_t)p->D * p->D, &g->Linv));
+    {
+        const dim3 b((p->D + 31) / 32, (p->D + 31) / 32);
+        if (f64) adj::k_transpose<double><<<b, 256>>>(p->d_LinvT64, (double*)g->Linv, p->D);
+        else adj::k_transpose<float><<<b, 256>>>(p->d_LinvT32, (float*)g->Linv, p->D);
+        NS_CUDA_TRY(cudaGetLastError());
+    }
     int wmax = 0;
     for (int l = 1; l <= L; ++l) wmax = std::max(wmax, p->dims[l]);
     if (f64) {
         g->H.assign(L, nullptr);
         for (int l = 1; l < L; ++l) NS_TRY(grad_alloc(g, 8 * (size_t)cap * p->dims[l], (void**)&g->H[l]));
         for (int i = 0; i < 2; ++i) NS_TRY(grad_alloc(g, 8 * (size_t)cap * wmax, (void**)&g->g64[i]));
+        NS_CUDA_TRY(cudaStreamSynchronize(nullptr));   // calls may come on any stream
         return NS_OK;
     }
     const bool f32 = p->precision == NS_PREC_FP32;
@@ -870,6 +307,12 @@ static int grad_state_create(const ns_problem* p, GradState* g) {
     return NS_OK;
 }
 
+static void grad_state_free(GradState* g) {
+    projection_adj_free(&g->proj);
+    for (void* q : g->owned) cudaFree(q);
+    delete g;
+}
+
 template <typename T>
 static int launch_finish_grad(const ns_problem* p, GradState* g, const T* gpre, int B, double* grad, cudaStream_t st) {
     auto kern = p->dims[0] <= 8 ? adj::k_finish_grad<T, 8> : adj::k_finish_grad<T, 32>;
@@ -883,6 +326,7 @@ static int launch_finish_grad(const ns_problem* p, GradState* g, const T* gpre, 
 static int run_grad_f64(const ns_problem* p, GradState* g, int B, double* logL, double* grad, cudaStream_t st) {
     const int L = p->n_layers, n_out = p->dims.back();
     const ShearParams& sp = p->sp;
+    NS_TRY(launch_projection_adj_windows<double>(sp, &g->proj, g->theta_full, g->d_nrows, B, st));
     const dim3 g0((p->dims[1] + 255) / 256, B);
     adj::k_emu_in_store<double><<<g0, 256, 0, st>>>(g->theta_full, p->P, p->d_inputs, p->d_in_center, p->d_in_scale,
                                                     p->dims[0], (const double*)p->d_W[0], (const double*)p->d_b[0],
@@ -900,8 +344,8 @@ static int run_grad_f64(const ns_problem* p, GradState* g, int B, double* logL, 
         NS_TRY(launch_zinterp_generic(p, g->table, g->table_fine, g->d_nrows, B, 8, st));
         tab = (const double*)g->table_fine;
     }
-    NS_TRY(launch_projection_adj<double>(sp, g->theta_full, tab, p->d_LinvT64, p->c0, (double*)g->scratch,
-                                         (double*)g->gtab, g->gfull, logL, g->d_nrows, B, st));
+    NS_TRY(launch_projection_adj<double>(sp, &g->proj, g->theta_full, tab, p->d_LinvT64, (const double*)g->Linv, p->c0,
+                                         TableGrad{g->gtab}, g->gfull, logL, g->d_nrows, B, g->d_err, st));
     // table adjoint -> emulator output adjoint (transpose of the z interpolation) -> g_pre_L
     const double* gt = (const double*)g->gtab;
     if (coarse) {
@@ -933,6 +377,7 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, double* log
         e.pitch = plane_pitch(width);
         e.plane_stride = g->rows_pad * e.pitch;
     };
+    NS_TRY(launch_projection_adj_windows<float>(sp, &g->proj, g->theta_full, g->d_nrows, B, st));
     NS_TRY(launch_emu_input_planes(p, g->theta_full, g->d_nrows, B, px, g->Hp[1],
                                    g->rows_pad * plane_pitch(p->dims[1]), st));
     for (int l = 1; l < L; ++l) {
@@ -956,8 +401,8 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, double* log
         NS_TRY(launch_zinterp_generic(p, g->table, g->table_fine, g->d_nrows, B, 4, st));
         tab = (const float*)g->table_fine;
     }
-    NS_TRY(launch_projection_adj<float>(sp, g->theta_full, tab, p->d_LinvT32, p->c0, (float*)g->scratch,
-                                        (float*)g->gtab, g->gfull, logL, g->d_nrows, B, st));
+    NS_TRY(launch_projection_adj<float>(sp, &g->proj, g->theta_full, tab, p->d_LinvT32, (const float*)g->Linv, p->c0,
+                                        TableGrad{g->gtab}, g->gfull, logL, g->d_nrows, B, g->d_err, st));
     // d log L / d (output pre-scaling) = sigma * d log L / d table
     const float* gt = (const float*)g->gtab;
     if (coarse) {
@@ -1027,8 +472,7 @@ extern "C" int loglike_grad_batch(const ns_problem* p, const double* theta_dev, 
             gs = new GradState();
             const int rc = grad_state_create(p, gs);
             if (rc != NS_OK) {
-                for (void* q : gs->owned) cudaFree(q);
-                delete gs;
+                grad_state_free(gs);
                 return rc;
             }
             g_grad_states.push_back(gs);
@@ -1047,8 +491,7 @@ void gpuns_release_grad_state(const ns_problem* p) {
     for (size_t i = 0; i < g_grad_states.size(); ++i) {
         GradState* s = g_grad_states[i];
         if (s->p != p) continue;
-        for (void* q : s->owned) cudaFree(q);
-        delete s;
+        grad_state_free(s);
         g_grad_states.erase(g_grad_states.begin() + i);
         return;
     }

@@ -172,13 +172,14 @@ int launch_cube_to_theta(const ns_problem* p, Workspace* ws, const double* cube,
 // the lensing/IA windows into `win` (rows x (nb + 1) x N); independent of the
 // emulator, so it may run on a second stream beside it.  Limber: P lookup,
 // Limber sums and the data vector; writes the residual d - m per row, or the
-// model vectors when model_out != nullptr.  FAST selects SFU transcendentals.
+// model vectors when model_out != nullptr, and into cl_out, when given, the
+// Limber sums C_ij(ell) themselves.  FAST selects SFU transcendentals.
 template <typename T, bool FAST>
 int launch_windows(const ShearParams& sp, const double* theta_full, T* win, const int* nrows, int grid_rows,
                    cudaStream_t st);
 template <typename T, bool FAST>
 int launch_limber(const ShearParams& sp, const double* theta_full, const T* table, const T* win, T* resid,
-                  double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st);
+                  double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st, T* cl_out = nullptr);
 // Whether both projection stages fit the shared memory of one CTA (elt = 4 or 8).
 bool projection_fits(const ShearParams& sp, int elt);
 // Whitened chi^2 and log L = c0 - chi^2 / 2 (projection.cu).  rows_ready: the
@@ -189,12 +190,6 @@ template <typename TR, typename TA>
 int launch_chi2(const TR* resid, int D, const TA* LinvT, double c0, double* logL, const int* nrows, int grid_rows,
                 cudaStream_t st, bool rows_ready = false);
 
-// Adjoint of the shear projection (adjoint.cu).
-int adjoint_scratch_elems(const ShearParams& sp);
-template <typename T>
-int launch_projection_adj(const ShearParams& sp, const double* theta_full, const T* table, const T* LinvT, double c0,
-                          T* scratch, T* gtab, double* gfull, double* logL, const int* nrows, int grid_rows,
-                          cudaStream_t st);
 int launch_free_to_full(const ns_problem* p, const double* theta, int B, double* theta_full, cudaStream_t st);
 int launch_zinterp_generic(const ns_problem* p, const void* coarse, void* fine, const int* nrows, int grid_rows,
                            int elt, cudaStream_t st);

@@ -437,7 +437,7 @@ template <typename T, int NB, bool FAST, int PKC>
 __global__ void __launch_bounds__(32 * kLimberWarps, sizeof(T) == 8 ? 1 : 2)
 k_limber(const ShearParams sp, const double* __restrict__ theta_full, const T* __restrict__ table,
          const T* __restrict__ win, T* __restrict__ resid, double* __restrict__ model_out,
-         const int* __restrict__ nrows, int* __restrict__ err) {
+         const int* __restrict__ nrows, int* __restrict__ err, T* __restrict__ cl_out) {
     using M = Math<T, FAST>;
     constexpr int NP = NB * (NB + 1) / 2;
     static_assert(2 * NP <= 32, "two multipoles of pair sums must fit one warp transpose");
@@ -605,6 +605,7 @@ k_limber(const ShearParams sp, const double* __restrict__ theta_full, const T* _
         if (lane < 2 * NP && l < n_ell) {
             // data vector (1 + m_i)(1 + m_j) C_ij(ell) + T b; residual d - m
             const int a = p * n_ell + l;
+            if (cl_out) cl_out[(size_t)row * sp.D + a] = cl;   // the adjoint keeps the Limber sums
             T m = (T(1) + thr[11 + NB + sp.pi[p]]) * (T(1) + thr[11 + NB + sp.pj[p]]) * cl;
             for (int t = 0; t < sp.n_tmpl; ++t) m += tm[(size_t)a * sp.n_tmpl + t] * thr[11 + 2 * NB + t];
             if (model_out) model_out[(size_t)row * sp.D + a] = (double)m;
@@ -905,7 +906,7 @@ static int windows_nb(const ShearParams& sp, const double* theta_full, T* win, c
 
 template <typename T, int NB, bool FAST, int PKC>
 static int limber_launch(const ShearParams& sp, const double* theta_full, const T* table, const T* win, T* resid,
-                         double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st) {
+                         double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st, T* cl_out) {
     const size_t smem = limber_smem<T>(sp);
     if (smem > kLimberSmemMax) return NS_ENOTSUP;
     static bool attr_done = false;
@@ -918,7 +919,7 @@ static int limber_launch(const ShearParams& sp, const double* theta_full, const 
     }
     const int warps = std::min(kLimberWarps, (sp.n_ell + 1) / 2);
     NS_CUDA_TRY(launch_pdl(k_limber<T, NB, FAST, PKC>, dim3(grid_rows), dim3(32 * warps), smem, st, sp, theta_full,
-                           table, win, resid, model_out, nrows, err));
+                           table, win, resid, model_out, nrows, err, cl_out));
     return NS_OK;
 }
 
@@ -928,13 +929,13 @@ static_assert(kPitch39 % 4 == 0, "padded rows stay 16-byte aligned");
 
 template <typename T, int NB, bool FAST>
 static int limber_nb(const ShearParams& sp, const double* theta_full, const T* table, const T* win, T* resid,
-                     double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st) {
+                     double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st, T* cl_out) {
     if constexpr (sizeof(T) == 4 && NB == 5) {
         if (limber_pitch(sp.n_k) == kPitch39)
             return limber_launch<T, NB, FAST, kPitch39>(sp, theta_full, table, win, resid, model_out, nrows,
-                                                        grid_rows, err, st);
+                                                        grid_rows, err, st, cl_out);
     }
-    return limber_launch<T, NB, FAST, 0>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st);
+    return limber_launch<T, NB, FAST, 0>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st, cl_out);
 }
 
 template <typename T, bool FAST>
@@ -952,13 +953,13 @@ int launch_windows(const ShearParams& sp, const double* theta_full, T* win, cons
 
 template <typename T, bool FAST>
 int launch_limber(const ShearParams& sp, const double* theta_full, const T* table, const T* win, T* resid,
-                  double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st) {
+                  double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st, T* cl_out) {
     switch (sp.nb) {
-        case 1: return limber_nb<T, 1, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st);
-        case 2: return limber_nb<T, 2, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st);
-        case 3: return limber_nb<T, 3, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st);
-        case 4: return limber_nb<T, 4, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st);
-        case 5: return limber_nb<T, 5, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st);
+        case 1: return limber_nb<T, 1, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st, cl_out);
+        case 2: return limber_nb<T, 2, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st, cl_out);
+        case 3: return limber_nb<T, 3, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st, cl_out);
+        case 4: return limber_nb<T, 4, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st, cl_out);
+        case 5: return limber_nb<T, 5, FAST>(sp, theta_full, table, win, resid, model_out, nrows, grid_rows, err, st, cl_out);
         default: return NS_ENOTSUP;
     }
 }
@@ -967,10 +968,10 @@ template int launch_windows<double, false>(const ShearParams&, const double*, do
 template int launch_windows<float, false>(const ShearParams&, const double*, float*, const int*, int, cudaStream_t);
 template int launch_windows<float, true>(const ShearParams&, const double*, float*, const int*, int, cudaStream_t);
 template int launch_limber<double, false>(const ShearParams&, const double*, const double*, const double*, double*,
-                                          double*, const int*, int, int*, cudaStream_t);
+                                          double*, const int*, int, int*, cudaStream_t, double*);
 template int launch_limber<float, false>(const ShearParams&, const double*, const float*, const float*, float*,
-                                         double*, const int*, int, int*, cudaStream_t);
+                                         double*, const int*, int, int*, cudaStream_t, float*);
 template int launch_limber<float, true>(const ShearParams&, const double*, const float*, const float*, float*,
-                                        double*, const int*, int, int*, cudaStream_t);
+                                        double*, const int*, int, int*, cudaStream_t, float*);
 
 }  // namespace gpuns
