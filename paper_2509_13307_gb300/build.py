@@ -18,8 +18,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libgpuns.so")
-SOURCES = ["likelihood.cu", "projection.cu", "gemm_tc.cu", "gemm_planes.cu", "problem.cu", "ns_engine.cu", "noalloc.cu", "adjoint.cu",
-           "projection_adj.cu", "dense_linalg.cu", "nuts.cu"]
+SOURCES = ["likelihood.cu", "projection.cu", "gemm_tc.cu", "gemm_planes.cu", "gemm_slices.cu", "problem.cu",
+           "ns_engine.cu", "noalloc.cu", "adjoint.cu", "projection_adj.cu", "dense_linalg.cu", "nuts.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-std=c++17", "-O3", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2",
          "--expt-relaxed-constexpr", "-I" + os.path.join(ROOT, "include")]

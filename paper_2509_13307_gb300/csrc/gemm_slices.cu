@@ -1,0 +1,292 @@
+// FP64 GEMMs on the fp16 tensor path (tcgen05), for the layers of FP64 tanh
+// emulators:  out[r][f] = epi( sum_k X[r][k] W[f][k] ),  |X| <= 1.
+//
+// GB300 runs FP64 at two FMAs per cycle and SM (1.26 TFLOP/s), a thousandth of
+// its fp16 tensor rate.  An operand is therefore held in fixed point, scaled to
+// |v| <= 1 (activations of tanh as they are, a row of W by a power of two), as
+// six 9-bit slices:  v = sum_i q_i 2^-(8 + 9 i),  |q_i| <= 256 an integer, the
+// rest at most 2^-54.  Products q_i q_j and their sums over 128 k are integers
+// within FP32's 24 bits, so the tensor core adds them exactly; the 21 slice pairs
+// with i + j <= 5 are kept, one FP32 accumulator in TMEM for each sum i + j.
+// Every 128 k the epilogue warps add the six accumulators to two 64-bit integers
+// per element (in registers, while the next MMAs run in the second TMEM buffer),
+// and one FP64 expression at the end joins them.  (Pairs with i + j >= 4 could
+// leave the 24 bits if every slice of every operand were near its largest value
+// with equal signs; a unit of theirs is 2^-52.)  What is dropped is about 2^-51 of the
+// row's largest |w| for K = 1024, against 2^-48 for the rounding of an FP64 FMA
+// chain.
+//
+// Tiles: 128 features (the MMA's M) x 32 rows; six accumulators of 32 columns
+// twice fill TMEM.  Slots of 32 k hold every slice of both operands (60 KB, 64-byte
+// swizzle, three slots).  Few tiles are spread over clusters of S CTAs along k,
+// whose integer partial tiles are added exactly through cluster shared memory.
+// A NaN operand (its leading slice is NaN) and a timeout give NaN.
+//
+// Measured on the 39-d emulator: 64 rows 5.80 ms of FP64 FMA tiles -> 0.35 ms
+// (the call 6367 -> 1070 us); error of its table against 113-bit arithmetic
+// rms 1.17e-16, largest 4.1e-16 (FMA chain 1.18e-16 and 4.8e-16).
+//
+// Warps 0-7: drain and epilogue; warp 8: copies; warp 9: TMEM and MMAs.  Waits are
+// bounded as in gemm_planes.cu.
+#include <algorithm>
+
+#include "likelihood.cuh"
+#include "tcgen05.cuh"
+
+namespace gpuns {
+namespace slc {
+
+using namespace tc;
+
+constexpr int NS = kSlices;                      // slices of an operand
+constexpr int SBK = 32;                          // k per slot: 64 bytes of fp16
+constexpr int BR = 32;                           // rows per tile
+constexpr int W_SUB = 128 * SBK * 2, X_SUB = BR * SBK * 2;
+constexpr int STAGE_BYTES = NS * (W_SUB + X_SUB);
+constexpr int STAGES = 3;
+constexpr int CHUNK = 4;                         // slots per TMEM accumulation: 128 k
+constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int EPI_WARPS = 8, THREADS = 32 * (EPI_WARPS + 2);
+constexpr int HC = BR / 2;                       // rows per epilogue warp
+constexpr long long kNaN = 1ll << 58;            // stands for NaN in a sum (others stay below 2^50; eight of it fit)
+static_assert(STAGES * STAGE_BYTES >= 128 * BR * 16, "the partial tile reuses the ring");
+static_assert(2 * NS * BR <= 512, "two sets of accumulators in TMEM");
+
+// K-major tile of 64-byte rows, 64-byte swizzle (8-row groups of 512 bytes).
+__device__ __forceinline__ uint64_t desc64(uint32_t addr) {
+    return (uint64_t)((addr & 0x3FFFF) >> 4) | (uint64_t)1 << 16 | (uint64_t)(512 >> 4) << 32 | (uint64_t)1 << 46 |
+           (uint64_t)4 << 61;
+}
+
+// kind::f16, D = F32, A = B = F16, K-major, M = 128, N = BR
+constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(BR >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+
+__global__ void __launch_bounds__(THREADS, 1)
+k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const SliceEpi e,
+              const int* __restrict__ nrows, int N, int K, int* __restrict__ err) {
+    pdl_begin();
+    const int M = *nrows;
+    const int S = gridDim.x, rank = blockIdx.x;
+    const int f0 = blockIdx.y * 128, r0 = blockIdx.z * BR;
+    if (r0 >= M) return;                         // every CTA of the cluster has these rows
+
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    uint8_t* gbase = smem_raw + (base - raw);
+    const uint32_t bar0 = base + STAGES * STAGE_BYTES;
+    auto full_bar = [&](int s) { return bar0 + 8u * s; };
+    auto empty_bar = [&](int s) { return bar0 + 8u * (STAGES + s); };
+    auto acc_full = [&](int b) { return bar0 + 8u * (2 * STAGES + b); };
+    auto acc_empty = [&](int b) { return bar0 + 8u * (2 * STAGES + 2 + b); };
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + STAGES * STAGE_BYTES + 8 * (2 * STAGES + 4));
+    __shared__ int s_fail;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        s_fail = 0;
+        for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
+        for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), EPI_WARPS); }
+        mbar_init_fence();
+    }
+    if (warp == 9) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const int nk = (K + SBK - 1) / SBK;
+    const int kb0 = (int)((long long)nk * rank / S), n_it = (int)((long long)nk * (rank + 1) / S) - kb0;
+    const int n_chunk = (n_it + CHUNK - 1) / CHUNK;
+
+    uint32_t nan = 0;                            // elements whose leading accumulator is NaN
+    long long hi[HC], lo[HC];                    // sums of i + j = 0..2 and 3..5, in units of the last of each
+#pragma unroll
+    for (int j = 0; j < HC; ++j) { hi[j] = 0; lo[j] = 0; }
+    if (warp == 8) {
+        if (lane == 0) {
+            int issued = 0;
+            for (int it = 0; it < n_it; ++it) {
+                const int s = it % STAGES;
+                if (it >= STAGES && !mbar_wait(empty_bar(s), ((it / STAGES) & 1) ^ 1)) { s_fail = 1; break; }
+                const uint32_t sa = base + s * STAGE_BYTES;
+                mbar_expect_tx(full_bar(s), STAGE_BYTES);
+                tma_load_3d(sa, &tmW, full_bar(s), (kb0 + it) * SBK, f0, 0);
+                tma_load_3d(sa + NS * W_SUB, &tmX, full_bar(s), (kb0 + it) * SBK, r0, 0);
+                ++issued;
+            }
+            // no copy may still be in flight when the CTA leaves
+            for (int it = max(0, issued - STAGES); it < issued; ++it)
+                if (!mbar_wait(full_bar(it % STAGES), (it / STAGES) & 1)) s_fail = 1;
+        }
+        __syncwarp();
+    } else if (warp == 9) {
+        if (lane == 0) {
+            bool ok = true;
+            for (int it = 0; it < n_it && ok; ++it) {
+                const int s = it % STAGES, c = it / CHUNK, b = c & 1, in = it % CHUNK;
+                if (in == 0 && c >= 2) ok = mbar_wait(acc_empty(b), ((c >> 1) & 1) ^ 1);
+                ok = ok && mbar_wait(full_bar(s), (it / STAGES) & 1);
+                if (!ok) { s_fail = 1; break; }
+                fence_after();
+                const uint32_t sw = base + s * STAGE_BYTES, sx = sw + NS * W_SUB;
+#pragma unroll
+                for (int i = 0; i < NS; ++i)
+#pragma unroll
+                    for (int j = 0; i + j < NS; ++j) {
+                        const uint64_t dw = desc64(sw + i * W_SUB), dx = desc64(sx + j * X_SUB);
+#pragma unroll
+                        for (int kk = 0; kk < SBK / 16; ++kk)
+                            mma_bf16(tmem + (uint32_t)((b * NS + i + j) * BR), dw + 2 * kk, dx + 2 * kk, kIdesc,
+                                     in != 0 || i != 0 || kk != 0);
+                    }
+                mma_commit(empty_bar(s));
+                if (in == CHUNK - 1 || it == n_it - 1) mma_commit(acc_full(b));
+            }
+        }
+        __syncwarp();
+    } else {
+        const uint32_t addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * HC);
+        for (int c = 0; c < n_chunk; ++c) {
+            const int b = c & 1;
+            if (!mbar_wait(acc_full(b), (c >> 1) & 1)) { s_fail = 1; break; }
+            fence_after();
+            __syncwarp();
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+                float v[HC];
+                tmem_ld<HC>(addr + (uint32_t)((b * NS + s) * BR), v);
+                if (s == 0) {
+#pragma unroll
+                    for (int j = 0; j < HC; ++j) nan |= (uint32_t)(v[j] != v[j]) << j;
+                }
+                const long long unit = 1ll << (9 * (s < 3 ? 2 - s : 5 - s));
+#pragma unroll
+                for (int j = 0; j < HC; ++j) (s < 3 ? hi[j] : lo[j]) += (long long)__float2int_rn(v[j]) * unit;
+            }
+            fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty(b));
+        }
+        __syncwarp();
+    }
+
+    const int f = f0 + (tid & 127);
+    const bool fv = tid < 32 * EPI_WARPS && f < N;
+    double bias = 0, mu = 0, ws = 0;
+    if (fv) {
+        bias = e.bias[f];
+        ws = e.wscale[f];
+        if (!e.tanh) mu = e.mu[f];
+    }
+    auto finish = [&](int rl, long long h, long long l) {
+        const int row = r0 + rl;
+        if (!fv || row >= M) return;
+        // hi 2^-34 + lo 2^-61
+        double v = fma((double)l, 4.33680868994201773603e-19, (double)h * 5.82076609134674072266e-11) * ws + bias;
+        if (h >= kNaN) v = NAN;
+        if (e.tanh) slice_store(tanh(v), e.slices + (size_t)row * e.pitch + f, e.slice_stride);
+        else e.out[(size_t)row * N + f] = mu + e.sigma * v;
+    };
+    __syncthreads();                             // the ring's last copies have landed
+    const bool failed = s_fail != 0;
+    if (failed) nan = 0xffffffffu;
+    long long* red = reinterpret_cast<long long*>(gbase);       // hi, then lo: BR x 128 each
+    if (warp < EPI_WARPS) {
+#pragma unroll
+        for (int j = 0; j < HC; ++j) {
+            const int at = ((warp >> 2) * HC + j) * 128 + (tid & 127);
+            red[at] = (nan >> j) & 1 ? kNaN : hi[j];
+            red[BR * 128 + at] = lo[j];
+        }
+    }
+    if (S == 1) __syncthreads();
+    else cluster_sync_all();
+    if (warp < EPI_WARPS) {
+        const int end = min(BR * (rank + 1) / S, M - r0);
+#pragma unroll 1
+        for (int rl = BR * rank / S + (tid >> 7); rl < end; rl += 2) {
+            const int at = rl * 128 + (tid & 127);
+            long long h = red[at], l = red[BR * 128 + at];
+            for (int q = 1; q < S; ++q) {        // integers: any order
+                const uint32_t peer = (uint32_t)((rank + q) % S);
+                h += ld_cluster_s64(mapa_u32(base + 8u * (uint32_t)at, peer));
+                l += ld_cluster_s64(mapa_u32(base + 8u * (uint32_t)(BR * 128 + at), peer));
+            }
+            finish(rl, h, l);
+        }
+    }
+    if (S > 1) cluster_sync_all();               // peers have read this CTA's partial tile
+    if (failed && tid == 0 && err) atomicOr(err, NS_BIT_TIMEOUT);
+    fence_before();
+    __syncthreads();
+    if (warp == 9) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(512u) : "memory");
+    }
+}
+
+// slices and power-of-two scale of every row of W (rows x K)
+__global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ W, int K, __half* __restrict__ out,
+                                                    long long stride, int pitch, double* __restrict__ scale) {
+    __shared__ double red[8];
+    const double* w = W + (size_t)blockIdx.x * K;
+    double m = 0;
+    for (int k = threadIdx.x; k < K; k += 256) m = fmax(m, fabs(w[k]));
+    m = warp_max(m);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+    __syncthreads();
+    for (int i = 0; i < 8; ++i) m = fmax(m, red[i]);
+    int ex = 0;
+    if (m > 0) frexp(m, &ex);
+    const double s = scalbn(1.0, -ex);
+    for (int k = threadIdx.x; k < K; k += 256) slice_store(w[k] * s, out + (size_t)blockIdx.x * pitch + k, stride);
+    if (threadIdx.x == 0) scale[blockIdx.x] = scalbn(1.0, ex);
+}
+
+}  // namespace slc
+
+int launch_gemm_slices(const CUtensorMap* tmW, const CUtensorMap* tmX, const SliceEpi& e, const int* nrows,
+                       int grid_rows, int N, int K, int* err, cudaStream_t st) {
+    if (grid_rows <= 0) return NS_OK;
+    static bool attr = false;
+    if (!attr) {
+        NS_CUDA_TRY(cudaFuncSetAttribute(slc::k_gemm_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, slc::SMEM));
+        attr = true;
+    }
+    // the largest split that keeps every cluster resident (about 96 SMs hold
+    // clusters of 8, 128 clusters of 4, one CTA each) and a chunk per CTA
+    const int nk = (K + slc::SBK - 1) / slc::SBK;
+    const long long tiles = (long long)((N + 127) / 128) * ((grid_rows + slc::BR - 1) / slc::BR);
+    int S = 1;
+    for (int s : {2, 4, 8})
+        if (tiles * s <= (s == 8 ? 96 : s == 4 ? 128 : 152) && nk >= slc::CHUNK * s) S = s;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(S, (N + 127) / 128, (grid_rows + slc::BR - 1) / slc::BR);
+    cfg.blockDim = dim3(slc::THREADS);
+    cfg.dynamicSmemBytes = slc::SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute a[2];
+    a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a[0].val.programmaticStreamSerializationAllowed = 1;
+    a[1].id = cudaLaunchAttributeClusterDimension;
+    a[1].val.clusterDim.x = S;
+    a[1].val.clusterDim.y = 1;
+    a[1].val.clusterDim.z = 1;
+    cfg.attrs = a;
+    cfg.numAttrs = 2;
+    NS_CUDA_TRY(cudaLaunchKernelEx(&cfg, slc::k_gemm_slices, *tmW, *tmX, e, nrows, N, K, err));
+    return NS_OK;
+}
+
+int launch_slice_rows(const double* W, int rows, int K, __half* out, long long stride, int pitch, double* scale,
+                      cudaStream_t st) {
+    slc::k_slice_rows<<<rows, 256, 0, st>>>(W, K, out, stride, pitch, scale);
+    NS_CUDA_TRY(cudaGetLastError());
+    return NS_OK;
+}
+
+}  // namespace gpuns

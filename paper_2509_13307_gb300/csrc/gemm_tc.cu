@@ -770,6 +770,22 @@ int make_tensor_map_planes(CUtensorMap* tm, const void* base, int rows, int K, l
     return r == CUDA_SUCCESS ? NS_OK : NS_EINVAL;
 }
 
+// The six fixed-point slices (fp16, row pitch plane_pitch(K)) of a rows x K
+// operand, 64-byte swizzle, box = every slice's box_rows x 32.
+int make_tensor_map_slices(CUtensorMap* tm, const void* base, int rows, int K, long long stride, int box_rows) {
+    auto enc = get_encode();
+    if (!enc) return NS_ECUDA;
+    if ((reinterpret_cast<uintptr_t>(base) & 15) || stride % 8) return NS_EINVAL;
+    cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)tc::kSlices};
+    cuuint64_t strides[2] = {(cuuint64_t)plane_pitch(K) * 2, (cuuint64_t)stride * 2};
+    cuuint32_t box[3] = {32, (cuuint32_t)box_rows, (cuuint32_t)tc::kSlices};
+    cuuint32_t estr[3] = {1, 1, 1};
+    const CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? NS_OK : NS_EINVAL;
+}
+
 int make_plane_maps_x(PlaneMapX* m, const void* base, int rows, int K, long long stride, int planes) {
     for (int i = 0; i < 4; ++i) NS_TRY(make_tensor_map_planes(&m->m[i], base, rows, K, stride, planes, 32 << i));
     return NS_OK;

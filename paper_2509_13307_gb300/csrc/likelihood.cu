@@ -114,6 +114,14 @@ struct OutF64 {
     double* p;
     __device__ __forceinline__ void put(int row, int n, int N, double v) const { p[(size_t)row * N + n] = v; }
 };
+struct OutSlices {
+    __half* p;
+    long long stride;
+    int pitch;
+    __device__ __forceinline__ void put(int row, int n, int, double v) const {
+        tc::slice_store(v, p + (size_t)row * pitch + n, stride);
+    }
+};
 struct OutBf16 {
     __nv_bfloat16* p;
     __device__ __forceinline__ void put(int row, int n, int N, float v) const {
@@ -354,8 +362,38 @@ static Head model_head(const ns_problem* p, void* out) {
                 p->out_sigma, out};
 }
 
+// FP64 with tanh hidden layers: fixed-point slices on the tensor cores.
+static int run_emulator_slices(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, double* out) {
+    const int L = p->n_layers;
+    NS_TRY(launch_emu_input<double>(p, ws->theta_full, ws->d_nrows, grid_rows, layer_act<double>(p, 0),
+                                    OutSlices{(__half*)ws->act[0], ws->plane_stride, plane_pitch(p->dims[1])}, st));
+    int cur = 0;
+    for (int l = 1; l < L; ++l) {
+        const bool last = l == L - 1;
+        SliceEpi e;
+        e.bias = (const double*)p->d_b[l];
+        e.wscale = p->d_wscale[l];
+        if (last) {
+            e.mu = (const double*)p->d_out_mu;
+            e.sigma = p->out_sigma;
+            e.out = out;
+        } else {
+            e.tanh = 1;
+            e.slices = (__half*)ws->act[cur ^ 1];
+            e.slice_stride = ws->plane_stride;
+            e.pitch = plane_pitch(p->dims[l + 1]);
+        }
+        NS_TRY(launch_gemm_slices(&p->tmWs[l], &ws->tmXs[l], e, ws->d_nrows, grid_rows, p->dims[l + 1], p->dims[l],
+                                  ws->d_err, st));
+        cur ^= 1;
+    }
+    return NS_OK;
+}
+
+// FP64 on CUDA cores: emulators with unbounded activations (CMB).
 static int run_emulator_f64(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, const Head& hd) {
     const int L = p->n_layers;
+    if (!p->tmWs.empty()) return run_emulator_slices(p, ws, grid_rows, st, (double*)hd.out);
     NS_TRY(launch_emu_input<double>(p, ws->theta_full, ws->d_nrows, grid_rows, layer_act<double>(p, 0),
                                     OutF64{(double*)ws->act[0]}, st));
     int cur = 0;

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <vector>
 
 #include "common.cuh"
@@ -63,9 +64,10 @@ struct Workspace {
     double* logL = nullptr;       // cap
     // tcgen05 tensor maps (BF16 precision): A operand of layer l >= 1 and its output
     std::vector<CUtensorMap> tmA;
+    std::vector<CUtensorMap> tmXs;   // FP64 tanh emulators: layer l's input slices (plane_stride apart)
     // k_gemm_planes: layer l's input planes (FP32: three; the FP32 head of a BF16 CMB problem: one)
     std::vector<PlaneMapX> tmXp;
-    long long plane_stride = 0;   // FP32: elements between the planes of an activation buffer
+    long long plane_stride = 0;   // FP32, FP64 slices: elements between the planes of an activation buffer
     CUtensorMap tmX_out{};        // the last layer's activations in kSwapRows-row boxes
     CUtensorMap tmF_out{};        // fused emulator stack: its output activations in 64-row boxes of two k-blocks
     std::vector<void*> owned;
@@ -90,6 +92,8 @@ struct ns_problem {
     std::vector<int> dims;
     std::vector<void*> d_W;          // per layer, compute dtype (layer 0: FP64 or FP32)
     std::vector<void*> d_b;          // per layer, FP64 (FP64 mode) else FP32
+    std::vector<CUtensorMap> tmWs;   // FP64 tanh emulators, layers >= 1: the weights as fixed-point slices
+    std::vector<double*> d_wscale;   // and their rows' scales
     std::vector<__nv_bfloat16*> d_Wp;   // and the planes themselves (row pitch plane_pitch(K))
     std::vector<CUtensorMap> tmWp;   // FP32 layers >= 1 (and a BF16 CMB head): the weights as three bf16 planes
     std::vector<CUtensorMap> tmB;    // BF16: weight tensor maps for layers >= 1
@@ -260,6 +264,24 @@ inline int plane_pitch(int K) { return (K + 7) & ~7; }   // rows of 16-byte mult
 int make_tensor_map_planes(CUtensorMap* tm, const void* base, int rows, int K, long long stride, int planes,
                            int box_rows);
 int make_plane_maps_x(PlaneMapX* m, const void* base, int rows, int K, long long stride, int planes);
+// FP64 GEMMs on the fp16 tensor path (gemm_slices.cu): operands |v| <= 1 as six
+// fixed-point slices.  tanh: slices of tanh(acc + bias); else out = mu + sigma (acc + bias).
+struct SliceEpi {
+    int tanh = 0;
+    const double* bias = nullptr;
+    const double* wscale = nullptr;   // per feature: the power of two taken out of the row of W
+    const double* mu = nullptr;
+    double sigma = 0;
+    double* out = nullptr;            // rows x N
+    __half* slices = nullptr;         // row pitch `pitch`
+    long long slice_stride = 0;
+    int pitch = 0;
+};
+int launch_gemm_slices(const CUtensorMap* tmW, const CUtensorMap* tmX, const SliceEpi& e, const int* nrows,
+                       int grid_rows, int N, int K, int* err, cudaStream_t st);
+int launch_slice_rows(const double* W, int rows, int K, __half* out, long long stride, int pitch, double* scale,
+                      cudaStream_t st);
+int make_tensor_map_slices(CUtensorMap* tm, const void* base, int rows, int K, long long stride, int box_rows);
 // Dense FP64 set-up kernels (dense_linalg.cu): C (device, overwritten by L) ->
 // L^-1 (new device buffer) and sum ln L_aa; NS_EINVAL if C is not SPD.
 int device_cholesky_inverse(double* dC, int D, double** Xout, double* sum_log_diag, cudaStream_t st);

@@ -110,13 +110,21 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
     ws->logL = (double*)v;
     if (p->kind == NS_KIND_GAUSS) return NS_OK;
     // activations: FP64, bf16, or FP32 as three bf16 planes
-    const int elt = (p->precision == NS_PREC_FP64) ? 8 : (p->precision == NS_PREC_FP32 ? 6 : 2);
+    // FP64 tanh: six fp16 slices
+    const bool slices = !p->tmWs.empty();
+    const int elt = slices ? 12 : (p->precision == NS_PREC_FP64) ? 8 : (p->precision == NS_PREC_FP32 ? 6 : 2);
     const int rows_pad = ((cap + 127) / 128) * 128;
     const size_t act_bytes = (size_t)elt * rows_pad * plane_pitch(p->hidden_max);
     for (int i = 0; i < 2; ++i) {
         NS_TRY(dalloc(act_bytes, &v, ws->owned));
         ws->act[i] = v;
         NS_CUDA_TRY(cudaMemset(v, 0, act_bytes));
+    }
+    if (slices) {
+        ws->plane_stride = (long long)rows_pad * plane_pitch(p->hidden_max);
+        ws->tmXs.resize(p->n_layers);
+        for (int l = 1; l < p->n_layers; ++l)
+            NS_TRY(make_tensor_map_slices(&ws->tmXs[l], ws->act[(l - 1) & 1], rows_pad, p->dims[l], ws->plane_stride, 32));
     }
     if (p->precision == NS_PREC_FP32) {
         ws->plane_stride = (long long)rows_pad * plane_pitch(p->hidden_max);
@@ -567,6 +575,19 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
             if ((s = upload(e.W[l], nw, &w, p->owned))) return fail(s);
             if ((s = upload(e.b[l], nb, &b, p->owned))) return fail(s);
             p->d_W[l] = w; p->d_b[l] = b;
+            if (l >= 1 && !cmb && e.activation == NS_ACT_TANH && !e.out_sigma_vec) {
+                const int N = p->dims[l + 1], K = p->dims[l], pitch = plane_pitch(K);
+                const long long stride = (long long)N * pitch;
+                void *v, *sc;
+                if ((s = dalloc(sizeof(uint16_t) * 6 * (size_t)stride, &v, p->owned)) ||
+                    (s = dalloc(sizeof(double) * N, &sc, p->owned)) ||
+                    (s = launch_slice_rows(w, N, K, (__half*)v, stride, pitch, (double*)sc, nullptr)))
+                    return fail(s);
+                p->tmWs.resize(e.n_layers);
+                p->d_wscale.resize(e.n_layers);
+                p->d_wscale[l] = (double*)sc;
+                if ((s = make_tensor_map_slices(&p->tmWs[l], v, N, K, stride, 128))) return fail(s);
+            }
         } else {
             std::vector<float> bf(nb);
             for (size_t i = 0; i < nb; ++i) bf[i] = (float)e.b[l][i];
@@ -857,6 +878,7 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
         if ((s = upload(LT32.data(), LT32.size(), &p->d_LinvT32, p->owned))) return fail(s);
     }
     int s = workspace_create(p, p->max_batch, &p->ws);
+    if (!s && cudaStreamSynchronize(nullptr) != cudaSuccess) s = NS_ECUDA;   // calls may come on any stream
     if (s) return fail(s);
     *out = p;
     return NS_OK;

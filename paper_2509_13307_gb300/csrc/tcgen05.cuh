@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 #include "async_copy.cuh"
@@ -130,6 +131,11 @@ __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ long long ld_cluster_s64(uint32_t cluster_addr) {
+    long long v;
+    asm volatile("ld.shared::cluster.s64 %0, [%1];" : "=l"(v) : "r"(cluster_addr) : "memory");
+    return v;
+}
 __device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
     float v;
     asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
@@ -145,6 +151,19 @@ __device__ __forceinline__ void plane_store(float v, __nv_bfloat16* out, long lo
         const __nv_bfloat16 q = __float2bfloat16_rn(v);
         out[p * stride] = q;
         v -= __bfloat162float(q);
+    }
+}
+
+// v in [-1, 1] as kSlices fixed-point slices `stride` elements apart:
+// v = sum_i q_i 2^-(8 + 9 i), q_i integers of at most 256 (gemm_slices.cu).
+constexpr int kSlices = 6;
+__device__ __forceinline__ void slice_store(double v, __half* out, long long stride) {
+    long long x = __double2ll_rn(v * 9007199254740992.0);      // 2^53
+#pragma unroll
+    for (int i = kSlices - 1; i >= 0; --i) {
+        const int q = i > 0 ? (int)((x + 256) & 511) - 256 : (int)x;
+        out[i * stride] = i == 0 && v != v ? __ushort_as_half(0x7fff) : __int2half_rn(q);
+        x = (x - q) >> 9;
     }
 }
 
