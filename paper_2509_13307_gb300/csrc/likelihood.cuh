@@ -34,6 +34,13 @@ struct ShearParams {
     const int* pj;
     const double* data;   // D
     const double* tmpl;   // D x n_tmpl
+    // theta-independent functions of the scale factor: 1/a at the nodes, and at
+    // the 4 Gauss-Legendre points of each interval [n][4] the triples
+    // (1/a, ln a, 1 - a) as separate arrays; ln of the IA pivot
+    const double *ia, *gl_ia, *gl_ln, *gl_1ma;
+    const float *ia_f, *gl_ia_f, *gl_ln_f, *gl_1ma_f;
+    double ln_pivot;
+    float ln_pivot_f;
     // FP32 copies read by the float kernels (GB300 runs FP64, conversions
     // included, at a small fraction of its FP32 rate, so float kernels take no
     // per-thread double -> float conversions)

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "likelihood.cuh"
+#include "tcgen05.cuh"
 
 static thread_local char g_last_err[512] = {0};
 
@@ -47,14 +48,6 @@ static int dalloc(size_t bytes, void** dev, std::vector<void*>& owned) {
     if (cudaMalloc(dev, bytes) != cudaSuccess) return NS_ENOMEM;
     owned.push_back(*dev);
     return NS_OK;
-}
-
-static uint16_t f32_to_bf16_rne(float f) {
-    uint32_t u;
-    std::memcpy(&u, &f, 4);
-    if ((u & 0x7f800000u) == 0x7f800000u) return (uint16_t)(u >> 16);   // inf / nan
-    u += 0x7fffu + ((u >> 16) & 1u);
-    return (uint16_t)(u >> 16);
 }
 
 // Catmull-Rom taps of coordinate s on a uniform grid [lo, lo + (n-1) step], ghosts folded.
@@ -220,30 +213,60 @@ static int upload_compute(const ns_problem* p, const double* h, size_t n, void**
     return NS_OK;
 }
 
-// An FP32 matrix (rows x K) on the device as three bf16 planes and their
-// tensor map (the weights of k_gemm_planes).
-static int make_planes(const float* d, int rows, int K, CUtensorMap* tm, __nv_bfloat16** planes,
-                       std::vector<void*>& owned) {
+// Weight matrices go to the device once as FP64 (reused staging) and are
+// converted there; the null stream orders the copies and the conversions.
+struct Staging {
+    double* d = nullptr;
+    size_t cap = 0;
+    ~Staging() { cudaFree(d); }
+    int put(const double* h, size_t n) {
+        if (n > cap) {
+            cudaFree(d);
+            d = nullptr;
+            cap = 0;
+            if (cudaMalloc((void**)&d, n * sizeof(double)) != cudaSuccess) return NS_ENOMEM;
+            cap = n;
+        }
+        NS_CUDA_TRY(cudaMemcpy(d, h, n * sizeof(double), cudaMemcpyHostToDevice));
+        return NS_OK;
+    }
+};
+
+__global__ void k_to_bf16(const double* __restrict__ in, size_t n, __nv_bfloat16* __restrict__ out) {
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+        out[i] = __float2bfloat16_rn((float)in[i]);
+}
+
+// the FP32 values of a rows x K matrix as three bf16 planes (row pitch `pitch`)
+__global__ void k_to_planes(const double* __restrict__ in, int rows, int K, __nv_bfloat16* __restrict__ out,
+                            long long stride, int pitch) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= K) return;
+    for (int r = blockIdx.y; r < rows; r += gridDim.y)
+        tc::plane_store<3>((float)in[(size_t)r * K + k], out + (size_t)r * pitch + k, stride);
+}
+
+// bf16 copy of a host FP64 matrix (rounded through FP32)
+static int upload_bf16(const double* h, size_t n, Staging* st, void** out, std::vector<void*>& owned) {
+    NS_TRY(st->put(h, n));
+    NS_TRY(dalloc(n * 2, out, owned));
+    k_to_bf16<<<(int)std::min<size_t>((n + 255) / 256, 4096), 256>>>(st->d, n, (__nv_bfloat16*)*out);
+    NS_CUDA_TRY(cudaGetLastError());
+    return NS_OK;
+}
+
+// a host FP64 matrix as the planes and tensor map of k_gemm_planes' weights
+static int upload_planes(const double* h, int rows, int K, Staging* st, CUtensorMap* tm, __nv_bfloat16** planes,
+                         std::vector<void*>& owned) {
     const int pitch = plane_pitch(K);
     const long long stride = (long long)rows * pitch;
     void* v = nullptr;
+    NS_TRY(st->put(h, (size_t)rows * K));
     NS_TRY(dalloc(sizeof(uint16_t) * 3 * (size_t)stride, &v, owned));
     if (planes) *planes = (__nv_bfloat16*)v;
-    NS_TRY(launch_split_planes(3, d, 1.f, rows, K, (__nv_bfloat16*)v, stride, pitch, nullptr, nullptr));
-    NS_CUDA_TRY(cudaStreamSynchronize(nullptr));   // calls may come on any stream
+    k_to_planes<<<dim3((K + 255) / 256, std::min(rows, 16384)), 256>>>(st->d, rows, K, (__nv_bfloat16*)v, stride, pitch);
+    NS_CUDA_TRY(cudaGetLastError());
     return make_tensor_map_planes(tm, v, rows, K, stride, 3, 128);
-}
-
-// FP32 copy of a host FP64 matrix as planes only; the copy is freed again.
-static int upload_planes(const double* h, int rows, int K, CUtensorMap* tm, __nv_bfloat16** planes,
-                         std::vector<void*>& owned) {
-    std::vector<float> f(h, h + (size_t)rows * K);
-    std::vector<void*> tmp;
-    float* d = nullptr;
-    int s = upload(f.data(), f.size(), &d, tmp);
-    if (!s) s = make_planes(d, rows, K, tm, planes, owned);
-    for (void* q : tmp) cudaFree(q);
-    return s;
 }
 
 // CMB set-up: FP64 factorisation of the covariance (host for D <= 256, else
@@ -251,6 +274,7 @@ static int upload_planes(const double* h, int rows, int K, CUtensorMap* tm, __nv
 // literal per-evaluation whitening or the fold of the linear head:
 // W' = L^-1 diag(sigma) W_out, c' = L^-1 (d - mu - sigma b_out).
 static int cmb_setup(ns_problem* p, const ns_problem_desc* desc) {
+    Staging staging;
     p->cmb_solve = desc->cmb.solve;
     p->cmb_form = desc->cmb.form;
     if (!p->has_lik) return NS_OK;
@@ -361,7 +385,7 @@ static int cmb_setup(ns_problem* p, const ns_problem_desc* desc) {
         done(NS_OK);
     }
     if (p->precision == NS_PREC_FP64) NS_TRY(upload_compute(p, Wf.data(), Wf.size(), &p->d_Wfold, p->owned));
-    else NS_TRY(upload_planes(Wf.data(), D, H, &p->tmWfold, nullptr, p->owned));
+    else NS_TRY(upload_planes(Wf.data(), D, H, &staging, &p->tmWfold, nullptr, p->owned));
     NS_TRY(upload_compute(p, cf.data(), cf.size(), &p->d_cfold, p->owned));
     return NS_OK;
 }
@@ -562,6 +586,7 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
     }
     p->d_W.assign(e.n_layers, nullptr);
     p->d_b.assign(e.n_layers, nullptr);
+    Staging staging;
     if (!f64) {
         p->tmWp.resize(e.n_layers);
         p->d_Wp.assign(e.n_layers, nullptr);
@@ -595,13 +620,10 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
             if ((s = upload(bf.data(), nb, &b, p->owned))) return fail(s);
             p->d_b[l] = b;
             if (tc_layer(l)) {
-                std::vector<uint16_t> wb(nw);
-                for (size_t i = 0; i < nw; ++i) wb[i] = f32_to_bf16_rne((float)e.W[l][i]);
-                uint16_t* w;
-                if ((s = upload(wb.data(), nw, &w, p->owned))) return fail(s);
-                p->d_W[l] = w;
+                if ((s = upload_bf16(e.W[l], nw, &staging, &p->d_W[l], p->owned))) return fail(s);
             } else if (l >= 1) {
-                if ((s = upload_planes(e.W[l], p->dims[l + 1], p->dims[l], &p->tmWp[l], &p->d_Wp[l], p->owned)))
+                if ((s = upload_planes(e.W[l], p->dims[l + 1], p->dims[l], &staging, &p->tmWp[l], &p->d_Wp[l],
+                                       p->owned)))
                     return fail(s);
             } else {
                 std::vector<float> wf(nw);
@@ -728,6 +750,7 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
     if (cmb) {
         int s = cmb_setup(p, desc);
         if (!s) s = workspace_create(p, p->max_batch, &p->ws);
+        if (!s && cudaStreamSynchronize(nullptr) != cudaSuccess) s = NS_ECUDA;   // calls may come on any stream
         if (s) return fail(s);
         *out = p;
         return NS_OK;
@@ -814,6 +837,35 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
                 (s = upload(z4f.data(), 4 * N, &dz4f, p->owned)))
                 return fail(s);
             sp.zrp = dzr; sp.zw4d = dz4; sp.zw4f = dz4f;
+        }
+        {
+            const double glx[4] = {-0.86113631159405257522, -0.33998104358485626480, 0.33998104358485626480,
+                                   0.86113631159405257522};
+            std::vector<double> ia(N), g1(4 * N, 1.0), g2(4 * N, 0.0), g3(4 * N, 0.0);
+            for (int n = 0; n < N; ++n) {
+                ia[n] = 1.0 / a[n];
+                for (int g = 0; n < N - 1 && g < 4; ++g) {
+                    const double ag = 0.5 * (a[n] + a[n + 1]) + 0.5 * (a[n] - a[n + 1]) * glx[g];
+                    g1[4 * n + g] = 1.0 / ag;
+                    g2[4 * n + g] = std::log(ag);
+                    g3[4 * n + g] = 1.0 - ag;
+                }
+            }
+            auto both = [&](const std::vector<double>& v, const double** d, const float** f) {
+                std::vector<float> vf(v.begin(), v.end());
+                double* dd;
+                float* df;
+                int e = upload(v.data(), v.size(), &dd, p->owned);
+                if (!e) e = upload(vf.data(), vf.size(), &df, p->owned);
+                *d = dd;
+                *f = df;
+                return e;
+            };
+            if ((s = both(ia, &sp.ia, &sp.ia_f)) || (s = both(g1, &sp.gl_ia, &sp.gl_ia_f)) ||
+                (s = both(g2, &sp.gl_ln, &sp.gl_ln_f)) || (s = both(g3, &sp.gl_1ma, &sp.gl_1ma_f)))
+                return fail(s);
+            sp.ln_pivot = std::log(sd.ia_pivot);
+            sp.ln_pivot_f = (float)sp.ln_pivot;
         }
         sp.nz_mean = dmu; sp.nz_sigma = dsg; sp.pi = dpi; sp.pj = dpj; sp.data = ddata; sp.tmpl = dtm;
         {

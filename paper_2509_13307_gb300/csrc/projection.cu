@@ -55,13 +55,13 @@ template <> __device__ __forceinline__ float pick_s<float>(double, float f) { re
 // Transcendentals: accurate library versions, or (FAST, BF16 modes) the SFU
 // approximations, whose ~1e-6 relative error is far below the bf16 emulator's.
 template <typename T, bool FAST> struct Math;
-// div / rsq: IEEE quotient and 1/sqrt, or (FAST) the SFU reciprocal forms.
+// div / rsq: IEEE quotient and 1/sqrt to an ulp, or (FAST) the SFU reciprocal forms.
 template <> struct Math<double, false> {
     static __device__ __forceinline__ double ex(double x) { return exp(x); }
     static __device__ __forceinline__ double lg(double x) { return log(x); }
     static __device__ __forceinline__ double p10(double v) { return exp(v * kLn10); }
     static __device__ __forceinline__ double div(double a, double b) { return a / b; }
-    static __device__ __forceinline__ double rsq(double x) { return 1.0 / sqrt(x); }
+    static __device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
 };
 template <> struct Math<float, false> {
     static __device__ __forceinline__ float ex(float x) { return expf(x); }
@@ -69,7 +69,10 @@ template <> struct Math<float, false> {
     static __device__ __forceinline__ float p10(float v) { return exp2f(v * 3.32192809488736234787f); }
     static __device__ __forceinline__ float e2(float v) { return exp2f(v); }
     static __device__ __forceinline__ float div(float a, float b) { return a / b; }
-    static __device__ __forceinline__ float rsq(float x) { return 1.f / sqrtf(x); }
+    static __device__ __forceinline__ float rsq(float x) {   // one Newton step on the SFU value
+        const float y = rsqrtf(x);
+        return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
+    }
 };
 template <> struct Math<float, true> {
     static __device__ __forceinline__ float ex(float x) { return __expf(x); }
@@ -159,6 +162,13 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
     const T* lna_ = pick<T>(sp.lna, sp.lna_f);
     const T* z_ = pick<T>(sp.z, sp.z_f);
     const T* wa_ = pick<T>(sp.wa, sp.wa_f);
+    // the accurate forms read the functions of the scale factor alone (1/a, and
+    // 1/a, ln a, 1 - a at the quadrature points) from tables made once, and share
+    // reciprocals: 64 evaluations in FP64 290 -> 180 us, 500 in FP32 56 -> 40 us
+    const T* ia_ = pick<T>(sp.ia, sp.ia_f);
+    const T* gl_ia = pick<T>(sp.gl_ia, sp.gl_ia_f);
+    const T* gl_ln = pick<T>(sp.gl_ln, sp.gl_ln_f);
+    const T* gl_1ma = pick<T>(sp.gl_1ma, sp.gl_1ma_f);
     const int tid = threadIdx.x, nt = kProjThreads;
     const int lane = tid & 31, wid = tid >> 5;
     (void)lane;
@@ -175,7 +185,9 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
     // 1. background: E(a), chi by composite 4-point Gauss-Legendre + scan, growth
     for (int n = tid; n < N; n += nt) {
         const T a = a_[n], lna = lna_[n];
-        const T e2 = om * M::ex(T(-3) * lna) + (T(1) - om) * M::ex(-pde * lna - T(3) * wa * (T(1) - a));
+        const T ian = FAST ? T(0) : ia_[n];
+        const T a3 = FAST ? M::ex(T(-3) * lna) : ian * ian * ian;
+        const T e2 = om * a3 + (T(1) - om) * M::ex(-pde * lna - T(3) * wa * (T(1) - a));
         Ez[n] = sqrt_<T>(e2);
         T inc = T(0);
         if (n < N - 1) {
@@ -184,9 +196,10 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
                 const T ag = mid + half * gl4_x<T>(g);
-                const T lg = M::lg(ag);
-                const T ia = M::div(T(1), ag);
-                const T eg = om * ia * ia * ia + (T(1) - om) * M::ex(-pde * lg - T(3) * wa * (T(1) - ag));
+                const T lg = FAST ? M::lg(ag) : gl_ln[4 * n + g];
+                const T ia = FAST ? M::div(T(1), ag) : gl_ia[4 * n + g];
+                const T oma = FAST ? T(1) - ag : gl_1ma[4 * n + g];
+                const T eg = om * ia * ia * ia + (T(1) - om) * M::ex(-pde * lg - T(3) * wa * oma);
                 inc += gl4_w<T>(g) * ia * ia * M::rsq(eg);
             }
             inc *= chiH * half;
@@ -199,9 +212,10 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
         const T c = t0[n];
         chi[n] = c;
         lnchi[n] = (n >= 1) ? M::lg(c) : T(0);
-        const T oma = M::div(om * M::ex(T(-3) * lna_[n]), Ez[n] * Ez[n]);
+        const T ian = FAST ? T(0) : ia_[n];
+        const T oma = M::div(om * (FAST ? M::ex(T(-3) * lna_[n]) : ian * ian * ian), Ez[n] * Ez[n]);
         t1[n] = M::ex(gamma * M::lg(oma));
-        omw[n] = M::div(wa_[n] * chiH, a_[n] * a_[n] * Ez[n]);
+        omw[n] = FAST ? M::div(wa_[n] * chiH, a_[n] * a_[n] * Ez[n]) : M::div(wa_[n] * chiH * (ian * ian), Ez[n]);
     }
     __syncthreads();
     for (int n = tid; n < N; n += nt)
@@ -224,10 +238,10 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
         isg[i] = M::div(T(1), nz_sg[i]);
     }
     for (int n = tid; n < N; n += nt) {
-        const T wz = M::div(wa_[n], a_[n] * a_[n]);
+        const T wz = FAST ? M::div(wa_[n], a_[n] * a_[n]) : wa_[n] * (ia_[n] * ia_[n]);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
-            const T u = FAST ? (z_[n] - zc[i]) * isg[i] : (z_[n] - th[11 + i] - nz_mu[i]) / nz_sg[i];
+            const T u = FAST ? (z_[n] - zc[i]) * isg[i] : (z_[n] - th[11 + i] - nz_mu[i]) * isg[i];
             const T raw = M::ex(T(-0.5) * u * u);
             V[i * N + n] = raw;
             pn[i] += wz * raw;
@@ -255,7 +269,7 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
     for (int i = 0; i < NB; ++i) { s0[i] = T(0); s1[i] = T(0); }
     for (int n = lo; n < hi; ++n) {
         const T e = Ez[n];
-        const T ichi = (FAST && n >= 1) ? M::div(T(1), chi[n]) : T(0);
+        const T ichi = (n >= 1) ? M::div(T(1), chi[n]) : T(0);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             const T nchi = V[i * N + n] * e * inv_norm[i];
@@ -263,7 +277,7 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
             if (n >= 1) {
                 const T wn = omw[n] * nchi;
                 s0[i] += wn;
-                s1[i] += FAST ? wn * ichi : wn / chi[n];
+                s1[i] += wn * ichi;
             }
         }
     }
@@ -290,14 +304,17 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
     const T A_IA = th[9], eta = th[10];
     const T pivot = pick_s<T>(sp.ia_pivot, sp.ia_pivot_f), c1rho = pick_s<T>(sp.c1rho, sp.c1rho_f);
     const T ipiv = M::div(T(1), pivot);
+    const T lnpiv = pick_s<T>(sp.ln_pivot, sp.ln_pivot_f);
     const T c1om = c1rho * om;
     for (int n = hi - 1; n >= lo; --n) {
         const T c = chi[n];
-        const T ic = (FAST && n >= 1) ? M::div(T(1), c) : T(0);
-        const T sq = (n >= 1) ? (FAST ? sqrt_<T>(omw[n]) * ic : sqrt_<T>(omw[n] / (c * c))) : T(0);
-        const T amp = FAST ? M::div(A_IA * M::ex(eta * M::lg((T(1) + z_[n]) * ipiv)) * c1om, Dg[n])
-                           : A_IA * M::ex(eta * M::lg((T(1) + z_[n]) / pivot)) * c1rho * om / Dg[n];
-        const T pc = FAST ? pref * c * M::div(T(1), a_[n]) : pref * c / a_[n];
+        const T ic = (n >= 1) ? M::div(T(1), c) : T(0);
+        const T sq = (n >= 1) ? sqrt_<T>(omw[n]) * ic : T(0);
+        // ln((1 + z) / pivot) = -ln a - ln pivot
+        const T lq = FAST ? M::lg((T(1) + z_[n]) * ipiv) : -lna_[n] - lnpiv;
+        const T amp = FAST ? M::div(A_IA * M::ex(eta * lq) * c1om, Dg[n])
+                           : M::div(A_IA * M::ex(eta * lq) * c1rho * om, Dg[n]);
+        const T pc = pref * c * (FAST ? M::div(T(1), a_[n]) : ia_[n]);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             const T nchi = V[i * N + n];
@@ -306,7 +323,7 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
                 v = sq * (pc * (e0[i] - c * e1[i]) - amp * nchi);
                 const T wn = omw[n] * nchi;
                 e0[i] += wn;
-                e1[i] += FAST ? wn * ic : wn / c;
+                e1[i] += wn * ic;
             }
             V[i * N + n] = v;
         }
@@ -548,7 +565,9 @@ k_limber(const ShearParams sp, const double* __restrict__ theta_full, const T* _
     const T* lnell = pick<T>(sp.lnell, sp.lnell_f);
     const T* tm = pick<T>(sp.tmpl, sp.tmpl_f);
     const T* dat = pick<T>(sp.data, sp.data_f);
-    for (int lp = wid; lp < n_lp; lp += nw) {
+    // FP64: the pairs of an evaluation may be split over gridDim.y CTAs
+    const int lp0 = sizeof(T) == 8 ? wid + nw * blockIdx.y : wid, lps = sizeof(T) == 8 ? nw * gridDim.y : nw;
+    for (int lp = lp0; lp < n_lp; lp += lps) {
         const int l0 = 2 * lp;
         const bool has1 = l0 + 1 < n_ell;
         const T lne0 = lnell[l0], lne1 = has1 ? lnell[l0 + 1] : lne0;
@@ -851,9 +870,54 @@ static int launch_whiten(const TR* resid, int D, const TA* LinvT, double c0, dou
     return NS_OK;
 }
 
+// FP64 chi^2 of short data vectors: one CTA per row, so that few rows use many
+// SMs' FP64 pipes (two FMAs per cycle each; 45 k for D = 300).  Two threads share
+// a column's reduction range, whose loads stay in flight eight deep.
+constexpr int kRowThreads = 640, kRowMaxD = 1024;
+template <typename TR>
+__global__ void __launch_bounds__(kRowThreads)
+k_whiten_row(const TR* __restrict__ resid, int D, const double* __restrict__ LinvT, double c0,
+             double* __restrict__ logL, const int* __restrict__ nrows) {
+    pdl_begin();
+    const int row = blockIdx.x;
+    if (row >= *nrows) return;
+    __shared__ double r[kRowMaxD], part[kRowMaxD], red[32];
+    constexpr int COLS = kRowThreads / 2;
+    const int half = threadIdx.x / COLS, t = threadIdx.x % COLS;
+    for (int b = threadIdx.x; b < D; b += kRowThreads) r[b] = (double)resid[(size_t)row * D + b];
+    __syncthreads();
+    double sq = 0.0;
+    for (int a0 = 0; a0 < D; a0 += COLS) {
+        const int a = a0 + t, mid = (a + 1) / 2;
+        double y = 0.0;
+        if (a < D) {
+#pragma unroll 8
+            for (int b = half ? mid : 0; b < (half ? a + 1 : mid); ++b) y = fma(LinvT[(size_t)b * D + a], r[b], y);
+            if (half) part[a] = y;
+        }
+        __syncthreads();
+        if (!half && a < D) {
+            y += part[a];
+            sq = fma(y, y, sq);
+        }
+    }
+    sq = block_sum(sq, red);
+    if (threadIdx.x == 0) logL[row] = c0 - 0.5 * sq;
+}
+
 template <typename TR, typename TA>
 int launch_chi2(const TR* resid, int D, const TA* LinvT, double c0, double* logL, const int* nrows, int grid_rows,
                 cudaStream_t st, bool rows_ready) {
+    // FP64: one CTA per row while half of L^-T, which every row reads, stays in
+    // L2 (8 MB at D = 1024): 64 rows of D = 300 take 29 us, against 510 us in
+    // 16-row blocks of 20 CTAs
+    if constexpr (sizeof(TA) == 8) {
+        if (D <= kRowMaxD) {
+            NS_CUDA_TRY(launch_pdl(k_whiten_row<TR>, dim3(grid_rows), dim3(kRowThreads), 0, st, resid, D, LinvT, c0, logL,
+                                   nrows));
+            return NS_OK;
+        }
+    }
     // 16-row blocks.  Short data vectors: CTAs of up to ~100 KB (two per SM),
     // so the clusters of a ~460-row batch fit one wave (8-row blocks needed
     // 58 five-CTA clusters there, two waves: 114.7 -> 111.6 us per 39-d
@@ -917,8 +981,16 @@ static int limber_launch(const ShearParams& sp, const double* theta_full, const 
                                          (int)(227 * 1024 - fa.sharedSizeBytes)));
         attr_done = true;
     }
-    const int warps = std::min(kLimberWarps, (sp.n_ell + 1) / 2);
-    NS_CUDA_TRY(launch_pdl(k_limber<T, NB, FAST, PKC>, dim3(grid_rows), dim3(32 * warps), smem, st, sp, theta_full,
+    const int n_lp = (sp.n_ell + 1) / 2;
+    int warps = std::min(kLimberWarps, n_lp), split = 1;
+    if (sizeof(T) == 8) {
+        // FP64: a CTA fills an SM (shared memory) and is bound by the SM's two FP64
+        // FMAs per cycle, so few evaluations are spread over all SMs, each CTA
+        // taking a share of the multipole pairs (64 evaluations: 425 -> 228 us)
+        split = std::max(1, std::min(n_lp, 152 / grid_rows));
+        warps = std::min(kLimberWarps, (n_lp + split - 1) / split);
+    }
+    NS_CUDA_TRY(launch_pdl(k_limber<T, NB, FAST, PKC>, dim3(grid_rows, split), dim3(32 * warps), smem, st, sp, theta_full,
                            table, win, resid, model_out, nrows, err, cl_out));
     return NS_OK;
 }
