@@ -401,19 +401,27 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, double* log
         NS_TRY(launch_zinterp_generic(p, g->table, g->table_fine, g->d_nrows, B, 4, st));
         tab = (const float*)g->table_fine;
     }
-    NS_TRY(launch_projection_adj<float>(sp, &g->proj, g->theta_full, tab, p->d_LinvT32, (const float*)g->Linv, p->c0,
-                                        TableGrad{g->gtab}, g->gfull, logL, g->d_nrows, B, g->d_err, st));
-    // d log L / d (output pre-scaling) = sigma * d log L / d table
-    const float* gt = (const float*)g->gtab;
+    // d log L / d (output pre-scaling) = sigma * d log L / d table, in planes
+    TableGrad tg;
+    if (coarse) {
+        tg.table = g->gtab;
+    } else {
+        tg.px = px;
+        tg.planes = g->Gp[0];
+        tg.pitch = plane_pitch(n_out);
+        tg.stride = g->rows_pad * tg.pitch;
+        tg.scale = (float)p->out_sigma;
+    }
+    NS_TRY(launch_projection_adj<float>(sp, &g->proj, g->theta_full, tab, p->d_LinvT32, (const float*)g->Linv, p->c0, tg,
+                                        g->gfull, logL, g->d_nrows, B, g->d_err, st));
     if (coarse) {
         const dim3 gz((n_out + 255) / 256, B);
-        adj::k_zinterp_adj<float><<<gz, 256, 0, st>>>(gt, sp.n_z, p->d_zi_row, p->d_zi_w, (float*)g->gcoarse,
-                                                      p->n_z_emu, sp.n_k, g->d_nrows);
+        adj::k_zinterp_adj<float><<<gz, 256, 0, st>>>((const float*)g->gtab, sp.n_z, p->d_zi_row, p->d_zi_w,
+                                                      (float*)g->gcoarse, p->n_z_emu, sp.n_k, g->d_nrows);
         NS_CUDA_TRY(cudaGetLastError());
-        gt = (const float*)g->gcoarse;
+        NS_TRY(launch_split_planes(px, (const float*)g->gcoarse, (float)p->out_sigma, B, n_out, g->Gp[0],
+                                   g->rows_pad * plane_pitch(n_out), plane_pitch(n_out), g->d_nrows, st));
     }
-    NS_TRY(launch_split_planes(px, gt, (float)p->out_sigma, B, n_out, g->Gp[0], g->rows_pad * plane_pitch(n_out),
-                               plane_pitch(n_out), g->d_nrows, st));
     // backward: G_l = (G_{l+1} W_l) (1 - h_l^2), l = L-1 .. 1 (the last in FP32)
     for (int l = L - 1; l >= 1; --l) {
         PlaneEpi e;

@@ -23,22 +23,21 @@
 // Bound: FP32 instruction issue.  The one-kernel form it replaced kept 250 KB
 // of intermediates per evaluation in global memory and added 16 atomics per
 // (node, multipole) to the table gradient.  Whole BF16 gradient calls of the
-// 39-d problem: 4096 rows 9978 -> 6496 us, 64 rows 608 -> 413 us.
+// 39-d problem: 4096 rows 9978 -> 5218 us, 64 rows 608 -> 369 us.  Per 2048
+// evaluations (BF16 problem): k_limber_adj 1334 us, k_windows_adj 382, k_table_adj
+// 149, k_chi2_adj 93.
 #include <algorithm>
 #include <vector>
 
 #include "likelihood.cuh"
 #include "projection_adj.cuh"
+#include "tcgen05.cuh"
 
 namespace gpuns {
 namespace adj {
 
-// 4-point Gauss-Legendre nodes and weights as compile-time constants of the
-// kernel's type (no double -> float conversions at run time).
-template <typename T> __device__ __forceinline__ T glx(int g) {
-    return g == 0 ? T(-0.86113631159405257522) : g == 1 ? T(-0.33998104358485626480)
-         : g == 2 ? T(0.33998104358485626480) : T(0.86113631159405257522);
-}
+// 4-point Gauss-Legendre weights as compile-time constants of the kernel's type
+// (no double -> float conversions at run time).
 template <typename T> __device__ __forceinline__ T glw(int g) {
     return (g == 0 || g == 3) ? T(0.34785484513745385737) : T(0.65214515486254614263);
 }
@@ -56,15 +55,29 @@ template <> __device__ __forceinline__ float ex<float>(float x) { return expf(x)
 template <typename T> __device__ __forceinline__ T lg(T x);
 template <> __device__ __forceinline__ double lg<double>(double x) { return log(x); }
 template <> __device__ __forceinline__ float lg<float>(float x) { return logf(x); }
+// 1 / sqrt: FP32 takes one Newton step on the SFU value
+__device__ __forceinline__ double rsq(double x) { return rsqrt(x); }
+__device__ __forceinline__ float rsq(float x) {
+    const float y = rsqrtf(x);
+    return fmaf(0.5f * y, fmaf(-x * y, y, 1.f), y);
+}
 // 10^v and its FP32 form on exp2
 __device__ __forceinline__ double p10(double v) { return exp(v * kLn10); }
 __device__ __forceinline__ float p10(float v) { return exp2f(v * 3.32192809488736234787f); }
 
 // ------------------------------------------------------------------ chi^2
 // RB rows per block: each entry of L^-1 read serves RB rows, whose values lie
-// beside one another in shared memory.
+// beside one another in shared memory.  Three threads share a column's reduction
+// range, with eight loads in flight each: a range walked by one thread is a chain
+// of L2 latencies (119 us for 64 rows, D = 300).
+constexpr int kChiCols = 320, kChiParts = 3, kChiThreads = kChiCols * kChiParts, kChiSeg = 16;
+
+__host__ __device__ inline size_t chi2_adj_elems(int D, int nb, int np, int nt, int rb) {
+    return (size_t)rb * ((2 + kChiParts - 1) * (size_t)D + nb + np + kChiSeg * (size_t)nt);
+}
+
 template <typename T, int RB>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kChiThreads)
 k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T* __restrict__ resid,
            const T* __restrict__ C, const T* __restrict__ LinvT, const T* __restrict__ Linv, double c0,
            T* __restrict__ gC, double* __restrict__ gfull, double* __restrict__ logL, const int* __restrict__ nrows) {
@@ -75,37 +88,57 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
     const int D = sp.D, P = sp.n_params, nb = sp.nb, n_ell = sp.n_ell, nt = sp.n_tmpl, np = sp.n_pairs;
     T* r = reinterpret_cast<T*>(smem_raw);     // D x RB, later g_m
     T* y = r + D * RB;                         // D x RB
-    T* th = y + D * RB;                        // RB x nb: 1 + m_i
+    T* part = y + D * RB;                      // (kChiParts - 1) x D x RB
+    T* th = part + (kChiParts - 1) * D * RB;   // RB x nb: 1 + m_i
     T* S = th + RB * nb;                       // np x RB: sum_ell g_m C
-    T* tp = S + np * RB;                       // 8 x RB x nt partial template sums
+    T* tp = S + np * RB;                       // kChiSeg x RB x nt partial template sums
     __shared__ T red[32];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    for (int i = tid; i < RB * D; i += 256) {
+    const int seg = tid / kChiCols, col = tid % kChiCols;
+    for (int i = tid; i < RB * D; i += kChiThreads) {
         const int j = i / D, a = i - j * D;
         r[a * RB + j] = r0 + j < M ? resid[(size_t)(r0 + j) * D + a] : T(0);
     }
-    for (int i = tid; i < RB * nb; i += 256) {
+    for (int i = tid; i < RB * nb; i += kChiThreads) {
         const int j = i / nb;
         th[i] = r0 + j < M ? T(1) + (T)theta_full[(size_t)(r0 + j) * P + 11 + nb + i % nb] : T(0);
     }
     __syncthreads();
+    // acc[j] = sum_{b = lo}^{hi-1} A[b][a] x[b][j], the parts of a column in order
+    auto column = [&](const T* A, const T* x, int a, int lo, int hi, T (&acc)[RB]) {
+        const int b0 = lo + (hi - lo) * seg / kChiParts, b1 = lo + (hi - lo) * (seg + 1) / kChiParts;
+#pragma unroll
+        for (int j = 0; j < RB; ++j) acc[j] = T(0);
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) {
+            const T l = A[(size_t)b * D + a];
+#pragma unroll
+            for (int j = 0; j < RB; ++j) acc[j] = fma(l, x[b * RB + j], acc[j]);
+        }
+        if (seg > 0)
+#pragma unroll
+            for (int j = 0; j < RB; ++j) part[((seg - 1) * D + a) * RB + j] = acc[j];
+    };
+    auto join = [&](int a, T (&acc)[RB]) {
+        for (int q = 0; q < kChiParts - 1; ++q)
+#pragma unroll
+            for (int j = 0; j < RB; ++j) acc[j] += part[(q * D + a) * RB + j];
+    };
     T sq[RB];
 #pragma unroll
     for (int j = 0; j < RB; ++j) sq[j] = T(0);
-    for (int a = tid; a < D; a += 256) {
+    for (int a0 = 0; a0 < D; a0 += kChiCols) {
+        const int a = a0 + col;
         T acc[RB];
+        if (a < D) column(LinvT, r, a, 0, a + 1, acc);
+        __syncthreads();
+        if (a < D && seg == 0) {
+            join(a, acc);
 #pragma unroll
-        for (int j = 0; j < RB; ++j) acc[j] = T(0);
-#pragma unroll 4
-        for (int b = 0; b <= a; ++b) {
-            const T l = LinvT[(size_t)b * D + a];
-#pragma unroll
-            for (int j = 0; j < RB; ++j) acc[j] = fma(l, r[b * RB + j], acc[j]);
-        }
-#pragma unroll
-        for (int j = 0; j < RB; ++j) {
-            y[a * RB + j] = acc[j];
-            sq[j] = fma(acc[j], acc[j], sq[j]);
+            for (int j = 0; j < RB; ++j) {
+                y[a * RB + j] = acc[j];
+                sq[j] = fma(acc[j], acc[j], sq[j]);
+            }
         }
     }
 #pragma unroll
@@ -114,38 +147,38 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
         if (tid == 0 && r0 + j < M) logL[r0 + j] = c0 - 0.5 * (double)s;
     }
     // g_m = L^-T y: (g_m)_a = sum_{b >= a} (L^-1)[b][a] y_b
-    for (int a = tid; a < D; a += 256) {
+    for (int a0 = 0; a0 < D; a0 += kChiCols) {
+        const int a = a0 + col;
         T acc[RB];
+        if (a < D) column(Linv, y, a, a, D, acc);
+        __syncthreads();
+        if (a < D && seg == 0) {
+            join(a, acc);
+            const int p = a / n_ell, i = sp.pi[p], k = sp.pj[p];
 #pragma unroll
-        for (int j = 0; j < RB; ++j) acc[j] = T(0);
-#pragma unroll 4
-        for (int b = a; b < D; ++b) {
-            const T l = Linv[(size_t)b * D + a];
-#pragma unroll
-            for (int j = 0; j < RB; ++j) acc[j] = fma(l, y[b * RB + j], acc[j]);
-        }
-        const int p = a / n_ell, i = sp.pi[p], k = sp.pj[p];
-#pragma unroll
-        for (int j = 0; j < RB; ++j) {
-            r[a * RB + j] = acc[j];
-            if (r0 + j < M) gC[(size_t)(r0 + j) * D + a] = acc[j] * th[j * nb + i] * th[j * nb + k];
+            for (int j = 0; j < RB; ++j) {
+                r[a * RB + j] = acc[j];
+                if (r0 + j < M) gC[(size_t)(r0 + j) * D + a] = acc[j] * th[j * nb + i] * th[j * nb + k];
+            }
         }
     }
     __syncthreads();
-    for (int q = tid; q < np * RB; q += 256) {
+    for (int q = tid; q < np * RB; q += kChiThreads) {
         const int p = q / RB, j = q % RB;
         T s = T(0);
         if (r0 + j < M)
+#pragma unroll 4
             for (int e = 0; e < n_ell; ++e) s = fma(r[(p * n_ell + e) * RB + j], C[(size_t)(r0 + j) * D + p * n_ell + e], s);
         S[q] = s;
     }
-    {   // templates: warp w sums the w-th eighth of the data vector, lanes over templates
+    if (wid < kChiSeg) {   // templates: warp w sums its share of the data vector, lanes over templates
         const T* tm = pick<T>(sp.tmpl, sp.tmpl_f);
-        const int lo = D * wid / 8, hi = D * (wid + 1) / 8;
+        const int lo = D * wid / kChiSeg, hi = D * (wid + 1) / kChiSeg;
         for (int t = lane; t < nt; t += 32) {
             T acc[RB];
 #pragma unroll
             for (int j = 0; j < RB; ++j) acc[j] = T(0);
+#pragma unroll 8
             for (int a = lo; a < hi; ++a) {
                 const T g = tm[(size_t)a * nt + t];
 #pragma unroll
@@ -156,7 +189,7 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
         }
     }
     __syncthreads();
-    for (int q = tid; q < RB * P; q += 256) {
+    for (int q = tid; q < RB * P; q += kChiThreads) {
         const int j = q / P, i = q % P - (11 + nb);
         if (r0 + j >= M) continue;
         T v = T(0);
@@ -166,15 +199,13 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
                 if (sp.pj[p] == i) v = fma(S[p * RB + j], th[j * nb + sp.pi[p]], v);
             }
         } else if (i >= nb) {
-            for (int w = 0; w < 8; ++w) v += tp[(w * RB + j) * nt + i - nb];
+            for (int w = 0; w < kChiSeg; ++w) v += tp[(w * RB + j) * nt + i - nb];
         }
         gfull[(size_t)(r0 + j) * P + q % P] = (double)v;
     }
 }
 
 // ------------------------------------------------------------------ Limber
-template <typename T> struct alignas(16) V4 { T x, y, z, w; };
-
 // Entry (r, c) of the table padded by one ghost row and column on every side
 // (linear extrapolation), rows 0 .. n_z + 1, columns 0 .. n_k + 1.
 template <typename T>
@@ -185,11 +216,35 @@ __device__ __forceinline__ T padded_row(const T* t, int n_k, int c) {
 }
 template <typename T>
 __device__ __forceinline__ T padded(const T* t, int n_z, int n_k, int r, int c) {
+    if (r >= 1 && r <= n_z && c >= 1 && c <= n_k) return t[(size_t)(r - 1) * n_k + c - 1];
     if (r == 0) return T(2) * padded_row(t, n_k, c) - padded_row(t + n_k, n_k, c);
     if (r == n_z + 1)
         return T(2) * padded_row(t + (size_t)(n_z - 1) * n_k, n_k, c) - padded_row(t + (size_t)(n_z - 2) * n_k, n_k, c);
     return padded_row(t + (size_t)(r - 1) * n_k, n_k, c);
 }
+
+// Pairs of values: packed FP32x2 instructions for float, two FMAs for double.
+template <typename T> struct P2;
+template <> struct P2<float> {
+    float2 v;
+    __device__ __forceinline__ P2() {}
+    __device__ __forceinline__ P2(float x, float y) : v(make_float2(x, y)) {}
+    static __device__ __forceinline__ P2 mul(P2 a, P2 b) { P2 r; r.v = __fmul2_rn(a.v, b.v); return r; }
+    static __device__ __forceinline__ P2 fma(P2 a, P2 b, P2 c) { P2 r; r.v = __ffma2_rn(a.v, b.v, c.v); return r; }
+    static __device__ __forceinline__ P2 add(P2 a, P2 b) { P2 r; r.v = __fadd2_rn(a.v, b.v); return r; }
+};
+template <> struct P2<double> {
+    double2 v;
+    __device__ __forceinline__ P2() {}
+    __device__ __forceinline__ P2(double x, double y) : v(make_double2(x, y)) {}
+    static __device__ __forceinline__ P2 mul(P2 a, P2 b) { return P2(a.v.x * b.v.x, a.v.y * b.v.y); }
+    static __device__ __forceinline__ P2 fma(P2 a, P2 b, P2 c) {
+        return P2(::fma(a.v.x, b.v.x, c.v.x), ::fma(a.v.y, b.v.y, c.v.y));
+    }
+    static __device__ __forceinline__ P2 add(P2 a, P2 b) { return P2(a.v.x + b.v.x, a.v.y + b.v.y); }
+};
+// four z-taps of a table column
+template <typename T> struct alignas(16) Z4 { P2<T> a, b; };
 
 // Sum of 8 values per lane over the warp: lane l gets the sum of value l & 7.
 template <typename T>
@@ -214,17 +269,19 @@ __device__ __forceinline__ T warp_transpose_sum8(T (&v)[8]) {
 // same ln k cell (u moves by ~0.05 cells per node), so a lane keeps the 16 taps
 // of its cell and their 16 gradients in registers and exchanges them only when
 // its cell changes (about one lane per node): the gradients go to the warp's own
-// columns in shared memory (four z-taps of a column side by side), and when the
-// warp enters the next z cell the rows it has left go to the warp's partial
-// rows in global memory.  No two lanes add to one column at a time: lanes with
-// equal cells take turns.  Sums over multipoles (g_V, g_ln chi) are warp
-// reductions of 8 values at once.
+// columns in shared memory (four z-taps of a column side by side, as are the
+// current table rows), and when the warp enters the next z cell the rows it has
+// left go to the warp's partial rows in global memory.  No two lanes add to one
+// column at a time: with ascending multipoles the lanes' cells ascend too, so only
+// neighbours can share one (clamped ln k); lanes with equal cells take turns.
+// Sums over multipoles (g_V, g_ln chi) are warp reductions of 8 values at once.
 template <typename T, int NB>
 __global__ void __launch_bounds__(32 * kAdjWarps, sizeof(T) == 4 ? 4 : 2)
 k_limber_adj(const ShearParams sp, const T* __restrict__ table, const T* __restrict__ win, const T* __restrict__ gC,
              const int4* __restrict__ ranges, int W, int part_rows, T* __restrict__ part, T* __restrict__ gV,
-             T* __restrict__ glnc, int stage, const int* __restrict__ nrows) {
-    constexpr int NP = NB * (NB + 1) / 2;
+             T* __restrict__ glnc, int stage, int sorted, const int* __restrict__ nrows) {
+    using Q = P2<T>;
+    constexpr int NB2 = (NB + 1) / 2;          // pairs of bins
     pdl_begin();
     const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int per_row = W / nw, row = blockIdx.x / per_row;
@@ -234,101 +291,123 @@ k_limber_adj(const ShearParams sp, const T* __restrict__ table, const T* __restr
     if (lo >= hi) return;                      // warps work alone: no block barrier below
     const int N = sp.N, n_k = sp.n_k, n_z = sp.n_z, n_ell = sp.n_ell, D = sp.D, PK = n_k + 2, Np = (N + 3) & ~3;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    V4<T>* acc = reinterpret_cast<V4<T>*>(smem_raw) + (size_t)wid * PK * (stage ? 2 : 1);
-    V4<T>* tab = acc + PK;                     // when staged: the four table rows of the current z cell
+    Z4<T>* acc = reinterpret_cast<Z4<T>*>(smem_raw) + (size_t)wid * PK * (stage ? 2 : 1);
+    Z4<T>* tab = acc + PK;                     // when staged: the four table rows of the current z cell
     const T* src = table + (size_t)row * n_z * n_k;
     const T* lnchi = win + (size_t)row * (NB + 1) * Np;
     const T* V = lnchi + Np;
     T* prow = part + ((size_t)row * part_rows + rg.z) * PK;
-    const T* zwp = pick<T>(sp.zw4d, sp.zw4f);
+    const Z4<T>* zwp = reinterpret_cast<const Z4<T>*>(pick<T>(sp.zw4d, sp.zw4f));
     const T* lnell = pick<T>(sp.lnell, sp.lnell_f);
     const T lkmin = pick_s<T>(sp.lnk_min, sp.lnk_min_f), lkmax = pick_s<T>(sp.lnk_max, sp.lnk_max_f);
     const T inv_dk = pick_s<T>(1.0 / sp.dlnk, sp.inv_dlnk_f);
+    const Q zero(T(0), T(0));
     for (int l0 = 0; l0 < n_ell; l0 += 32) {
         const int l = l0 + lane;
         const bool act = l < n_ell;
         const T lne = lnell[act ? l : n_ell - 1];
-        T G[NP];
+        // symmetric g_C with a doubled diagonal, rows of bins in pairs: h_i = sum_j G_ij V_j is
+        // the derivative of g_P = 1/2 sum_ij G_ij V_i V_j by V_i
+        Q G[NB2][NB];
+        {
+            auto g = [&](int i, int j) {
+                if (i >= NB || !act) return T(0);
+                const int p = min(i, j) * NB - min(i, j) * (min(i, j) - 1) / 2 + abs(i - j);
+                const T v = gC[(size_t)row * D + p * n_ell + l];
+                return i == j ? T(2) * v : v;
+            };
 #pragma unroll
-        for (int p = 0; p < NP; ++p) G[p] = act ? gC[(size_t)row * D + p * n_ell + l] : T(0);
+            for (int i = 0; i < NB2; ++i)
+#pragma unroll
+                for (int j = 0; j < NB; ++j) G[i][j] = Q(g(2 * i, j), g(2 * i + 1, j));
+        }
         int jc = sp.zrp[lo], ik = -1;
-        T c[4][4], a[4][4];                    // [column tap][row tap]
+        Z4<T> c[4], a[4];                      // by column tap
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-            for (int r = 0; r < 4; ++r) { c[q][r] = T(0); a[q][r] = T(0); }
-        auto load_rows = [&]() {
-            if (stage)
-                for (int k = lane; k < PK; k += 32)
-                    tab[k] = V4<T>{padded(src, n_z, n_k, jc, k), padded(src, n_z, n_k, jc + 1, k),
-                                   padded(src, n_z, n_k, jc + 2, k), padded(src, n_z, n_k, jc + 3, k)};
+        for (int q = 0; q < 4; ++q) { c[q].a = c[q].b = zero; a[q].a = a[q].b = zero; }
+        auto rows_at = [&](int k) {
+            Z4<T> s;
+            s.a = Q(padded(src, n_z, n_k, jc, k), padded(src, n_z, n_k, jc + 1, k));
+            s.b = Q(padded(src, n_z, n_k, jc + 2, k), padded(src, n_z, n_k, jc + 3, k));
+            return s;
         };
         // add the register gradients of the lanes with f to their columns
-        auto flush = [&](bool f) {
-            const unsigned same = __match_any_sync(0xffffffffu, f ? ik : -1 - lane);
-            const int turn = __popc(same & ((1u << lane) - 1u));
-            for (int t = 0; __any_sync(0xffffffffu, f && turn >= t); ++t) {
-                const bool mine = f && turn == t;
+        auto add_columns = [&](bool mine) {
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    if (mine) {
-                        V4<T> s = acc[ik + q];
-                        s.x += a[q][0]; s.y += a[q][1]; s.z += a[q][2]; s.w += a[q][3];
-                        acc[ik + q] = s;
-                    }
-                    __syncwarp();
+            for (int q = 0; q < 4; ++q) {
+                if (mine) {
+                    Z4<T> s = acc[ik + q];
+                    s.a = Q::add(s.a, a[q].a);
+                    s.b = Q::add(s.b, a[q].b);
+                    acc[ik + q] = s;
                 }
+                __syncwarp();
             }
         };
-        // rows jc .. to - 1 are complete for this warp: write them out, shift the rest
-        auto advance = [&](int to) {
+        auto flush = [&](bool f) {
+            const int before = __shfl_up_sync(0xffffffffu, f ? ik : -1 - lane, 1);
+            if (sorted && !__any_sync(0xffffffffu, f && lane > 0 && before == ik)) {
+                add_columns(f);
+                return;
+            }
+            const unsigned same = __match_any_sync(0xffffffffu, f ? ik : -1 - lane);
+            const int turn = __popc(same & ((1u << lane) - 1u));
+            for (int t = 0; __any_sync(0xffffffffu, f && turn >= t); ++t) add_columns(f && turn == t);
+        };
+        // rows jc .. to - 1 are complete for this warp: write them out, move the rest up
+        // and (when rows follow) bring in the table's next ones
+        auto advance = [&](int to, bool more) {
             const int n = to - jc;
             T* out = prow + (size_t)(jc - rg.w) * PK;
             for (int k = lane; k < PK; k += 32) {
-                V4<T> s = acc[k];
+                Z4<T> s = acc[k], t;
+                if (more && stage) t = tab[k];
                 for (int i = 0; i < n; ++i) {
                     T* o = out + (size_t)i * PK + k;
-                    *o = l0 ? *o + s.x : s.x;
-                    s = V4<T>{s.y, s.z, s.w, T(0)};
+                    *o = l0 ? *o + s.a.v.x : s.a.v.x;
+                    s.a = Q(s.a.v.y, s.b.v.x);
+                    s.b = Q(s.b.v.y, T(0));
+                    if (more && stage) {
+                        t.a = Q(t.a.v.y, t.b.v.x);
+                        t.b = Q(t.b.v.y, padded(src, n_z, n_k, jc + i + 4, k));
+                    }
                 }
                 acc[k] = s;
+                if (more && stage) tab[k] = t;
             }
+            jc = to;
             __syncwarp();
         };
-        for (int k = lane; k < PK; k += 32) acc[k] = V4<T>{T(0), T(0), T(0), T(0)};
-        load_rows();
+        for (int k = lane; k < PK; k += 32) {
+            acc[k].a = acc[k].b = zero;
+            if (stage) tab[k] = rows_at(k);
+        }
         __syncwarp();
         // node constants one node ahead
         int zr_n = jc;
-        T lc_n = lnchi[lo], w_n[4], v_n[NB];
-#pragma unroll
-        for (int r = 0; r < 4; ++r) w_n[r] = zwp[4 * lo + r];
+        T lc_n = lnchi[lo], v_n[NB];
+        Z4<T> w_n = zwp[lo];
 #pragma unroll
         for (int i = 0; i < NB; ++i) v_n[i] = V[i * Np + lo];
 #pragma unroll 1
         for (int n = lo; n < hi; ++n) {
             const int zr = zr_n;
             const T lc = lc_n;
-            T wz[4], vv[NB];
-#pragma unroll
-            for (int r = 0; r < 4; ++r) wz[r] = w_n[r];
+            const Z4<T> wz = w_n;
+            T vv[NB];
 #pragma unroll
             for (int i = 0; i < NB; ++i) vv[i] = v_n[i];
             if (n + 1 < hi) {
                 zr_n = sp.zrp[n + 1];
                 lc_n = lnchi[n + 1];
-#pragma unroll
-                for (int r = 0; r < 4; ++r) w_n[r] = zwp[4 * (n + 1) + r];
+                w_n = zwp[n + 1];
 #pragma unroll
                 for (int i = 0; i < NB; ++i) v_n[i] = V[i * Np + n + 1];
             }
             if (zr != jc) {
                 flush(ik >= 0);
-                advance(zr);
-                jc = zr;
+                advance(zr, true);
                 ik = -1;
-                load_rows();
-                __syncwarp();
             }
             const T s_raw = lne - lc;
             const bool clamped = (s_raw < lkmin) || (s_raw > lkmax);
@@ -341,68 +420,61 @@ k_limber_adj(const ShearParams sp, const T* __restrict__ table, const T* __restr
                     ik = ik_n;
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        V4<T> s;
-                        if (stage) s = tab[ik + q];
-                        else s = V4<T>{padded(src, n_z, n_k, jc, ik + q), padded(src, n_z, n_k, jc + 1, ik + q),
-                                       padded(src, n_z, n_k, jc + 2, ik + q), padded(src, n_z, n_k, jc + 3, ik + q)};
-                        c[q][0] = s.x; c[q][1] = s.y; c[q][2] = s.z; c[q][3] = s.w;
-                        a[q][0] = a[q][1] = a[q][2] = a[q][3] = T(0);
+                        c[q] = stage ? tab[ik + q] : rows_at(ik + q);
+                        a[q].a = a[q].b = zero;
                     }
                 }
                 __syncwarp();
             }
             // doubled Catmull-Rom weights in ln k and their derivatives (the z-weights are doubled too)
-            const T t = uk - (T)ik_n, t2 = t * t;
-            const T wk[4] = {t * (t * (T(2) - t) - T(1)), T(2) + t2 * (T(3) * t - T(5)),
-                             t * (T(1) + t * (T(4) - T(3) * t)), t2 * (t - T(1))};
-            const T dk[4] = {T(-1) + t * (T(4) - T(3) * t), t * (T(9) * t - T(10)), T(1) + t * (T(8) - T(9) * t),
-                             t * (T(3) * t - T(2))};
+            const T t = uk - (T)ik_n, t2 = t * t, m = t * (T(4) - T(3) * t);
+            const T wk[4] = {t * (t * (T(2) - t) - T(1)), T(2) + t2 * (T(3) * t - T(5)), t * (T(1) + m), t2 * (t - T(1))};
+            const T dk[4] = {m - T(1), t * (T(9) * t - T(10)), T(1) + t * (T(8) - T(9) * t), t * (T(3) * t - T(2))};
             T v = T(0), dv = T(0);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const T col = wz[0] * c[q][0] + wz[1] * c[q][1] + wz[2] * c[q][2] + wz[3] * c[q][3];
+                const Q s = Q::fma(wz.b, c[q].b, Q::mul(wz.a, c[q].a));
+                const T col = s.v.x + s.v.y;
                 v = fma(wk[q], col, v);
                 dv = fma(dk[q], col, dv);
             }
             const T Pw = p10(T(0.25) * v);
-            // h_i = sum_{j >= i} G_ij V_j; g_P = sum_i V_i h_i; g_V_i = P (h_i + sum_{j <= i} G_ji V_j)
+            Q h[NB2];
+#pragma unroll
+            for (int i = 0; i < NB2; ++i) h[i] = zero;
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                const Q vj(vv[j], vv[j]);
+#pragma unroll
+                for (int i = 0; i < NB2; ++i) h[i] = Q::fma(G[i][j], vj, h[i]);
+            }
             T red[8];
             T gP = T(0);
 #pragma unroll
             for (int i = 0; i < 8; ++i) red[i] = T(0);
-            {
-                int p = 0;
 #pragma unroll
-                for (int i = 0; i < NB; ++i) {
-                    T h = T(0);
-#pragma unroll
-                    for (int j = i; j < NB; ++j) {
-                        h = fma(G[p], vv[j], h);
-                        red[j] = fma(G[p], vv[i], red[j]);
-                        ++p;
-                    }
-                    gP = fma(vv[i], h, gP);
-                    red[i] += h;
-                }
+            for (int i = 0; i < NB; ++i) {
+                const T hi_ = (i & 1) ? h[i / 2].v.y : h[i / 2].v.x;
+                gP = fma(vv[i], hi_, gP);
+                red[i] = hi_ * Pw;
             }
-#pragma unroll
-            for (int i = 0; i < NB; ++i) red[i] *= Pw;
-            const T gv = gP * Pw * (T)(kLn10 * 0.25);     // d log L / d (doubled-weight sum)
+            const T gv = gP * Pw * (T)(kLn10 * 0.125);    // d log L / d (doubled-weight sum); gP is twice g_P
             red[NB] = clamped ? T(0) : -gv * dv * inv_dk; // s = ln(ell + 1/2) - ln chi
+            const Q ga = Q::mul(Q(gv, gv), wz.a), gb = Q::mul(Q(gv, gv), wz.b);
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                const T g = gv * wz[r];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) a[q][r] = fma(g, wk[q], a[q][r]);
+            for (int q = 0; q < 4; ++q) {
+                const Q w(wk[q], wk[q]);
+                a[q].a = Q::fma(ga, w, a[q].a);
+                a[q].b = Q::fma(gb, w, a[q].b);
             }
-            T sum = warp_transpose_sum8(red);
+            const T sum = warp_transpose_sum8(red);
             if (lane <= NB) {
                 T* o = lane < NB ? gV + ((size_t)row * NB + lane) * N + n : glnc + (size_t)row * N + n;
                 *o = l0 ? *o + sum : sum;
             }
         }
         flush(ik >= 0);
-        advance(jc + 4);
+        advance(jc + 4, false);
     }
 }
 
@@ -430,13 +502,13 @@ k_table_adj(const T* __restrict__ part, int part_rows, const int* __restrict__ p
         if (c >= n_k - 1) s += (c == n_k ? T(2) : T(-1)) * at(r, n_k + 1);
         return s;
     };
-    for (int i = blockIdx.y * 256 + threadIdx.x; i < n_z * n_k; i += gridDim.y * 256) {
-        const int r = i / n_k + 1, c = i % n_k + 1;
-        T s = cols(r, c);
-        if (r <= 2) s += (r == 1 ? T(2) : T(-1)) * cols(0, c);
-        if (r >= n_z - 1) s += (r == n_z ? T(2) : T(-1)) * cols(n_z + 1, c);
-        out.put(row, i, n_z * n_k, s);
-    }
+    for (int r = 1 + blockIdx.y; r <= n_z; r += gridDim.y)
+        for (int c = 1 + threadIdx.x; c <= n_k; c += blockDim.x) {
+            T s = cols(r, c);
+            if (r <= 2) s += (r == 1 ? T(2) : T(-1)) * cols(0, c);
+            if (r >= n_z - 1) s += (r == n_z ? T(2) : T(-1)) * cols(n_z + 1, c);
+            out.put(row, (r - 1) * n_k + c - 1, n_z * n_k, s);
+        }
 }
 
 // ------------------------------------------------------------------ windows and distances
@@ -509,7 +581,11 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
     const T* wa_ = pick<T>(sp.wa, sp.wa_f);
     const T* nz_mu = pick<T>(sp.nz_mean, sp.nz_mean_f);
     const T* nz_sg = pick<T>(sp.nz_sigma, sp.nz_sigma_f);
-    const T ia_piv = pick_s<T>(sp.ia_pivot, sp.ia_pivot_f), c1rho = pick_s<T>(sp.c1rho, sp.c1rho_f);
+    const T* ia_ = pick<T>(sp.ia, sp.ia_f);
+    const T* gl_ia = pick<T>(sp.gl_ia, sp.gl_ia_f);
+    const T* gl_ln = pick<T>(sp.gl_ln, sp.gl_ln_f);
+    const T* gl_1ma = pick<T>(sp.gl_1ma, sp.gl_1ma_f);
+    const T lnpiv = pick_s<T>(sp.ln_pivot, sp.ln_pivot_f), c1rho = pick_s<T>(sp.c1rho, sp.c1rho_f);
     if (tid < 11 + NB) th[tid] = (T)theta_full[(size_t)row * sp.n_params + tid];
     __syncthreads();
     const T h = th[2];
@@ -519,47 +595,45 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
     const T chiH = T(kCover100) / h;
     const T gamma = T(0.55) + T(0.05) * (T(1) + w0 + T(0.5) * wa);
     const T pref = T(1.5) * om / (chiH * chiH);
-    const T A_IA = th[9], eta = th[10];
+    const T A_IA = th[9], eta = th[10], iom = T(1) / om, ichiH = T(1) / chiH;
     T sum[NS];                                  // scalars, then per bin: g_nchi nchi u / sigma, g_nchi nchi, d norm / d D_z
 #pragma unroll
     for (int q = 0; q < NS; ++q) sum[q] = T(0);
 
     // ---- forward
     for (int n = tid; n < N; n += nt) {
-        const T a = a_[n], lna = lna_[n];
-        const T de = ex<T>(-pde * lna - T(3) * wa * (T(1) - a));
-        Ez[n] = sqrt(om * ex<T>(T(-3) * lna) + (T(1) - om) * de);
+        const T a = a_[n], ia = ia_[n];
+        const T de = ex<T>(-pde * lna_[n] - T(3) * wa * (T(1) - a));
+        Ez[n] = sqrt(om * (ia * ia * ia) + (T(1) - om) * de);
         T inc = T(0);
         if (n < N - 1) {
-            const T a1 = a_[n + 1];
-            const T mid = T(0.5) * (a + a1), half = T(0.5) * (a - a1);
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
-                const T ag = mid + half * glx<T>(g);
-                const T e2 = om / (ag * ag * ag) + (T(1) - om) * ex<T>(-pde * lg<T>(ag) - T(3) * wa * (T(1) - ag));
-                inc += glw<T>(g) / (ag * ag * sqrt(e2));
+                const T ig = gl_ia[4 * n + g];
+                const T e2 = om * ig * ig * ig + (T(1) - om) * ex<T>(-pde * gl_ln[4 * n + g] - T(3) * wa * gl_1ma[4 * n + g]);
+                inc += glw<T>(g) * ig * ig * rsq(e2);
             }
-            inc *= chiH * half;
+            inc *= chiH * T(0.5) * (a - a_[n + 1]);
         }
         chi[n] = inc;
     }
     __syncthreads();
     block_scan<1, false>(chi, N, N, red);
-    T pn[NB];
+    T pn[NB], isg[NB];
 #pragma unroll
-    for (int i = 0; i < NB; ++i) pn[i] = T(0);
+    for (int i = 0; i < NB; ++i) { pn[i] = T(0); isg[i] = T(1) / nz_sg[i]; }
     for (int n = tid; n < N; n += nt) {
-        const T e = Ez[n], ia2 = wa_[n] / (a_[n] * a_[n]);
-        const T oma = om * ex<T>(T(-3) * lna_[n]) / (e * e);
+        const T ie = T(1) / Ez[n], ia = ia_[n], ia2 = wa_[n] * (ia * ia);
+        const T oma = om * (ia * ia * ia) * (ie * ie);
         fg[n] = ex<T>(gamma * lg<T>(oma));
-        omw[n] = ia2 * chiH / e;
+        omw[n] = ia2 * chiH * ie;
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
-            const T u = (z_[n] - th[11 + i] - nz_mu[i]) / nz_sg[i];
+            const T u = (z_[n] - th[11 + i] - nz_mu[i]) * isg[i];
             const T rw = ex<T>(T(-0.5) * u * u);
             raw[i * N + n] = rw;
             pn[i] += ia2 * rw;
-            sum[S_COUNT + 2 * NB + i] += ia2 * rw * u / nz_sg[i];
+            sum[S_COUNT + 2 * NB + i] += ia2 * rw * u * isg[i];
         }
     }
 #pragma unroll
@@ -568,19 +642,20 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
         if (lane == 0) red[wid * NB + i] = s;
     }
     __syncthreads();
-    T norm[NB];
+    T inorm[NB];                                // 1 / (chiH norm)
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
-        norm[i] = T(0);
-        for (int w = 0; w < nt / 32; ++w) norm[i] += red[w * NB + i];
+        T s = T(0);
+        for (int w = 0; w < nt / 32; ++w) s += red[w * NB + i];
+        inorm[i] = T(1) / (chiH * s);
     }
     __syncthreads();
     for (int n = tid; n < N; n += nt) {
         Dg[n] = (n < N - 1) ? T(0.5) * (fg[n] + fg[n + 1]) * (lna_[n] - lna_[n + 1]) : T(0);
-        const T o = omw[n], ic = n >= 1 ? T(1) / chi[n] : T(0);
+        const T o = omw[n], e = Ez[n], ic = n >= 1 ? T(1) / chi[n] : T(0);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
-            const T nc = raw[i * N + n] * Ez[n] / (chiH * norm[i]);
+            const T nc = raw[i * N + n] * e * inorm[i];
             nchi[i * N + n] = nc;
             E0[i * N + n] = (n >= 1) ? o * nc : T(0);
             E1[i * N + n] = (n >= 1) ? o * nc * ic : T(0);
@@ -599,10 +674,10 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
             gchi[0] = T(0); gomw[0] = T(0); t1[0] = T(0);
             continue;
         }
-        const T c = chi[n], an = a_[n], so = sqrt(omw[n]), ic = T(1) / c;
-        const T lq = lg<T>((T(1) + z_[n]) / ia_piv);
+        const T c = chi[n], ian = ia_[n], so = sqrt(omw[n]), ic = T(1) / c;
+        const T lq = -lna_[n] - lnpiv;          // ln((1 + z) / pivot)
         const T ampc = ex<T>(eta * lq) * c1rho * om / D_n;   // amp = A_IA * ampc
-        const T pc = pref * c / an;
+        const T pc = pref * c * ian;
         T g_so = T(0), g_c = T(0), g_amp = T(0);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
@@ -613,8 +688,8 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
             g_so += gVv * W * ic;
             g_c += -gVv * so * W * ic * ic;
             const T gpc = gW * (e0 - c * e1);
-            sum[S_PREF] += gpc * c / an;
-            g_c += gpc * pref / an - gW * pc * e1;
+            sum[S_PREF] += gpc * c * ian;
+            g_c += gpc * pref * ian - gW * pc * e1;
             E0[i * N + n] = gW * pc;            // the adjoints take the place of the suffix sums
             E1[i * N + n] = -gW * pc * c;
             g_amp += -gW * nc;
@@ -624,36 +699,35 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
         gchi[n] = glnc[(size_t)row * N + n] * ic + g_c;
         sum[S_AIA] += g_amp * ampc;
         sum[S_ETA] += g_amp * A_IA * ampc * lq;
-        sum[S_OM] += g_amp * A_IA * ampc / om;
+        sum[S_OM] += g_amp * A_IA * ampc * iom;
         t1[n] = g_amp * A_IA * ampc;            // g_S = -g_D D, g_D = -g_amp amp / D
     }
     __syncthreads();
     // E0_i(n) = sum_{m>n} omw_m nchi_m  ->  G0(m) = sum_{n<m} gE0(n)
     block_scan<2 * NB, false>(E0, N, N, red);
     for (int m = tid; m < N; m += nt) {
-        const T e = Ez[m], o = omw[m];
+        const T ie = T(1) / Ez[m], o = omw[m], ic = m >= 1 ? T(1) / chi[m] : T(0);
         T go = gomw[m], gc = gchi[m], ge = T(0);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             T gnc = raw[i * N + m];
             const T nc = nchi[i * N + m];
             if (m >= 1) {
-                const T ic = T(1) / chi[m];
-                const T G0 = E0[i * N + m], G1 = E1[i * N + m] * ic, G = G0 + G1;
+                const T G1 = E1[i * N + m] * ic, G = E0[i * N + m] + G1;
                 go += nc * G;
                 gnc += o * G;
                 gc += -o * nc * G1 * ic;
             }
             // nchi = raw E / (chiH norm); raw and norm depend on D_z through u
-            const T u = (z_[m] - th[11 + i] - nz_mu[i]) / nz_sg[i];
+            const T u = (z_[m] - th[11 + i] - nz_mu[i]) * isg[i];
             const T gn = gnc * nc;
-            ge += gn / e;
-            sum[S_COUNT + i] += gn * u / nz_sg[i];
+            ge += gn * ie;
+            sum[S_COUNT + i] += gn * u * isg[i];
             sum[S_COUNT + NB + i] += gn;
         }
         // omw = wa chiH / (a^2 E)
-        sum[S_CHIH] += go * o / chiH;
-        gE[m] = ge - go * o / e;
+        sum[S_CHIH] += go * o * ichiH;
+        gE[m] = ge - go * o * ie;
         t2[m] = gc;
     }
     __syncthreads();
@@ -661,37 +735,35 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
     // distances: chi_n = sum_{m<n} dchi_m -> g_dchi_m = sum_{n>m} g_chi_n
     block_scan<2, true>(t1, N, N, red);
     for (int m = tid; m < N; m += nt) {
-        const T a = a_[m], lna = lna_[m], e = Ez[m];
+        const T a = a_[m], lna = lna_[m], ie = T(1) / Ez[m], ia = ia_[m];
         T gf = T(0);
         if (m < N - 1) gf += T(0.5) * t1[m] * (lna - lna_[m + 1]);
         if (m >= 1) gf += T(0.5) * t1[m - 1] * (lna_[m - 1] - lna);
-        const T ia3 = ex<T>(T(-3) * lna);
-        const T oma = om * ia3 / (e * e);
+        const T ia3 = ia * ia * ia;
+        const T oma = om * ia3 * (ie * ie);
         const T gff = gf * fg[m];
         sum[S_GAMMA] += gff * lg<T>(oma);
-        sum[S_OM] += gff * gamma / om;
+        sum[S_OM] += gff * gamma * iom;
         // node E: E^2 = om a^-3 + (1 - om) de
-        const T ge2 = (gE[m] - T(2) * gff * gamma / e) / (T(2) * e);
+        const T ge2 = (gE[m] - T(2) * gff * gamma * ie) * T(0.5) * ie;
         const T de = ex<T>(-pde * lna - T(3) * wa * (T(1) - a));
         sum[S_OM] += ge2 * (ia3 - de);
         sum[S_W0] += ge2 * (T(1) - om) * de * (T(-3) * lna);
         sum[S_WA] += ge2 * (T(1) - om) * de * (T(-3) * lna - T(3) * (T(1) - a));
         if (m < N - 1) {
-            const T g = t2[m], a1 = a_[m + 1];
-            const T mid = T(0.5) * (a + a1), half = T(0.5) * (a - a1);
+            const T g = t2[m], half = T(0.5) * (a - a_[m + 1]);
             T inc = T(0);
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const T ag = mid + half * glx<T>(q);
-                const T lgg = lg<T>(ag), i3 = T(1) / (ag * ag * ag);
-                const T deg = ex<T>(-pde * lgg - T(3) * wa * (T(1) - ag));
-                const T e2 = om * i3 + (T(1) - om) * deg;
-                const T F = T(1) / (ag * ag * sqrt(e2));
+                const T lgg = gl_ln[4 * m + q], ig = gl_ia[4 * m + q], oma_q = gl_1ma[4 * m + q], i3 = ig * ig * ig;
+                const T deg = ex<T>(-pde * lgg - T(3) * wa * oma_q);
+                const T rs = rsq(om * i3 + (T(1) - om) * deg);
+                const T F = ig * ig * rs;
                 inc += glw<T>(q) * F;
-                const T gE2 = g * chiH * half * glw<T>(q) * T(-0.5) * F / e2;
+                const T gE2 = g * chiH * half * glw<T>(q) * T(-0.5) * F * (rs * rs);
                 sum[S_OM] += gE2 * (i3 - deg);
                 sum[S_W0] += gE2 * (T(1) - om) * deg * (T(-3) * lgg);
-                sum[S_WA] += gE2 * (T(1) - om) * deg * (T(-3) * lgg - T(3) * (T(1) - ag));
+                sum[S_WA] += gE2 * (T(1) - om) * deg * (T(-3) * lgg - T(3) * oma_q);
             }
             sum[S_CHIH] += g * half * inc;
         }
@@ -714,8 +786,8 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
         double* g = gfull + (size_t)row * sp.n_params;
         for (int i = 0; i < NB; ++i) {
             const T gn = gs[S_COUNT + NB + i];
-            chih -= gn / chiH;                  // nchi ~ 1 / chiH
-            g[11 + i] += (double)(gs[S_COUNT + i] - gn / norm[i] * gs[S_COUNT + 2 * NB + i]);
+            chih -= gn * ichiH;                 // nchi ~ 1 / chiH
+            g[11 + i] += (double)(gs[S_COUNT + i] - gn * (inorm[i] * chiH) * gs[S_COUNT + 2 * NB + i]);
         }
         // pref = 1.5 om / chiH^2; gamma = 0.55 + 0.05 (1 + w0 + wa/2)
         const T g_om = gs[S_OM] + gs[S_PREF] * pref / om;
@@ -734,6 +806,17 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
 struct OutT64 {
     double* p;
     __device__ __forceinline__ void put(int row, int i, int n, double v) const { p[(size_t)row * n + i] = v; }
+};
+// scaled and in bf16 planes: the operand of the emulator's backward GEMMs
+template <int P>
+struct OutPlaneT {
+    __nv_bfloat16* p;
+    long long stride;
+    int pitch;
+    float s;
+    __device__ __forceinline__ void put(int row, int i, int, float v) const {
+        tc::plane_store<P>(s * v, p + (size_t)row * pitch + i, stride);
+    }
 };
 struct OutT32 {
     float* p;
@@ -785,6 +868,9 @@ int projection_adj_create(const ShearParams& sp, int elt, int cap, ProjectionAdj
     NS_TRY(alloc(n * sp.D, &a->gC));
     NS_TRY(alloc(n * sp.nb * sp.N, &a->gV));
     NS_TRY(alloc(n * sp.N, &a->glnc));
+    std::vector<double> lnell(sp.n_ell);
+    NS_CUDA_TRY(cudaMemcpy(lnell.data(), sp.lnell, sizeof(double) * sp.n_ell, cudaMemcpyDeviceToHost));
+    a->sorted = std::is_sorted(lnell.begin(), lnell.end());
     std::vector<int> zrp(sp.N);
     NS_CUDA_TRY(cudaMemcpy(zrp.data(), sp.zrp, sizeof(int) * sp.N, cudaMemcpyDeviceToHost));
     size_t part = 0;
@@ -842,13 +928,13 @@ template <typename T, int RB>
 static int launch_chi2_adj(const ShearParams& sp, ProjectionAdj* a, const double* theta_full, const T* LinvT,
                            const T* Linv, double c0, double* gfull, double* logL, const int* nrows, int grid_rows,
                            cudaStream_t st) {
-    const size_t smem = sizeof(T) * RB * (2 * (size_t)sp.D + sp.nb + sp.n_pairs + 8 * (size_t)sp.n_tmpl);
+    const size_t smem = sizeof(T) * adj::chi2_adj_elems(sp.D, sp.nb, sp.n_pairs, sp.n_tmpl, RB);
     static bool attr = false;
     if (!attr) {
         NS_CUDA_TRY(cudaFuncSetAttribute(adj::k_chi2_adj<T, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmemMax));
         attr = true;
     }
-    NS_CUDA_TRY(launch_pdl(adj::k_chi2_adj<T, RB>, dim3((grid_rows + RB - 1) / RB), dim3(256), smem, st, sp, theta_full,
+    NS_CUDA_TRY(launch_pdl(adj::k_chi2_adj<T, RB>, dim3((grid_rows + RB - 1) / RB), dim3(adj::kChiThreads), smem, st, sp, theta_full,
                            (const T*)a->resid, (const T*)a->C, LinvT, Linv, c0, (T*)a->gC, gfull, logL, nrows));
     return NS_OK;
 }
@@ -859,7 +945,7 @@ static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double*
     const int k = limber_adj_split(grid_rows), W = 8 << k, PK = sp.n_k + 2;
     // a warp's columns of gradients and of the current table rows; the rows stay
     // in global memory, and CTAs shrink to one warp, where tables are very wide
-    const size_t col = sizeof(adj::V4<T>) * (size_t)PK;
+    const size_t col = sizeof(adj::Z4<T>) * (size_t)PK;
     const int stage = 2 * col <= kAdjSmemMax;
     int nw = kAdjWarps;
     while (nw > 1 && nw * col * (stage ? 2 : 1) > kAdjSmemMax) nw >>= 1;
@@ -873,16 +959,21 @@ static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double*
     }
     NS_CUDA_TRY(launch_pdl(adj::k_limber_adj<T, NB>, dim3(grid_rows * (W / nw)), dim3(32 * nw), smem, st, sp, table,
                            (const T*)a->win, (const T*)a->gC, (const int4*)a->ranges[k], W, a->part_rows[k],
-                           (T*)a->part, (T*)a->gV, (T*)a->glnc, stage, nrows));
-    const dim3 g(grid_rows, grid_rows < 256 ? 8 : 2);
+                           (T*)a->part, (T*)a->gV, (T*)a->glnc, stage, a->sorted, nrows));
+    // a table row per block for few evaluations, a third of the table for many
+    const dim3 g(grid_rows, grid_rows < 256 ? sp.n_z : 3);
+    const dim3 b(std::min(256, (sp.n_k + 31) & ~31));
+    auto table_adj = [&](auto o) -> int {
+        NS_CUDA_TRY(launch_pdl(adj::k_table_adj<T, decltype(o)>, g, b, 0, st, (const T*)a->part, a->part_rows[k],
+                               (const int*)a->ptr[k], (const int*)a->idx[k], sp.n_z, sp.n_k, o, nrows));
+        return NS_OK;
+    };
     if constexpr (sizeof(T) == 8) {
-        NS_CUDA_TRY(launch_pdl(adj::k_table_adj<T, adj::OutT64>, g, dim3(256), 0, st, (const T*)a->part, a->part_rows[k],
-                               (const int*)a->ptr[k], (const int*)a->idx[k], sp.n_z, sp.n_k,
-                               adj::OutT64{(double*)out.table}, nrows));
+        NS_TRY(table_adj(adj::OutT64{(double*)out.table}));
     } else {
-        NS_CUDA_TRY(launch_pdl(adj::k_table_adj<T, adj::OutT32>, g, dim3(256), 0, st, (const T*)a->part, a->part_rows[k],
-                               (const int*)a->ptr[k], (const int*)a->idx[k], sp.n_z, sp.n_k,
-                               adj::OutT32{(float*)out.table}, nrows));
+        if (out.px == 3) NS_TRY(table_adj(adj::OutPlaneT<3>{out.planes, out.stride, out.pitch, out.scale}));
+        else if (out.px == 2) NS_TRY(table_adj(adj::OutPlaneT<2>{out.planes, out.stride, out.pitch, out.scale}));
+        else NS_TRY(table_adj(adj::OutT32{(float*)out.table}));
     }
     NS_CUDA_TRY(launch_pdl(adj::k_windows_adj<T, NB>, dim3(grid_rows), dim3(adj::kWinAdjThreads), a->win_smem, st, sp,
                            theta_full, (const T*)a->gV, (const T*)a->glnc, (T*)a->scratch, gfull, nrows));
@@ -896,9 +987,9 @@ int launch_projection_adj(const ShearParams& sp, ProjectionAdj* a, const double*
     NS_CUDA_TRY(cudaStreamWaitEvent(st, a->ev_join, 0));
     NS_TRY((launch_limber<T, false>(sp, theta_full, table, (const T*)a->win, (T*)a->resid, nullptr, nrows, grid_rows,
                                     err, st, (T*)a->C)));
-    // two rows per block spread few rows over the chip, eight share the reads of L^-1
-    if (grid_rows < 1024)
-        NS_TRY((launch_chi2_adj<T, 2>(sp, a, theta_full, LinvT, Linv, c0, gfull, logL, nrows, grid_rows, st)));
+    // one row per block spreads few rows over the chip, eight share the reads of L^-1
+    if (grid_rows < 1024 || sizeof(T) * adj::chi2_adj_elems(sp.D, sp.nb, sp.n_pairs, sp.n_tmpl, 8) > kAdjSmemMax)
+        NS_TRY((launch_chi2_adj<T, 1>(sp, a, theta_full, LinvT, Linv, c0, gfull, logL, nrows, grid_rows, st)));
     else
         NS_TRY((launch_chi2_adj<T, 8>(sp, a, theta_full, LinvT, Linv, c0, gfull, logL, nrows, grid_rows, st)));
     switch (sp.nb) {

@@ -16,6 +16,7 @@ struct ProjectionAdj {
     void* part = nullptr;              // partial rows of the table gradient
     void* scratch = nullptr;           // arrays of k_windows_adj where shared memory does not hold them
     size_t win_smem = 0;
+    int sorted = 0;                    // ascending multipoles
     int4* ranges[3] = {};              // node ranges for 8, 16, 32 warps per evaluation
     int *ptr[3] = {}, *idx[3] = {}, part_rows[3] = {};
     cudaStream_t side = nullptr;       // the windows run beside the emulator
@@ -23,8 +24,15 @@ struct ProjectionAdj {
     std::vector<void*> owned;
 };
 
+// Where d log L / d table goes: rows x (n_z n_k) in FP64 or FP32, or (px = 2, 3)
+// scaled into px bf16 planes.
 struct TableGrad {
-    void* table = nullptr;             // rows x (n_z n_k), FP64 or FP32
+    void* table = nullptr;
+    int px = 0;
+    __nv_bfloat16* planes = nullptr;
+    long long stride = 0;
+    int pitch = 0;
+    float scale = 1.f;
 };
 
 int projection_adj_create(const ShearParams& sp, int elt, int cap, ProjectionAdj* a);
