@@ -392,8 +392,9 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, double* log
         } else {
             planes_out(e, g->Hp[l + 1], p->dims[l + 1]);
         }
+        // BF16: no K split, so that every activation has the bits of the one chain
         NS_TRY(launch_gemm_planes(px, pw, &g->tmW[l], &g->tmH[l], e, g->d_nrows, B, p->dims[l + 1], p->dims[l],
-                                  g->d_err, st));
+                                  pw == 1 ? 1 : 0, g->d_err, st));
     }
     const float* tab = (const float*)g->table;
     const bool coarse = p->n_z_emu != sp.n_z;
@@ -427,11 +428,12 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, double* log
         PlaneEpi e;
         e.mode = l == 1 ? PLN_DTANH32 : PLN_DTANH;
         e.aux = g->Hp[l];
+        e.aux_planes = px;
         e.aux_pitch = plane_pitch(p->dims[l]);
         e.aux_stride = g->rows_pad * e.aux_pitch;
         if (l == 1) e.out = g->G1;
         else planes_out(e, g->Gp[(L - l) & 1], p->dims[l]);
-        NS_TRY(launch_gemm_planes(px, pw, &g->tmWT[l], &g->tmG[l], e, g->d_nrows, B, p->dims[l], p->dims[l + 1],
+        NS_TRY(launch_gemm_planes(px, pw, &g->tmWT[l], &g->tmG[l], e, g->d_nrows, B, p->dims[l], p->dims[l + 1], 0,
                                   g->d_err, st));
     }
     return launch_finish_grad<float>(p, g, g->G1, B, grad, st);

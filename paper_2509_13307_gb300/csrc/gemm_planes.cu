@@ -14,7 +14,8 @@
 // accuracy.  Each 64-deep k-block is therefore summed in TMEM by itself,
 // small plane products first, and the epilogue warps add the block sums in
 // FP32 registers (round to nearest) while the next block's MMAs run in the
-// second TMEM buffer.
+// second TMEM buffer.  (BF16 gradients, two planes of 16 bits on bf16 weights,
+// are far from that limit: one accumulator for all of K, leading plane first.)
 //
 // Tiles.  The MMA's M is 128 features (rows of W), its N is BR rows of X, so
 // few rows waste no tensor work; BR = 32, 64, 128, or 256 where two ring slots
@@ -73,6 +74,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
 k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const PlaneEpi e,
               const int* __restrict__ nrows, int N, int K, int* __restrict__ err) {
     using C = CfgP<PX, PW, BR>;
+    constexpr bool CHAIN = PX == 2;                  // all of K in one accumulator
     constexpr int HC = BR / 2;                       // rows per epilogue warp
     pdl_begin();
     const int M = *nrows;
@@ -136,10 +138,22 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
             constexpr uint32_t idesc = instr_desc<BR>();
             for (int it = 0; it < n_it; ++it) {
                 const int s = it % C::STAGES, b = it & 1;
-                if (it >= 2 && !mbar_wait(acc_empty(b), ((it >> 1) & 1) ^ 1)) { s_fail = 1; break; }
+                if (!CHAIN && it >= 2 && !mbar_wait(acc_empty(b), ((it >> 1) & 1) ^ 1)) { s_fail = 1; break; }
                 if (!mbar_wait(full_bar(s), (it / C::STAGES) & 1)) { s_fail = 1; break; }
                 fence_after();
-                const uint32_t sa = base + s * C::STAGE_BYTES, d = tmem + (uint32_t)(b * BR);
+                const uint32_t sa = base + s * C::STAGE_BYTES, sx = sa + C::W_BYTES;
+                if constexpr (CHAIN) {
+#pragma unroll
+                    for (int kk = 0; kk < BK / 16; ++kk)
+#pragma unroll
+                        for (int q = 0; q < PX; ++q)
+                            mma_bf16(tmem, smem_desc(sa) + 2 * kk, smem_desc(sx + q * C::X_SUB) + 2 * kk, idesc,
+                                     (it | kk | q) != 0);
+                    mma_commit(empty_bar(s));
+                    if (it == n_it - 1) mma_commit(acc_full(0));
+                    continue;
+                }
+                const uint32_t d = tmem + (uint32_t)(b * BR);
                 uint32_t accumulate = 0;
                 // plane pairs in ascending order of size: p + q = 2, 1, 0
 #pragma unroll
@@ -149,7 +163,7 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
                         const int p = sum - q;
                         if (p < 0 || p >= PW) continue;
                         const uint64_t dw = smem_desc(sa + p * C::W_SUB);
-                        const uint64_t dx = smem_desc(sa + C::W_BYTES + q * C::X_SUB);
+                        const uint64_t dx = smem_desc(sx + q * C::X_SUB);
 #pragma unroll
                         for (int kk = 0; kk < BK / 16; ++kk) {
                             mma_bf16(d, dw + 2 * kk, dx + 2 * kk, idesc, accumulate);
@@ -164,7 +178,7 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     } else {
         const uint32_t addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * HC);
         constexpr int CW = HC < 32 ? HC : 32;
-        for (int it = 0; it < n_it; ++it) {
+        for (int it = 0; it < (CHAIN ? 1 : n_it); ++it) {
             const int b = it & 1;
             if (!mbar_wait(acc_full(b), (it >> 1) & 1)) { s_fail = 1; break; }
             fence_after();
@@ -210,8 +224,7 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
             v = (g + (1.f - g) / (1.f + expf(-beta * v))) * v;
         } else {
             float h = 0.f;
-#pragma unroll
-            for (int p = PX - 1; p >= 0; --p)
+            for (int p = e.aux_planes - 1; p >= 0; --p)
                 h += __bfloat162float(e.aux[p * e.aux_stride + (size_t)row * e.aux_pitch + f]);
             v *= 1.f - h * h;
             if (e.mode == PLN_DTANH32) {
@@ -339,7 +352,7 @@ __global__ void __launch_bounds__(256) k_split_planes(const float* __restrict__ 
 
 }  // namespace tc
 
-// Rows per tile and K split of one launch, by the cycles of the SM that ends
+// Rows per tile and K split (unless given) of one launch, by the cycles of the SM that ends
 // last.  A k-block costs its MMAs (N / 2 cycles each, or the shared-memory
 // reads of both operands) or its copies (54 B per cycle and SM with every SM
 // loading, 450 cycles at least); a CTA adds 2500 for set-up and the first
@@ -350,16 +363,16 @@ __global__ void __launch_bounds__(256) k_split_planes(const float* __restrict__ 
 // 10000 and 512 -> 512 -> 2507 layers: the choice is the fastest of the 12 or
 // within 7 % of it everywhere (1024 -> 1024, emulator at 64 rows: 90 us with
 // the chosen 64 / 8, 101 with 32 / 8, 130 with 64 / 1, 181 with 128 / 1).
-PlaneTiling plane_tiling(int rows, int N, int K, int px, int pw) {
+PlaneTiling plane_tiling(int rows, int N, int K, int px, int pw, int split) {
     int prod = 0;
     for (int p = 0; p < pw; ++p)
         for (int q = 0; q < px; ++q) prod += p + q <= 2;
     const int nk = (K + tc::BK - 1) / tc::BK, mt = (N + 127) / 128;
-    PlaneTiling best{128, 1};
+    PlaneTiling best{128, std::max(split, 1)};
     double best_t = 1e300;
     for (int br : {32, 64, 128, 256})
         for (int s : {1, 2, 4, 8}) {
-            if (s > nk || (br == 256 && 256 * (128 * pw + 256 * px) > 192 * 1024)) continue;
+            if (s > nk || (split && s != split) || (br == 256 && 256 * (128 * pw + 256 * px) > 192 * 1024)) continue;
             const double mma = prod * 4.0 * std::max(br / 2.0, (128 + br) / 4.0);
             const double load = std::max(450.0, 128.0 * (128 * pw + br * px) / 54.0);
             const int sms = s == 8 ? 96 : s == 4 ? 128 : 152;
@@ -372,10 +385,20 @@ PlaneTiling plane_tiling(int rows, int N, int K, int px, int pw) {
     return best;
 }
 
+// The K split of a likelihood's layer, by its shape alone: a row's log L must not
+// depend on the batch it comes in (the shards of a run evaluate their own
+// chains), and the split fixes the order of the sums.  Four ways while that
+// leaves a chip of SMs to the row tiles: on 1024 -> 1024 within 5 % of the best split
+// at 1 to 1000 rows.
+int plane_split(int N, int K) {
+    const int mt = (N + 127) / 128, nk = (K + tc::BK - 1) / tc::BK;
+    return mt <= 8 && nk >= 4 ? 4 : mt <= 16 && nk >= 2 ? 2 : 1;
+}
+
 int launch_gemm_planes(int px, int pw, const CUtensorMap* tmW, const PlaneMapX* tmX, const PlaneEpi& e,
-                       const int* nrows, int grid_rows, int N, int K, int* err, cudaStream_t st) {
+                       const int* nrows, int grid_rows, int N, int K, int split, int* err, cudaStream_t st) {
     if (grid_rows <= 0) return NS_OK;
-    const PlaneTiling t = plane_tiling(grid_rows, N, K, px, pw);
+    const PlaneTiling t = plane_tiling(grid_rows, N, K, px, pw, split);
     if (px == 3 && pw == 3) return tc::launch_planes_p<3, 3>(tmW, tmX, e, nrows, grid_rows, N, K, t, err, st);
     if (px == 2 && pw == 1) return tc::launch_planes_p<2, 1>(tmW, tmX, e, nrows, grid_rows, N, K, t, err, st);
     if (px == 1 && pw == 3) return tc::launch_planes_p<1, 3>(tmW, tmX, e, nrows, grid_rows, N, K, t, err, st);

@@ -424,8 +424,9 @@ static int launch_head_f32(const ns_problem* p, Workspace* ws, int grid_rows, in
     e.sig_vec = (const float*)hd.sig_vec;
     e.sigma = (float)hd.sigma;
     e.out = (float*)hd.out;
-    return launch_gemm_planes(px, 3, hd.tmW, &ws->tmXp[L - 1], e, ws->d_nrows, grid_rows,
-                              hd.n_out ? hd.n_out : p->dims[L], p->dims[L - 1], ws->d_err, st);
+    const int N = hd.n_out ? hd.n_out : p->dims[L], K = p->dims[L - 1];
+    return launch_gemm_planes(px, 3, hd.tmW, &ws->tmXp[L - 1], e, ws->d_nrows, grid_rows, N, K, plane_split(N, K),
+                              ws->d_err, st);
 }
 
 // FP32: the input layer on CUDA cores, every further layer as an FP32-accurate
@@ -447,7 +448,7 @@ static int run_emulator_f32(const ns_problem* p, Workspace* ws, int grid_rows, c
         e.plane_stride = ws->plane_stride;
         e.pitch = plane_pitch(p->dims[l + 1]);
         NS_TRY(launch_gemm_planes(3, 3, &p->tmWp[l], &ws->tmXp[l], e, ws->d_nrows, grid_rows, p->dims[l + 1],
-                                  p->dims[l], ws->d_err, st));
+                                  p->dims[l], plane_split(p->dims[l + 1], p->dims[l]), ws->d_err, st));
         cur ^= 1;
     }
     return launch_head_f32(p, ws, grid_rows, 3, hd, st);

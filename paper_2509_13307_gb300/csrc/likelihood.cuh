@@ -250,16 +250,19 @@ struct PlaneEpi {
     __nv_bfloat16* planes = nullptr;  // TANH, SIGLIN, DTANH: px planes of row pitch `pitch`
     long long plane_stride = 0;
     int pitch = 0;
-    const __nv_bfloat16* aux = nullptr;  // DTANH: acc (1 - h^2), h in px planes
+    const __nv_bfloat16* aux = nullptr;  // DTANH: acc (1 - h^2), h in aux_planes planes
+    int aux_planes = 0;
     long long aux_stride = 0;
     int aux_pitch = 0;
 };
 struct PlaneTiling {
     int br, split;                    // rows per tile; CTAs of a cluster sharing the k-blocks
 };
-PlaneTiling plane_tiling(int rows, int N, int K, int px, int pw);
+PlaneTiling plane_tiling(int rows, int N, int K, int px, int pw, int split);
+int plane_split(int N, int K);        // the split of a likelihood's layer (by shape, not by rows)
 int launch_gemm_planes(int px, int pw, const CUtensorMap* tmW, const PlaneMapX* tmX, const PlaneEpi& e,
-                       const int* nrows, int grid_rows, int N, int K, int* err, cudaStream_t st);
+                       const int* nrows, int grid_rows, int N, int K, int split /* 0: by rows too */, int* err,
+                       cudaStream_t st);
 // planes of s * in (rows x cols, packed); nrows: device row count or null
 int launch_split_planes(int planes, const float* in, float s, int rows, int cols, __nv_bfloat16* out, long long stride,
                         int pitch, const int* nrows, cudaStream_t st);

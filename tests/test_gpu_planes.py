@@ -93,3 +93,17 @@ def test_gradient_tiles(precision, hidden, rows):
         ratio = float(((got[b] - ref[b]).abs() / bound).max())
         print(f"{precision} {hidden} row {b} of {rows}: error / bound = {ratio:.3f}")
         assert ratio <= 1.0
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_rows_do_not_depend_on_their_batch(precision):
+    """The shards of a run evaluate their own chains: the same row gives the same
+    bits in every batch size (every row tile, and both sides of the FP64 rules)."""
+    from paper_2509_13307_gb300 import Problem
+    inp = w.make_shear_inputs(replace(w.shear_tiny(), emu_hidden=(1024, 1024)))
+    D, rows = len(inp["noise_eps"]), 400
+    p = Problem(inp, precision, max_batch=rows, data=np.ones(D), cov=np.eye(D))
+    theta = torch.tensor(free_theta(inp, random_cube(rows, p.d, 3)), device="cuda")
+    whole = p.loglike(theta)
+    for n in (1, 5, 33, 64, 100, 153, 250):
+        assert torch.equal(p.loglike(theta[:n]), whole[:n])
