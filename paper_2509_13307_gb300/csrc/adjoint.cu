@@ -488,9 +488,7 @@ extern "C" int loglike_grad_batch(const ns_problem* p, const double* theta_dev, 
             g_grad_states.push_back(gs);
         }
     }
-    NS_TRY(launch_free_to_full_ext(p, theta_dev, B, gs->theta_full, st));
-    k_set_int<<<1, 1, 0, st>>>(gs->d_nrows, B);
-    NS_CUDA_TRY(cudaGetLastError());
+    NS_TRY(launch_free_to_full(p, theta_dev, B, gs->theta_full, gs->d_nrows, st));
     if (p->precision == NS_PREC_FP64) return run_grad_f64(p, gs, B, logL_dev, grad_dev, st);
     return run_grad_planes(p, gs, B, logL_dev, grad_dev, st);
 }

@@ -16,9 +16,9 @@
 // row's largest |w| for K = 1024, against 2^-48 for the rounding of an FP64 FMA
 // chain.
 //
-// Tiles: 128 features (the MMA's M) x 32 rows; six accumulators of 32 columns
-// twice fill TMEM.  Slots of 32 k hold every slice of both operands (60 KB, 64-byte
-// swizzle, three slots).  Few tiles are spread over clusters of S CTAs along k,
+// Tiles: 128 features (the MMA's M) x 16, 32 or 64 rows, six accumulators each
+// (twice in TMEM for up to 32 rows).  Slots of 32 k hold every slice of both
+// operands (60 KB for 32 rows, 64-byte swizzle, three slots).  Few tiles are spread over clusters of S CTAs along k,
 // whose integer partial tiles are added exactly through cluster shared memory.
 // A NaN operand (its leading slice is NaN) and a timeout give NaN.
 //
@@ -26,8 +26,8 @@
 // (the call 6367 -> 1070 us); error of its table against 113-bit arithmetic
 // rms 1.17e-16, largest 4.1e-16 (FMA chain 1.18e-16 and 4.8e-16).
 //
-// Warps 0-7: drain and epilogue; warp 8: copies; warp 9: TMEM and MMAs.  Waits are
-// bounded as in gemm_planes.cu.
+// Warps 0-7 (0-15 for 64 rows): drain and epilogue; then one warp for the copies
+// and one for TMEM and MMAs.  Waits are bounded as in gemm_planes.cu.
 #include <algorithm>
 
 #include "likelihood.cuh"
@@ -40,17 +40,23 @@ using namespace tc;
 
 constexpr int NS = kSlices;                      // slices of an operand
 constexpr int SBK = 32;                          // k per slot: 64 bytes of fp16
-constexpr int BR = 32;                           // rows per tile
-constexpr int W_SUB = 128 * SBK * 2, X_SUB = BR * SBK * 2;
-constexpr int STAGE_BYTES = NS * (W_SUB + X_SUB);
+constexpr int W_SUB = 128 * SBK * 2;
 constexpr int STAGES = 3;
 constexpr int CHUNK = 4;                         // slots per TMEM accumulation: 128 k
-constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256;
-constexpr int EPI_WARPS = 8, THREADS = 32 * (EPI_WARPS + 2);
-constexpr int HC = BR / 2;                       // rows per epilogue warp
 constexpr long long kNaN = 1ll << 58;            // stands for NaN in a sum (others stay below 2^50; eight of it fit)
-static_assert(STAGES * STAGE_BYTES >= 128 * BR * 16, "the partial tile reuses the ring");
-static_assert(2 * NS * BR <= 512, "two sets of accumulators in TMEM");
+
+template <int BR>                                // rows per tile
+struct CfgL {
+    static constexpr int X_SUB = BR * SBK * 2;
+    static constexpr int STAGE_BYTES = NS * (W_SUB + X_SUB);
+    static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 256;
+    static constexpr int NBUF = BR <= 32 ? 2 : 1;    // sets of accumulators that fit TMEM
+    static constexpr uint32_t TMEM_COLS = BR == 16 ? 256 : 512;
+    static constexpr int EPI_WARPS = BR == 64 ? 16 : 8, THREADS = 32 * (EPI_WARPS + 2);
+    static constexpr int HC = BR / (EPI_WARPS / 4);  // rows per epilogue warp
+    static_assert(STAGES * STAGE_BYTES >= 128 * BR * 16, "the partial tile reuses the ring");
+    static_assert(NBUF * NS * BR <= (int)TMEM_COLS, "accumulators in TMEM");
+};
 
 // K-major tile of 64-byte rows, 64-byte swizzle (8-row groups of 512 bytes).
 __device__ __forceinline__ uint64_t desc64(uint32_t addr) {
@@ -59,11 +65,16 @@ __device__ __forceinline__ uint64_t desc64(uint32_t addr) {
 }
 
 // kind::f16, D = F32, A = B = F16, K-major, M = 128, N = BR
+template <int BR>
 constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(BR >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 
-__global__ void __launch_bounds__(THREADS, 1)
+template <int BR>
+__global__ void __launch_bounds__(CfgL<BR>::THREADS, 1)
 k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, const SliceEpi e,
               const int* __restrict__ nrows, int N, int K, int* __restrict__ err) {
+    using C = CfgL<BR>;
+    constexpr int STAGE_BYTES = C::STAGE_BYTES, X_SUB = C::X_SUB, EPI_WARPS = C::EPI_WARPS, HC = C::HC, NBUF = C::NBUF;
+    constexpr int W_LOAD = EPI_WARPS, W_MMA = EPI_WARPS + 1;   // the other two warps
     pdl_begin();
     const int M = *nrows;
     const int S = gridDim.x, rank = blockIdx.x;
@@ -89,9 +100,9 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
         for (int b = 0; b < 2; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), EPI_WARPS); }
         mbar_init_fence();
     }
-    if (warp == 9) {
+    if (warp == W_MMA) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     :: "r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+                     :: "r"(smem_u32(tmem_slot)), "r"(C::TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     fence_before();
@@ -106,7 +117,7 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     long long hi[HC], lo[HC];                    // sums of i + j = 0..2 and 3..5, in units of the last of each
 #pragma unroll
     for (int j = 0; j < HC; ++j) { hi[j] = 0; lo[j] = 0; }
-    if (warp == 8) {
+    if (warp == W_LOAD) {
         if (lane == 0) {
             int issued = 0;
             for (int it = 0; it < n_it; ++it) {
@@ -123,12 +134,12 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
                 if (!mbar_wait(full_bar(it % STAGES), (it / STAGES) & 1)) s_fail = 1;
         }
         __syncwarp();
-    } else if (warp == 9) {
+    } else if (warp == W_MMA) {
         if (lane == 0) {
             bool ok = true;
             for (int it = 0; it < n_it && ok; ++it) {
-                const int s = it % STAGES, c = it / CHUNK, b = c & 1, in = it % CHUNK;
-                if (in == 0 && c >= 2) ok = mbar_wait(acc_empty(b), ((c >> 1) & 1) ^ 1);
+                const int s = it % STAGES, c = it / CHUNK, b = c % NBUF, in = it % CHUNK;
+                if (in == 0 && c >= NBUF) ok = mbar_wait(acc_empty(b), ((c / NBUF) & 1) ^ 1);
                 ok = ok && mbar_wait(full_bar(s), (it / STAGES) & 1);
                 if (!ok) { s_fail = 1; break; }
                 fence_after();
@@ -140,7 +151,7 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
                         const uint64_t dw = desc64(sw + i * W_SUB), dx = desc64(sx + j * X_SUB);
 #pragma unroll
                         for (int kk = 0; kk < SBK / 16; ++kk)
-                            mma_bf16(tmem + (uint32_t)((b * NS + i + j) * BR), dw + 2 * kk, dx + 2 * kk, kIdesc,
+                            mma_bf16(tmem + (uint32_t)((b * NS + i + j) * BR), dw + 2 * kk, dx + 2 * kk, kIdesc<BR>,
                                      in != 0 || i != 0 || kk != 0);
                     }
                 mma_commit(empty_bar(s));
@@ -151,8 +162,8 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     } else {
         const uint32_t addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * HC);
         for (int c = 0; c < n_chunk; ++c) {
-            const int b = c & 1;
-            if (!mbar_wait(acc_full(b), (c >> 1) & 1)) { s_fail = 1; break; }
+            const int b = c % NBUF;
+            if (!mbar_wait(acc_full(b), (c / NBUF) & 1)) { s_fail = 1; break; }
             fence_after();
             __syncwarp();
 #pragma unroll
@@ -208,7 +219,7 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     if (warp < EPI_WARPS) {
         const int end = min(BR * (rank + 1) / S, M - r0);
 #pragma unroll 1
-        for (int rl = BR * rank / S + (tid >> 7); rl < end; rl += 2) {
+        for (int rl = BR * rank / S + (tid >> 7); rl < end; rl += EPI_WARPS / 4) {
             const int at = rl * 128 + (tid & 127);
             long long h = red[at], l = red[BR * 128 + at];
             for (int q = 1; q < S; ++q) {        // integers: any order
@@ -223,9 +234,9 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     if (failed && tid == 0 && err) atomicOr(err, NS_BIT_TIMEOUT);
     fence_before();
     __syncthreads();
-    if (warp == 9) {
+    if (warp == W_MMA) {
         fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(512u) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(C::TMEM_COLS) : "memory");
     }
 }
 
@@ -249,25 +260,19 @@ __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ W
 
 }  // namespace slc
 
-int launch_gemm_slices(const CUtensorMap* tmW, const CUtensorMap* tmX, const SliceEpi& e, const int* nrows,
-                       int grid_rows, int N, int K, int* err, cudaStream_t st) {
-    if (grid_rows <= 0) return NS_OK;
+template <int BR>
+static int launch_slices_t(const CUtensorMap* tmW, const CUtensorMap* tmX, const SliceEpi& e, const int* nrows,
+                           int grid_rows, int N, int K, int S, int* err, cudaStream_t st) {
+    using C = slc::CfgL<BR>;
     static bool attr = false;
     if (!attr) {
-        NS_CUDA_TRY(cudaFuncSetAttribute(slc::k_gemm_slices, cudaFuncAttributeMaxDynamicSharedMemorySize, slc::SMEM));
+        NS_CUDA_TRY(cudaFuncSetAttribute(slc::k_gemm_slices<BR>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
         attr = true;
     }
-    // the largest split that keeps every cluster resident (about 96 SMs hold
-    // clusters of 8, 128 clusters of 4, one CTA each) and a chunk per CTA
-    const int nk = (K + slc::SBK - 1) / slc::SBK;
-    const long long tiles = (long long)((N + 127) / 128) * ((grid_rows + slc::BR - 1) / slc::BR);
-    int S = 1;
-    for (int s : {2, 4, 8})
-        if (tiles * s <= (s == 8 ? 96 : s == 4 ? 128 : 152) && nk >= slc::CHUNK * s) S = s;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(S, (N + 127) / 128, (grid_rows + slc::BR - 1) / slc::BR);
-    cfg.blockDim = dim3(slc::THREADS);
-    cfg.dynamicSmemBytes = slc::SMEM;
+    cfg.gridDim = dim3(S, (N + 127) / 128, (grid_rows + BR - 1) / BR);
+    cfg.blockDim = dim3(C::THREADS);
+    cfg.dynamicSmemBytes = C::SMEM;
     cfg.stream = st;
     cudaLaunchAttribute a[2];
     a[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -278,8 +283,38 @@ int launch_gemm_slices(const CUtensorMap* tmW, const CUtensorMap* tmX, const Sli
     a[1].val.clusterDim.z = 1;
     cfg.attrs = a;
     cfg.numAttrs = 2;
-    NS_CUDA_TRY(cudaLaunchKernelEx(&cfg, slc::k_gemm_slices, *tmW, *tmX, e, nrows, N, K, err));
+    NS_CUDA_TRY(cudaLaunchKernelEx(&cfg, slc::k_gemm_slices<BR>, *tmW, *tmX, e, nrows, N, K, err));
     return NS_OK;
+}
+
+int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const SliceEpi& e, const int* nrows,
+                       int grid_rows, int N, int K, int* err, cudaStream_t st) {
+    if (grid_rows <= 0) return NS_OK;
+    // Rows per tile and K split by the cycles of the SM that ends last (sums are
+    // exact, so the choice does not change a bit).  A slot is 42 MMAs of ~65 cycles
+    // each up to N = 64; the epilogue's FP64 runs at two operations per cycle (tanh
+    // and slicing ~75 per element, the output 6); 64-row tiles have one set of
+    // accumulators and wait for each drain; clusters of 8 (4) find room on about 96
+    // (128) SMs.  64 rows: 64-row output tiles 1 wave of 79 CTAs against two of 158
+    // (111 us); 16-row hidden tiles spread the FP64 of tanh over 128 SMs.
+    const int nk = (K + slc::SBK - 1) / slc::SBK, mt = (N + 127) / 128;
+    int best_br = 32, best_s = 1;
+    double best = 1e300;
+    for (int br : {16, 32, 64})
+        for (int s : {1, 2, 4, 8}) {
+            if (s > 1 && nk < slc::CHUNK * s) continue;
+            const int sms = s == 8 ? 96 : s == 4 ? 128 : 152, slots = (nk + s - 1) / s;
+            const long long ctas = (long long)mt * ((grid_rows + br - 1) / br) * s;
+            const double t = (double)((ctas + sms - 1) / sms) *
+                             (3000.0 + 2750.0 * slots + (br == 64 ? 3000.0 * (slots / slc::CHUNK) : 0.0) +
+                              64.0 * br / s * (e.tanh ? 75 : 6) + (s > 1 ? 2500.0 : 0.0));
+            if (t < 0.97 * best) { best = t; best_br = br; best_s = s; }
+        }
+    switch (best_br) {
+        case 16: return launch_slices_t<16>(tmW, &tmX->m[0], e, nrows, grid_rows, N, K, best_s, err, st);
+        case 32: return launch_slices_t<32>(tmW, &tmX->m[1], e, nrows, grid_rows, N, K, best_s, err, st);
+        default: return launch_slices_t<64>(tmW, &tmX->m[2], e, nrows, grid_rows, N, K, best_s, err, st);
+    }
 }
 
 int launch_slice_rows(const double* W, int rows, int K, __half* out, long long stride, int pitch, double* scale,

@@ -7,6 +7,7 @@
 //   projection.cu     App. A projection (distances, windows, P lookup, Limber,
 //                     data vector) and the whitened chi^2.
 #include <algorithm>
+#include <type_traits>
 
 #include "likelihood.cuh"
 #include "tcgen05.cuh"
@@ -62,9 +63,10 @@ __global__ void k_cube_to_free(const double* __restrict__ cube, int d, int P,
 
 __global__ void k_free_to_full(const double* __restrict__ theta, int d, int P,
                                const double* __restrict__ pa, const int* __restrict__ free_of_full,
-                               double* __restrict__ theta_full, int B) {
+                               double* __restrict__ theta_full, int B, int* __restrict__ nrows) {
     const int row = blockIdx.x;
     if (row >= B) return;
+    if (row == 0 && threadIdx.x == 0) *nrows = B;
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         const int f = free_of_full[i];
         theta_full[(size_t)row * P + i] = (f < 0) ? pa[i] : theta[(size_t)row * d + f];
@@ -153,11 +155,14 @@ k_emu_input(const double* __restrict__ theta_full, int P, const int* __restrict_
             const OUT out, const int* __restrict__ nrows) {
     // the weights of a thread's first UP units are problem constants: in
     // registers before the dependency wait
-    constexpr int UP = KMAX <= 8 ? 4 : 1;
+    constexpr int UP = sizeof(T) == 4 && KMAX <= 8 ? 4 : 1;
+    // FP64 (tanh is ~50 operations on a pipe of two per cycle and SM): the units
+    // are spread over gridDim.y CTAs too
+    const int n0 = sizeof(T) == 8 ? 256 * blockIdx.y : 0, nstep = sizeof(T) == 8 ? 256 * gridDim.y : blockDim.x;
     T wp[UP][KMAX], bp[UP];
 #pragma unroll
     for (int u = 0; u < UP; ++u) {
-        const int n = threadIdx.x + u * blockDim.x;
+        const int n = n0 + threadIdx.x + u * blockDim.x;
 #pragma unroll
         for (int j = 0; j < KMAX; ++j) wp[u][j] = (n < N && j < K0) ? W0[(size_t)n * K0 + j] : T(0);
         bp[u] = n < N ? b0[n] : T(0);
@@ -187,10 +192,10 @@ k_emu_input(const double* __restrict__ theta_full, int P, const int* __restrict_
     };
 #pragma unroll
     for (int u = 0; u < UP; ++u) {
-        const int n = threadIdx.x + u * blockDim.x;
+        const int n = n0 + threadIdx.x + u * blockDim.x;
         if (n < N) unit(n, wp[u], bp[u]);
     }
-    for (int n = threadIdx.x + UP * blockDim.x; n < N; n += blockDim.x) {
+    for (int n = n0 + threadIdx.x + UP * nstep; n < N; n += nstep) {
         T w[KMAX];
 #pragma unroll
         for (int j = 0; j < KMAX; ++j) w[j] = j < K0 ? W0[(size_t)n * K0 + j] : T(0);
@@ -265,22 +270,61 @@ k_gemm_simt(const T* __restrict__ A, const T* __restrict__ W, const T* __restric
 }
 
 // Coarse-z emulator table -> n_z table: out[jz][ik] = sum_q w[jz][q] in[row[jz][q]][ik]
-// (Catmull-Rom in z with folded ghosts).
-template <typename T>
-__global__ void k_zinterp(const T* __restrict__ coarse, int nzc, const int* __restrict__ zr,
-                          const double* __restrict__ zwt, T* __restrict__ fine, int nz, int nk,
-                          const int* __restrict__ nrows) {
+// (Catmull-Rom in z with folded ghosts).  A block takes a share of an
+// evaluation's z nodes, threads V columns each (16-byte accesses where rows
+// allow); the taps and weights, converted once, sit in shared memory.  375 rows of
+// 10 -> 50 nodes: 29 us with a division and four FP64 conversions per entry.
+template <typename T, int V>
+__global__ void __launch_bounds__(256) k_zinterp(const T* __restrict__ coarse, int nzc, const int* __restrict__ zr,
+                                                 const double* __restrict__ zwt, T* __restrict__ fine, int nz, int nk,
+                                                 const int* __restrict__ nrows) {
+    struct alignas(sizeof(T) * V) Vec { T v[V]; };
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* w = reinterpret_cast<T*>(smem_raw);
+    int* tap = reinterpret_cast<int*>(w + 4 * nz);
+    for (int i = threadIdx.x; i < 4 * nz; i += 256) {
+        w[i] = (T)zwt[i];
+        tap[i] = zr[i] * nk;
+    }
+    pdl_begin();
     const int row = blockIdx.y;
     if (row >= *nrows) return;
+    __syncthreads();
     const T* c = coarse + (size_t)row * nzc * nk;
     T* f = fine + (size_t)row * nz * nk;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nz * nk; i += gridDim.x * blockDim.x) {
-        const int jz = i / nk, ik = i % nk;
-        T v = T(0);
+    const int cols = nk / V, per = min(cols, 256), lines = 256 / per;
+    if (threadIdx.x >= per * lines) return;
+    const int k0 = threadIdx.x % per;
+    for (int jz = blockIdx.x * lines + threadIdx.x / per; jz < nz; jz += gridDim.x * lines)
+        for (int k = k0; k < cols; k += per) {
+            Vec o;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v += (T)zwt[jz * 4 + q] * c[zr[jz * 4 + q] * nk + ik];
-        f[i] = v;
+            for (int e = 0; e < V; ++e) o.v[e] = T(0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const Vec x = *reinterpret_cast<const Vec*>(c + tap[jz * 4 + q] + k * V);
+#pragma unroll
+                for (int e = 0; e < V; ++e) o.v[e] += w[jz * 4 + q] * x.v[e];
+            }
+            *reinterpret_cast<Vec*>(f + (size_t)jz * nk + k * V) = o;
+        }
+}
+
+template <typename T>
+static int launch_zinterp(const ns_problem* p, const T* coarse, T* fine, const int* nrows, int grid_rows,
+                          cudaStream_t st) {
+    constexpr int V = 16 / sizeof(T);
+    const ShearParams& sp = p->sp;
+    const bool vec = sp.n_k % V == 0;          // rows of 16-byte multiples in cudaMalloc'ed buffers
+    const size_t smem = 4 * (size_t)sp.n_z * (sizeof(T) + sizeof(int));
+    if (smem > 48 * 1024) {
+        auto k = vec ? k_zinterp<T, V> : k_zinterp<T, 1>;
+        NS_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     }
+    NS_CUDA_TRY(launch_pdl(vec ? k_zinterp<T, V> : k_zinterp<T, 1>, dim3(grid_rows < 304 ? 4 : 2, grid_rows), dim3(256),
+                           smem, st, coarse, p->n_z_emu, (const int*)p->d_zi_row, (const double*)p->d_zi_w, fine, sp.n_z,
+                           sp.n_k, nrows));
+    return NS_OK;
 }
 
 static int launch_gemm_simt(const double* A, const double* W, const double* bias, ActDev<double> act, const double* mu,
@@ -326,7 +370,7 @@ template <typename T, typename OUT>
 static int launch_emu_input(const ns_problem* p, const double* theta_full, const int* nrows, int grid_rows,
                             const ActDev<T>& act, const OUT& out, cudaStream_t st) {
     const int K0 = p->dims[0], H1 = p->dims[1];
-    const dim3 g((grid_rows + kInRows - 1) / kInRows);
+    const dim3 g((grid_rows + kInRows - 1) / kInRows, sizeof(T) == 8 ? std::min(8, (H1 + 255) / 256) : 1);
     auto kern = K0 <= 8 ? k_emu_input<T, OUT, 8> : k_emu_input<T, OUT, 32>;
     NS_CUDA_TRY(launch_pdl(kern, g, dim3(256), 0, st, theta_full, p->P, (const int*)p->d_inputs,
                            (const double*)p->d_in_center, (const double*)p->d_in_scale,
@@ -526,6 +570,7 @@ __global__ void k_to_double(const T* __restrict__ in, double* __restrict__ out, 
 template <typename T>
 __global__ void __launch_bounds__(256) k_rowsq(const T* __restrict__ y, int D, double c0, double* __restrict__ logL,
                                                const int* __restrict__ nrows) {
+    pdl_begin();
     const int row = blockIdx.x;
     if (row >= *nrows) return;
     __shared__ double part[256];
@@ -548,6 +593,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_cmb_tt(const T* __restrict__ C, int n_tt, int ld, const T* __restrict__ dobs,
                                                 const T* __restrict__ halfk, double c0, double* __restrict__ logL,
                                                 const int* __restrict__ nrows) {
+    pdl_begin();
     const int row = blockIdx.x;
     if (row >= *nrows) return;
     __shared__ double part[256];
@@ -600,15 +646,15 @@ static int run_cmb(const ns_problem* p, Workspace* ws, int grid_rows, double* lo
         else if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_f32(p, ws, grid_rows, st, hd));
         else NS_TRY(run_emulator_bf16(p, ws, grid_rows, st, probe, &hd));
         NS_TRY(probe_begin(probe, PROBE_CHI2, ws, st));
-        if (f64)
-            k_cmb_tt<double><<<grid_rows, 256, 0, st>>>((const double*)ws->table, p->n_tt, p->n_tt,
-                                                        (const double*)p->d_tt_obs, (const double*)p->d_tt_halfk,
-                                                        p->c0, logL_out, ws->d_nrows);
-        else
-            k_cmb_tt<float><<<grid_rows, 256, 0, st>>>((const float*)ws->table, p->n_tt, p->n_tt,
-                                                       (const float*)p->d_tt_obs, (const float*)p->d_tt_halfk,
-                                                       p->c0, logL_out, ws->d_nrows);
-        NS_CUDA_TRY(cudaGetLastError());
+        auto tt = [&](auto kern, auto* tab) -> int {
+            using T = std::remove_pointer_t<decltype(tab)>;
+            NS_CUDA_TRY(launch_pdl(kern, dim3(grid_rows), dim3(256), 0, st, (const T*)tab, p->n_tt, p->n_tt,
+                                   (const T*)p->d_tt_obs, (const T*)p->d_tt_halfk, p->c0, logL_out,
+                                   (const int*)ws->d_nrows));
+            return NS_OK;
+        };
+        if (f64) NS_TRY(tt(k_cmb_tt<double>, (double*)ws->table));
+        else NS_TRY(tt(k_cmb_tt<float>, (float*)ws->table));
         return probe_end(probe, PROBE_CHI2, st);
     }
     if (p->cmb_solve == NS_SOLVE_LITERAL) {
@@ -625,9 +671,12 @@ static int run_cmb(const ns_problem* p, Workspace* ws, int grid_rows, double* lo
     else if (p->precision == NS_PREC_FP32) NS_TRY(run_emulator_f32(p, ws, grid_rows, st, hd));
     else NS_TRY(run_emulator_bf16(p, ws, grid_rows, st, probe, &hd));
     NS_TRY(probe_begin(probe, PROBE_CHI2, ws, st));
-    if (f64) k_rowsq<double><<<grid_rows, 256, 0, st>>>((const double*)ws->table, D, p->c0, logL_out, ws->d_nrows);
-    else k_rowsq<float><<<grid_rows, 256, 0, st>>>((const float*)ws->table, D, p->c0, logL_out, ws->d_nrows);
-    NS_CUDA_TRY(cudaGetLastError());
+    if (f64)
+        NS_CUDA_TRY(launch_pdl(k_rowsq<double>, dim3(grid_rows), dim3(256), 0, st, (const double*)ws->table, D, p->c0,
+                               logL_out, (const int*)ws->d_nrows));
+    else
+        NS_CUDA_TRY(launch_pdl(k_rowsq<float>, dim3(grid_rows), dim3(256), 0, st, (const float*)ws->table, D, p->c0,
+                               logL_out, (const int*)ws->d_nrows));
     return probe_end(probe, PROBE_CHI2, st);
 }
 
@@ -649,7 +698,7 @@ int run_likelihood(const ns_problem* p, Workspace* ws, int grid_rows, double* lo
     NS_CUDA_TRY(cudaEventRecord(ws->ev_fork, st));
     NS_CUDA_TRY(cudaStreamWaitEvent(ws->side, ws->ev_fork, 0));
     NS_TRY(probe_begin(probe, PROBE_WINDOWS, ws, ws->side));
-    if (f64) NS_TRY(launch_windows<double, false>(sp, ws->theta_full, (double*)ws->win, ws->d_nrows, grid_rows, ws->side));
+    if (f64) NS_TRY(launch_windows<double, false>(sp, ws->theta_full, (double*)ws->win, ws->d_nrows, grid_rows, ws->side, (double*)ws->win_nodes));
     else if (p->precision == NS_PREC_FP32)
         NS_TRY(launch_windows<float, false>(sp, ws->theta_full, (float*)ws->win, ws->d_nrows, grid_rows, ws->side));
     else NS_TRY(launch_windows<float, true>(sp, ws->theta_full, (float*)ws->win, ws->d_nrows, grid_rows, ws->side));
@@ -659,10 +708,7 @@ int run_likelihood(const ns_problem* p, Workspace* ws, int grid_rows, double* lo
         NS_TRY(run_emulator_f64(p, ws, grid_rows, st, model_head(p, ws->table)));
         const double* tab = (const double*)ws->table;
         if (coarse) {
-            dim3 g((sp.n_z * sp.n_k + 255) / 256, grid_rows);
-            k_zinterp<double><<<g, 256, 0, st>>>(tab, p->n_z_emu, p->d_zi_row, p->d_zi_w,
-                                                 (double*)ws->table_fine, sp.n_z, sp.n_k, ws->d_nrows);
-            NS_CUDA_TRY(cudaGetLastError());
+            NS_TRY(launch_zinterp<double>(p, tab, (double*)ws->table_fine, ws->d_nrows, grid_rows, st));
             tab = (const double*)ws->table_fine;
         }
         NS_CUDA_TRY(cudaStreamWaitEvent(st, ws->ev_join, 0));
@@ -677,10 +723,7 @@ int run_likelihood(const ns_problem* p, Workspace* ws, int grid_rows, double* lo
     else NS_TRY(run_emulator_bf16(p, ws, grid_rows, st, probe, nullptr));
     const float* tab = (const float*)ws->table;
     if (coarse) {
-        dim3 g((sp.n_z * sp.n_k + 255) / 256, grid_rows);
-        k_zinterp<float><<<g, 256, 0, st>>>(tab, p->n_z_emu, p->d_zi_row, p->d_zi_w, (float*)ws->table_fine,
-                                            sp.n_z, sp.n_k, ws->d_nrows);
-        NS_CUDA_TRY(cudaGetLastError());
+        NS_TRY(launch_zinterp<float>(p, tab, (float*)ws->table_fine, ws->d_nrows, grid_rows, st));
         tab = (const float*)ws->table_fine;
     }
     NS_CUDA_TRY(cudaStreamWaitEvent(st, ws->ev_join, 0));
@@ -714,8 +757,9 @@ int launch_cube_to_free(const ns_problem* p, const double* cube, int B, double* 
     NS_CUDA_TRY(cudaGetLastError());
     return NS_OK;
 }
-int launch_free_to_full(const ns_problem* p, const double* theta, int B, double* theta_full, cudaStream_t st) {
-    k_free_to_full<<<B, 64, 0, st>>>(theta, p->d, p->P, p->d_pa, p->d_free_of_full, theta_full, B);
+int launch_free_to_full(const ns_problem* p, const double* theta, int B, double* theta_full, int* nrows,
+                        cudaStream_t st) {
+    k_free_to_full<<<B, 64, 0, st>>>(theta, p->d, p->P, p->d_pa, p->d_free_of_full, theta_full, B, nrows);
     NS_CUDA_TRY(cudaGetLastError());
     return NS_OK;
 }
@@ -724,18 +768,7 @@ int launch_free_to_full(const ns_problem* p, const double* theta, int B, double*
 namespace gpuns {
 int launch_zinterp_generic(const ns_problem* p, const void* coarse, void* fine, const int* nrows, int grid_rows, int elt,
                            cudaStream_t st) {
-    const ShearParams& sp = p->sp;
-    dim3 g((sp.n_z * sp.n_k + 255) / 256, grid_rows);
-    if (elt == 8)
-        k_zinterp<double><<<g, 256, 0, st>>>((const double*)coarse, p->n_z_emu, p->d_zi_row, p->d_zi_w, (double*)fine,
-                                             sp.n_z, sp.n_k, nrows);
-    else
-        k_zinterp<float><<<g, 256, 0, st>>>((const float*)coarse, p->n_z_emu, p->d_zi_row, p->d_zi_w, (float*)fine,
-                                            sp.n_z, sp.n_k, nrows);
-    NS_CUDA_TRY(cudaGetLastError());
-    return NS_OK;
-}
-int launch_free_to_full_ext(const ns_problem* p, const double* theta, int B, double* theta_full, cudaStream_t st) {
-    return launch_free_to_full(p, theta, B, theta_full, st);
+    if (elt == 8) return launch_zinterp<double>(p, (const double*)coarse, (double*)fine, nrows, grid_rows, st);
+    return launch_zinterp<float>(p, (const float*)coarse, (float*)fine, nrows, grid_rows, st);
 }
 }  // namespace gpuns

@@ -57,6 +57,11 @@ struct PlaneMapX {
     CUtensorMap m[4];
 };
 
+// Of k_gemm_slices: row tiles 16, 32, 64.
+struct SliceMapX {
+    CUtensorMap m[3];
+};
+
 struct Workspace {
     int cap = 0;
     int* d_nrows = nullptr;       // device row count used by every stage
@@ -68,10 +73,11 @@ struct Workspace {
     void* table_fine = nullptr;   // cap x n_z*n_k (coarse-z emulators)
     void* resid = nullptr;        // cap x D residuals
     void* win = nullptr;          // cap x (nb + 1) x pitch: ln chi and windows (pitch = N rounded up to 4)
+    void* win_nodes = nullptr;    // FP64: the windows' node-local functions
     double* logL = nullptr;       // cap
     // tcgen05 tensor maps (BF16 precision): A operand of layer l >= 1 and its output
     std::vector<CUtensorMap> tmA;
-    std::vector<CUtensorMap> tmXs;   // FP64 tanh emulators: layer l's input slices (plane_stride apart)
+    std::vector<SliceMapX> tmXs;   // FP64 tanh emulators: layer l's input slices (plane_stride apart)
     // k_gemm_planes: layer l's input planes (FP32: three; the FP32 head of a BF16 CMB problem: one)
     std::vector<PlaneMapX> tmXp;
     long long plane_stride = 0;   // FP32, FP64 slices: elements between the planes of an activation buffer
@@ -187,7 +193,9 @@ int launch_cube_to_theta(const ns_problem* p, Workspace* ws, const double* cube,
 // Limber sums C_ij(ell) themselves.  FAST selects SFU transcendentals.
 template <typename T, bool FAST>
 int launch_windows(const ShearParams& sp, const double* theta_full, T* win, const int* nrows, int grid_rows,
-                   cudaStream_t st);
+                   cudaStream_t st, T* nodes = nullptr);
+// values per chi node that a separate launch prepares for the windows (FP64: nodes, rows x values x N)
+constexpr int window_node_values(int nb) { return 4 + nb; }
 template <typename T, bool FAST>
 int launch_limber(const ShearParams& sp, const double* theta_full, const T* table, const T* win, T* resid,
                   double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st, T* cl_out = nullptr);
@@ -201,10 +209,11 @@ template <typename TR, typename TA>
 int launch_chi2(const TR* resid, int D, const TA* LinvT, double c0, double* logL, const int* nrows, int grid_rows,
                 cudaStream_t st, bool rows_ready = false);
 
-int launch_free_to_full(const ns_problem* p, const double* theta, int B, double* theta_full, cudaStream_t st);
+// free -> full parameter vectors, and the device row count
+int launch_free_to_full(const ns_problem* p, const double* theta, int B, double* theta_full, int* nrows,
+                        cudaStream_t st);
 int launch_zinterp_generic(const ns_problem* p, const void* coarse, void* fine, const int* nrows, int grid_rows,
                            int elt, cudaStream_t st);
-int launch_free_to_full_ext(const ns_problem* p, const double* theta, int B, double* theta_full, cudaStream_t st);
 
 // BF16 tcgen05 GEMM: C[M x N] = epi(A[M x K] * W[N x K]^T + bias), M = *d_nrows.
 // epi 0: tanh -> bf16 C (ldc = N); epi 1: mu + sigma * v -> fp32 C.
@@ -287,7 +296,7 @@ struct SliceEpi {
     long long slice_stride = 0;
     int pitch = 0;
 };
-int launch_gemm_slices(const CUtensorMap* tmW, const CUtensorMap* tmX, const SliceEpi& e, const int* nrows,
+int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const SliceEpi& e, const int* nrows,
                        int grid_rows, int N, int K, int* err, cudaStream_t st);
 int launch_slice_rows(const double* W, int rows, int K, __half* out, long long stride, int pitch, double* scale,
                       cudaStream_t st);

@@ -117,7 +117,9 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
         ws->plane_stride = (long long)rows_pad * plane_pitch(p->hidden_max);
         ws->tmXs.resize(p->n_layers);
         for (int l = 1; l < p->n_layers; ++l)
-            NS_TRY(make_tensor_map_slices(&ws->tmXs[l], ws->act[(l - 1) & 1], rows_pad, p->dims[l], ws->plane_stride, 32));
+            for (int i = 0; i < 3; ++i)
+                NS_TRY(make_tensor_map_slices(&ws->tmXs[l].m[i], ws->act[(l - 1) & 1], rows_pad, p->dims[l],
+                                              ws->plane_stride, 16 << i));
     }
     if (p->precision == NS_PREC_FP32) {
         ws->plane_stride = (long long)rows_pad * plane_pitch(p->hidden_max);
@@ -161,6 +163,10 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
     ws->resid = v;
     NS_TRY(dalloc((size_t)tab_elt * cap * (p->sp.nb + 1) * ((p->sp.N + 3) & ~3), &v, ws->owned));
     ws->win = v;
+    if (p->precision == NS_PREC_FP64) {
+        NS_TRY(dalloc(sizeof(double) * (size_t)cap * window_node_values(p->sp.nb) * p->sp.N, &v, ws->owned));
+        ws->win_nodes = v;
+    }
     NS_CUDA_TRY(cudaStreamCreateWithFlags(&ws->side, cudaStreamNonBlocking));
     NS_CUDA_TRY(cudaEventCreateWithFlags(&ws->ev_fork, cudaEventDisableTiming));
     NS_CUDA_TRY(cudaEventCreateWithFlags(&ws->ev_join, cudaEventDisableTiming));
@@ -951,7 +957,6 @@ extern "C" int ns_problem_dim(const ns_problem* p, int* d) {
 
 namespace gpuns {
 int launch_cube_to_free(const ns_problem* p, const double* cube, int B, double* theta, cudaStream_t st);
-int launch_free_to_full(const ns_problem* p, const double* theta, int B, double* theta_full, cudaStream_t st);
 }
 
 extern "C" int ns_prior_transform(const ns_problem* p, const double* cube_dev, int B, double* theta_dev,
@@ -963,10 +968,7 @@ extern "C" int ns_prior_transform(const ns_problem* p, const double* cube_dev, i
 
 static int batch_common(const ns_problem* p, const double* theta_dev, int B, cudaStream_t st) {
     ns_problem* mp = const_cast<ns_problem*>(p);
-    NS_TRY(launch_free_to_full(p, theta_dev, B, mp->ws.theta_full, st));
-    k_set_int<<<1, 1, 0, st>>>(mp->ws.d_nrows, B);
-    NS_CUDA_TRY(cudaGetLastError());
-    return NS_OK;
+    return launch_free_to_full(p, theta_dev, B, mp->ws.theta_full, mp->ws.d_nrows, st);
 }
 
 extern "C" int loglike_batch(const ns_problem* p, const double* theta_dev, int B, double* logL_dev, void* stream) {

@@ -137,10 +137,61 @@ __device__ __forceinline__ T warp_transpose_sum16(T (&v)[16]) {
 // win_pitch(N) (16-byte multiples, for the Limber stage's bulk copy), to `win`.
 __host__ __device__ inline int win_pitch(int N) { return (N + 3) & ~3; }
 
+// Node-local functions of the FP64 windows: E, the chi increment of the interval,
+// Omega_m(a)^gamma, the IA power ((1 + z) / pivot)^eta and the shifted Gaussians.  They hold three
+// quarters of the stage's FP64 work, which one CTA per evaluation would put on one
+// SM's two FMAs per cycle; here every SM takes nodes.
+template <typename T, int NB>
+__global__ void __launch_bounds__(128)
+k_window_nodes(const ShearParams sp, const double* __restrict__ theta_full, T* __restrict__ nodes,
+               const int* __restrict__ nrows) {
+    using M = Math<T, false>;
+    const int row = blockIdx.y, n = blockIdx.x * 128 + threadIdx.x, N = sp.N;
+    if (row >= *nrows || n >= N) return;
+    const double* t = theta_full + (size_t)row * sp.n_params;
+    const T h = (T)t[2];
+    const T om = ((T)t[0] + (T)t[1]) / (h * h);
+    const T w0 = (T)t[5], wa = (T)t[6];
+    const T pde = T(3) * (T(1) + w0 + wa);
+    const T chiH = T(kCover100) / h;
+    const T gamma = T(0.55) + T(0.05) * (T(1) + w0 + T(0.5) * wa);
+    const T* a_ = pick<T>(sp.a, sp.a_f);
+    const T* lna_ = pick<T>(sp.lna, sp.lna_f);
+    const T* z_ = pick<T>(sp.z, sp.z_f);
+    const T* ia_ = pick<T>(sp.ia, sp.ia_f);
+    const T* gl_ia = pick<T>(sp.gl_ia, sp.gl_ia_f);
+    const T* gl_ln = pick<T>(sp.gl_ln, sp.gl_ln_f);
+    const T* gl_1ma = pick<T>(sp.gl_1ma, sp.gl_1ma_f);
+    const T* nz_mu = pick<T>(sp.nz_mean, sp.nz_mean_f);
+    const T* nz_sg = pick<T>(sp.nz_sigma, sp.nz_sigma_f);
+    T* o = nodes + (size_t)row * window_node_values(NB) * N + n;
+    const T a = a_[n], lna = lna_[n], ia = ia_[n], a3 = ia * ia * ia;
+    const T e = sqrt_<T>(om * a3 + (T(1) - om) * M::ex(-pde * lna - T(3) * wa * (T(1) - a)));
+    T inc = T(0);
+    if (n < N - 1) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+            const T ig = gl_ia[4 * n + g];
+            const T eg = om * ig * ig * ig + (T(1) - om) * M::ex(-pde * gl_ln[4 * n + g] - T(3) * wa * gl_1ma[4 * n + g]);
+            inc += gl4_w<T>(g) * ig * ig * M::rsq(eg);
+        }
+        inc *= chiH * (T(0.5) * (a - a_[n + 1]));
+    }
+    o[0] = e;
+    o[N] = inc;
+    o[2 * (size_t)N] = M::ex(gamma * M::lg(M::div(om * a3, e * e)));
+    o[3 * (size_t)N] = M::ex((T)t[10] * (-lna - pick_s<T>(sp.ln_pivot, sp.ln_pivot_f)));
+#pragma unroll
+    for (int i = 0; i < NB; ++i) {
+        const T u = (z_[n] - (T)t[11 + i] - nz_mu[i]) * M::div(T(1), nz_sg[i]);
+        o[(4 + i) * (size_t)N] = M::ex(T(-0.5) * u * u);
+    }
+}
+
 template <typename T, int NB, bool FAST>
 __global__ void __launch_bounds__(kProjThreads)
 k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __restrict__ win,
-          const int* __restrict__ nrows) {
+          const int* __restrict__ nrows, const T* __restrict__ nodes) {
     using M = Math<T, FAST>;
     const int row = blockIdx.x;
     if (row >= *nrows) return;
@@ -182,8 +233,16 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
     const T chiH = T(kCover100) / h;
     const T gamma = T(0.55) + T(0.05) * (T(1) + w0 + T(0.5) * wa);
 
+    // FP64: the node-local functions come from k_window_nodes
+    constexpr bool PRE = sizeof(T) == 8;
+    const T* pre = PRE ? nodes + (size_t)row * window_node_values(NB) * N : nullptr;
     // 1. background: E(a), chi by composite 4-point Gauss-Legendre + scan, growth
     for (int n = tid; n < N; n += nt) {
+        if constexpr (PRE) {
+            Ez[n] = pre[n];
+            t0[n] = pre[N + n];
+            continue;
+        }
         const T a = a_[n], lna = lna_[n];
         const T ian = FAST ? T(0) : ia_[n];
         const T a3 = FAST ? M::ex(T(-3) * lna) : ian * ian * ian;
@@ -213,8 +272,12 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
         chi[n] = c;
         lnchi[n] = (n >= 1) ? M::lg(c) : T(0);
         const T ian = FAST ? T(0) : ia_[n];
-        const T oma = M::div(om * (FAST ? M::ex(T(-3) * lna_[n]) : ian * ian * ian), Ez[n] * Ez[n]);
-        t1[n] = M::ex(gamma * M::lg(oma));
+        if constexpr (PRE) {
+            t1[n] = pre[2 * (size_t)N + n];
+        } else {
+            const T oma = M::div(om * (FAST ? M::ex(T(-3) * lna_[n]) : ian * ian * ian), Ez[n] * Ez[n]);
+            t1[n] = M::ex(gamma * M::lg(oma));
+        }
         omw[n] = FAST ? M::div(wa_[n] * chiH, a_[n] * a_[n] * Ez[n]) : M::div(wa_[n] * chiH * (ian * ian), Ez[n]);
     }
     __syncthreads();
@@ -242,7 +305,7 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             const T u = FAST ? (z_[n] - zc[i]) * isg[i] : (z_[n] - th[11 + i] - nz_mu[i]) * isg[i];
-            const T raw = M::ex(T(-0.5) * u * u);
+            const T raw = PRE ? pre[(4 + i) * (size_t)N + n] : M::ex(T(-0.5) * u * u);
             V[i * N + n] = raw;
             pn[i] += wz * raw;
         }
@@ -313,7 +376,7 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
         // ln((1 + z) / pivot) = -ln a - ln pivot
         const T lq = FAST ? M::lg((T(1) + z_[n]) * ipiv) : -lna_[n] - lnpiv;
         const T amp = FAST ? M::div(A_IA * M::ex(eta * lq) * c1om, Dg[n])
-                           : M::div(A_IA * M::ex(eta * lq) * c1rho * om, Dg[n]);
+                           : M::div(A_IA * (PRE ? pre[3 * (size_t)N + n] : M::ex(eta * lq)) * c1rho * om, Dg[n]);
         const T pc = pref * c * (FAST ? M::div(T(1), a_[n]) : ia_[n]);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
@@ -871,9 +934,10 @@ static int launch_whiten(const TR* resid, int D, const TA* LinvT, double c0, dou
 }
 
 // FP64 chi^2 of short data vectors: one CTA per row, so that few rows use many
-// SMs' FP64 pipes (two FMAs per cycle each; 45 k for D = 300).  Two threads share
-// a column's reduction range, whose loads stay in flight eight deep.
-constexpr int kRowThreads = 640, kRowMaxD = 1024;
+// SMs' FP64 pipes (two FMAs per cycle each; 45 k for D = 300).  A thread takes
+// two neighbouring columns (one 16-byte load) of one of `parts` shares of the
+// reduction range: a share is a short chain of L2 latencies.
+constexpr int kRowThreads = 1024, kRowMaxD = 1024;
 template <typename TR>
 __global__ void __launch_bounds__(kRowThreads)
 k_whiten_row(const TR* __restrict__ resid, int D, const double* __restrict__ LinvT, double c0,
@@ -881,25 +945,42 @@ k_whiten_row(const TR* __restrict__ resid, int D, const double* __restrict__ Lin
     pdl_begin();
     const int row = blockIdx.x;
     if (row >= *nrows) return;
-    __shared__ double r[kRowMaxD], part[kRowMaxD], red[32];
-    constexpr int COLS = kRowThreads / 2;
-    const int half = threadIdx.x / COLS, t = threadIdx.x % COLS;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[32];
+    const int groups = (D + 1) / 2, parts = max(1, kRowThreads / groups);
+    double* r = reinterpret_cast<double*>(smem_raw);         // D
+    double* part = r + D;                                    // parts x 2 groups
     for (int b = threadIdx.x; b < D; b += kRowThreads) r[b] = (double)resid[(size_t)row * D + b];
     __syncthreads();
-    double sq = 0.0;
-    for (int a0 = 0; a0 < D; a0 += COLS) {
-        const int a = a0 + t, mid = (a + 1) / 2;
-        double y = 0.0;
-        if (a < D) {
+    const bool vec = D % 2 == 0;                             // rows of L^-T on 16-byte boundaries
+    for (int i = threadIdx.x; i < groups * parts; i += kRowThreads) {
+        const int seg = i / groups, a = 2 * (i - seg * groups), end = min(D, a + 2);
+        const int b0 = end * seg / parts, b1 = end * (seg + 1) / parts;
+        const double* l = LinvT + a;
+        double y0 = 0.0, y1 = 0.0;
+        if (vec) {
 #pragma unroll 8
-            for (int b = half ? mid : 0; b < (half ? a + 1 : mid); ++b) y = fma(LinvT[(size_t)b * D + a], r[b], y);
-            if (half) part[a] = y;
+            for (int b = b0; b < b1; ++b) {
+                const double2 v = *reinterpret_cast<const double2*>(l + (size_t)b * D);
+                y0 = fma(v.x, r[b], y0);
+                y1 = fma(v.y, r[b], y1);
+            }
+        } else {
+#pragma unroll 8
+            for (int b = b0; b < b1; ++b) {
+                y0 = fma(l[(size_t)b * D], r[b], y0);
+                if (a + 1 < D) y1 = fma(l[(size_t)b * D + 1], r[b], y1);
+            }
         }
-        __syncthreads();
-        if (!half && a < D) {
-            y += part[a];
-            sq = fma(y, y, sq);
-        }
+        part[seg * 2 * groups + a] = y0;
+        part[seg * 2 * groups + a + 1] = y1;
+    }
+    __syncthreads();
+    double sq = 0.0;
+    for (int a = threadIdx.x; a < D; a += kRowThreads) {
+        double y = 0.0;
+        for (int q = 0; q < parts; ++q) y += part[q * 2 * groups + a];
+        sq = fma(y, y, sq);
     }
     sq = block_sum(sq, red);
     if (threadIdx.x == 0) logL[row] = c0 - 0.5 * sq;
@@ -913,8 +994,10 @@ int launch_chi2(const TR* resid, int D, const TA* LinvT, double c0, double* logL
     // 16-row blocks of 20 CTAs
     if constexpr (sizeof(TA) == 8) {
         if (D <= kRowMaxD) {
-            NS_CUDA_TRY(launch_pdl(k_whiten_row<TR>, dim3(grid_rows), dim3(kRowThreads), 0, st, resid, D, LinvT, c0, logL,
-                                   nrows));
+            const int groups = (D + 1) / 2, parts = std::max(1, kRowThreads / groups);
+            const size_t smem = sizeof(double) * ((size_t)D + 2 * (size_t)groups * parts);   // at most 26 KB
+            NS_CUDA_TRY(launch_pdl(k_whiten_row<TR>, dim3(grid_rows), dim3(kRowThreads), smem, st, resid, D, LinvT, c0,
+                                   logL, nrows));
             return NS_OK;
         }
     }
@@ -955,7 +1038,7 @@ bool projection_fits(const ShearParams& sp, int elt) {
 
 template <typename T, int NB, bool FAST>
 static int windows_nb(const ShearParams& sp, const double* theta_full, T* win, const int* nrows, int grid_rows,
-                      cudaStream_t st) {
+                      cudaStream_t st, T* nodes) {
     const size_t smem = windows_smem<T>(sp);
     if (smem > 227 * 1024) return NS_ENOTSUP;
     static bool attr_done = false;
@@ -963,7 +1046,12 @@ static int windows_nb(const ShearParams& sp, const double* theta_full, T* win, c
         NS_CUDA_TRY(cudaFuncSetAttribute(k_windows<T, NB, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
         attr_done = true;
     }
-    k_windows<T, NB, FAST><<<grid_rows, kProjThreads, smem, st>>>(sp, theta_full, win, nrows);
+    if constexpr (sizeof(T) == 8) {
+        if (!nodes) return NS_EINVAL;
+        k_window_nodes<T, NB><<<dim3((sp.N + 127) / 128, grid_rows), 128, 0, st>>>(sp, theta_full, nodes, nrows);
+        NS_CUDA_TRY(cudaGetLastError());
+    }
+    k_windows<T, NB, FAST><<<grid_rows, kProjThreads, smem, st>>>(sp, theta_full, win, nrows, nodes);
     NS_CUDA_TRY(cudaGetLastError());
     return NS_OK;
 }
@@ -1012,13 +1100,13 @@ static int limber_nb(const ShearParams& sp, const double* theta_full, const T* t
 
 template <typename T, bool FAST>
 int launch_windows(const ShearParams& sp, const double* theta_full, T* win, const int* nrows, int grid_rows,
-                   cudaStream_t st) {
+                   cudaStream_t st, T* nodes) {
     switch (sp.nb) {
-        case 1: return windows_nb<T, 1, FAST>(sp, theta_full, win, nrows, grid_rows, st);
-        case 2: return windows_nb<T, 2, FAST>(sp, theta_full, win, nrows, grid_rows, st);
-        case 3: return windows_nb<T, 3, FAST>(sp, theta_full, win, nrows, grid_rows, st);
-        case 4: return windows_nb<T, 4, FAST>(sp, theta_full, win, nrows, grid_rows, st);
-        case 5: return windows_nb<T, 5, FAST>(sp, theta_full, win, nrows, grid_rows, st);
+        case 1: return windows_nb<T, 1, FAST>(sp, theta_full, win, nrows, grid_rows, st, nodes);
+        case 2: return windows_nb<T, 2, FAST>(sp, theta_full, win, nrows, grid_rows, st, nodes);
+        case 3: return windows_nb<T, 3, FAST>(sp, theta_full, win, nrows, grid_rows, st, nodes);
+        case 4: return windows_nb<T, 4, FAST>(sp, theta_full, win, nrows, grid_rows, st, nodes);
+        case 5: return windows_nb<T, 5, FAST>(sp, theta_full, win, nrows, grid_rows, st, nodes);
         default: return NS_ENOTSUP;
     }
 }
@@ -1036,9 +1124,12 @@ int launch_limber(const ShearParams& sp, const double* theta_full, const T* tabl
     }
 }
 
-template int launch_windows<double, false>(const ShearParams&, const double*, double*, const int*, int, cudaStream_t);
-template int launch_windows<float, false>(const ShearParams&, const double*, float*, const int*, int, cudaStream_t);
-template int launch_windows<float, true>(const ShearParams&, const double*, float*, const int*, int, cudaStream_t);
+template int launch_windows<double, false>(const ShearParams&, const double*, double*, const int*, int, cudaStream_t,
+                                            double*);
+template int launch_windows<float, false>(const ShearParams&, const double*, float*, const int*, int, cudaStream_t,
+                                          float*);
+template int launch_windows<float, true>(const ShearParams&, const double*, float*, const int*, int, cudaStream_t,
+                                          float*);
 template int launch_limber<double, false>(const ShearParams&, const double*, const double*, const double*, double*,
                                           double*, const int*, int, int*, cudaStream_t, double*);
 template int launch_limber<float, false>(const ShearParams&, const double*, const float*, const float*, float*,

@@ -67,13 +67,19 @@ __device__ __forceinline__ float p10(float v) { return exp2f(v * 3.3219280948873
 
 // ------------------------------------------------------------------ chi^2
 // RB rows per block: each entry of L^-1 read serves RB rows, whose values lie
-// beside one another in shared memory.  Three threads share a column's reduction
-// range, with eight loads in flight each: a range walked by one thread is a chain
-// of L2 latencies (119 us for 64 rows, D = 300).
-constexpr int kChiCols = 320, kChiParts = 3, kChiThreads = kChiCols * kChiParts, kChiSeg = 16;
+// beside one another in shared memory.  A thread takes V neighbouring columns (one
+// 16-byte load) of one of `parts` shares of the reduction range, a short chain of
+// L2 latencies (one thread per column: 119 us for 64 rows, D = 300).
+constexpr int kChiThreads = 960, kChiSeg = 16;
+template <typename T> constexpr int kChiV = 16 / sizeof(T);
 
-__host__ __device__ inline size_t chi2_adj_elems(int D, int nb, int np, int nt, int rb) {
-    return (size_t)rb * ((2 + kChiParts - 1) * (size_t)D + nb + np + kChiSeg * (size_t)nt);
+// shares of the reduction range: what the threads allow, four for many rows
+__host__ __device__ inline int chi2_adj_parts(int D, int v, int rb) {
+    const int p = kChiThreads / ((D + v - 1) / v);
+    return p < 1 ? 1 : (rb > 1 && p > 4) ? 4 : p;
+}
+__host__ __device__ inline size_t chi2_adj_elems(int D, int v, int nb, int np, int nt, int rb) {
+    return (size_t)rb * ((2 + chi2_adj_parts(D, v, rb)) * (size_t)((D + v - 1) / v * v) + nb + np + kChiSeg * (size_t)nt);
 }
 
 template <typename T, int RB>
@@ -85,16 +91,19 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
     const int M = *nrows, r0 = blockIdx.x * RB;
     if (r0 >= M) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int V = kChiV<T>;
     const int D = sp.D, P = sp.n_params, nb = sp.nb, n_ell = sp.n_ell, nt = sp.n_tmpl, np = sp.n_pairs;
-    T* r = reinterpret_cast<T*>(smem_raw);     // D x RB, later g_m
-    T* y = r + D * RB;                         // D x RB
-    T* part = y + D * RB;                      // (kChiParts - 1) x D x RB
-    T* th = part + (kChiParts - 1) * D * RB;   // RB x nb: 1 + m_i
+    const int groups = (D + V - 1) / V, Dv = groups * V, parts = chi2_adj_parts(D, V, RB);
+    T* r = reinterpret_cast<T*>(smem_raw);     // Dv x RB, later g_m
+    T* y = r + Dv * RB;                        // Dv x RB
+    T* part = y + Dv * RB;                     // parts x Dv x RB
+    T* th = part + (size_t)parts * Dv * RB;    // RB x nb: 1 + m_i
     T* S = th + RB * nb;                       // np x RB: sum_ell g_m C
     T* tp = S + np * RB;                       // kChiSeg x RB x nt partial template sums
-    __shared__ T red[32];
+    __shared__ T wsum[(kChiThreads / 32) * RB];
+    __shared__ int pi[16], pj[16];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int seg = tid / kChiCols, col = tid % kChiCols;
+    if (tid < np) { pi[tid] = sp.pi[tid]; pj[tid] = sp.pj[tid]; }
     for (int i = tid; i < RB * D; i += kChiThreads) {
         const int j = i / D, a = i - j * D;
         r[a * RB + j] = r0 + j < M ? resid[(size_t)(r0 + j) * D + a] : T(0);
@@ -104,63 +113,66 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
         th[i] = r0 + j < M ? T(1) + (T)theta_full[(size_t)(r0 + j) * P + 11 + nb + i % nb] : T(0);
     }
     __syncthreads();
-    // acc[j] = sum_{b = lo}^{hi-1} A[b][a] x[b][j], the parts of a column in order
-    auto column = [&](const T* A, const T* x, int a, int lo, int hi, T (&acc)[RB]) {
-        const int b0 = lo + (hi - lo) * seg / kChiParts, b1 = lo + (hi - lo) * (seg + 1) / kChiParts;
+    // part[seg][a][j] = share seg of sum_b A[b][a] x[b][j]; lower: b <= a, else b >= a (A is zero elsewhere)
+    const bool vec = D % V == 0;
+    auto columns = [&](const T* A, const T* x, bool lower) {
+        for (int i = tid; i < groups * parts; i += kChiThreads) {
+            const int seg = i / groups, a = V * (i - seg * groups);
+            const int lo = lower ? 0 : a, hi = lower ? min(D, a + V) : D;
+            const int b0 = lo + (hi - lo) * seg / parts, b1 = lo + (hi - lo) * (seg + 1) / parts;
+            T acc[V][RB];
 #pragma unroll
-        for (int j = 0; j < RB; ++j) acc[j] = T(0);
+            for (int v = 0; v < V; ++v)
+#pragma unroll
+                for (int j = 0; j < RB; ++j) acc[v][j] = T(0);
 #pragma unroll 8
-        for (int b = b0; b < b1; ++b) {
-            const T l = A[(size_t)b * D + a];
+            for (int b = b0; b < b1; ++b) {
+                struct alignas(16) { T v[V]; } l;
+                if (vec) l = *reinterpret_cast<const decltype(l)*>(A + (size_t)b * D + a);
+                else
 #pragma unroll
-            for (int j = 0; j < RB; ++j) acc[j] = fma(l, x[b * RB + j], acc[j]);
-        }
-        if (seg > 0)
+                    for (int v = 0; v < V; ++v) l.v[v] = a + v < D ? A[(size_t)b * D + a + v] : T(0);
 #pragma unroll
-            for (int j = 0; j < RB; ++j) part[((seg - 1) * D + a) * RB + j] = acc[j];
-    };
-    auto join = [&](int a, T (&acc)[RB]) {
-        for (int q = 0; q < kChiParts - 1; ++q)
+                for (int v = 0; v < V; ++v)
 #pragma unroll
-            for (int j = 0; j < RB; ++j) acc[j] += part[(q * D + a) * RB + j];
-    };
-    T sq[RB];
-#pragma unroll
-    for (int j = 0; j < RB; ++j) sq[j] = T(0);
-    for (int a0 = 0; a0 < D; a0 += kChiCols) {
-        const int a = a0 + col;
-        T acc[RB];
-        if (a < D) column(LinvT, r, a, 0, a + 1, acc);
-        __syncthreads();
-        if (a < D && seg == 0) {
-            join(a, acc);
-#pragma unroll
-            for (int j = 0; j < RB; ++j) {
-                y[a * RB + j] = acc[j];
-                sq[j] = fma(acc[j], acc[j], sq[j]);
+                    for (int j = 0; j < RB; ++j) acc[v][j] = fma(l.v[v], x[b * RB + j], acc[v][j]);
             }
-        }
-    }
 #pragma unroll
-    for (int j = 0; j < RB; ++j) {
-        const T s = block_sum(sq[j], red);     // also orders y before its reads
-        if (tid == 0 && r0 + j < M) logL[r0 + j] = c0 - 0.5 * (double)s;
+            for (int v = 0; v < V; ++v)
+#pragma unroll
+                for (int j = 0; j < RB; ++j) part[((size_t)seg * Dv + a + v) * RB + j] = acc[v][j];
+        }
+        __syncthreads();
+    };
+    auto join = [&](int i) {                   // i = a * RB + j
+        T s = T(0);
+        for (int q = 0; q < parts; ++q) s += part[(size_t)q * Dv * RB + i];
+        return s;
+    };
+    columns(LinvT, r, true);
+    T sq = T(0);                               // kChiThreads is a multiple of RB: a thread keeps its row
+    static_assert(kChiThreads % RB == 0, "rows of a thread");
+    for (int i = tid; i < D * RB; i += kChiThreads) {
+        y[i] = join(i);
+        sq = fma(y[i], y[i], sq);
+    }
+    // row sums: lanes of equal row (stride RB), then over warps
+#pragma unroll
+    for (int o = 16; o >= RB; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+    if (lane < RB) wsum[wid * RB + lane] = sq;
+    __syncthreads();
+    if (tid < RB && r0 + tid < M) {
+        T s = T(0);
+        for (int w = 0; w < kChiThreads / 32; ++w) s += wsum[w * RB + tid];
+        logL[r0 + tid] = c0 - 0.5 * (double)s;
     }
     // g_m = L^-T y: (g_m)_a = sum_{b >= a} (L^-1)[b][a] y_b
-    for (int a0 = 0; a0 < D; a0 += kChiCols) {
-        const int a = a0 + col;
-        T acc[RB];
-        if (a < D) column(Linv, y, a, a, D, acc);
-        __syncthreads();
-        if (a < D && seg == 0) {
-            join(a, acc);
-            const int p = a / n_ell, i = sp.pi[p], k = sp.pj[p];
-#pragma unroll
-            for (int j = 0; j < RB; ++j) {
-                r[a * RB + j] = acc[j];
-                if (r0 + j < M) gC[(size_t)(r0 + j) * D + a] = acc[j] * th[j * nb + i] * th[j * nb + k];
-            }
-        }
+    columns(Linv, y, false);
+    for (int i = tid; i < D * RB; i += kChiThreads) {
+        const int a = i / RB, j = i % RB, p = a / n_ell;
+        const T g = join(i);
+        r[i] = g;
+        if (r0 + j < M) gC[(size_t)(r0 + j) * D + a] = g * th[j * nb + pi[p]] * th[j * nb + pj[p]];
     }
     __syncthreads();
     for (int q = tid; q < np * RB; q += kChiThreads) {
@@ -195,8 +207,8 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
         T v = T(0);
         if (i >= 0 && i < nb) {
             for (int p = 0; p < np; ++p) {
-                if (sp.pi[p] == i) v = fma(S[p * RB + j], th[j * nb + sp.pj[p]], v);
-                if (sp.pj[p] == i) v = fma(S[p * RB + j], th[j * nb + sp.pi[p]], v);
+                if (pi[p] == i) v = fma(S[p * RB + j], th[j * nb + pj[p]], v);
+                if (pj[p] == i) v = fma(S[p * RB + j], th[j * nb + pi[p]], v);
             }
         } else if (i >= nb) {
             for (int w = 0; w < kChiSeg; ++w) v += tp[(w * RB + j) * nt + i - nb];
@@ -486,14 +498,21 @@ template <typename T, typename OUT>
 __global__ void __launch_bounds__(256)
 k_table_adj(const T* __restrict__ part, int part_rows, const int* __restrict__ ptr, const int* __restrict__ idx, int n_z,
             int n_k, const OUT out, const int* __restrict__ nrows) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int* sp_ = reinterpret_cast<int*>(smem_raw);   // n_z + 3 offsets, then the partial rows in order
+    int* si = sp_ + n_z + 3;
+    const int PK = n_k + 2;
+    for (int i = threadIdx.x; i < n_z + 3; i += blockDim.x) sp_[i] = ptr[i];
+    for (int i = threadIdx.x; i < part_rows; i += blockDim.x) si[i] = idx[i] * PK;
     pdl_begin();
     const int row = blockIdx.x;
     if (row >= *nrows) return;
-    const int PK = n_k + 2;
+    __syncthreads();
     const T* p = part + (size_t)row * part_rows * PK;
     auto at = [&](int r, int c) {
         T s = T(0);
-        for (int x = ptr[r]; x < ptr[r + 1]; ++x) s += p[(size_t)idx[x] * PK + c];
+#pragma unroll 4
+        for (int x = sp_[r]; x < sp_[r + 1]; ++x) s += p[si[x] + c];
         return s;
     };
     auto cols = [&](int r, int c) {
@@ -863,6 +882,7 @@ int projection_adj_create(const ShearParams& sp, int elt, int cap, ProjectionAdj
     };
     const size_t n = (size_t)elt * cap, Np = (sp.N + 3) & ~3;
     NS_TRY(alloc(n * (sp.nb + 1) * Np, &a->win));
+    if (elt == 8) NS_TRY(alloc(n * window_node_values(sp.nb) * sp.N, &a->win_nodes));
     NS_TRY(alloc(n * sp.D, &a->resid));
     NS_TRY(alloc(n * sp.D, &a->C));
     NS_TRY(alloc(n * sp.D, &a->gC));
@@ -919,7 +939,7 @@ int launch_projection_adj_windows(const ShearParams& sp, ProjectionAdj* a, const
                                   int grid_rows, cudaStream_t st) {
     NS_CUDA_TRY(cudaEventRecord(a->ev_fork, st));
     NS_CUDA_TRY(cudaStreamWaitEvent(a->side, a->ev_fork, 0));
-    NS_TRY((launch_windows<T, false>(sp, theta_full, (T*)a->win, nrows, grid_rows, a->side)));
+    NS_TRY((launch_windows<T, false>(sp, theta_full, (T*)a->win, nrows, grid_rows, a->side, (T*)a->win_nodes)));
     NS_CUDA_TRY(cudaEventRecord(a->ev_join, a->side));
     return NS_OK;
 }
@@ -928,7 +948,7 @@ template <typename T, int RB>
 static int launch_chi2_adj(const ShearParams& sp, ProjectionAdj* a, const double* theta_full, const T* LinvT,
                            const T* Linv, double c0, double* gfull, double* logL, const int* nrows, int grid_rows,
                            cudaStream_t st) {
-    const size_t smem = sizeof(T) * adj::chi2_adj_elems(sp.D, sp.nb, sp.n_pairs, sp.n_tmpl, RB);
+    const size_t smem = sizeof(T) * adj::chi2_adj_elems(sp.D, adj::kChiV<T>, sp.nb, sp.n_pairs, sp.n_tmpl, RB);
     static bool attr = false;
     if (!attr) {
         NS_CUDA_TRY(cudaFuncSetAttribute(adj::k_chi2_adj<T, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmemMax));
@@ -964,7 +984,8 @@ static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double*
     const dim3 g(grid_rows, grid_rows < 256 ? sp.n_z : 3);
     const dim3 b(std::min(256, (sp.n_k + 31) & ~31));
     auto table_adj = [&](auto o) -> int {
-        NS_CUDA_TRY(launch_pdl(adj::k_table_adj<T, decltype(o)>, g, b, 0, st, (const T*)a->part, a->part_rows[k],
+        NS_CUDA_TRY(launch_pdl(adj::k_table_adj<T, decltype(o)>, g, b, sizeof(int) * (sp.n_z + 3 + a->part_rows[k]), st,
+                               (const T*)a->part, a->part_rows[k],
                                (const int*)a->ptr[k], (const int*)a->idx[k], sp.n_z, sp.n_k, o, nrows));
         return NS_OK;
     };
@@ -988,7 +1009,7 @@ int launch_projection_adj(const ShearParams& sp, ProjectionAdj* a, const double*
     NS_TRY((launch_limber<T, false>(sp, theta_full, table, (const T*)a->win, (T*)a->resid, nullptr, nrows, grid_rows,
                                     err, st, (T*)a->C)));
     // one row per block spreads few rows over the chip, eight share the reads of L^-1
-    if (grid_rows < 1024 || sizeof(T) * adj::chi2_adj_elems(sp.D, sp.nb, sp.n_pairs, sp.n_tmpl, 8) > kAdjSmemMax)
+    if (grid_rows < 1024 || sizeof(T) * adj::chi2_adj_elems(sp.D, adj::kChiV<T>, sp.nb, sp.n_pairs, sp.n_tmpl, 8) > kAdjSmemMax)
         NS_TRY((launch_chi2_adj<T, 1>(sp, a, theta_full, LinvT, Linv, c0, gfull, logL, nrows, grid_rows, st)));
     else
         NS_TRY((launch_chi2_adj<T, 8>(sp, a, theta_full, LinvT, Linv, c0, gfull, logL, nrows, grid_rows, st)));
