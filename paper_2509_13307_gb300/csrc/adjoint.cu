@@ -100,8 +100,7 @@ template <typename T, int KMAX>
 __global__ void __launch_bounds__(256)
 k_finish_grad(const T* __restrict__ gpre, const T* __restrict__ W0, int N1, int K0, const int* __restrict__ inputs,
               const double* __restrict__ scale, const double* __restrict__ gfull, int P,
-              const int* __restrict__ free_of_full, double* __restrict__ grad, int d,
-              const int* __restrict__ nrows) {
+              const int* __restrict__ free_of_full, const OutPtr grad, int d, const int* __restrict__ nrows) {
     pdl_begin();
     const int row = blockIdx.x;
     if (row >= *nrows) return;
@@ -135,7 +134,7 @@ k_finish_grad(const T* __restrict__ gpre, const T* __restrict__ W0, int N1, int 
         double v = gfull[(size_t)row * P + i];
         for (int j = 0; j < K0; ++j)
             if (inputs[j] == i) v += gx[j];
-        grad[(size_t)row * d + f] = v;
+        grad.get()[(size_t)row * d + f] = v;
     }
 }
 
@@ -228,10 +227,27 @@ struct GradState {
     float* G1 = nullptr;                     // gradient of layer 1's input pre-activations (rows x dims[1])
     std::vector<CUtensorMap> tmW, tmWT;      // W_l and its transpose
     std::vector<PlaneMapX> tmH, tmG;         // layer l's forward and backward operands
+    CallGraphs graphs;
     std::vector<void*> owned;
 };
 
 static std::mutex g_grad_mu;
+
+int CallGraphs::create(std::vector<void*>& owned) {
+    void* v;
+    if (cudaMalloc(&v, 2 * sizeof(double*)) != cudaSuccess) return NS_ENOMEM;
+    owned.push_back(v);
+    d_out = (double**)v;
+    return NS_OK;
+}
+
+void CallGraphs::release() {
+    for (Entry& e : entries)
+        if (e.exec) cudaGraphExecDestroy(e.exec);
+    entries.clear();
+    if (cap) cudaStreamDestroy(cap);
+    cap = nullptr;
+}
 
 static int grad_alloc(GradState* g, size_t bytes, void** out) {
     if (cudaMalloc(out, bytes) != cudaSuccess) return NS_ENOMEM;
@@ -245,6 +261,7 @@ static int grad_state_create(const ns_problem* p, GradState* g) {
     const size_t T = f64 ? 8 : 4;
     void* v;
     g->p = p;
+    NS_TRY(g->graphs.create(g->owned));
     NS_TRY(grad_alloc(g, sizeof(int), (void**)&g->d_nrows));
     NS_TRY(grad_alloc(g, sizeof(int), (void**)&g->d_err));
     NS_CUDA_TRY(cudaMemset(g->d_err, 0, sizeof(int)));
@@ -308,13 +325,14 @@ static int grad_state_create(const ns_problem* p, GradState* g) {
 }
 
 static void grad_state_free(GradState* g) {
+    g->graphs.release();
     projection_adj_free(&g->proj);
     for (void* q : g->owned) cudaFree(q);
     delete g;
 }
 
 template <typename T>
-static int launch_finish_grad(const ns_problem* p, GradState* g, const T* gpre, int B, double* grad, cudaStream_t st) {
+static int launch_finish_grad(const ns_problem* p, GradState* g, const T* gpre, int B, OutPtr grad, cudaStream_t st) {
     auto kern = p->dims[0] <= 8 ? adj::k_finish_grad<T, 8> : adj::k_finish_grad<T, 32>;
     NS_CUDA_TRY(launch_pdl(kern, dim3(B), dim3(256), 0, st, gpre, (const T*)p->d_W[0], p->dims[1], p->dims[0],
                            (const int*)p->d_inputs, (const double*)p->d_in_scale, (const double*)g->gfull, p->P,
@@ -323,7 +341,7 @@ static int launch_finish_grad(const ns_problem* p, GradState* g, const T* gpre, 
 }
 
 // FP64 problems: the emulator forward and backward on CUDA cores.
-static int run_grad_f64(const ns_problem* p, GradState* g, int B, double* logL, double* grad, cudaStream_t st) {
+static int run_grad_f64(const ns_problem* p, GradState* g, int B, OutPtr logL, OutPtr grad, cudaStream_t st) {
     const int L = p->n_layers, n_out = p->dims.back();
     const ShearParams& sp = p->sp;
     NS_TRY(launch_projection_adj_windows<double>(sp, &g->proj, g->theta_full, g->d_nrows, B, st));
@@ -369,7 +387,7 @@ static int run_grad_f64(const ns_problem* p, GradState* g, int B, double* logL, 
 
 // FP32 and BF16 problems: the emulator forward and backward as plane GEMMs
 // (gemm_planes.cu), the projection adjoint in FP32.
-static int run_grad_planes(const ns_problem* p, GradState* g, int B, double* logL, double* grad, cudaStream_t st) {
+static int run_grad_planes(const ns_problem* p, GradState* g, int B, OutPtr logL, OutPtr grad, cudaStream_t st) {
     const int L = p->n_layers, n_out = p->dims.back(), px = g->px, pw = g->pw;
     const ShearParams& sp = p->sp;
     auto planes_out = [&](PlaneEpi& e, __nv_bfloat16* buf, int width) {
@@ -488,9 +506,13 @@ extern "C" int loglike_grad_batch(const ns_problem* p, const double* theta_dev, 
             g_grad_states.push_back(gs);
         }
     }
-    NS_TRY(launch_free_to_full(p, theta_dev, B, gs->theta_full, gs->d_nrows, st));
-    if (p->precision == NS_PREC_FP64) return run_grad_f64(p, gs, B, logL_dev, grad_dev, st);
-    return run_grad_planes(p, gs, B, logL_dev, grad_dev, st);
+    double** out = gs->graphs.d_out;
+    NS_TRY(launch_free_to_full(p, theta_dev, B, gs->theta_full, gs->d_nrows, out, logL_dev, grad_dev, st));
+    const int rows = call_rows(B, p->max_batch);
+    return gs->graphs.run(rows, st, [&](cudaStream_t s) {
+        return p->precision == NS_PREC_FP64 ? run_grad_f64(p, gs, rows, OutPtr{out}, OutPtr{out + 1}, s)
+                                            : run_grad_planes(p, gs, rows, OutPtr{out}, OutPtr{out + 1}, s);
+    });
 }
 
 // Called by ns_problem_free: release the gradient state of a problem.

@@ -63,10 +63,17 @@ __global__ void k_cube_to_free(const double* __restrict__ cube, int d, int P,
 
 __global__ void k_free_to_full(const double* __restrict__ theta, int d, int P,
                                const double* __restrict__ pa, const int* __restrict__ free_of_full,
-                               double* __restrict__ theta_full, int B, int* __restrict__ nrows) {
+                               double* __restrict__ theta_full, int B, int* __restrict__ nrows,
+                               double** __restrict__ slots, double* out0, double* out1) {
     const int row = blockIdx.x;
     if (row >= B) return;
-    if (row == 0 && threadIdx.x == 0) *nrows = B;
+    if (row == 0 && threadIdx.x == 0) {
+        *nrows = B;
+        if (slots) {
+            slots[0] = out0;
+            slots[1] = out1;
+        }
+    }
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
         const int f = free_of_full[i];
         theta_full[(size_t)row * P + i] = (f < 0) ? pa[i] : theta[(size_t)row * d + f];
@@ -758,8 +765,9 @@ int launch_cube_to_free(const ns_problem* p, const double* cube, int B, double* 
     return NS_OK;
 }
 int launch_free_to_full(const ns_problem* p, const double* theta, int B, double* theta_full, int* nrows,
-                        cudaStream_t st) {
-    k_free_to_full<<<B, 64, 0, st>>>(theta, p->d, p->P, p->d_pa, p->d_free_of_full, theta_full, B, nrows);
+                        double** slots, double* out0, double* out1, cudaStream_t st) {
+    k_free_to_full<<<B, 64, 0, st>>>(theta, p->d, p->P, p->d_pa, p->d_free_of_full, theta_full, B, nrows, slots, out0,
+                                     out1);
     NS_CUDA_TRY(cudaGetLastError());
     return NS_OK;
 }

@@ -209,9 +209,10 @@ template <typename TR, typename TA>
 int launch_chi2(const TR* resid, int D, const TA* LinvT, double c0, double* logL, const int* nrows, int grid_rows,
                 cudaStream_t st, bool rows_ready = false);
 
-// free -> full parameter vectors, and the device row count
+// A batch call's set-up: free -> full parameter vectors, the device row count and
+// (slots given) where its results go.
 int launch_free_to_full(const ns_problem* p, const double* theta, int B, double* theta_full, int* nrows,
-                        cudaStream_t st);
+                        double** slots, double* out0, double* out1, cudaStream_t st);
 int launch_zinterp_generic(const ns_problem* p, const void* coarse, void* fine, const int* nrows, int grid_rows,
                            int elt, cudaStream_t st);
 

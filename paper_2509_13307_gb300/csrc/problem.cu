@@ -968,7 +968,7 @@ extern "C" int ns_prior_transform(const ns_problem* p, const double* cube_dev, i
 
 static int batch_common(const ns_problem* p, const double* theta_dev, int B, cudaStream_t st) {
     ns_problem* mp = const_cast<ns_problem*>(p);
-    return launch_free_to_full(p, theta_dev, B, mp->ws.theta_full, mp->ws.d_nrows, st);
+    return launch_free_to_full(p, theta_dev, B, mp->ws.theta_full, mp->ws.d_nrows, nullptr, nullptr, nullptr, st);
 }
 
 extern "C" int loglike_batch(const ns_problem* p, const double* theta_dev, int B, double* logL_dev, void* stream) {

@@ -86,7 +86,7 @@ template <typename T, int RB>
 __global__ void __launch_bounds__(kChiThreads)
 k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T* __restrict__ resid,
            const T* __restrict__ C, const T* __restrict__ LinvT, const T* __restrict__ Linv, double c0,
-           T* __restrict__ gC, double* __restrict__ gfull, double* __restrict__ logL, const int* __restrict__ nrows) {
+           T* __restrict__ gC, double* __restrict__ gfull, const OutPtr logL, const int* __restrict__ nrows) {
     pdl_begin();
     const int M = *nrows, r0 = blockIdx.x * RB;
     if (r0 >= M) return;
@@ -164,7 +164,7 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
     if (tid < RB && r0 + tid < M) {
         T s = T(0);
         for (int w = 0; w < kChiThreads / 32; ++w) s += wsum[w * RB + tid];
-        logL[r0 + tid] = c0 - 0.5 * (double)s;
+        logL.get()[r0 + tid] = c0 - 0.5 * (double)s;
     }
     // g_m = L^-T y: (g_m)_a = sum_{b >= a} (L^-1)[b][a] y_b
     columns(Linv, y, false);
@@ -946,7 +946,7 @@ int launch_projection_adj_windows(const ShearParams& sp, ProjectionAdj* a, const
 
 template <typename T, int RB>
 static int launch_chi2_adj(const ShearParams& sp, ProjectionAdj* a, const double* theta_full, const T* LinvT,
-                           const T* Linv, double c0, double* gfull, double* logL, const int* nrows, int grid_rows,
+                           const T* Linv, double c0, double* gfull, OutPtr logL, const int* nrows, int grid_rows,
                            cudaStream_t st) {
     const size_t smem = sizeof(T) * adj::chi2_adj_elems(sp.D, adj::kChiV<T>, sp.nb, sp.n_pairs, sp.n_tmpl, RB);
     static bool attr = false;
@@ -1003,7 +1003,7 @@ static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double*
 
 template <typename T>
 int launch_projection_adj(const ShearParams& sp, ProjectionAdj* a, const double* theta_full, const T* table,
-                          const T* LinvT, const T* Linv, double c0, const TableGrad& out, double* gfull, double* logL,
+                          const T* LinvT, const T* Linv, double c0, const TableGrad& out, double* gfull, OutPtr logL,
                           const int* nrows, int grid_rows, int* err, cudaStream_t st) {
     NS_CUDA_TRY(cudaStreamWaitEvent(st, a->ev_join, 0));
     NS_TRY((launch_limber<T, false>(sp, theta_full, table, (const T*)a->win, (T*)a->resid, nullptr, nrows, grid_rows,
@@ -1027,7 +1027,7 @@ int launch_projection_adj(const ShearParams& sp, ProjectionAdj* a, const double*
     template int launch_projection_adj_windows<T>(const ShearParams&, ProjectionAdj*, const double*, const int*, int, \
                                                   cudaStream_t);                                                      \
     template int launch_projection_adj<T>(const ShearParams&, ProjectionAdj*, const double*, const T*, const T*,      \
-                                          const T*, double, const TableGrad&, double*, double*, const int*, int,      \
+                                          const T*, double, const TableGrad&, double*, OutPtr, const int*, int,      \
                                           int*, cudaStream_t);
 NS_INST(double)
 NS_INST(float)

@@ -1,10 +1,77 @@
 // Interfaces of the projection adjoint (projection_adj.cu).
 #pragma once
+#include <mutex>
 #include <vector>
 
 #include "likelihood.cuh"
 
 namespace gpuns {
+
+// Where a gradient call's results go: a device slot that its set-up kernel writes,
+// so that the launches behind it hold no pointer of the caller's.
+struct OutPtr {
+    double* const* slot;
+    __device__ __forceinline__ double* get() const { return *slot; }
+};
+
+// Those launches (some twenty, with a fork and a join) as CUDA graphs, one per row
+// bucket, made at a bucket's third call: a lockstep NUTS step or a training step
+// of 64 rows is bound by the host (359 -> 304 us per call through autograd).  At most
+// kMost graphs per problem; other buckets, and calls on a stream that is being
+// captured, are launched one by one.  (Log-likelihood calls have half the launches
+// and their host keeps ahead of the GPU: replaying them cost 2 - 8 us per call.)
+struct CallGraphs {
+    static constexpr int kMost = 8;
+    struct Entry { int rows, seen; cudaGraphExec_t exec; };
+    std::mutex mu;                // a graph is launched by one thread at a time
+    std::vector<Entry> entries;
+    cudaStream_t cap = nullptr;
+    double** d_out = nullptr;     // device slots: log L, gradient
+    int create(std::vector<void*>& owned);
+    void release();
+    template <typename F>
+    int run(int rows, cudaStream_t st, F&& body);
+};
+// Rows a call's grids are sized for: powers of two up to 16, then multiples of 16.
+inline int call_rows(int B, int max_batch) {
+    int r = 1;
+    if (B > 16) r = (B + 15) & ~15;
+    else while (r < B) r *= 2;
+    return r < max_batch ? r : max_batch;
+}
+
+template <typename F>
+int CallGraphs::run(int rows, cudaStream_t st, F&& body) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return body(st);
+    std::lock_guard<std::mutex> lk(mu);
+    Entry* e = nullptr;
+    for (Entry& x : entries)
+        if (x.rows == rows) e = &x;
+    if (!e) {
+        if ((int)entries.size() >= kMost) return body(st);
+        entries.push_back(Entry{rows, 0, nullptr});
+        e = &entries.back();
+    }
+    if (!e->exec && ++e->seen == 3) {
+        cudaGraph_t g = nullptr;
+        if (!cap) NS_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
+        NS_CUDA_TRY(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
+        const int s = body(cap);
+        const cudaError_t c = cudaStreamEndCapture(cap, &g);
+        if (s != NS_OK) {
+            if (c == cudaSuccess) cudaGraphDestroy(g);
+            return s;
+        }
+        NS_CUDA_TRY(c);
+        const cudaError_t i = cudaGraphInstantiate(&e->exec, g, 0);
+        cudaGraphDestroy(g);
+        NS_CUDA_TRY(i);
+    }
+    if (!e->exec) return body(st);
+    NS_CUDA_TRY(cudaGraphLaunch(e->exec, st));
+    return NS_OK;
+}
 
 constexpr int kAdjWarps = 4;                            // warps per CTA of the Limber adjoint
 constexpr size_t kAdjSmemMax = 227 * 1024 - 8 * 1024;   // dynamic shared memory beside the kernels' static arrays
@@ -46,7 +113,7 @@ int launch_projection_adj_windows(const ShearParams& sp, ProjectionAdj* a, const
                                   int grid_rows, cudaStream_t st);
 template <typename T>
 int launch_projection_adj(const ShearParams& sp, ProjectionAdj* a, const double* theta_full, const T* table,
-                          const T* LinvT, const T* Linv, double c0, const TableGrad& out, double* gfull, double* logL,
+                          const T* LinvT, const T* Linv, double c0, const TableGrad& out, double* gfull, OutPtr logL,
                           const int* nrows, int grid_rows, int* err, cudaStream_t st);
 
 }  // namespace gpuns
