@@ -446,7 +446,6 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, OutPtr logL
         PlaneEpi e;
         e.mode = l == 1 ? PLN_DTANH32 : PLN_DTANH;
         e.aux = g->Hp[l];
-        e.aux_planes = px;
         e.aux_pitch = plane_pitch(p->dims[l]);
         e.aux_stride = g->rows_pad * e.aux_pitch;
         if (l == 1) e.out = g->G1;

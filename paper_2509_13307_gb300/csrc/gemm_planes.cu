@@ -211,7 +211,18 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
             beta = __ldg(e.beta + f);
         }
     }
-    auto finish = [&](int rl, float v) {
+    // h of row rl for the backward epilogues (loaded ahead of their use)
+    const bool dtanh = e.mode == PLN_DTANH || e.mode == PLN_DTANH32;
+    auto h_of = [&](int rl) {
+        float h = 0.f;
+        if (dtanh && fv && r0 + rl < M) {
+#pragma unroll
+            for (int p = PX - 1; p >= 0; --p)
+                h += __bfloat162float(e.aux[p * e.aux_stride + (size_t)(r0 + rl) * e.aux_pitch + f]);
+        }
+        return h;
+    };
+    auto finish = [&](int rl, float v, float h) {
         const int row = r0 + rl;
         if (!fv || row >= M) return;
         if (e.mode == PLN_OUT) {
@@ -223,9 +234,6 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
             v += bias;
             v = (g + (1.f - g) / (1.f + expf(-beta * v))) * v;
         } else {
-            float h = 0.f;
-            for (int p = e.aux_planes - 1; p >= 0; --p)
-                h += __bfloat162float(e.aux[p * e.aux_stride + (size_t)row * e.aux_pitch + f]);
             v *= 1.f - h * h;
             if (e.mode == PLN_DTANH32) {
                 e.out[(size_t)row * N + f] = v;
@@ -250,9 +258,17 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     if (S == 1) {
         __syncthreads();
         if (warp < kPlaneEpiWarps) {
+            // four rows at a time: the backward epilogues' loads of h overlap
             const int hi = min(BR, M - r0);
-#pragma unroll 2
-            for (int rl = tid >> 7; rl < hi; rl += 2) finish(rl, red[rl * 128 + (tid & 127)]);
+#pragma unroll 1
+            for (int rl = tid >> 7; rl < hi; rl += 8) {
+                float h[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) h[q] = h_of(rl + 2 * q);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (rl + 2 * q < hi) finish(rl + 2 * q, red[(rl + 2 * q) * 128 + (tid & 127)], h[q]);
+            }
         }
     } else {
         cluster_sync_all();
@@ -262,8 +278,9 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
 #pragma unroll 1
             for (int rl = BR * rank / S + (tid >> 7); rl < hi; rl += 2) {
                 float v = 0.f;
+#pragma unroll 4
                 for (int q = 0; q < S; ++q) v += ld_cluster_f32(mapa_u32(off + 512u * (uint32_t)rl, (uint32_t)q));
-                finish(rl, v);
+                finish(rl, v, h_of(rl));
             }
         }
         cluster_sync_all();                          // peers have read this CTA's partial tile

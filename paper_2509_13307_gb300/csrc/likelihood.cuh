@@ -3,6 +3,7 @@
 
 #include <cuda.h>
 #include <cuda_fp16.h>
+#include <utility>
 #include <vector>
 
 #include "common.cuh"
@@ -111,6 +112,7 @@ struct ns_problem {
     std::vector<CUtensorMap> tmWp;   // FP32 layers >= 1 (and a BF16 CMB head): the weights as three bf16 planes
     std::vector<CUtensorMap> tmB;    // BF16: weight tensor maps for layers >= 1
     std::vector<int> tile_n;         // BF16: N tile per layer (hidden layers autotuned at creation)
+    std::vector<CUtensorMap> tmB64;  // BF16, autotuned hidden layers: weight maps of 64-wide tiles (many rows)
     std::vector<float> tile_ms;      // BF16: measured time per launch of the chosen hidden tiles
     int fused_cs = 0;                // BF16: > 0 when the input and hidden layers run as one clustered kernel
                                      // (cluster of fused_cs CTAs, hidden width 128 fused_cs)
@@ -154,6 +156,31 @@ struct ns_problem {
 
 namespace gpuns {
 
+// Several device buffers in one allocation: a run or workspace has some forty,
+// and cudaMalloc / cudaFree cost its creation and end a call each.
+struct Carve {
+    std::vector<std::pair<void**, size_t>> parts;
+    template <typename T>
+    void want(T** p, size_t bytes) {
+        *p = nullptr;
+        if (bytes) parts.emplace_back((void**)p, bytes);
+    }
+    int alloc(std::vector<void*>& owned) {
+        size_t total = 0;
+        for (auto& q : parts) total += (q.second + 1023) & ~(size_t)1023;
+        void* base = nullptr;
+        if (cudaMalloc(&base, total) != cudaSuccess) return NS_ENOMEM;
+        owned.push_back(base);
+        char* at = (char*)base;
+        for (auto& q : parts) {
+            *q.first = at;
+            at += (q.second + 1023) & ~(size_t)1023;
+        }
+        parts.clear();
+        return NS_OK;
+    }
+};
+
 int workspace_create(const ns_problem* p, int cap, Workspace* ws);
 // Queue a copy of the device status bits into the pinned mirror on `st`; after
 // the stream has synchronised, workspace_err_bits returns them.
@@ -195,7 +222,7 @@ template <typename T, bool FAST>
 int launch_windows(const ShearParams& sp, const double* theta_full, T* win, const int* nrows, int grid_rows,
                    cudaStream_t st, T* nodes = nullptr);
 // values per chi node that a separate launch prepares for the windows (FP64: nodes, rows x values x N)
-constexpr int window_node_values(int nb) { return 4 + nb; }
+constexpr int window_node_values(int nb) { return 5 + nb; }
 template <typename T, bool FAST>
 int launch_limber(const ShearParams& sp, const double* theta_full, const T* table, const T* win, T* resid,
                   double* model_out, const int* nrows, int grid_rows, int* err, cudaStream_t st, T* cl_out = nullptr);
@@ -260,8 +287,7 @@ struct PlaneEpi {
     __nv_bfloat16* planes = nullptr;  // TANH, SIGLIN, DTANH: px planes of row pitch `pitch`
     long long plane_stride = 0;
     int pitch = 0;
-    const __nv_bfloat16* aux = nullptr;  // DTANH: acc (1 - h^2), h in aux_planes planes
-    int aux_planes = 0;
+    const __nv_bfloat16* aux = nullptr;  // DTANH: acc (1 - h^2), h in px planes
     long long aux_stride = 0;
     int aux_pitch = 0;
 };

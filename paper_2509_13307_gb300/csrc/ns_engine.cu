@@ -987,7 +987,8 @@ extern "C" int ns_init(const ns_problem* p, const ns_config* cfg, void* stream, 
     rd.n = n; rd.k = k; rd.d = d; rd.R = r->R; rd.cap_steps = cfg->step_cap;
     rd.width = cfg->width; rd.tol = cfg->tol; rd.seed = cfg->seed;
     void* v;
-#define RA(field, bytes) do { if ((s = run_alloc(r, (bytes), &v))) return fail(s); rd.field = (decltype(rd.field))v; } while (0)
+    Carve carve;
+#define RA(field, bytes) carve.want(&rd.field, (bytes))
     RA(live_x, sizeof(double) * n * d);
     RA(live_L, sizeof(double) * n);
     RA(order, sizeof(int) * r->n_pad);
@@ -1014,6 +1015,7 @@ extern "C" int ns_init(const ns_problem* p, const ns_config* cfg, void* stream, 
     RA(prop, sizeof(double) * cap * d);
     RA(sc, sizeof(Scalars));
 #undef RA
+    if ((s = carve.alloc(r->owned))) return fail(s);
     rd.logL = r->ws.logL;
     k_reset_chains<<<(k + 127) / 128, 128, 0, r->st>>>(rd);
     rd.batch_ctr = &rd.sc->batch;

@@ -89,30 +89,37 @@ static bool cholesky_inverse(const double* C, int D, std::vector<double>& L, std
 
 int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
     ws->cap = cap;
-    void* v;
-    NS_TRY(dalloc(sizeof(int), &v, ws->owned));
-    ws->d_nrows = (int*)v;
-    NS_TRY(dalloc(sizeof(int), &v, ws->owned));
-    ws->d_err = (int*)v;
-    NS_CUDA_TRY(cudaMemset(ws->d_err, 0, sizeof(int)));
     if (cudaMallocHost(&ws->h_err, sizeof(int)) != cudaSuccess) return NS_ENOMEM;
     *ws->h_err = 0;
-    NS_TRY(dalloc(sizeof(double) * (size_t)cap * p->P, &v, ws->owned));
-    ws->theta_full = (double*)v;
-    NS_TRY(dalloc(sizeof(double) * (size_t)cap, &v, ws->owned));
-    ws->logL = (double*)v;
-    if (p->kind == NS_KIND_GAUSS) return NS_OK;
-    // activations: FP64, bf16, or FP32 as three bf16 planes
-    // FP64 tanh: six fp16 slices
-    const bool slices = !p->tmWs.empty();
-    const int elt = slices ? 12 : (p->precision == NS_PREC_FP64) ? 8 : (p->precision == NS_PREC_FP32 ? 6 : 2);
+    Carve c;
+    c.want(&ws->d_nrows, sizeof(int));
+    c.want(&ws->d_err, sizeof(int));
+    c.want(&ws->theta_full, sizeof(double) * (size_t)cap * p->P);
+    c.want(&ws->logL, sizeof(double) * (size_t)cap);
+    const bool gauss = p->kind == NS_KIND_GAUSS, cmb = p->kind == NS_KIND_CMB;
+    const bool f64 = p->precision == NS_PREC_FP64, slices = !p->tmWs.empty();
+    // activations: FP64 (tanh: six fp16 slices), bf16, or FP32 as three bf16 planes
+    const int elt = slices ? 12 : f64 ? 8 : (p->precision == NS_PREC_FP32 ? 6 : 2), tab_elt = f64 ? 8 : 4;
     const int rows_pad = ((cap + 127) / 128) * 128;
     const size_t act_bytes = (size_t)elt * rows_pad * plane_pitch(p->hidden_max);
-    for (int i = 0; i < 2; ++i) {
-        NS_TRY(dalloc(act_bytes, &v, ws->owned));
-        ws->act[i] = v;
-        NS_CUDA_TRY(cudaMemset(v, 0, act_bytes));
+    if (!gauss)
+        for (int i = 0; i < 2; ++i) c.want(&ws->act[i], act_bytes);
+    if (cmb) {
+        c.want(&ws->table, (size_t)tab_elt * cap * std::max(p->D, p->dims.back()));
+        if (p->cmb_solve == NS_SOLVE_LITERAL && p->cmb_form == NS_CMB_GAUSS)
+            c.want(&ws->resid, sizeof(double) * (size_t)cap * p->D);
+    } else if (!gauss) {
+        const ShearParams& sp = p->sp;
+        c.want(&ws->table, (size_t)tab_elt * cap * p->dims.back());
+        if (p->n_z_emu != sp.n_z) c.want(&ws->table_fine, (size_t)tab_elt * cap * sp.n_z * sp.n_k);
+        c.want(&ws->resid, (size_t)tab_elt * cap * sp.D);
+        c.want(&ws->win, (size_t)tab_elt * cap * (sp.nb + 1) * ((sp.N + 3) & ~3));
+        if (f64) c.want(&ws->win_nodes, sizeof(double) * (size_t)cap * window_node_values(sp.nb) * sp.N);
     }
+    NS_TRY(c.alloc(ws->owned));
+    NS_CUDA_TRY(cudaMemset(ws->d_err, 0, sizeof(int)));
+    if (gauss) return NS_OK;
+    for (int i = 0; i < 2; ++i) NS_CUDA_TRY(cudaMemset(ws->act[i], 0, act_bytes));
     if (slices) {
         ws->plane_stride = (long long)rows_pad * plane_pitch(p->hidden_max);
         ws->tmXs.resize(p->n_layers);
@@ -127,14 +134,7 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
         for (int l = 1; l < p->n_layers; ++l)
             NS_TRY(make_plane_maps_x(&ws->tmXp[l], ws->act[(l - 1) & 1], rows_pad, p->dims[l], ws->plane_stride, 3));
     }
-    if (p->kind == NS_KIND_CMB) {
-        const int tab_elt = (p->precision == NS_PREC_FP64) ? 8 : 4;
-        NS_TRY(dalloc((size_t)tab_elt * cap * std::max(p->D, p->dims.back()), &v, ws->owned));
-        ws->table = v;
-        if (p->cmb_solve == NS_SOLVE_LITERAL && p->cmb_form == NS_CMB_GAUSS) {
-            NS_TRY(dalloc(sizeof(double) * (size_t)cap * p->D, &v, ws->owned));
-            ws->resid = v;
-        }
+    if (cmb) {
         if (p->precision == NS_PREC_BF16) {
             ws->tmA.resize(p->n_layers);
             int cur = 0;
@@ -150,22 +150,6 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
                                      (long long)rows_pad * plane_pitch(Kh), 1));
         }
         return NS_OK;
-    }
-    const int tab_elt = (p->precision == NS_PREC_FP64) ? 8 : 4;
-    const int n_out = p->dims.back();
-    NS_TRY(dalloc((size_t)tab_elt * cap * n_out, &v, ws->owned));
-    ws->table = v;
-    if (p->n_z_emu != p->sp.n_z) {
-        NS_TRY(dalloc((size_t)tab_elt * cap * p->sp.n_z * p->sp.n_k, &v, ws->owned));
-        ws->table_fine = v;
-    }
-    NS_TRY(dalloc((size_t)tab_elt * cap * p->sp.D, &v, ws->owned));
-    ws->resid = v;
-    NS_TRY(dalloc((size_t)tab_elt * cap * (p->sp.nb + 1) * ((p->sp.N + 3) & ~3), &v, ws->owned));
-    ws->win = v;
-    if (p->precision == NS_PREC_FP64) {
-        NS_TRY(dalloc(sizeof(double) * (size_t)cap * window_node_values(p->sp.nb) * p->sp.N, &v, ws->owned));
-        ws->win_nodes = v;
     }
     NS_CUDA_TRY(cudaStreamCreateWithFlags(&ws->side, cudaStreamNonBlocking));
     NS_CUDA_TRY(cudaEventCreateWithFlags(&ws->ev_fork, cudaEventDisableTiming));
@@ -746,6 +730,11 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
             }
         } else {
             s = autotune_hidden_tiles(p, e.n_layers - 2);   // hidden layers 1 .. L-2
+            p->tmB64.resize(e.n_layers);
+            for (int l = 1; l <= e.n_layers - 2 && !s; ++l) {
+                const int K = p->dims[l], N = p->dims[l + 1];
+                s = make_tensor_map_bf16(&p->tmB64[l], p->d_W[l], N, K, 64, gemm_tc_kps(K));
+            }
         }
         if (s) return fail(s);
     }

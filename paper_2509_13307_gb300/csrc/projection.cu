@@ -137,8 +137,8 @@ __device__ __forceinline__ T warp_transpose_sum16(T (&v)[16]) {
 // win_pitch(N) (16-byte multiples, for the Limber stage's bulk copy), to `win`.
 __host__ __device__ inline int win_pitch(int N) { return (N + 3) & ~3; }
 
-// Node-local functions of the FP64 windows: E, the chi increment of the interval,
-// Omega_m(a)^gamma, the IA power ((1 + z) / pivot)^eta and the shifted Gaussians.  They hold three
+// Node-local functions of the FP64 windows: E and 1/E, the chi increment of the
+// interval, Omega_m(a)^gamma, the IA power ((1 + z) / pivot)^eta and the shifted Gaussians.  They hold three
 // quarters of the stage's FP64 work, which one CTA per evaluation would put on one
 // SM's two FMAs per cycle; here every SM takes nodes.
 template <typename T, int NB>
@@ -166,7 +166,7 @@ k_window_nodes(const ShearParams sp, const double* __restrict__ theta_full, T* _
     const T* nz_sg = pick<T>(sp.nz_sigma, sp.nz_sigma_f);
     T* o = nodes + (size_t)row * window_node_values(NB) * N + n;
     const T a = a_[n], lna = lna_[n], ia = ia_[n], a3 = ia * ia * ia;
-    const T e = sqrt_<T>(om * a3 + (T(1) - om) * M::ex(-pde * lna - T(3) * wa * (T(1) - a)));
+    const T e2 = om * a3 + (T(1) - om) * M::ex(-pde * lna - T(3) * wa * (T(1) - a)), ie = M::rsq(e2);
     T inc = T(0);
     if (n < N - 1) {
 #pragma unroll
@@ -177,14 +177,15 @@ k_window_nodes(const ShearParams sp, const double* __restrict__ theta_full, T* _
         }
         inc *= chiH * (T(0.5) * (a - a_[n + 1]));
     }
-    o[0] = e;
+    o[0] = e2 * ie;
     o[N] = inc;
-    o[2 * (size_t)N] = M::ex(gamma * M::lg(M::div(om * a3, e * e)));
+    o[2 * (size_t)N] = M::ex(gamma * M::lg(om * a3 * (ie * ie)));
     o[3 * (size_t)N] = M::ex((T)t[10] * (-lna - pick_s<T>(sp.ln_pivot, sp.ln_pivot_f)));
+    o[4 * (size_t)N] = ie;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         const T u = (z_[n] - (T)t[11 + i] - nz_mu[i]) * M::div(T(1), nz_sg[i]);
-        o[(4 + i) * (size_t)N] = M::ex(T(-0.5) * u * u);
+        o[(5 + i) * (size_t)N] = M::ex(T(-0.5) * u * u);
     }
 }
 
@@ -274,6 +275,8 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
         const T ian = FAST ? T(0) : ia_[n];
         if constexpr (PRE) {
             t1[n] = pre[2 * (size_t)N + n];
+            omw[n] = wa_[n] * chiH * (ian * ian) * pre[4 * (size_t)N + n];
+            continue;
         } else {
             const T oma = M::div(om * (FAST ? M::ex(T(-3) * lna_[n]) : ian * ian * ian), Ez[n] * Ez[n]);
             t1[n] = M::ex(gamma * M::lg(oma));
@@ -285,7 +288,7 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
         t0[n] = (n < N - 1) ? T(0.5) * (t1[n] + t1[n + 1]) * (lna_[n] - lna_[n + 1]) : T(0);
     __syncthreads();
     block_exclusive_scan(t0, N, red);
-    for (int n = tid; n < N; n += nt) Dg[n] = M::ex(-t0[n]);
+    for (int n = tid; n < N; n += nt) Dg[n] = M::ex(PRE ? t0[n] : -t0[n]);   // FP64: 1 / D, a factor below
 
     // 2. windows for all bins at once: n_i(chi) into V, then one multi-value
     //    exclusive suffix scan of (w n_i, w n_i / chi) over contiguous chunks.
@@ -305,7 +308,7 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             const T u = FAST ? (z_[n] - zc[i]) * isg[i] : (z_[n] - th[11 + i] - nz_mu[i]) * isg[i];
-            const T raw = PRE ? pre[(4 + i) * (size_t)N + n] : M::ex(T(-0.5) * u * u);
+            const T raw = PRE ? pre[(5 + i) * (size_t)N + n] : M::ex(T(-0.5) * u * u);
             V[i * N + n] = raw;
             pn[i] += wz * raw;
         }
@@ -333,6 +336,7 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
     for (int n = lo; n < hi; ++n) {
         const T e = Ez[n];
         const T ichi = (n >= 1) ? M::div(T(1), chi[n]) : T(0);
+        if (PRE) t1[n] = ichi;                  // this thread's nodes again below
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
             const T nchi = V[i * N + n] * e * inv_norm[i];
@@ -371,12 +375,13 @@ k_windows(const ShearParams sp, const double* __restrict__ theta_full, T* __rest
     const T c1om = c1rho * om;
     for (int n = hi - 1; n >= lo; --n) {
         const T c = chi[n];
-        const T ic = (n >= 1) ? M::div(T(1), c) : T(0);
+        const T ic = PRE ? t1[n] : (n >= 1) ? M::div(T(1), c) : T(0);
         const T sq = (n >= 1) ? sqrt_<T>(omw[n]) * ic : T(0);
         // ln((1 + z) / pivot) = -ln a - ln pivot
         const T lq = FAST ? M::lg((T(1) + z_[n]) * ipiv) : -lna_[n] - lnpiv;
         const T amp = FAST ? M::div(A_IA * M::ex(eta * lq) * c1om, Dg[n])
-                           : M::div(A_IA * (PRE ? pre[3 * (size_t)N + n] : M::ex(eta * lq)) * c1rho * om, Dg[n]);
+                     : PRE ? A_IA * pre[3 * (size_t)N + n] * c1rho * om * Dg[n]
+                           : M::div(A_IA * M::ex(eta * lq) * c1rho * om, Dg[n]);
         const T pc = pref * c * (FAST ? M::div(T(1), a_[n]) : ia_[n]);
 #pragma unroll
         for (int i = 0; i < NB; ++i) {
