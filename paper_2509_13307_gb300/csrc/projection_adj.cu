@@ -572,10 +572,13 @@ __device__ __forceinline__ void block_scan(T* x, int pitch, int n, T* red) {
 }
 
 enum { S_OM = 0, S_CHIH, S_W0, S_WA, S_GAMMA, S_PREF, S_AIA, S_ETA, S_COUNT };
+// Threads: 512 while an SM holds one evaluation, 256 from 153 evaluations on: two
+// CTAs then share the SM (27 arrays of 1025 FP32 nodes are 111 KB) and run through
+// one another's barriers (4096 evaluations: XXX).
 constexpr int kWinAdjThreads = 512;
 
 // elements of the per-evaluation arrays of k_windows_adj
-__host__ __device__ inline size_t windows_adj_elems(int N, int nb) { return (size_t)(10 + 4 * nb) * N; }
+__host__ __device__ inline size_t windows_adj_elems(int N, int nb) { return (size_t)(7 + 4 * nb) * N; }
 
 template <typename T, int NB>
 __global__ void __launch_bounds__(kWinAdjThreads)
@@ -586,11 +589,13 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
     const int row = blockIdx.x;
     if (row >= *nrows) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = sp.N, tid = threadIdx.x, nt = kWinAdjThreads, lane = tid & 31, wid = tid >> 5;
+    const int N = sp.N, tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
     T* S = scratch ? scratch + (size_t)row * windows_adj_elems(N, NB) : reinterpret_cast<T*>(smem_raw);
-    T *chi = S, *Ez = S + N, *Dg = S + 2 * N, *omw = S + 3 * N, *fg = S + 4 * N;
-    T *gchi = S + 5 * N, *gE = S + 6 * N, *gomw = S + 7 * N, *t1 = S + 8 * N, *t2 = S + 9 * N;
-    T *raw = S + 10 * N, *nchi = raw + NB * N, *E0 = nchi + NB * N, *E1 = E0 + NB * N;
+    T *chi = S, *Ez = S + N, *omw = S + 2 * N, *fg = S + 3 * N;
+    T *gomw = S + 4 * N, *gE = gomw;             // g_omw makes room for g_E node by node,
+    T *Dg = S + 5 * N, *t1 = Dg;                 // ln D and D for g_S,
+    T *gchi = S + 6 * N, *t2 = gchi;             // g_chi for its suffix sums (beside t1)
+    T *raw = S + 7 * N, *nchi = raw + NB * N, *E0 = nchi + NB * N, *E1 = E0 + NB * N;
     constexpr int NS = S_COUNT + 3 * NB, NR = NS > 2 * NB ? NS : 2 * NB;
     __shared__ T red[(kWinAdjThreads / 32) * NR];
     __shared__ T th[16];
@@ -687,7 +692,6 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
     // ---- windows: V = sqrt(omw)/chi * W, W = pc (E0 - chi E1) - amp nchi, amp = A_IA q c1rho Om / D
     for (int n = tid; n < N; n += nt) {
         const T D_n = ex<T>(-Dg[n]);
-        Dg[n] = D_n;
         if (n == 0) {                           // carries no window value
             for (int i = 0; i < NB; ++i) { raw[i * N] = T(0); E0[i * N] = T(0); E1[i * N] = T(0); }
             gchi[0] = T(0); gomw[0] = T(0); t1[0] = T(0);
@@ -996,7 +1000,8 @@ static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double*
         else if (out.px == 2) NS_TRY(table_adj(adj::OutPlaneT<2>{out.planes, out.stride, out.pitch, out.scale}));
         else NS_TRY(table_adj(adj::OutT32{(float*)out.table}));
     }
-    NS_CUDA_TRY(launch_pdl(adj::k_windows_adj<T, NB>, dim3(grid_rows), dim3(adj::kWinAdjThreads), a->win_smem, st, sp,
+    NS_CUDA_TRY(launch_pdl(adj::k_windows_adj<T, NB>, dim3(grid_rows), dim3(grid_rows > 152 ? 256 : adj::kWinAdjThreads),
+                           a->win_smem, st, sp,
                            theta_full, (const T*)a->gV, (const T*)a->glnc, (T*)a->scratch, gfull, nrows));
     return NS_OK;
 }
