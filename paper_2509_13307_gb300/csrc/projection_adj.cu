@@ -1,4 +1,4 @@
-// Adjoint of the shear projection (row A14): from the emulator table and theta
+// Adjoint of the shear projection: from the emulator table and theta
 // to log L, d log L / d table and d log L / d theta (emulator inputs' share
 // through the emulator excluded).  The forward stages are the likelihood's own
 // kernels (projection.cu), with the Limber sums kept; the reverse stages are
@@ -258,42 +258,167 @@ template <> struct P2<double> {
 // four z-taps of a table column
 template <typename T> struct alignas(16) Z4 { P2<T> a, b; };
 
-// Sum of 8 values per lane over the warp: lane l gets the sum of value l & 7.
-template <typename T>
-__device__ __forceinline__ T warp_transpose_sum8(T (&v)[8]) {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int off = 4; off >= 1; off >>= 1) {
-        const bool upper = (lane & off) != 0;
-#pragma unroll
-        for (int i = 0; i < off; ++i) {
-            const T send = upper ? v[i] : v[i + off];
-            const T keep = upper ? v[i + off] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+// Reverse of the Limber sums, node by node: one lane per chi node, its windows and
+// their gradients in registers, two multipoles at a time as the halves of packed
+// values; g_C, the same for every lane, and the padded table come from shared
+// memory.  Sums over multipoles stay in the lane.  The gradient of the
+// interpolated table value (doubled-weight sum), g_v, goes to global memory for
+// k_limber_adj, whose lanes are multipoles.  With both halves in one kernel and one
+// multipole per lane, 20 of 32 lanes worked and each node took a warp reduction of
+// six values and the loads of its windows: 460 k warp instructions per evaluation,
+// 2560 us for 4096 evaluations of the 39-d problem; the two kernels: XXX us.
+template <typename T, int NB> constexpr int kGQuads = (NB * (NB + 1) / 2 + 1) / 2;   // pairs of g_C entries
+constexpr int kNodeThreads = 256;
+
+template <typename T, int NB, bool STAGE>
+__global__ void __launch_bounds__(kNodeThreads, sizeof(T) == 4 ? 2 : 1)
+k_limber_nodes(const ShearParams sp, const T* __restrict__ table, const T* __restrict__ win, const T* __restrict__ gC,
+               T* __restrict__ gv_out, T* __restrict__ gV, T* __restrict__ glnc, const int* __restrict__ nrows) {
+    using Q = P2<T>;
+    constexpr int NP = NB * (NB + 1) / 2, NG = kGQuads<T, NB>;
+    pdl_begin();
+    const int row = blockIdx.x;
+    if (row >= *nrows) return;
+    const int N = sp.N, n_k = sp.n_k, n_z = sp.n_z, n_ell = sp.n_ell, D = sp.D, PK = n_k + 2, Np = (N + 3) & ~3;
+    const int n_lp = (n_ell + 1) / 2, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    Z4<T>* Gs = reinterpret_cast<Z4<T>*>(smem_raw);
+    T* U = reinterpret_cast<T*>(Gs + n_lp * NG);
+    const T* src = table + (size_t)row * n_z * n_k;
+    const T* lnchi = win + (size_t)row * (NB + 1) * Np;
+    const T* V = lnchi + Np;
+    const Z4<T>* zwp = reinterpret_cast<const Z4<T>*>(pick<T>(sp.zw4d, sp.zw4f));
+    const T* lnell = pick<T>(sp.lnell, sp.lnell_f);
+    const T lkmin = pick_s<T>(sp.lnk_min, sp.lnk_min_f), lkmax = pick_s<T>(sp.lnk_max, sp.lnk_max_f);
+    const T inv_dk = pick_s<T>(1.0 / sp.dlnk, sp.inv_dlnk_f);
+    if (STAGE)
+        for (int r = wid; r < n_z + 2; r += kNodeThreads / 32)
+            for (int c = lane; c < PK; c += 32) U[r * PK + c] = padded(src, n_z, n_k, r, c);
+    // symmetric g_C with a doubled diagonal: h_i = sum_j G_ij V_j is the derivative of
+    // g_P = 1/2 sum_ij G_ij V_i V_j by V_i
+    for (int x = tid; x < n_lp * 2 * NG; x += kNodeThreads) {
+        const int lp = x / (2 * NG), p = x % (2 * NG);
+        T g0 = T(0), g1 = T(0);
+        if (p < NP) {
+            const T f = sp.pi[p] == sp.pj[p] ? T(2) : T(1);
+            const T* g = gC + (size_t)row * D + p * n_ell + 2 * lp;
+            g0 = f * g[0];
+            if (2 * lp + 1 < n_ell) g1 = f * g[1];
         }
+        reinterpret_cast<Q*>(Gs)[x] = Q(g0, g1);
     }
-    T s = v[0] + __shfl_xor_sync(0xffffffffu, v[0], 8);
-    return s + __shfl_xor_sync(0xffffffffu, s, 16);
+    __syncthreads();
+    auto two = [](T x) { return Q(x, x); };
+    for (int n = 1 + blockIdx.y * kNodeThreads + tid; n < N; n += kNodeThreads * gridDim.y) {
+        const T lc = lnchi[n];
+        const Z4<T> wz = zwp[n];
+        const Q w[4] = {two(wz.a.v.x), two(wz.a.v.y), two(wz.b.v.x), two(wz.b.v.y)};
+        const int zr = sp.zrp[n];
+        const T* rz = U + zr * PK;
+        Q v[NB], sV[NB];
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            v[i] = two(V[i * Np + n]);
+            sV[i] = two(T(0));
+        }
+        T sl = T(0);
+        T* gvp = gv_out + (size_t)row * n_ell * Np + n;
+#pragma unroll 1
+        for (int lp = 0; lp < n_lp; ++lp) {
+            const bool both = 2 * lp + 1 < n_ell;
+            const T s0 = lnell[2 * lp] - lc, s1 = lnell[both ? 2 * lp + 1 : 2 * lp] - lc;
+            const T c0 = fmin(fmax(s0, lkmin), lkmax), c1 = fmin(fmax(s1, lkmin), lkmax);
+            const T u0 = (c0 - lkmin) * inv_dk, u1 = (c1 - lkmin) * inv_dk;
+            const int k0 = min(max((int)floor(u0), 0), n_k - 2), k1 = min(max((int)floor(u1), 0), n_k - 2);
+            // taps folded over z
+            Q col[4];
+            if (STAGE) {
+                const T *p0 = rz + k0, *p1 = rz + k1;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    col[q] = Q::mul(w[0], Q(p0[q], p1[q]));
+#pragma unroll
+                    for (int r = 1; r < 4; ++r) col[q] = Q::fma(w[r], Q(p0[r * PK + q], p1[r * PK + q]), col[q]);
+                }
+            } else {
+#pragma unroll 1
+                for (int q = 0; q < 4; ++q) {
+                    Q x = two(T(0));
+                    for (int r = 0; r < 4; ++r)
+                        x = Q::fma(two(r == 0 ? wz.a.v.x : r == 1 ? wz.a.v.y : r == 2 ? wz.b.v.x : wz.b.v.y),
+                                   Q(padded(src, n_z, n_k, zr + r, k0 + q), padded(src, n_z, n_k, zr + r, k1 + q)), x);
+#pragma unroll
+                    for (int y = 0; y < 4; ++y)
+                        if (y == q) col[y] = x;
+                }
+            }
+            // doubled Catmull-Rom weights in ln k and their derivatives (the z-weights are doubled too)
+            const Q t(u0 - (T)k0, u1 - (T)k1), t2 = Q::mul(t, t);
+            const Q m = Q::mul(t, Q::fma(two(T(-3)), t, two(T(4))));
+            const Q one = two(T(1)), neg = two(T(-1));
+            const Q w0 = Q::mul(t, Q::fma(t, Q::fma(t, neg, two(T(2))), neg));
+            const Q w1 = Q::fma(t2, Q::fma(two(T(3)), t, two(T(-5))), two(T(2)));
+            const Q w2 = Q::fma(t, m, t), w3 = Q::mul(t2, Q::add(t, neg));
+            const Q d0 = Q::add(m, neg), d1 = Q::mul(t, Q::fma(two(T(9)), t, two(T(-10))));
+            const Q d2 = Q::fma(t, Q::fma(two(T(-9)), t, two(T(8))), one);
+            const Q d3 = Q::mul(t, Q::fma(two(T(3)), t, two(T(-2))));
+            const Q f = Q::fma(w3, col[3], Q::fma(w2, col[2], Q::fma(w1, col[1], Q::mul(w0, col[0]))));
+            const Q df = Q::fma(d3, col[3], Q::fma(d2, col[2], Q::fma(d1, col[1], Q::mul(d0, col[0]))));
+            const Q P(p10(T(0.25) * f.v.x), p10(T(0.25) * f.v.y));
+            Q h[NB];
+#pragma unroll
+            for (int i = 0; i < NB; ++i) h[i] = two(T(0));
+            {
+                const Z4<T>* G = Gs + lp * NG;
+                int p = 0;
+                Z4<T> g;
+#pragma unroll
+                for (int i = 0; i < NB; ++i)
+#pragma unroll
+                    for (int j = i; j < NB; ++j) {
+                        if ((p & 1) == 0) g = G[p / 2];
+                        const Q e = (p & 1) ? g.b : g.a;
+                        h[i] = Q::fma(e, v[j], h[i]);
+                        if (j != i) h[j] = Q::fma(e, v[i], h[j]);
+                        ++p;
+                    }
+            }
+            Q gP = Q::mul(v[0], h[0]);
+#pragma unroll
+            for (int i = 1; i < NB; ++i) gP = Q::fma(v[i], h[i], gP);
+#pragma unroll
+            for (int i = 0; i < NB; ++i) sV[i] = Q::fma(h[i], P, sV[i]);
+            // d log L / d (doubled-weight sum); gP is twice g_P; s = ln(ell + 1/2) - ln chi
+            const Q gv = Q::mul(Q::mul(gP, P), two((T)(kLn10 * 0.125)));
+            const Q gs = Q::mul(gv, df);
+            if (s0 == c0) sl = fma(-inv_dk, gs.v.x, sl);
+            if (s1 == c1) sl = fma(-inv_dk, gs.v.y, sl);
+            gvp[(size_t)(2 * lp) * Np] = gv.v.x;
+            if (both) gvp[(size_t)(2 * lp + 1) * Np] = gv.v.y;
+        }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) gV[((size_t)row * NB + i) * N + n] = sV[i].v.x + sV[i].v.y;
+        glnc[(size_t)row * N + n] = sl;
+    }
 }
 
-// One warp walks a contiguous range of chi nodes, one multipole per lane.
-// Neighbouring nodes fall into the same z cell, and at most distances into the
-// same ln k cell (u moves by ~0.05 cells per node), so a lane keeps the 16 taps
-// of its cell and their 16 gradients in registers and exchanges them only when
-// its cell changes (about one lane per node): the gradients go to the warp's own
-// columns in shared memory (four z-taps of a column side by side, as are the
-// current table rows), and when the warp enters the next z cell the rows it has
-// left go to the warp's partial rows in global memory.  No two lanes add to one
-// column at a time: with ascending multipoles the lanes' cells ascend too, so only
-// neighbours can share one (clamped ln k); lanes with equal cells take turns.
-// Sums over multipoles (g_V, g_ln chi) are warp reductions of 8 values at once.
-template <typename T, int NB>
-__global__ void __launch_bounds__(32 * kAdjWarps, sizeof(T) == 4 ? 4 : 2)
-k_limber_adj(const ShearParams sp, const T* __restrict__ table, const T* __restrict__ win, const T* __restrict__ gC,
-             const int4* __restrict__ ranges, int W, int part_rows, T* __restrict__ part, T* __restrict__ gV,
-             T* __restrict__ glnc, int stage, int sorted, const int* __restrict__ nrows) {
+// Table gradient of g_v.  One warp walks a contiguous range of chi nodes, one
+// multipole per lane.  Neighbouring nodes fall into the same z cell, and at most
+// distances into the same ln k cell (u moves by ~0.05 cells per node), so a lane
+// keeps the 16 gradients of its cell's taps in registers.  A step to the
+// next cell down adds the one column that leaves to the warp's own columns in shared
+// memory (four z-taps of a column side by side), any other step all four; when the
+// warp enters the next z cell the rows it has left go to the warp's partial
+// rows in global memory.  No two lanes add to one column at a time: with
+// ascending multipoles the lanes' cells ascend too, so only neighbours can share one
+// (clamped ln k); lanes with equal cells take turns.
+template <typename T>
+__global__ void __launch_bounds__(32 * kAdjWarps, sizeof(T) == 4 ? 6 : 3)
+k_limber_adj(const ShearParams sp, const T* __restrict__ win, const T* __restrict__ gv_in,
+             const int4* __restrict__ ranges, int W, int part_rows, T* __restrict__ part, int sorted,
+             const int* __restrict__ nrows) {
     using Q = P2<T>;
-    constexpr int NB2 = (NB + 1) / 2;          // pairs of bins
+    constexpr unsigned ALL = 0xffffffffu;
     pdl_begin();
     const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int per_row = W / nw, row = blockIdx.x / per_row;
@@ -301,52 +426,31 @@ k_limber_adj(const ShearParams sp, const T* __restrict__ table, const T* __restr
     const int4 rg = ranges[(blockIdx.x % per_row) * nw + wid];
     const int lo = rg.x, hi = rg.y;
     if (lo >= hi) return;                      // warps work alone: no block barrier below
-    const int N = sp.N, n_k = sp.n_k, n_z = sp.n_z, n_ell = sp.n_ell, D = sp.D, PK = n_k + 2, Np = (N + 3) & ~3;
+    const int N = sp.N, n_k = sp.n_k, n_ell = sp.n_ell, PK = n_k + 2, Np = (N + 3) & ~3;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Z4<T>* acc = reinterpret_cast<Z4<T>*>(smem_raw) + (size_t)wid * PK * (stage ? 2 : 1);
-    Z4<T>* tab = acc + PK;                     // when staged: the four table rows of the current z cell
-    const T* src = table + (size_t)row * n_z * n_k;
-    const T* lnchi = win + (size_t)row * (NB + 1) * Np;
-    const T* V = lnchi + Np;
+    Z4<T>* acc = reinterpret_cast<Z4<T>*>(smem_raw) + (size_t)wid * PK;
+    const T* lnchi = win + (size_t)row * (sp.nb + 1) * Np;
     T* prow = part + ((size_t)row * part_rows + rg.z) * PK;
     const Z4<T>* zwp = reinterpret_cast<const Z4<T>*>(pick<T>(sp.zw4d, sp.zw4f));
     const T* lnell = pick<T>(sp.lnell, sp.lnell_f);
     const T lkmin = pick_s<T>(sp.lnk_min, sp.lnk_min_f), lkmax = pick_s<T>(sp.lnk_max, sp.lnk_max_f);
     const T inv_dk = pick_s<T>(1.0 / sp.dlnk, sp.inv_dlnk_f);
     const Q zero(T(0), T(0));
+    const std::integral_constant<int, 0> all_taps;
+    const std::integral_constant<int, 3> last_tap;
     for (int l0 = 0; l0 < n_ell; l0 += 32) {
         const int l = l0 + lane;
         const bool act = l < n_ell;
         const T lne = lnell[act ? l : n_ell - 1];
-        // symmetric g_C with a doubled diagonal, rows of bins in pairs: h_i = sum_j G_ij V_j is
-        // the derivative of g_P = 1/2 sum_ij G_ij V_i V_j by V_i
-        Q G[NB2][NB];
-        {
-            auto g = [&](int i, int j) {
-                if (i >= NB || !act) return T(0);
-                const int p = min(i, j) * NB - min(i, j) * (min(i, j) - 1) / 2 + abs(i - j);
-                const T v = gC[(size_t)row * D + p * n_ell + l];
-                return i == j ? T(2) * v : v;
-            };
-#pragma unroll
-            for (int i = 0; i < NB2; ++i)
-#pragma unroll
-                for (int j = 0; j < NB; ++j) G[i][j] = Q(g(2 * i, j), g(2 * i + 1, j));
-        }
+        const T* gvp = gv_in + ((size_t)row * n_ell + (act ? l : n_ell - 1)) * Np;
         int jc = sp.zrp[lo], ik = -1;
-        Z4<T> c[4], a[4];                      // by column tap
+        Z4<T> a[4];                            // by column tap
 #pragma unroll
-        for (int q = 0; q < 4; ++q) { c[q].a = c[q].b = zero; a[q].a = a[q].b = zero; }
-        auto rows_at = [&](int k) {
-            Z4<T> s;
-            s.a = Q(padded(src, n_z, n_k, jc, k), padded(src, n_z, n_k, jc + 1, k));
-            s.b = Q(padded(src, n_z, n_k, jc + 2, k), padded(src, n_z, n_k, jc + 3, k));
-            return s;
-        };
-        // add the register gradients of the lanes with f to their columns
-        auto add_columns = [&](bool mine) {
+        for (int q = 0; q < 4; ++q) a[q].a = a[q].b = zero;
+        // add the register gradients of the lanes with f to their columns, from tap q0 on
+        auto add_columns = [&](bool mine, auto q0) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
+            for (int q = decltype(q0)::value; q < 4; ++q) {
                 if (mine) {
                     Z4<T> s = acc[ik + q];
                     s.a = Q::add(s.a, a[q].a);
@@ -356,137 +460,99 @@ k_limber_adj(const ShearParams sp, const T* __restrict__ table, const T* __restr
                 __syncwarp();
             }
         };
-        auto flush = [&](bool f) {
-            const int before = __shfl_up_sync(0xffffffffu, f ? ik : -1 - lane, 1);
-            if (sorted && !__any_sync(0xffffffffu, f && lane > 0 && before == ik)) {
-                add_columns(f);
+        auto flush = [&](bool f, auto q0) {
+            const int before = __shfl_up_sync(ALL, f ? ik : -1 - lane, 1);
+            if (sorted && !__any_sync(ALL, f && lane > 0 && before == ik)) {
+                add_columns(f, q0);
                 return;
             }
-            const unsigned same = __match_any_sync(0xffffffffu, f ? ik : -1 - lane);
+            const unsigned same = __match_any_sync(ALL, f ? ik : -1 - lane);
             const int turn = __popc(same & ((1u << lane) - 1u));
-            for (int t = 0; __any_sync(0xffffffffu, f && turn >= t); ++t) add_columns(f && turn == t);
+            for (int t = 0; __any_sync(ALL, f && turn >= t); ++t) add_columns(f && turn == t, q0);
         };
         // rows jc .. to - 1 are complete for this warp: write them out, move the rest up
-        // and (when rows follow) bring in the table's next ones
-        auto advance = [&](int to, bool more) {
-            const int n = to - jc;
+        auto advance = [&](int to) {
+            const int steps = to - jc;
             T* out = prow + (size_t)(jc - rg.w) * PK;
             for (int k = lane; k < PK; k += 32) {
-                Z4<T> s = acc[k], t;
-                if (more && stage) t = tab[k];
-                for (int i = 0; i < n; ++i) {
+                Z4<T> s = acc[k];
+                for (int i = 0; i < steps; ++i) {
                     T* o = out + (size_t)i * PK + k;
                     *o = l0 ? *o + s.a.v.x : s.a.v.x;
                     s.a = Q(s.a.v.y, s.b.v.x);
                     s.b = Q(s.b.v.y, T(0));
-                    if (more && stage) {
-                        t.a = Q(t.a.v.y, t.b.v.x);
-                        t.b = Q(t.b.v.y, padded(src, n_z, n_k, jc + i + 4, k));
-                    }
                 }
                 acc[k] = s;
-                if (more && stage) tab[k] = t;
             }
             jc = to;
             __syncwarp();
         };
-        for (int k = lane; k < PK; k += 32) {
-            acc[k].a = acc[k].b = zero;
-            if (stage) tab[k] = rows_at(k);
-        }
+        for (int k = lane; k < PK; k += 32) acc[k].a = acc[k].b = zero;
         __syncwarp();
-        // node constants one node ahead
-        int zr_n = jc;
-        T lc_n = lnchi[lo], v_n[NB];
-        Z4<T> w_n = zwp[lo];
-#pragma unroll
-        for (int i = 0; i < NB; ++i) v_n[i] = V[i * Np + lo];
+        // four nodes per load of g_v and ln chi (both padded to 4), requested one quad ahead
+        Z4<T> g_n = *reinterpret_cast<const Z4<T>*>(gvp + (lo & ~3));
+        Z4<T> lc_n = *reinterpret_cast<const Z4<T>*>(lnchi + (lo & ~3));
 #pragma unroll 1
-        for (int n = lo; n < hi; ++n) {
-            const int zr = zr_n;
-            const T lc = lc_n;
-            const Z4<T> wz = w_n;
-            T vv[NB];
-#pragma unroll
-            for (int i = 0; i < NB; ++i) vv[i] = v_n[i];
-            if (n + 1 < hi) {
-                zr_n = sp.zrp[n + 1];
-                lc_n = lnchi[n + 1];
-                w_n = zwp[n + 1];
-#pragma unroll
-                for (int i = 0; i < NB; ++i) v_n[i] = V[i * Np + n + 1];
+        for (int n4 = lo & ~3; n4 < hi; n4 += 4) {
+            const Z4<T> g4 = g_n, lc4 = lc_n;
+            if (n4 + 4 < hi) {
+                g_n = *reinterpret_cast<const Z4<T>*>(gvp + n4 + 4);
+                lc_n = *reinterpret_cast<const Z4<T>*>(lnchi + n4 + 4);
             }
-            if (zr != jc) {
-                flush(ik >= 0);
-                advance(zr, true);
-                ik = -1;
-            }
-            const T s_raw = lne - lc;
-            const bool clamped = (s_raw < lkmin) || (s_raw > lkmax);
-            const T uk = (fmin(fmax(s_raw, lkmin), lkmax) - lkmin) * inv_dk;
-            const int ik_n = min(max((int)floor(uk), 0), n_k - 2);
-            const bool move = act && ik_n != ik;
-            if (__any_sync(0xffffffffu, move)) {
-                flush(move && ik >= 0);
-                if (move) {
-                    ik = ik_n;
+            const T gn[4] = {g4.a.v.x, g4.a.v.y, g4.b.v.x, g4.b.v.y};
+            const T ln[4] = {lc4.a.v.x, lc4.a.v.y, lc4.b.v.x, lc4.b.v.y};
+            int zn[4];
+            Z4<T> wn[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        c[q] = stage ? tab[ik + q] : rows_at(ik + q);
-                        a[q].a = a[q].b = zero;
+            for (int i = 0; i < 4; ++i) {
+                const int n = min(max(n4 + i, lo), hi - 1);
+                zn[i] = sp.zrp[n];
+                wn[i] = zwp[n];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (n4 + i < lo || n4 + i >= hi) continue;
+                if (zn[i] != jc) {
+                    flush(ik >= 0, all_taps);
+                    advance(zn[i]);
+                    ik = -1;
+                }
+                const T uk = (fmin(fmax(lne - ln[i], lkmin), lkmax) - lkmin) * inv_dk;
+                const int ik_n = min(max((int)floor(uk), 0), n_k - 2);
+                const bool move = act && ik_n != ik, slide = move && ik_n == ik - 1;
+                if (__any_sync(ALL, slide)) {             // one column leaves, one enters
+                    flush(slide, last_tap);
+                    if (slide) {
+                        ik = ik_n;
+#pragma unroll
+                        for (int q = 3; q > 0; --q) a[q] = a[q - 1];
+                        a[0].a = a[0].b = zero;
                     }
                 }
-                __syncwarp();
-            }
-            // doubled Catmull-Rom weights in ln k and their derivatives (the z-weights are doubled too)
-            const T t = uk - (T)ik_n, t2 = t * t, m = t * (T(4) - T(3) * t);
-            const T wk[4] = {t * (t * (T(2) - t) - T(1)), T(2) + t2 * (T(3) * t - T(5)), t * (T(1) + m), t2 * (t - T(1))};
-            const T dk[4] = {m - T(1), t * (T(9) * t - T(10)), T(1) + t * (T(8) - T(9) * t), t * (T(3) * t - T(2))};
-            T v = T(0), dv = T(0);
+                const bool jump = act && ik_n != ik;
+                if (__any_sync(ALL, jump)) {
+                    flush(jump && ik >= 0, all_taps);
+                    if (jump) {
+                        ik = ik_n;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const Q s = Q::fma(wz.b, c[q].b, Q::mul(wz.a, c[q].a));
-                const T col = s.v.x + s.v.y;
-                v = fma(wk[q], col, v);
-                dv = fma(dk[q], col, dv);
-            }
-            const T Pw = p10(T(0.25) * v);
-            Q h[NB2];
+                        for (int q = 0; q < 4; ++q) a[q].a = a[q].b = zero;
+                    }
+                }
+                // doubled Catmull-Rom weights in ln k (the z-weights are doubled too)
+                const T t = uk - (T)ik_n, t2 = t * t;
+                const T wk[4] = {t * (t * (T(2) - t) - T(1)), T(2) + t2 * (T(3) * t - T(5)),
+                                 t * (T(1) + t * (T(4) - T(3) * t)), t2 * (t - T(1))};
+                const Q ga = Q::mul(Q(gn[i], gn[i]), wn[i].a), gb = Q::mul(Q(gn[i], gn[i]), wn[i].b);
 #pragma unroll
-            for (int i = 0; i < NB2; ++i) h[i] = zero;
-#pragma unroll
-            for (int j = 0; j < NB; ++j) {
-                const Q vj(vv[j], vv[j]);
-#pragma unroll
-                for (int i = 0; i < NB2; ++i) h[i] = Q::fma(G[i][j], vj, h[i]);
-            }
-            T red[8];
-            T gP = T(0);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) red[i] = T(0);
-#pragma unroll
-            for (int i = 0; i < NB; ++i) {
-                const T hi_ = (i & 1) ? h[i / 2].v.y : h[i / 2].v.x;
-                gP = fma(vv[i], hi_, gP);
-                red[i] = hi_ * Pw;
-            }
-            const T gv = gP * Pw * (T)(kLn10 * 0.125);    // d log L / d (doubled-weight sum); gP is twice g_P
-            red[NB] = clamped ? T(0) : -gv * dv * inv_dk; // s = ln(ell + 1/2) - ln chi
-            const Q ga = Q::mul(Q(gv, gv), wz.a), gb = Q::mul(Q(gv, gv), wz.b);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const Q w(wk[q], wk[q]);
-                a[q].a = Q::fma(ga, w, a[q].a);
-                a[q].b = Q::fma(gb, w, a[q].b);
-            }
-            const T sum = warp_transpose_sum8(red);
-            if (lane <= NB) {
-                T* o = lane < NB ? gV + ((size_t)row * NB + lane) * N + n : glnc + (size_t)row * N + n;
-                *o = l0 ? *o + sum : sum;
+                for (int q = 0; q < 4; ++q) {
+                    const Q w(wk[q], wk[q]);
+                    a[q].a = Q::fma(ga, w, a[q].a);
+                    a[q].b = Q::fma(gb, w, a[q].b);
+                }
             }
         }
-        flush(ik >= 0);
-        advance(jc + 4, false);
+        flush(ik >= 0, all_taps);
+        advance(jc + 4);
     }
 }
 
@@ -574,7 +640,7 @@ __device__ __forceinline__ void block_scan(T* x, int pitch, int n, T* red) {
 enum { S_OM = 0, S_CHIH, S_W0, S_WA, S_GAMMA, S_PREF, S_AIA, S_ETA, S_COUNT };
 // Threads: 512 while an SM holds one evaluation, 256 from 153 evaluations on: two
 // CTAs then share the SM (27 arrays of 1025 FP32 nodes are 111 KB) and run through
-// one another's barriers (4096 evaluations: XXX).
+// one another's barriers (4096 evaluations: 769 -> 556 us).
 constexpr int kWinAdjThreads = 512;
 
 // elements of the per-evaluation arrays of k_windows_adj
@@ -892,6 +958,7 @@ int projection_adj_create(const ShearParams& sp, int elt, int cap, ProjectionAdj
     NS_TRY(alloc(n * sp.D, &a->gC));
     NS_TRY(alloc(n * sp.nb * sp.N, &a->gV));
     NS_TRY(alloc(n * sp.N, &a->glnc));
+    NS_TRY(alloc(n * sp.n_ell * Np, &a->gv));
     std::vector<double> lnell(sp.n_ell);
     NS_CUDA_TRY(cudaMemcpy(lnell.data(), sp.lnell, sizeof(double) * sp.n_ell, cudaMemcpyDeviceToHost));
     a->sorted = std::is_sorted(lnell.begin(), lnell.end());
@@ -967,23 +1034,32 @@ template <typename T, int NB>
 static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double* theta_full, const T* table,
                           const TableGrad& out, double* gfull, const int* nrows, int grid_rows, cudaStream_t st) {
     const int k = limber_adj_split(grid_rows), W = 8 << k, PK = sp.n_k + 2;
-    // a warp's columns of gradients and of the current table rows; the rows stay
-    // in global memory, and CTAs shrink to one warp, where tables are very wide
+    // the padded table beside g_C in shared memory; very wide tables stay in global memory
+    const size_t g_bytes = sizeof(adj::Z4<T>) * (size_t)((sp.n_ell + 1) / 2) * adj::kGQuads<T, NB>;
+    const size_t t_bytes = sizeof(T) * (size_t)(sp.n_z + 2) * PK;
+    // a warp's columns of gradients; CTAs shrink to one warp where tables are very wide
     const size_t col = sizeof(adj::Z4<T>) * (size_t)PK;
-    const int stage = 2 * col <= kAdjSmemMax;
     int nw = kAdjWarps;
-    while (nw > 1 && nw * col * (stage ? 2 : 1) > kAdjSmemMax) nw >>= 1;
-    const size_t smem = nw * col * (stage ? 2 : 1);
-    if (smem > kAdjSmemMax) return NS_ENOTSUP;
+    while (nw > 1 && nw * col > kAdjSmemMax) nw >>= 1;
+    if (nw * col > kAdjSmemMax) return NS_ENOTSUP;
     static bool attr = false;
     if (!attr) {
-        NS_CUDA_TRY(cudaFuncSetAttribute(adj::k_limber_adj<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmemMax));
+        NS_CUDA_TRY(cudaFuncSetAttribute(adj::k_limber_nodes<T, NB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmemMax));
+        NS_CUDA_TRY(cudaFuncSetAttribute(adj::k_limber_adj<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmemMax));
         NS_CUDA_TRY(cudaFuncSetAttribute(adj::k_windows_adj<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAdjSmemMax));
         attr = true;
     }
-    NS_CUDA_TRY(launch_pdl(adj::k_limber_adj<T, NB>, dim3(grid_rows * (W / nw)), dim3(32 * nw), smem, st, sp, table,
-                           (const T*)a->win, (const T*)a->gC, (const int4*)a->ranges[k], W, a->part_rows[k],
-                           (T*)a->part, (T*)a->gV, (T*)a->glnc, stage, a->sorted, nrows));
+    auto nodes = [&](auto kern, size_t smem) -> int {
+        // few evaluations: the nodes of one over several CTAs
+        NS_CUDA_TRY(launch_pdl(kern, dim3(grid_rows, 1 << k), dim3(adj::kNodeThreads), smem, st, sp, table,
+                               (const T*)a->win, (const T*)a->gC, (T*)a->gv, (T*)a->gV, (T*)a->glnc, nrows));
+        return NS_OK;
+    };
+    if (g_bytes + t_bytes <= kAdjSmemMax) NS_TRY(nodes(adj::k_limber_nodes<T, NB, true>, g_bytes + t_bytes));
+    else NS_TRY(nodes(adj::k_limber_nodes<T, NB, false>, g_bytes));
+    NS_CUDA_TRY(launch_pdl(adj::k_limber_adj<T>, dim3(grid_rows * (W / nw)), dim3(32 * nw), nw * col, st, sp,
+                           (const T*)a->win, (const T*)a->gv, (const int4*)a->ranges[k], W, a->part_rows[k],
+                           (T*)a->part, a->sorted, nrows));
     // a table row per block for few evaluations, a third of the table for many
     const dim3 g(grid_rows, grid_rows < 256 ? sp.n_z : 3);
     const dim3 b(std::min(256, (sp.n_k + 31) & ~31));

@@ -79,7 +79,7 @@ constexpr size_t kAdjSmemMax = 227 * 1024 - 8 * 1024;   // dynamic shared memory
 // Per-problem buffers of the projection adjoint for `cap` rows, in the problem's
 // arithmetic type.
 struct ProjectionAdj {
-    void *win = nullptr, *resid = nullptr, *C = nullptr, *gC = nullptr, *gV = nullptr, *glnc = nullptr;
+    void *win = nullptr, *resid = nullptr, *C = nullptr, *gC = nullptr, *gV = nullptr, *glnc = nullptr, *gv = nullptr;
     void* win_nodes = nullptr;         // FP64: the windows' node-local functions
     void* part = nullptr;              // partial rows of the table gradient
     void* scratch = nullptr;           // arrays of k_windows_adj where shared memory does not hold them
