@@ -5,9 +5,10 @@
 //
 //   k_chi2_adj     y = L^-1 r, log L, g_m = L^-T y; g_C = g_m (1+m_i)(1+m_j);
 //                  gradients of the biases and the noise templates
-//   k_limber_adj   per node and multipole: g_P = sum_p g_C V_i V_j;
-//                  g_V_i += g_C V_j P; g_v = ln 10 P g_P spread over the 16 table
-//                  taps; d v / d ln k (Catmull-Rom derivative) gives g_ln chi
+//   k_limber_nodes per node and multipole: g_P = sum_p g_C V_i V_j;
+//                  g_V_i += g_C V_j P; g_v = ln 10 P g_P; d v / d ln k (Catmull-Rom
+//                  derivative) gives g_ln chi
+//   k_limber_adj   g_v spread over the 16 table taps of each node and multipole
 //   k_table_adj    the table gradient: the warps' partial rows summed in order,
 //                  ghost rows and columns folded back
 //   k_windows_adj  windows (Eq. 5-6: the exclusive suffix sums transpose to
@@ -20,12 +21,12 @@
 //
 // No stage uses atomics, so gradients repeat bit for bit.
 //
-// Bound: FP32 instruction issue.  The one-kernel form it replaced kept 250 KB
-// of intermediates per evaluation in global memory and added 16 atomics per
-// (node, multipole) to the table gradient.  Whole BF16 gradient calls of the
-// 39-d problem: 4096 rows 9978 -> 5218 us, 64 rows 608 -> 369 us.  Per 2048
-// evaluations (BF16 problem): k_limber_adj 1334 us, k_windows_adj 382, k_table_adj
-// 149, k_chi2_adj 93.
+// Bound: FP32 instruction issue and the latencies behind it (16 to 28 warps per
+// SM).  The one-kernel form it replaced kept 250 KB of intermediates per evaluation
+// in global memory and added 16 atomics per (node, multipole) to the table
+// gradient.  Whole BF16 gradient calls of the 39-d problem: 4096 rows 9978 -> 3290
+// us, 64 rows 608 -> 290 us.  Per 4096 evaluations (BF16 problem): k_limber_adj 714
+// us, k_limber_nodes 527, k_windows_adj 519, k_chi2_adj 157, k_table_adj 153.
 #include <algorithm>
 #include <vector>
 
@@ -256,7 +257,10 @@ template <> struct P2<double> {
     static __device__ __forceinline__ P2 add(P2 a, P2 b) { return P2(a.v.x + b.v.x, a.v.y + b.v.y); }
 };
 // four z-taps of a table column
-template <typename T> struct alignas(16) Z4 { P2<T> a, b; };
+template <typename T> struct alignas(16) Z4 {
+    P2<T> a, b;
+    __device__ __forceinline__ T operator[](int i) const { return i == 0 ? a.v.x : i == 1 ? a.v.y : i == 2 ? b.v.x : b.v.y; }
+};
 
 // Reverse of the Limber sums, node by node: one lane per chi node, its windows and
 // their gradients in registers, two multipoles at a time as the halves of packed
@@ -266,7 +270,8 @@ template <typename T> struct alignas(16) Z4 { P2<T> a, b; };
 // k_limber_adj, whose lanes are multipoles.  With both halves in one kernel and one
 // multipole per lane, 20 of 32 lanes worked and each node took a warp reduction of
 // six values and the loads of its windows: 460 k warp instructions per evaluation,
-// 2560 us for 4096 evaluations of the 39-d problem; the two kernels: XXX us.
+// 2560 us for 4096 evaluations of the 39-d problem; the two kernels: 66 k and
+// 155 k instructions, 527 + 714 us.
 template <typename T, int NB> constexpr int kGQuads = (NB * (NB + 1) / 2 + 1) / 2;   // pairs of g_C entries
 constexpr int kNodeThreads = 256;
 
@@ -283,7 +288,8 @@ k_limber_nodes(const ShearParams sp, const T* __restrict__ table, const T* __res
     const int n_lp = (n_ell + 1) / 2, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Z4<T>* Gs = reinterpret_cast<Z4<T>*>(smem_raw);
-    T* U = reinterpret_cast<T*>(Gs + n_lp * NG);
+    Q* Ls = reinterpret_cast<Q*>(Gs + n_lp * NG);          // ln(ell + 1/2) of the pairs
+    T* U = reinterpret_cast<T*>(Ls + n_lp + (n_lp & 1));
     const T* src = table + (size_t)row * n_z * n_k;
     const T* lnchi = win + (size_t)row * (NB + 1) * Np;
     const T* V = lnchi + Np;
@@ -292,8 +298,10 @@ k_limber_nodes(const ShearParams sp, const T* __restrict__ table, const T* __res
     const T lkmin = pick_s<T>(sp.lnk_min, sp.lnk_min_f), lkmax = pick_s<T>(sp.lnk_max, sp.lnk_max_f);
     const T inv_dk = pick_s<T>(1.0 / sp.dlnk, sp.inv_dlnk_f);
     if (STAGE)
-        for (int r = wid; r < n_z + 2; r += kNodeThreads / 32)
-            for (int c = lane; c < PK; c += 32) U[r * PK + c] = padded(src, n_z, n_k, r, c);
+        for (int r = wid; r < n_z; r += kNodeThreads / 32)
+#pragma unroll 8
+            for (int c = lane; c < n_k; c += 32) U[(r + 1) * PK + c + 1] = src[(size_t)r * n_k + c];
+    for (int x = tid; x < n_lp; x += kNodeThreads) Ls[x] = Q(lnell[2 * x], lnell[min(2 * x + 1, n_ell - 1)]);
     // symmetric g_C with a doubled diagonal: h_i = sum_j G_ij V_j is the derivative of
     // g_P = 1/2 sum_ij G_ij V_i V_j by V_i
     for (int x = tid; x < n_lp * 2 * NG; x += kNodeThreads) {
@@ -308,6 +316,18 @@ k_limber_nodes(const ShearParams sp, const T* __restrict__ table, const T* __res
         reinterpret_cast<Q*>(Gs)[x] = Q(g0, g1);
     }
     __syncthreads();
+    if (STAGE) {                               // ghost rows, then ghost columns (linear extrapolation)
+        for (int c = 1 + tid; c <= n_k; c += kNodeThreads) {
+            U[c] = T(2) * U[PK + c] - U[2 * PK + c];
+            U[(n_z + 1) * PK + c] = T(2) * U[n_z * PK + c] - U[(n_z - 1) * PK + c];
+        }
+        __syncthreads();
+        for (int r = tid; r < n_z + 2; r += kNodeThreads) {
+            U[r * PK] = T(2) * U[r * PK + 1] - U[r * PK + 2];
+            U[r * PK + n_k + 1] = T(2) * U[r * PK + n_k] - U[r * PK + n_k - 1];
+        }
+        __syncthreads();
+    }
     auto two = [](T x) { return Q(x, x); };
     for (int n = 1 + blockIdx.y * kNodeThreads + tid; n < N; n += kNodeThreads * gridDim.y) {
         const T lc = lnchi[n];
@@ -326,10 +346,11 @@ k_limber_nodes(const ShearParams sp, const T* __restrict__ table, const T* __res
 #pragma unroll 1
         for (int lp = 0; lp < n_lp; ++lp) {
             const bool both = 2 * lp + 1 < n_ell;
-            const T s0 = lnell[2 * lp] - lc, s1 = lnell[both ? 2 * lp + 1 : 2 * lp] - lc;
+            const Q le = Ls[lp];
+            const T s0 = le.v.x - lc, s1 = le.v.y - lc;
             const T c0 = fmin(fmax(s0, lkmin), lkmax), c1 = fmin(fmax(s1, lkmin), lkmax);
             const T u0 = (c0 - lkmin) * inv_dk, u1 = (c1 - lkmin) * inv_dk;
-            const int k0 = min(max((int)floor(u0), 0), n_k - 2), k1 = min(max((int)floor(u1), 0), n_k - 2);
+            const int k0 = min((int)u0, n_k - 2), k1 = min((int)u1, n_k - 2);
             // taps folded over z
             Q col[4];
             if (STAGE) {
@@ -402,7 +423,10 @@ k_limber_nodes(const ShearParams sp, const T* __restrict__ table, const T* __res
     }
 }
 
-// Table gradient of g_v.  One warp walks a contiguous range of chi nodes, one
+// Table gradient of g_v.  Bound by instruction issue (155 k warp instructions per
+// evaluation, 2.5 per cycle); node constants are read where they are used, which
+// leaves registers for 28 warps per SM (held for four nodes at a time: 870 us against
+// 714 for 4096 evaluations).  One warp walks a contiguous range of chi nodes, one
 // multipole per lane.  Neighbouring nodes fall into the same z cell, and at most
 // distances into the same ln k cell (u moves by ~0.05 cells per node), so a lane
 // keeps the 16 gradients of its cell's taps in registers.  A step to the
@@ -413,7 +437,7 @@ k_limber_nodes(const ShearParams sp, const T* __restrict__ table, const T* __res
 // ascending multipoles the lanes' cells ascend too, so only neighbours can share one
 // (clamped ln k); lanes with equal cells take turns.
 template <typename T>
-__global__ void __launch_bounds__(32 * kAdjWarps, sizeof(T) == 4 ? 6 : 3)
+__global__ void __launch_bounds__(32 * kAdjWarps, sizeof(T) == 4 ? 7 : 3)
 k_limber_adj(const ShearParams sp, const T* __restrict__ win, const T* __restrict__ gv_in,
              const int4* __restrict__ ranges, int W, int part_rows, T* __restrict__ part, int sorted,
              const int* __restrict__ nrows) {
@@ -501,48 +525,44 @@ k_limber_adj(const ShearParams sp, const T* __restrict__ win, const T* __restric
             }
             const T gn[4] = {g4.a.v.x, g4.a.v.y, g4.b.v.x, g4.b.v.y};
             const T ln[4] = {lc4.a.v.x, lc4.a.v.y, lc4.b.v.x, lc4.b.v.y};
-            int zn[4];
-            Z4<T> wn[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int n = min(max(n4 + i, lo), hi - 1);
-                zn[i] = sp.zrp[n];
-                wn[i] = zwp[n];
-            }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 if (n4 + i < lo || n4 + i >= hi) continue;
-                if (zn[i] != jc) {
+                const int zr = sp.zrp[n4 + i];
+                const Z4<T> wz = zwp[n4 + i];
+                if (zr != jc) {
                     flush(ik >= 0, all_taps);
-                    advance(zn[i]);
+                    advance(zr);
                     ik = -1;
                 }
                 const T uk = (fmin(fmax(lne - ln[i], lkmin), lkmax) - lkmin) * inv_dk;
-                const int ik_n = min(max((int)floor(uk), 0), n_k - 2);
-                const bool move = act && ik_n != ik, slide = move && ik_n == ik - 1;
-                if (__any_sync(ALL, slide)) {             // one column leaves, one enters
-                    flush(slide, last_tap);
-                    if (slide) {
-                        ik = ik_n;
+                const int ik_n = min((int)uk, n_k - 2);   // uk >= 0
+                if (__any_sync(ALL, act && ik_n != ik)) {
+                    const bool slide = act && ik_n == ik - 1;
+                    if (__any_sync(ALL, slide)) {         // one column leaves, one enters
+                        flush(slide, last_tap);
+                        if (slide) {
+                            ik = ik_n;
 #pragma unroll
-                        for (int q = 3; q > 0; --q) a[q] = a[q - 1];
-                        a[0].a = a[0].b = zero;
+                            for (int q = 3; q > 0; --q) a[q] = a[q - 1];
+                            a[0].a = a[0].b = zero;
+                        }
                     }
-                }
-                const bool jump = act && ik_n != ik;
-                if (__any_sync(ALL, jump)) {
-                    flush(jump && ik >= 0, all_taps);
-                    if (jump) {
-                        ik = ik_n;
+                    const bool jump = act && ik_n != ik;
+                    if (__any_sync(ALL, jump)) {
+                        flush(jump && ik >= 0, all_taps);
+                        if (jump) {
+                            ik = ik_n;
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) a[q].a = a[q].b = zero;
+                            for (int q = 0; q < 4; ++q) a[q].a = a[q].b = zero;
+                        }
                     }
                 }
                 // doubled Catmull-Rom weights in ln k (the z-weights are doubled too)
                 const T t = uk - (T)ik_n, t2 = t * t;
                 const T wk[4] = {t * (t * (T(2) - t) - T(1)), T(2) + t2 * (T(3) * t - T(5)),
                                  t * (T(1) + t * (T(4) - T(3) * t)), t2 * (t - T(1))};
-                const Q ga = Q::mul(Q(gn[i], gn[i]), wn[i].a), gb = Q::mul(Q(gn[i], gn[i]), wn[i].b);
+                const Q ga = Q::mul(Q(gn[i], gn[i]), wz.a), gb = Q::mul(Q(gn[i], gn[i]), wz.b);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     const Q w(wk[q], wk[q]);
@@ -587,13 +607,57 @@ k_table_adj(const T* __restrict__ part, int part_rows, const int* __restrict__ p
         if (c >= n_k - 1) s += (c == n_k ? T(2) : T(-1)) * at(r, n_k + 1);
         return s;
     };
-    for (int r = 1 + blockIdx.y; r <= n_z; r += gridDim.y)
-        for (int c = 1 + threadIdx.x; c <= n_k; c += blockDim.x) {
+    // rows r0 .. r1 - 1 of this block; ra .. rb - 1 of them take no ghost row, and their
+    // partial rows, contiguous in the index, are loaded eight at a time (one row's two or
+    // three at a time left a load's latency between any two rows: 188 us for 4096
+    // evaluations of the 39-d problem, 153 us so); a block with one row has none to overlap
+    const int per = (n_z + gridDim.y - 1) / gridDim.y;
+    const int r0 = 1 + blockIdx.y * per, r1 = min(n_z + 1, r0 + per);
+    const int ra = n_k >= 4 && per > 1 ? min(max(r0, 3), r1) : r1, rb = max(ra, min(r1, n_z - 1));
+    for (int c = 1 + threadIdx.x; c <= n_k; c += blockDim.x) {
+        auto put = [&](int r, T s) { out.put(row, (r - 1) * n_k + c - 1, n_z * n_k, s); };
+        auto edge_row = [&](int r) {
             T s = cols(r, c);
             if (r <= 2) s += (r == 1 ? T(2) : T(-1)) * cols(0, c);
             if (r >= n_z - 1) s += (r == n_z ? T(2) : T(-1)) * cols(n_z + 1, c);
-            out.put(row, (r - 1) * n_k + c - 1, n_z * n_k, s);
+            put(r, s);
+        };
+        for (int r = r0; r < ra; ++r) edge_row(r);
+        if (ra < rb) {
+            const bool ghost = c <= 2 || c >= n_k - 1;
+            const int cg = c <= 2 ? 0 : n_k + 1;
+            const T f = (c == 1 || c == n_k) ? T(2) : T(-1);
+            int r = ra, end = sp_[ra + 1];
+            const int last = sp_[rb];
+            T s = T(0);
+            for (int x = sp_[ra]; x < last; x += 8) {
+                T v[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    v[i] = T(0);
+                    if (x + i < last) {
+                        v[i] = p[si[x + i] + c];
+                        if (ghost) v[i] += f * p[si[x + i] + cg];
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    if (x + i >= last) break;
+                    while (x + i >= end) {
+                        put(r, s);
+                        s = T(0);
+                        end = sp_[++r + 1];
+                    }
+                    s += v[i];
+                }
+            }
+            for (; r < rb; ++r) {
+                put(r, s);
+                s = T(0);
+            }
         }
+        for (int r = rb; r < r1; ++r) edge_row(r);
+    }
 }
 
 // ------------------------------------------------------------------ windows and distances
@@ -638,16 +702,18 @@ __device__ __forceinline__ void block_scan(T* x, int pitch, int n, T* red) {
 }
 
 enum { S_OM = 0, S_CHIH, S_W0, S_WA, S_GAMMA, S_PREF, S_AIA, S_ETA, S_COUNT };
-// Threads: 512 while an SM holds one evaluation, 256 from 153 evaluations on: two
-// CTAs then share the SM (27 arrays of 1025 FP32 nodes are 111 KB) and run through
-// one another's barriers (4096 evaluations: 769 -> 556 us).
-constexpr int kWinAdjThreads = 512;
+// Threads per SM: one CTA while an SM holds one evaluation; from 153 evaluations on
+// two CTAs share the SM (27 arrays of 1025 FP32 nodes are 111 KB) and run through one
+// another's barriers (4096 evaluations: 769 -> 556 us).  A CTA's share is cut to the
+// warps that keep the number of passes over the nodes (1025 nodes: 352 threads in
+// 3 passes 519 us, 288 in 4 601, 256 in 5 550, 224 in 5 586).
+template <typename T> constexpr int kWinAdjThreads = sizeof(T) == 4 ? 704 : 512;
 
 // elements of the per-evaluation arrays of k_windows_adj
 __host__ __device__ inline size_t windows_adj_elems(int N, int nb) { return (size_t)(7 + 4 * nb) * N; }
 
 template <typename T, int NB>
-__global__ void __launch_bounds__(kWinAdjThreads)
+__global__ void __launch_bounds__(kWinAdjThreads<T>)
 k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const T* __restrict__ gV,
               const T* __restrict__ glnc, T* __restrict__ scratch, double* __restrict__ gfull,
               const int* __restrict__ nrows) {
@@ -663,7 +729,7 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
     T *gchi = S + 6 * N, *t2 = gchi;             // g_chi for its suffix sums (beside t1)
     T *raw = S + 7 * N, *nchi = raw + NB * N, *E0 = nchi + NB * N, *E1 = E0 + NB * N;
     constexpr int NS = S_COUNT + 3 * NB, NR = NS > 2 * NB ? NS : 2 * NB;
-    __shared__ T red[(kWinAdjThreads / 32) * NR];
+    __shared__ T red[(kWinAdjThreads<T> / 32) * NR];
     __shared__ T th[16];
     const T* a_ = pick<T>(sp.a, sp.a_f);
     const T* lna_ = pick<T>(sp.lna, sp.lna_f);
@@ -672,9 +738,9 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
     const T* nz_mu = pick<T>(sp.nz_mean, sp.nz_mean_f);
     const T* nz_sg = pick<T>(sp.nz_sigma, sp.nz_sigma_f);
     const T* ia_ = pick<T>(sp.ia, sp.ia_f);
-    const T* gl_ia = pick<T>(sp.gl_ia, sp.gl_ia_f);
-    const T* gl_ln = pick<T>(sp.gl_ln, sp.gl_ln_f);
-    const T* gl_1ma = pick<T>(sp.gl_1ma, sp.gl_1ma_f);
+    const Z4<T>* gl_ia = reinterpret_cast<const Z4<T>*>(pick<T>(sp.gl_ia, sp.gl_ia_f));   // four points per interval
+    const Z4<T>* gl_ln = reinterpret_cast<const Z4<T>*>(pick<T>(sp.gl_ln, sp.gl_ln_f));
+    const Z4<T>* gl_1ma = reinterpret_cast<const Z4<T>*>(pick<T>(sp.gl_1ma, sp.gl_1ma_f));
     const T lnpiv = pick_s<T>(sp.ln_pivot, sp.ln_pivot_f), c1rho = pick_s<T>(sp.c1rho, sp.c1rho_f);
     if (tid < 11 + NB) th[tid] = (T)theta_full[(size_t)row * sp.n_params + tid];
     __syncthreads();
@@ -697,10 +763,11 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
         Ez[n] = sqrt(om * (ia * ia * ia) + (T(1) - om) * de);
         T inc = T(0);
         if (n < N - 1) {
+            const Z4<T> qi = gl_ia[n], ql = gl_ln[n], qa = gl_1ma[n];
 #pragma unroll
             for (int g = 0; g < 4; ++g) {
-                const T ig = gl_ia[4 * n + g];
-                const T e2 = om * ig * ig * ig + (T(1) - om) * ex<T>(-pde * gl_ln[4 * n + g] - T(3) * wa * gl_1ma[4 * n + g]);
+                const T ig = qi[g];
+                const T e2 = om * ig * ig * ig + (T(1) - om) * ex<T>(-pde * ql[g] - T(3) * wa * qa[g]);
                 inc += glw<T>(g) * ig * ig * rsq(e2);
             }
             inc *= chiH * T(0.5) * (a - a_[n + 1]);
@@ -842,9 +909,10 @@ k_windows_adj(const ShearParams sp, const double* __restrict__ theta_full, const
         if (m < N - 1) {
             const T g = t2[m], half = T(0.5) * (a - a_[m + 1]);
             T inc = T(0);
+            const Z4<T> qi = gl_ia[m], ql = gl_ln[m], qa = gl_1ma[m];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                const T lgg = gl_ln[4 * m + q], ig = gl_ia[4 * m + q], oma_q = gl_1ma[4 * m + q], i3 = ig * ig * ig;
+                const T lgg = ql[q], ig = qi[q], oma_q = qa[q], i3 = ig * ig * ig;
                 const T deg = ex<T>(-pde * lgg - T(3) * wa * oma_q);
                 const T rs = rsq(om * i3 + (T(1) - om) * deg);
                 const T F = ig * ig * rs;
@@ -1035,7 +1103,8 @@ static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double*
                           const TableGrad& out, double* gfull, const int* nrows, int grid_rows, cudaStream_t st) {
     const int k = limber_adj_split(grid_rows), W = 8 << k, PK = sp.n_k + 2;
     // the padded table beside g_C in shared memory; very wide tables stay in global memory
-    const size_t g_bytes = sizeof(adj::Z4<T>) * (size_t)((sp.n_ell + 1) / 2) * adj::kGQuads<T, NB>;
+    const size_t g_bytes = sizeof(adj::Z4<T>) * (size_t)((sp.n_ell + 1) / 2) * adj::kGQuads<T, NB> +
+                           sizeof(adj::P2<T>) * (size_t)(((sp.n_ell + 1) / 2 + 1) & ~1);
     const size_t t_bytes = sizeof(T) * (size_t)(sp.n_z + 2) * PK;
     // a warp's columns of gradients; CTAs shrink to one warp where tables are very wide
     const size_t col = sizeof(adj::Z4<T>) * (size_t)PK;
@@ -1060,8 +1129,9 @@ static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double*
     NS_CUDA_TRY(launch_pdl(adj::k_limber_adj<T>, dim3(grid_rows * (W / nw)), dim3(32 * nw), nw * col, st, sp,
                            (const T*)a->win, (const T*)a->gv, (const int4*)a->ranges[k], W, a->part_rows[k],
                            (T*)a->part, a->sorted, nrows));
-    // a table row per block for few evaluations, a third of the table for many
-    const dim3 g(grid_rows, grid_rows < 256 ? sp.n_z : 3);
+    // a table row per block for few evaluations, the whole table from 1024 on (4096
+    // evaluations: one block 153 us, three 161, six 173)
+    const dim3 g(grid_rows, grid_rows < 256 ? sp.n_z : grid_rows < 1024 ? 3 : 1);
     const dim3 b(std::min(256, (sp.n_k + 31) & ~31));
     auto table_adj = [&](auto o) -> int {
         NS_CUDA_TRY(launch_pdl(adj::k_table_adj<T, decltype(o)>, g, b, sizeof(int) * (sp.n_z + 3 + a->part_rows[k]), st,
@@ -1076,7 +1146,9 @@ static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double*
         else if (out.px == 2) NS_TRY(table_adj(adj::OutPlaneT<2>{out.planes, out.stride, out.pitch, out.scale}));
         else NS_TRY(table_adj(adj::OutT32{(float*)out.table}));
     }
-    NS_CUDA_TRY(launch_pdl(adj::k_windows_adj<T, NB>, dim3(grid_rows), dim3(grid_rows > 152 ? 256 : adj::kWinAdjThreads),
+    const int share = grid_rows > 152 ? adj::kWinAdjThreads<T> / 2 : adj::kWinAdjThreads<T>;
+    const int passes = (sp.N + share - 1) / share, threads = ((sp.N + passes - 1) / passes + 31) & ~31;
+    NS_CUDA_TRY(launch_pdl(adj::k_windows_adj<T, NB>, dim3(grid_rows), dim3(threads),
                            a->win_smem, st, sp,
                            theta_full, (const T*)a->gV, (const T*)a->glnc, (T*)a->scratch, gfull, nrows));
     return NS_OK;
