@@ -1,95 +1,118 @@
-// Hand-written adjoint of the shear likelihood (row A14): d log L / d theta.
+// Hand-written adjoint of the shear likelihood: d log L / d theta.
 //
 // The emulator forward with stored activations, the projection and its reverse
 // (projection_adj.cu: log L, the table gradient and the gradient of the
 // parameters that enter the projection), the emulator backward (transposed
 // GEMMs, tanh' from the stored activations), and the emulator inputs' share
 // added to the parameter gradient in k_finish_grad.
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <vector>
 
 #include "likelihood.cuh"
 #include "projection_adj.cuh"
+#include "tcgen05.cuh"
 
 namespace gpuns {
 
 // ------------------------------------------------------------------ emulator backward
 namespace adj {
 
-// Forward layer with stored activation: out = tanh(A W^T + b) (hidden) or
-// mu + sigma (A W^T + b) (output); A: rows x K, W: N x K.
-template <typename T, int BM, int BN, int BK, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN))
-k_dense(const T* __restrict__ A, const T* __restrict__ W, const T* __restrict__ bias, const T* __restrict__ mu,
-        T sigma, T* __restrict__ C, const int* __restrict__ nrows, int N, int K, int mode,
-        const T* __restrict__ aux) {
-    // mode 0: tanh(acc + b); 1: mu + sigma (acc + b); 2: acc * (1 - aux^2)  [W read transposed: W is K_out x N]
-    constexpr int TX = BN / TN, TY = BM / TM, NT = TX * TY;
+// FP64 backward layer: share z of the contraction C = A W (A: rows x K, W: K x N
+// row-major), k in [z kc, (z + 1) kc).  Bound by the FP64 pipe (2 FMA per cycle and
+// SM): the output layer of the 39-d problem contracts 10000 outputs into 16 tiles of
+// 64 units, so that without shares 16 of 152 SMs worked (24 gradients 21.6 ms, 2.1
+// with them and the forward pass on the tensor cores).
+constexpr int kBackN = 64, kBackK = 8, kBackThreads = 256;
+template <int BM>
+__global__ void __launch_bounds__(kBackThreads)
+k_back(const double* __restrict__ A, const double* __restrict__ W, double* __restrict__ part, int cap,
+       const int* __restrict__ nrows, int N, int K, int kc) {
+    constexpr int TN = 4, TX = kBackN / TN, TY = kBackThreads / TX, TM = BM / TY;
     const int M = *nrows;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * kBackN;
     if (m0 >= M) return;
-    __shared__ T As[BK][BM + 1];
-    __shared__ T Bs[BK][BN + 1];
+    __shared__ double As[kBackK][BM + 1];
+    __shared__ double Bs[kBackK][kBackN + 1];
     const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
-    T acc[TM][TN];
+    const int k_end = min(K, ((int)blockIdx.z + 1) * kc);
+    double acc[TM][TN];
+#pragma unroll
     for (int i = 0; i < TM; ++i)
-        for (int j = 0; j < TN; ++j) acc[i][j] = T(0);
-    for (int k0 = 0; k0 < K; k0 += BK) {
-        for (int i = tid; i < BM * BK; i += NT) {
-            const int rr = i / BK, c = i % BK;
-            As[c][rr] = (m0 + rr < M && k0 + c < K) ? A[(size_t)(m0 + rr) * K + k0 + c] : T(0);
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = 0.0;
+    for (int k0 = blockIdx.z * kc; k0 < k_end; k0 += kBackK) {
+        for (int i = tid; i < BM * kBackK; i += kBackThreads) {
+            const int rr = i / kBackK, c = i % kBackK;
+            As[c][rr] = (m0 + rr < M && k0 + c < k_end) ? A[(size_t)(m0 + rr) * K + k0 + c] : 0.0;
         }
-        if (mode == 2) {
-            // contraction index k over rows of W (K x N row-major): element (n, k) = W[k * N + n]
-            for (int i = tid; i < BN * BK; i += NT) {
-                const int c = i / BN, nn = i % BN;
-                Bs[c][nn] = (n0 + nn < N && k0 + c < K) ? W[(size_t)(k0 + c) * N + n0 + nn] : T(0);
-            }
-        } else {
-            for (int i = tid; i < BN * BK; i += NT) {
-                const int rr = i / BK, c = i % BK;
-                Bs[c][rr] = (n0 + rr < N && k0 + c < K) ? W[(size_t)(n0 + rr) * K + k0 + c] : T(0);
-            }
+        for (int i = tid; i < kBackN * kBackK; i += kBackThreads) {
+            const int c = i / kBackN, nn = i % kBackN;
+            Bs[c][nn] = (n0 + nn < N && k0 + c < k_end) ? W[(size_t)(k0 + c) * N + n0 + nn] : 0.0;
         }
         __syncthreads();
-        for (int kk = 0; kk < BK; ++kk) {
-            T a[TM], b[TN];
+#pragma unroll
+        for (int kk = 0; kk < kBackK; ++kk) {
+            double a[TM], b[TN];
+#pragma unroll
             for (int i = 0; i < TM; ++i) a[i] = As[kk][ty + i * TY];
+#pragma unroll
             for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx + j * TX];
+#pragma unroll
             for (int i = 0; i < TM; ++i)
+#pragma unroll
                 for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
         }
         __syncthreads();
     }
+#pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int gm = m0 + ty + i * TY;
         if (gm >= M) continue;
+#pragma unroll
         for (int j = 0; j < TN; ++j) {
             const int gn = n0 + tx + j * TX;
-            if (gn >= N) continue;
-            T v = acc[i][j];
-            if (mode == 0) v = tanh(v + bias[gn]);
-            else if (mode == 1) v = mu[gn] + sigma * (v + bias[gn]);
-            else { const T hh = aux[(size_t)gm * N + gn]; v = v * (T(1) - hh * hh); }
-            C[(size_t)gm * N + gn] = v;
+            if (gn < N) part[((size_t)blockIdx.z * cap + gm) * N + gn] = acc[i][j];
         }
     }
 }
 
-template <typename T>
+// the shares added in order, times tanh' from the stored activations
+__global__ void k_back_sum(const double* __restrict__ part, int cap, int shares, const double* __restrict__ h, int N,
+                           double* __restrict__ out, const int* __restrict__ nrows) {
+    const int row = blockIdx.y, n = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= *nrows || n >= N) return;
+    double s = 0.0;
+    for (int z = 0; z < shares; ++z) s += part[((size_t)z * cap + row) * N + n];
+    const double hh = h[(size_t)row * N + n];
+    out[(size_t)row * N + n] = s * (1.0 - hh * hh);
+}
+
+// Shares of a backward contraction: enough for one block per SM at one row tile,
+// at least 64 terms each.  By shape only: a row's gradient does not depend on
+// its batch.
+static int back_shares(int N, int K) {
+    const int tiles = (N + kBackN - 1) / kBackN;
+    return std::max(1, std::min((K + 63) / 64, 152 / tiles));
+}
+
+// FP64 input layer: the activations and their slices for the next layer
 __global__ void k_emu_in_store(const double* __restrict__ theta_full, int P, const int* __restrict__ inputs,
                                const double* __restrict__ center, const double* __restrict__ scale, int K0,
-                               const T* __restrict__ W0, const T* __restrict__ b0, int N, T* __restrict__ out,
+                               const double* __restrict__ W0, const double* __restrict__ b0, int N,
+                               double* __restrict__ out, __half* __restrict__ slices, int pitch, long long stride,
                                const int* __restrict__ nrows) {
     const int row = blockIdx.y;
     if (row >= *nrows) return;
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= N) return;
-    T acc = b0[n];
+    double acc = b0[n];
     for (int j = 0; j < K0; ++j)
-        acc += W0[(size_t)n * K0 + j] * (T)((theta_full[(size_t)row * P + inputs[j]] - center[j]) / scale[j]);
-    out[(size_t)row * N + n] = tanh(acc);
+        acc += W0[(size_t)n * K0 + j] * ((theta_full[(size_t)row * P + inputs[j]] - center[j]) / scale[j]);
+    const double h = tanh(acc);
+    out[(size_t)row * N + n] = h;
+    tc::slice_store(h, slices + (size_t)row * pitch + n, stride);
 }
 
 // The emulator inputs' share g_x = g_pre_1 W0 (rows x K0, K0 <= KMAX) added to
@@ -189,12 +212,18 @@ __global__ void __launch_bounds__(256) k_transpose_planes(const __nv_bfloat16* _
         if (k0 + y < K && n0 + x < N) o[(size_t)(k0 + y) * tp + n0 + x] = t[x][y];
 }
 
-template <typename T>
-static int dense(const T* A, const T* W, const T* bias, const T* mu, T sigma, T* C, const int* nrows, int grid_rows,
-                 int N, int K, int mode, const T* aux, cudaStream_t st) {
-    constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4;
-    dim3 g((N + BN - 1) / BN, (grid_rows + BM - 1) / BM);
-    k_dense<T, BM, BN, BK, TM, TN><<<g, 256, 0, st>>>(A, W, bias, mu, sigma, C, nrows, N, K, mode, aux);
+// g_pre_l = (g_pre_{l+1} W_l) * (1 - h_l^2)
+static int back_layer(const double* A, const double* W, const double* h, double* part, int cap, double* out,
+                      const int* nrows, int grid_rows, int N, int K, cudaStream_t st) {
+    const int S = back_shares(N, K), kc = ((K + S - 1) / S + kBackK - 1) / kBackK * kBackK;
+    // 24 rows fill three quarters of a 32-row tile and three eighths of a 64-row one
+    const int bm = grid_rows <= 16 ? 16 : grid_rows <= 32 ? 32 : 64;
+    const dim3 g((N + kBackN - 1) / kBackN, (grid_rows + bm - 1) / bm, S);
+    if (bm == 16) k_back<16><<<g, kBackThreads, 0, st>>>(A, W, part, cap, nrows, N, K, kc);
+    else if (bm == 32) k_back<32><<<g, kBackThreads, 0, st>>>(A, W, part, cap, nrows, N, K, kc);
+    else k_back<64><<<g, kBackThreads, 0, st>>>(A, W, part, cap, nrows, N, K, kc);
+    NS_CUDA_TRY(cudaGetLastError());
+    k_back_sum<<<dim3((N + 255) / 256, grid_rows), 256, 0, st>>>(part, cap, S, h, N, out, nrows);
     NS_CUDA_TRY(cudaGetLastError());
     return NS_OK;
 }
@@ -214,7 +243,15 @@ struct GradState {
     void* Linv = nullptr;      // D x D, L^-1 row-major in the arithmetic type
     ProjectionAdj proj;
     double* gfull = nullptr;   // cap x P
-    // FP64: stored activations per hidden layer and ping-pong adjoints
+    // FP64: stored activations per hidden layer, their slices (ping-pong), adjoints
+    // (ping-pong) and the shares of a backward contraction
+    __half* Hs[2] = {};
+    long long slice_stride = 0;
+    std::vector<SliceMapX> tmHs;
+    std::vector<CUtensorMap> tmWs;           // the problem's weight slices, or its own
+    std::vector<double*> wscale;
+    double* part = nullptr;
+    int cap = 0;
     std::vector<double*> H;
     double* g64[2] = {nullptr, nullptr};
     // FP32 and BF16: activations and adjoints in px bf16 planes (3: FP32; 2: the
@@ -287,6 +324,38 @@ static int grad_state_create(const ns_problem* p, GradState* g) {
         g->H.assign(L, nullptr);
         for (int l = 1; l < L; ++l) NS_TRY(grad_alloc(g, 8 * (size_t)cap * p->dims[l], (void**)&g->H[l]));
         for (int i = 0; i < 2; ++i) NS_TRY(grad_alloc(g, 8 * (size_t)cap * wmax, (void**)&g->g64[i]));
+        g->cap = cap;
+        size_t part = 0;
+        for (int l = 1; l < L; ++l)
+            part = std::max(part, (size_t)adj::back_shares(p->dims[l], p->dims[l + 1]) * p->dims[l]);
+        NS_TRY(grad_alloc(g, 8 * part * cap, (void**)&g->part));
+        const long long rows_pad = ((cap + 127) / 128) * 128;
+        g->slice_stride = rows_pad * plane_pitch(p->hidden_max);
+        for (int i = 0; i < 2; ++i) {
+            const size_t n = sizeof(__half) * tc::kSlices * (size_t)g->slice_stride;
+            NS_TRY(grad_alloc(g, n, (void**)&g->Hs[i]));
+            NS_CUDA_TRY(cudaMemsetAsync(g->Hs[i], 0, n, nullptr));
+        }
+        g->tmWs = p->tmWs;
+        g->wscale = p->d_wscale;
+        if (g->tmWs.empty()) {               // a problem whose likelihood takes no slices
+            g->tmWs.resize(L);
+            g->wscale.assign(L, nullptr);
+            for (int l = 1; l < L; ++l) {
+                const int N = p->dims[l + 1], K = p->dims[l], pitch = plane_pitch(K);
+                void* v;
+                NS_TRY(grad_alloc(g, sizeof(__half) * tc::kSlices * (size_t)N * pitch, &v));
+                NS_TRY(grad_alloc(g, sizeof(double) * N, (void**)&g->wscale[l]));
+                NS_TRY(launch_slice_rows((const double*)p->d_W[l], N, K, (__half*)v, (long long)N * pitch, pitch,
+                                         g->wscale[l], nullptr));
+                NS_TRY(make_tensor_map_slices(&g->tmWs[l], v, N, K, (long long)N * pitch, 128));
+            }
+        }
+        g->tmHs.resize(L);
+        for (int l = 1; l < L; ++l)
+            for (int i = 0; i < 3; ++i)
+                NS_TRY(make_tensor_map_slices(&g->tmHs[l].m[i], g->Hs[(l - 1) & 1], (int)rows_pad, p->dims[l],
+                                              g->slice_stride, 16 << i));
         NS_CUDA_TRY(cudaStreamSynchronize(nullptr));   // calls may come on any stream
         return NS_OK;
     }
@@ -340,21 +409,35 @@ static int launch_finish_grad(const ns_problem* p, GradState* g, const T* gpre, 
     return NS_OK;
 }
 
-// FP64 problems: the emulator forward and backward on CUDA cores.
+// FP64 problems: the emulator forward as fixed-point slices on the tensor cores (as the
+// likelihood's), backward on the FP64 pipe.
 static int run_grad_f64(const ns_problem* p, GradState* g, int B, OutPtr logL, OutPtr grad, cudaStream_t st) {
     const int L = p->n_layers, n_out = p->dims.back();
     const ShearParams& sp = p->sp;
     NS_TRY(launch_projection_adj_windows<double>(sp, &g->proj, g->theta_full, g->d_nrows, B, st));
     const dim3 g0((p->dims[1] + 255) / 256, B);
-    adj::k_emu_in_store<double><<<g0, 256, 0, st>>>(g->theta_full, p->P, p->d_inputs, p->d_in_center, p->d_in_scale,
-                                                    p->dims[0], (const double*)p->d_W[0], (const double*)p->d_b[0],
-                                                    p->dims[1], g->H[1], g->d_nrows);
+    adj::k_emu_in_store<<<g0, 256, 0, st>>>(g->theta_full, p->P, p->d_inputs, p->d_in_center, p->d_in_scale,
+                                            p->dims[0], (const double*)p->d_W[0], (const double*)p->d_b[0],
+                                            p->dims[1], g->H[1], g->Hs[0], plane_pitch(p->dims[1]), g->slice_stride,
+                                            g->d_nrows);
     NS_CUDA_TRY(cudaGetLastError());
     for (int l = 1; l < L; ++l) {
         const bool last = (l == L - 1);
-        NS_TRY(adj::dense<double>(g->H[l], (const double*)p->d_W[l], (const double*)p->d_b[l],
-                                  (const double*)p->d_out_mu, p->out_sigma, last ? (double*)g->table : g->H[l + 1],
-                                  g->d_nrows, B, p->dims[l + 1], p->dims[l], last ? 1 : 0, nullptr, st));
+        SliceEpi e;
+        e.bias = (const double*)p->d_b[l];
+        e.wscale = g->wscale[l];
+        if (last) {
+            e.mu = (const double*)p->d_out_mu;
+            e.sigma = p->out_sigma;
+            e.out = (double*)g->table;
+        } else {
+            e.tanh = 1;
+            e.out = g->H[l + 1];
+            e.slices = g->Hs[l & 1];
+            e.slice_stride = g->slice_stride;
+            e.pitch = plane_pitch(p->dims[l + 1]);
+        }
+        NS_TRY(launch_gemm_slices(&g->tmWs[l], &g->tmHs[l], e, g->d_nrows, B, p->dims[l + 1], p->dims[l], g->d_err, st));
     }
     const double* tab = (const double*)g->table;
     const bool coarse = p->n_z_emu != sp.n_z;
@@ -378,8 +461,8 @@ static int run_grad_f64(const ns_problem* p, GradState* g, int B, OutPtr logL, O
     // g_pre_{l} = (g_pre_{l+1} W_l) * (1 - h_l^2), l = L-1 .. 1
     int cur = 0;
     for (int l = L - 1; l >= 1; --l) {
-        NS_TRY(adj::dense<double>(g->g64[cur], (const double*)p->d_W[l], nullptr, nullptr, 0.0, g->g64[cur ^ 1],
-                                  g->d_nrows, B, p->dims[l], p->dims[l + 1], 2, g->H[l], st));
+        NS_TRY(adj::back_layer(g->g64[cur], (const double*)p->d_W[l], g->H[l], g->part, g->cap, g->g64[cur ^ 1],
+                               g->d_nrows, B, p->dims[l], p->dims[l + 1], st));
         cur ^= 1;
     }
     return launch_finish_grad<double>(p, g, g->g64[cur], B, grad, st);

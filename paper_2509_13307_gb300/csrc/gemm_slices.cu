@@ -199,8 +199,13 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
         // hi 2^-34 + lo 2^-61
         double v = fma((double)l, 4.33680868994201773603e-19, (double)h * 5.82076609134674072266e-11) * ws + bias;
         if (h >= kNaN) v = NAN;
-        if (e.tanh) slice_store(tanh(v), e.slices + (size_t)row * e.pitch + f, e.slice_stride);
-        else e.out[(size_t)row * N + f] = mu + e.sigma * v;
+        if (e.tanh) {
+            const double t = tanh(v);
+            if (e.out) e.out[(size_t)row * N + f] = t;
+            slice_store(t, e.slices + (size_t)row * e.pitch + f, e.slice_stride);
+        } else {
+            e.out[(size_t)row * N + f] = mu + e.sigma * v;
+        }
     };
     __syncthreads();                             // the ring's last copies have landed
     const bool failed = s_fail != 0;

@@ -318,7 +318,7 @@ struct SliceEpi {
     const double* wscale = nullptr;   // per feature: the power of two taken out of the row of W
     const double* mu = nullptr;
     double sigma = 0;
-    double* out = nullptr;            // rows x N
+    double* out = nullptr;            // rows x N (tanh: the activations in FP64, if wanted)
     __half* slices = nullptr;         // row pitch `pitch`
     long long slice_stride = 0;
     int pitch = 0;

@@ -1146,7 +1146,9 @@ static int launch_reverse(const ShearParams& sp, ProjectionAdj* a, const double*
         else if (out.px == 2) NS_TRY(table_adj(adj::OutPlaneT<2>{out.planes, out.stride, out.pitch, out.scale}));
         else NS_TRY(table_adj(adj::OutT32{(float*)out.table}));
     }
-    const int share = grid_rows > 152 ? adj::kWinAdjThreads<T> / 2 : adj::kWinAdjThreads<T>;
+    // two CTAs per SM where their arrays fit (FP64: 221 KB for 1025 nodes, one)
+    const bool pairs = grid_rows > 152 && 2 * a->win_smem <= kAdjSmemMax;
+    const int share = pairs ? adj::kWinAdjThreads<T> / 2 : adj::kWinAdjThreads<T>;
     const int passes = (sp.N + share - 1) / share, threads = ((sp.N + passes - 1) / passes + 31) & ~31;
     NS_CUDA_TRY(launch_pdl(adj::k_windows_adj<T, NB>, dim3(grid_rows), dim3(threads),
                            a->win_smem, st, sp,

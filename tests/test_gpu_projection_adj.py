@@ -113,3 +113,12 @@ def test_fp32_gradient_variants(name, rows):
         ratio = float(((got[b] - ref[b]).abs() / bound).max())
         print(f"{name} row {b} of {rows}: error / bound = {ratio:.3f}")
         assert ratio <= 1.0
+
+
+@pytest.mark.parametrize("hidden", [(100, 72), (20, 136), (130, 1028), (64,)])
+@pytest.mark.parametrize("rows", [1, 17, 33, 65])
+def test_fp64_gradient_tiles(hidden, rows):
+    """FP64 emulator layers around the 16, 32 and 64 row tiles of the backward pass,
+    widths that are no multiple of 64 units or of a share of the contraction."""
+    inp = w.make_shear_inputs(replace(w.shear_tiny(), emu_hidden=hidden))
+    _check(inp, ShearOracle(inp), rows, (0, rows - 1))
