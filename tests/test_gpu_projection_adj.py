@@ -24,6 +24,7 @@ VARIANTS = {
     "few_nodes": dict(n_chi=14),
     "skipped_cells": dict(n_chi=41, n_z=38),
     "one_bin": dict(n_bins=1, nz_mean=(0.8,), nz_sigma=(0.2,), n_ell=33),
+    "wide_table": dict(n_k=4700, n_z=4, n_chi=14),     # table read from global memory, one warp per CTA
 }
 
 
@@ -69,7 +70,7 @@ FP32_VARIANTS = {
     "few_nodes": dict(n_chi=14),
     "skipped_cells": dict(n_chi=41, n_z=38),
     "one_bin": dict(n_bins=1, nz_mean=(0.8,), nz_sigma=(0.2,), n_ell=20),
-    "wide_table": dict(n_k=2000, n_z=4),           # table rows stay in global memory
+    "wide_table": dict(n_k=2000, n_z=4),           # 32 KB of columns per warp
     "unsorted": dict(),
 }
 
