@@ -54,9 +54,10 @@ extern "C" {
 
 /* ---- enums -------------------------------------------------------------- */
 enum ns_kind { NS_KIND_GAUSS = 0, NS_KIND_SHEAR = 1, NS_KIND_CMB = 2 };
-/* Arithmetic of the likelihood.  FP64: every stage in double.  FP32: every
- * stage in float (emulator on CUDA cores), the constant and the final log L in
- * double.  BF16: emulator hidden/output GEMMs as tcgen05 BF16 x BF16 -> FP32
+/* Arithmetic of the likelihood.  FP64: every stage in double (the GEMMs of a
+ * tanh emulator as exact sums of fixed-point fp16 slices on the tensor cores).
+ * FP32: every stage in float (GEMMs as sums of three bf16 planes per operand,
+ * FP32 accumulation), the constant and the final log L in double.  BF16: emulator hidden/output GEMMs as tcgen05 BF16 x BF16 -> FP32
  * tensor-core MMAs, all other stages FP32.  BF16_F64CHI2: as BF16 but the
  * whitening solve and chi^2 in FP64. */
 enum ns_precision { NS_PREC_FP64 = 0, NS_PREC_FP32 = 1, NS_PREC_BF16 = 2, NS_PREC_BF16_F64CHI2 = 3 };

@@ -2,8 +2,10 @@
 //
 //   prior transform   Table 1 (uniform, Gaussian via Phi^-1, fixed)
 //   emulator          MLP stand-in for CosmoPower (Sec. 2.5): input layer on
-//                     CUDA cores, hidden/output layers as GEMMs (SIMT here,
-//                     tcgen05 tensor cores for BF16 in gemm_tc.cu)
+//                     CUDA cores, hidden/output layers as tcgen05 GEMMs: BF16
+//                     (gemm_tc.cu), FP32 as three bf16 planes (gemm_planes.cu),
+//                     FP64 with tanh as six fp16 slices (gemm_slices.cu); FP64
+//                     with other activations on CUDA cores here
 //   projection.cu     App. A projection (distances, windows, P lookup, Limber,
 //                     data vector) and the whitened chi^2.
 #include <algorithm>
@@ -520,7 +522,7 @@ static int probe_end(const StageProbe* pr, int stage, cudaStream_t st) {
 // BF16: input layer on CUDA cores, hidden layers as tcgen05 GEMMs with the
 // activation in the epilogue.  The last layer: for the shear kind a tcgen05
 // GEMM with the de-standardising epilogue into the FP32 table; for the CMB
-// kind `hd` on CUDA cores in FP32 (the folded head needs FP32 weights).
+// kind `hd` with FP32 weights as three bf16 planes (gemm_planes.cu).
 static int run_emulator_bf16(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st,
                              const StageProbe* probe, const Head* hd) {
     const int L = p->n_layers;

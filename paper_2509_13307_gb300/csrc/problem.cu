@@ -566,7 +566,7 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
     for (int l = 1; l < e.n_layers; ++l) p->hidden_max = std::max(p->hidden_max, p->dims[l]);
     const bool cmb = p->kind == NS_KIND_CMB;
     // BF16 layers on tensor cores: every layer >= 1 for shear; the hidden
-    // layers only for CMB (its head runs on CUDA cores in FP32)
+    // layers only for CMB (its FP32 head takes the plane GEMMs)
     auto tc_layer = [&](int l) { return bf16 && l >= 1 && !(cmb && l == e.n_layers - 1); };
     if (bf16) {
         for (int l = 1; l < e.n_layers; ++l)
