@@ -1006,9 +1006,11 @@ static void build_split(const std::vector<int>& zrp, int N, int n_z, int W, std:
     ptr.push_back((int)idx.size());
 }
 
-// Warps per evaluation: eight keep the chip's 2432 resident warps busy from 304
-// evaluations on; fewer evaluations get shorter node ranges (64 evaluations of
-// the 39-d problem: 32 warps).
+// Warps per evaluation: with eight, 152 evaluations and more give every SM eight to
+// its limit of 28 warps; fewer evaluations get shorter node ranges (64 evaluations of
+// the 39-d problem: 32 warps, 14 per SM), at the price of four more partial rows a
+// range.  k_limber_nodes splits an evaluation's nodes over 4, 2 or 1 CTAs by the
+// same lines.
 static int limber_adj_split(int rows) { return rows <= 76 ? 2 : rows <= 152 ? 1 : 0; }
 
 int projection_adj_create(const ShearParams& sp, int elt, int cap, ProjectionAdj* a) {
