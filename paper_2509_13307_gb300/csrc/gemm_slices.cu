@@ -43,7 +43,9 @@ constexpr int SBK = 32;                          // k per slot: 64 bytes of fp16
 constexpr int W_SUB = 128 * SBK * 2;
 constexpr int STAGES = 3;
 constexpr int CHUNK = 4;                         // slots per TMEM accumulation: 128 k
-constexpr long long kNaN = 1ll << 58;            // stands for NaN in a sum (others stay below 2^50; eight of it fit)
+// Stands for NaN in a rank's sum: ordinary sums, of either sign, stay below 2^50, so a
+// total of one to eight markers and ordinary sums lies above kNaN / 2, any other below.
+constexpr long long kNaN = 1ll << 58;
 
 template <int BR>                                // rows per tile
 struct CfgL {
@@ -198,7 +200,7 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
         if (!fv || row >= M) return;
         // hi 2^-34 + lo 2^-61
         double v = fma((double)l, 4.33680868994201773603e-19, (double)h * 5.82076609134674072266e-11) * ws + bias;
-        if (h >= kNaN) v = NAN;
+        if (h >= kNaN / 2) v = NAN;
         if (e.tanh) {
             const double t = tanh(v);
             if (e.out) e.out[(size_t)row * N + f] = t;

@@ -1,0 +1,57 @@
+"""FP64 slice GEMMs (gemm_slices.cu) outside the well-behaved middle of their range."""
+
+from dataclasses import replace
+
+import numpy as np
+import pytest
+import torch
+
+import workloads as w
+from gpu_helpers import free_theta, random_cube
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(hidden, seed=0):
+    """shear_tiny with random-normal layers of the given widths (fan-in scaled)."""
+    inp = w.make_shear_inputs(replace(w.shear_tiny(), emu_hidden=hidden))
+    rng = np.random.default_rng([seed, *hidden])
+    dims = [len(inp["emu_inputs"]), *hidden, len(inp["emu_out_mu"])]
+    inp["emu_W"] = [rng.standard_normal((n, k)) / np.sqrt(k) for k, n in zip(dims[:-1], dims[1:])]
+    inp["emu_b"] = [0.1 * rng.standard_normal(n) for n in dims[1:]]
+    return inp
+
+
+def _problem(inp, rows):
+    from paper_2509_13307_gb300 import Problem
+    D = len(inp["noise_eps"])
+    return Problem(inp, "fp64", max_batch=rows, data=np.zeros(D), cov=np.eye(D))
+
+
+def _emulator(inp, full):
+    h = (full[:, inp["emu_inputs"]] - inp["emu_in_center"]) / inp["emu_in_scale"]
+    with np.errstate(invalid="ignore"):
+        for W, b in zip(inp["emu_W"][:-1], inp["emu_b"][:-1]):
+            h = np.tanh(h @ W.T + b)
+        return inp["emu_out_mu"] + inp["emu_out_sigma"] * (h @ inp["emu_W"][-1].T + inp["emu_b"][-1])
+
+
+@pytest.mark.parametrize("layer", [1, 2])
+@pytest.mark.parametrize("rows", [1, 16, 64])
+def test_nan_weight_marks_exactly_its_features(layer, rows):
+    """A NaN seen by one CTA of a cluster that splits K, beside partial sums of
+    either sign: a NaN weight of the output layer shows in its own outputs only, one
+    of a hidden layer in all of them."""
+    inp = _inputs((1024, 1024))
+    W = inp["emu_W"][layer]
+    rng = np.random.default_rng(layer)
+    if layer == 2:
+        for f in range(0, W.shape[0], 3):
+            W[f, rng.integers(W.shape[1])] = np.nan
+    else:
+        W[700, 300] = np.nan
+    p = _problem(inp, rows)
+    full = free_theta(inp, random_cube(rows, p.d, rows))
+    got = p.emulator(torch.tensor(full, device="cuda")).cpu().numpy()
+    assert p.device_status() == 0
+    assert np.array_equal(np.isnan(got), np.isnan(_emulator(inp, full)))
