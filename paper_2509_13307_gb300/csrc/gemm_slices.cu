@@ -5,16 +5,17 @@
 // its fp16 tensor rate.  An operand is therefore held in fixed point, scaled to
 // |v| <= 1 (activations of tanh as they are, a row of W by a power of two), as
 // six 9-bit slices:  v = sum_i q_i 2^-(8 + 9 i),  |q_i| <= 256 an integer, the
-// rest at most 2^-54.  Products q_i q_j and their sums over 128 k are integers
-// within FP32's 24 bits, so the tensor core adds them exactly; the 21 slice pairs
-// with i + j <= 5 are kept, one FP32 accumulator in TMEM for each sum i + j.
-// Every 128 k the epilogue warps add the six accumulators to two 64-bit integers
-// per element (in registers, while the next MMAs run in the second TMEM buffer),
-// and one FP64 expression at the end joins them.  (Pairs with i + j >= 4 could
-// leave the 24 bits if every slice of every operand were near its largest value
-// with equal signs; a unit of theirs is 2^-52.)  What is dropped is about 2^-51 of the
-// row's largest |w| for K = 1024, against 2^-48 for the rounding of an FP64 FMA
-// chain.
+// rest at most 2^-54.  Products q_i q_j are integers of at most 2^16; the 21 slice pairs
+// with i + j <= 5 are kept, one FP32 accumulator in TMEM for each sum i + j, whose
+// i + j + 1 pairs over 64 k stay within FP32's 24 bits up to i + j = 3: the tensor core
+// adds them exactly.  (Those of i + j = 4 and 5 could leave the 24 bits if every slice of
+// every operand were near its largest value with equal signs, in a total near 64; a unit of
+// theirs is 2^-52 and less.)  Every 64 k the epilogue warps add the six accumulators to two
+// 64-bit integers per element (in registers, while the next MMAs run in the second TMEM
+// buffer), and one FP64 expression at the end joins them.  What is dropped is about 2^-51 of
+// the row's largest |w| for K = 1024, against 2^-48 for the rounding of an FP64 FMA
+// chain.  The ranks of a cluster take whole groups of 64 k, so that every group is added
+// alike in every split: a row's bits do not depend on its batch.
 //
 // Tiles: 128 features (the MMA's M) x 16, 32 or 64 rows, six accumulators each
 // (twice in TMEM for up to 32 rows).  Slots of 32 k hold every slice of both
@@ -42,7 +43,7 @@ constexpr int NS = kSlices;                      // slices of an operand
 constexpr int SBK = 32;                          // k per slot: 64 bytes of fp16
 constexpr int W_SUB = 128 * SBK * 2;
 constexpr int STAGES = 3;
-constexpr int CHUNK = 4;                         // slots per TMEM accumulation: 128 k
+constexpr int CHUNK = 2;                         // slots per TMEM accumulation: 64 k
 // Stands for NaN in a rank's sum: ordinary sums, of either sign, stay below 2^50, so a
 // total of one to eight markers and ordinary sums lies above kNaN / 2, any other below.
 constexpr long long kNaN = 1ll << 58;
@@ -112,7 +113,8 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     fence_after();
     const uint32_t tmem = *tmem_slot;
     const int nk = (K + SBK - 1) / SBK;
-    const int kb0 = (int)((long long)nk * rank / S), n_it = (int)((long long)nk * (rank + 1) / S) - kb0;
+    const int nc = (nk + CHUNK - 1) / CHUNK;     // at least one for every rank (launch_gemm_slices)
+    const int kb0 = nc * rank / S * CHUNK, n_it = min(nk, nc * (rank + 1) / S * CHUNK) - kb0;
     const int n_chunk = (n_it + CHUNK - 1) / CHUNK;
 
     uint32_t nan = 0;                            // elements whose leading accumulator is NaN
@@ -297,8 +299,8 @@ static int launch_slices_t(const CUtensorMap* tmW, const CUtensorMap* tmX, const
 int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const SliceEpi& e, const int* nrows,
                        int grid_rows, int N, int K, int* err, cudaStream_t st) {
     if (grid_rows <= 0) return NS_OK;
-    // Rows per tile and K split by the cycles of the SM that ends last (sums are
-    // exact, so the choice does not change a bit).  A slot is 42 MMAs of ~65 cycles
+    // Rows per tile and K split by the cycles of the SM that ends last (every group of
+    // 64 k is added alike in each, so the choice does not change a bit).  A slot is 42 MMAs of ~65 cycles
     // each up to N = 64; the epilogue's FP64 runs at two operations per cycle (tanh
     // and slicing ~75 per element, the output 6); 64-row tiles have one set of
     // accumulators and wait for each drain; clusters of 8 (4) find room on about 96

@@ -55,3 +55,37 @@ def test_nan_weight_marks_exactly_its_features(layer, rows):
     got = p.emulator(torch.tensor(full, device="cuda")).cpu().numpy()
     assert p.device_status() == 0
     assert np.array_equal(np.isnan(got), np.isnan(_emulator(inp, full)))
+
+
+def _near_largest(rng, shape):
+    """Values whose 9-bit digits lie in 250 .. 255 in all of the first five slices."""
+    return sum(rng.integers(250, 256, shape) * 2.0 ** -(8 + 9 * i) for i in range(5))
+
+
+@pytest.mark.parametrize("width", [1024, 1000])
+def test_slices_near_their_largest_values(width):
+    """Operands with every slice near its largest value and equal signs: the sums
+    of 64 products still fit FP32's 24 bits where their unit matters, and a row's
+    bits do not depend on the batch, which chooses the split of K.
+
+    Bound, of the sum (about `width`): 2^-54 of the scale for each operand, one
+    unit in the last place of tanh, the slice pairs left out (below 2^-50 of the
+    scale in all), the roundings of the total, bias and output: under 2^-49."""
+    inp = _inputs((width,))
+    rng = np.random.default_rng(width)
+    h = _near_largest(rng, width)
+    inp["emu_W"][0][:] = 0.0
+    inp["emu_b"][0][:] = np.arctanh(h)
+    inp["emu_W"][1][:] = _near_largest(rng, inp["emu_W"][1].shape)
+    inp["emu_b"][1][:] = 0.0
+    inp["emu_out_mu"][:] = 0.0
+    p = _problem(inp, 200)
+    full = free_theta(inp, random_cube(200, p.d, 1))
+    theta = torch.tensor(full, device="cuda")
+    whole = p.emulator(theta)
+    ld = np.longdouble
+    ref = ld(inp["emu_out_sigma"]) * (np.tanh(inp["emu_b"][0]).astype(ld) @ inp["emu_W"][1].T.astype(ld))
+    err = np.abs(whole.cpu().numpy().astype(ld) / ref - 1).max()
+    assert err < 2.0 ** -49, float(err)
+    for n in (1, 16, 17, 33, 64, 100):
+        assert torch.equal(p.emulator(theta[:n]), whole[:n])
