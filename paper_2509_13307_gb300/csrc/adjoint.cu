@@ -97,12 +97,11 @@ static int back_shares(int N, int K) {
     return std::max(1, std::min((K + 63) / 64, 152 / tiles));
 }
 
-// FP64 input layer: the activations and their slices for the next layer
+// FP64 input layer
 __global__ void k_emu_in_store(const double* __restrict__ theta_full, int P, const int* __restrict__ inputs,
                                const double* __restrict__ center, const double* __restrict__ scale, int K0,
                                const double* __restrict__ W0, const double* __restrict__ b0, int N,
-                               double* __restrict__ out, __half* __restrict__ slices, int pitch, long long stride,
-                               const int* __restrict__ nrows) {
+                               double* __restrict__ out, const int* __restrict__ nrows) {
     const int row = blockIdx.y;
     if (row >= *nrows) return;
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
@@ -110,9 +109,7 @@ __global__ void k_emu_in_store(const double* __restrict__ theta_full, int P, con
     double acc = b0[n];
     for (int j = 0; j < K0; ++j)
         acc += W0[(size_t)n * K0 + j] * ((theta_full[(size_t)row * P + inputs[j]] - center[j]) / scale[j]);
-    const double h = tanh(acc);
-    out[(size_t)row * N + n] = h;
-    tc::slice_store(h, slices + (size_t)row * pitch + n, stride);
+    out[(size_t)row * N + n] = tanh(acc);
 }
 
 // The emulator inputs' share g_x = g_pre_1 W0 (rows x K0, K0 <= KMAX) added to
@@ -243,13 +240,9 @@ struct GradState {
     void* Linv = nullptr;      // D x D, L^-1 row-major in the arithmetic type
     ProjectionAdj proj;
     double* gfull = nullptr;   // cap x P
-    // FP64: stored activations per hidden layer, their slices (ping-pong), adjoints
+    // FP64: stored activations per hidden layer, the slices of one, adjoints
     // (ping-pong) and the shares of a backward contraction
-    __half* Hs[2] = {};
-    long long slice_stride = 0;
-    std::vector<SliceMapX> tmHs;
-    std::vector<CUtensorMap> tmWs;           // the problem's weight slices, or its own
-    std::vector<double*> wscale;
+    SliceInput xs;
     double* part = nullptr;
     int cap = 0;
     std::vector<double*> H;
@@ -329,33 +322,13 @@ static int grad_state_create(const ns_problem* p, GradState* g) {
         for (int l = 1; l < L; ++l)
             part = std::max(part, (size_t)adj::back_shares(p->dims[l], p->dims[l + 1]) * p->dims[l]);
         NS_TRY(grad_alloc(g, 8 * part * cap, (void**)&g->part));
-        const long long rows_pad = ((cap + 127) / 128) * 128;
-        g->slice_stride = rows_pad * plane_pitch(p->hidden_max);
-        for (int i = 0; i < 2; ++i) {
-            const size_t n = sizeof(__half) * tc::kSlices * (size_t)g->slice_stride;
-            NS_TRY(grad_alloc(g, n, (void**)&g->Hs[i]));
-            NS_CUDA_TRY(cudaMemsetAsync(g->Hs[i], 0, n, nullptr));
+        if (!p->tmWs.empty()) {
+            const size_t n = slice_input_bytes(p, cap);
+            NS_TRY(grad_alloc(g, n, (void**)&g->xs.slices));
+            NS_CUDA_TRY(cudaMemsetAsync(g->xs.slices, 0, n, nullptr));
+            NS_TRY(grad_alloc(g, sizeof(double) * cap, (void**)&g->xs.scale));
+            NS_TRY(slice_input_maps(p, cap, &g->xs));
         }
-        g->tmWs = p->tmWs;
-        g->wscale = p->d_wscale;
-        if (g->tmWs.empty()) {               // a problem whose likelihood takes no slices
-            g->tmWs.resize(L);
-            g->wscale.assign(L, nullptr);
-            for (int l = 1; l < L; ++l) {
-                const int N = p->dims[l + 1], K = p->dims[l], pitch = plane_pitch(K);
-                void* v;
-                NS_TRY(grad_alloc(g, sizeof(__half) * tc::kSlices * (size_t)N * pitch, &v));
-                NS_TRY(grad_alloc(g, sizeof(double) * N, (void**)&g->wscale[l]));
-                NS_TRY(launch_slice_rows((const double*)p->d_W[l], N, K, (__half*)v, (long long)N * pitch, pitch,
-                                         g->wscale[l], nullptr));
-                NS_TRY(make_tensor_map_slices(&g->tmWs[l], v, N, K, (long long)N * pitch, 128));
-            }
-        }
-        g->tmHs.resize(L);
-        for (int l = 1; l < L; ++l)
-            for (int i = 0; i < 3; ++i)
-                NS_TRY(make_tensor_map_slices(&g->tmHs[l].m[i], g->Hs[(l - 1) & 1], (int)rows_pad, p->dims[l],
-                                              g->slice_stride, 16 << i));
         NS_CUDA_TRY(cudaStreamSynchronize(nullptr));   // calls may come on any stream
         return NS_OK;
     }
@@ -418,27 +391,11 @@ static int run_grad_f64(const ns_problem* p, GradState* g, int B, OutPtr logL, O
     const dim3 g0((p->dims[1] + 255) / 256, B);
     adj::k_emu_in_store<<<g0, 256, 0, st>>>(g->theta_full, p->P, p->d_inputs, p->d_in_center, p->d_in_scale,
                                             p->dims[0], (const double*)p->d_W[0], (const double*)p->d_b[0],
-                                            p->dims[1], g->H[1], g->Hs[0], plane_pitch(p->dims[1]), g->slice_stride,
-                                            g->d_nrows);
+                                            p->dims[1], g->H[1], g->d_nrows);
     NS_CUDA_TRY(cudaGetLastError());
-    for (int l = 1; l < L; ++l) {
-        const bool last = (l == L - 1);
-        SliceEpi e;
-        e.bias = (const double*)p->d_b[l];
-        e.wscale = g->wscale[l];
-        if (last) {
-            e.mu = (const double*)p->d_out_mu;
-            e.sigma = p->out_sigma;
-            e.out = (double*)g->table;
-        } else {
-            e.tanh = 1;
-            e.out = g->H[l + 1];
-            e.slices = g->Hs[l & 1];
-            e.slice_stride = g->slice_stride;
-            e.pitch = plane_pitch(p->dims[l + 1]);
-        }
-        NS_TRY(launch_gemm_slices(&g->tmWs[l], &g->tmHs[l], e, g->d_nrows, B, p->dims[l + 1], p->dims[l], g->d_err, st));
-    }
+    for (int l = 1; l < L; ++l)
+        NS_TRY(launch_layer_f64(p, l, g->xs, g->H[l], l == L - 1 ? (double*)g->table : g->H[l + 1], g->d_nrows, B,
+                                g->d_err, st));
     const double* tab = (const double*)g->table;
     const bool coarse = p->n_z_emu != sp.n_z;
     if (coarse) {

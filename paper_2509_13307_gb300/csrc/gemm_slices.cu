@@ -1,23 +1,29 @@
 // FP64 GEMMs on the fp16 tensor path (tcgen05), for the layers of FP64 tanh
-// emulators:  out[r][f] = epi( sum_k X[r][k] W[f][k] ),  |X| <= 1.
+// emulators:  out[r][f] = epi( sum_k X[r][k] W[f][k] ).
 //
 // GB300 runs FP64 at two FMAs per cycle and SM (1.26 TFLOP/s), a thousandth of
-// its fp16 tensor rate.  An operand is therefore held in fixed point, scaled to
-// |v| <= 1 (activations of tanh as they are, a row of W by a power of two), as
+// its fp16 tensor rate.  An operand is therefore held in fixed point, every row of W and
+// every row of activations scaled to |v| <= 1 by a power of two of its own, as
 // six 9-bit slices:  v = sum_i q_i 2^-(8 + 9 i),  |q_i| <= 256 an integer, the
-// rest at most 2^-54.  Products q_i q_j are integers of at most 2^16; the 21 slice pairs
-// with i + j <= 5 are kept, one FP32 accumulator in TMEM for each sum i + j, whose
+// rest at most 2^-54.  Products q_i q_j are integers of at most 2^16; the 26 slice pairs
+// with i + j <= 6 are kept, one FP32 accumulator in TMEM for each sum i + j, whose
 // i + j + 1 pairs over 64 k stay within FP32's 24 bits up to i + j = 3: the tensor core
-// adds them exactly.  (Those of i + j = 4 and 5 could leave the 24 bits if every slice of
+// adds them exactly.  (Those of i + j = 4, 5 and 6 could leave the 24 bits if every slice of
 // every operand were near its largest value with equal signs, in a total near 64; a unit of
-// theirs is 2^-52 and less.)  Every 64 k the epilogue warps add the six accumulators to two
+// theirs is 2^-52 and less.)  Every 64 k the epilogue warps add the seven accumulators to two
 // 64-bit integers per element (in registers, while the next MMAs run in the second TMEM
-// buffer), and one FP64 expression at the end joins them.  What is dropped is about 2^-51 of
-// the row's largest |w| for K = 1024, against 2^-48 for the rounding of an FP64 FMA
-// chain.  The ranks of a cluster take whole groups of 64 k, so that every group is added
+// buffer), and one FP64 expression at the end joins them.
+//
+// Error, of sum |w| |h|, in an emulation of the digits (rms, normal weights): K = 1024,
+// activations of order 1 6.9e-18, of order 1e-3 or 1e-6 1.1e-17, spread over four decades
+// 1.5e-17; K = 64 2.6e-17, 3.9e-17, 5.5e-17; an FP64 FMA chain 4.7e-17 to 8.9e-17 throughout.  Without
+// the activations' scale order 1e-6 gave 7.7e-12; without the pairs of i + j = 6 (2^-54 of the
+// scale each) K = 64 1.5e-16 where the chain has 5.5e-17.
+//
+// The ranks of a cluster take whole groups of 64 k, so that every group is added
 // alike in every split: a row's bits do not depend on its batch.
 //
-// Tiles: 128 features (the MMA's M) x 16, 32 or 64 rows, six accumulators each
+// Tiles: 128 features (the MMA's M) x 16, 32 or 64 rows, seven accumulators each
 // (twice in TMEM for up to 32 rows).  Slots of 32 k hold every slice of both
 // operands (60 KB for 32 rows, 64-byte swizzle, three slots).  Few tiles are spread over clusters of S CTAs along k,
 // whose integer partial tiles are added exactly through cluster shared memory.
@@ -40,6 +46,7 @@ namespace slc {
 using namespace tc;
 
 constexpr int NS = kSlices;                      // slices of an operand
+constexpr int NSUM = NS + 1;                     // sums i + j kept
 constexpr int SBK = 32;                          // k per slot: 64 bytes of fp16
 constexpr int W_SUB = 128 * SBK * 2;
 constexpr int STAGES = 3;
@@ -58,7 +65,7 @@ struct CfgL {
     static constexpr int EPI_WARPS = BR == 64 ? 16 : 8, THREADS = 32 * (EPI_WARPS + 2);
     static constexpr int HC = BR / (EPI_WARPS / 4);  // rows per epilogue warp
     static_assert(STAGES * STAGE_BYTES >= 128 * BR * 16, "the partial tile reuses the ring");
-    static_assert(NBUF * NS * BR <= (int)TMEM_COLS, "accumulators in TMEM");
+    static_assert(NBUF * NSUM * BR <= (int)TMEM_COLS, "accumulators in TMEM");
 };
 
 // K-major tile of 64-byte rows, 64-byte swizzle (8-row groups of 512 bytes).
@@ -118,7 +125,7 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     const int n_chunk = (n_it + CHUNK - 1) / CHUNK;
 
     uint32_t nan = 0;                            // elements whose leading accumulator is NaN
-    long long hi[HC], lo[HC];                    // sums of i + j = 0..2 and 3..5, in units of the last of each
+    long long hi[HC], lo[HC];                    // sums of i + j = 0..2 and 3..6, in units of the last of each
 #pragma unroll
     for (int j = 0; j < HC; ++j) { hi[j] = 0; lo[j] = 0; }
     if (warp == W_LOAD) {
@@ -151,12 +158,12 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
 #pragma unroll
                 for (int i = 0; i < NS; ++i)
 #pragma unroll
-                    for (int j = 0; i + j < NS; ++j) {
+                    for (int j = 0; j < NS && i + j < NSUM; ++j) {
                         const uint64_t dw = desc64(sw + i * W_SUB), dx = desc64(sx + j * X_SUB);
 #pragma unroll
                         for (int kk = 0; kk < SBK / 16; ++kk)
-                            mma_bf16(tmem + (uint32_t)((b * NS + i + j) * BR), dw + 2 * kk, dx + 2 * kk, kIdesc<BR>,
-                                     in != 0 || i != 0 || kk != 0);
+                            mma_bf16(tmem + (uint32_t)((b * NSUM + i + j) * BR), dw + 2 * kk, dx + 2 * kk, kIdesc<BR>,
+                                     in != 0 || !(i == 0 || j == NS - 1) || kk != 0);
                     }
                 mma_commit(empty_bar(s));
                 if (in == CHUNK - 1 || it == n_it - 1) mma_commit(acc_full(b));
@@ -171,14 +178,14 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
             fence_after();
             __syncwarp();
 #pragma unroll
-            for (int s = 0; s < NS; ++s) {
+            for (int s = 0; s < NSUM; ++s) {
                 float v[HC];
-                tmem_ld<HC>(addr + (uint32_t)((b * NS + s) * BR), v);
+                tmem_ld<HC>(addr + (uint32_t)((b * NSUM + s) * BR), v);
                 if (s == 0) {
 #pragma unroll
                     for (int j = 0; j < HC; ++j) nan |= (uint32_t)(v[j] != v[j]) << j;
                 }
-                const long long unit = 1ll << (9 * (s < 3 ? 2 - s : 5 - s));
+                const long long unit = 1ll << (9 * (s < 3 ? 2 - s : NSUM - 1 - s));
 #pragma unroll
                 for (int j = 0; j < HC; ++j) (s < 3 ? hi[j] : lo[j]) += (long long)__float2int_rn(v[j]) * unit;
             }
@@ -200,16 +207,9 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     auto finish = [&](int rl, long long h, long long l) {
         const int row = r0 + rl;
         if (!fv || row >= M) return;
-        // hi 2^-34 + lo 2^-61
-        double v = fma((double)l, 4.33680868994201773603e-19, (double)h * 5.82076609134674072266e-11) * ws + bias;
+        double v = fma((double)l, 0x1p-70, (double)h * 0x1p-34) * ws * e.xscale[row] + bias;
         if (h >= kNaN / 2) v = NAN;
-        if (e.tanh) {
-            const double t = tanh(v);
-            if (e.out) e.out[(size_t)row * N + f] = t;
-            slice_store(t, e.slices + (size_t)row * e.pitch + f, e.slice_stride);
-        } else {
-            e.out[(size_t)row * N + f] = mu + e.sigma * v;
-        }
+        e.out[(size_t)row * N + f] = e.tanh ? tanh(v) : mu + e.sigma * v;
     };
     __syncthreads();                             // the ring's last copies have landed
     const bool failed = s_fail != 0;
@@ -249,9 +249,14 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
     }
 }
 
-// slices and power-of-two scale of every row of W (rows x K)
+// Slices and power-of-two scale of every row of a matrix (rows x K): the weights once, the
+// activations before each layer (64 rows of 1024: beside the windows, off the call's
+// longest path).
 __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ W, int K, __half* __restrict__ out,
-                                                    long long stride, int pitch, double* __restrict__ scale) {
+                                                    long long stride, int pitch, double* __restrict__ scale,
+                                                    const int* __restrict__ nrows) {
+    pdl_begin();
+    if (nrows && (int)blockIdx.x >= *nrows) return;
     __shared__ double red[8];
     const double* w = W + (size_t)blockIdx.x * K;
     double m = 0;
@@ -260,8 +265,10 @@ __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ W
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
     __syncthreads();
     for (int i = 0; i < 8; ++i) m = fmax(m, red[i]);
+    // the least power of two that is no smaller than the row's largest |v|
     int ex = 0;
-    if (m > 0) frexp(m, &ex);
+    if (m > 0 && frexp(m, &ex) == 0.5) --ex;
+    ex = max(ex, -900);                          // 1 / scale stays finite
     const double s = scalbn(1.0, -ex);
     for (int k = threadIdx.x; k < K; k += 256) slice_store(w[k] * s, out + (size_t)blockIdx.x * pitch + k, stride);
     if (threadIdx.x == 0) scale[blockIdx.x] = scalbn(1.0, ex);
@@ -300,9 +307,9 @@ int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const Slice
                        int grid_rows, int N, int K, int* err, cudaStream_t st) {
     if (grid_rows <= 0) return NS_OK;
     // Rows per tile and K split by the cycles of the SM that ends last (every group of
-    // 64 k is added alike in each, so the choice does not change a bit).  A slot is 42 MMAs of ~65 cycles
+    // 64 k is added alike in each, so the choice does not change a bit).  A slot is 52 MMAs of ~65 cycles
     // each up to N = 64; the epilogue's FP64 runs at two operations per cycle (tanh
-    // and slicing ~75 per element, the output 6); 64-row tiles have one set of
+    // ~75 per element, the output 6); 64-row tiles have one set of
     // accumulators and wait for each drain; clusters of 8 (4) find room on about 96
     // (128) SMs.  64 rows: 64-row output tiles 1 wave of 79 CTAs against two of 158
     // (111 us); 16-row hidden tiles spread the FP64 of tanh over 128 SMs.
@@ -315,7 +322,7 @@ int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const Slice
             const int sms = s == 8 ? 96 : s == 4 ? 128 : 152, slots = (nk + s - 1) / s;
             const long long ctas = (long long)mt * ((grid_rows + br - 1) / br) * s;
             const double t = (double)((ctas + sms - 1) / sms) *
-                             (3000.0 + 2750.0 * slots + (br == 64 ? 3000.0 * (slots / slc::CHUNK) : 0.0) +
+                             (3000.0 + 3400.0 * slots + (br == 64 ? 3000.0 * (slots / slc::CHUNK) : 0.0) +
                               64.0 * br / s * (e.tanh ? 75 : 6) + (s > 1 ? 2500.0 : 0.0));
             if (t < 0.97 * best) { best = t; best_br = br; best_s = s; }
         }
@@ -326,10 +333,9 @@ int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const Slice
     }
 }
 
-int launch_slice_rows(const double* W, int rows, int K, __half* out, long long stride, int pitch, double* scale,
-                      cudaStream_t st) {
-    slc::k_slice_rows<<<rows, 256, 0, st>>>(W, K, out, stride, pitch, scale);
-    NS_CUDA_TRY(cudaGetLastError());
+int launch_slice_rows(const double* in, int rows, int K, __half* out, long long stride, int pitch, double* scale,
+                      const int* nrows, cudaStream_t st) {
+    NS_CUDA_TRY(launch_pdl(slc::k_slice_rows, dim3(rows), dim3(256), 0, st, in, K, out, stride, pitch, scale, nrows));
     return NS_OK;
 }
 

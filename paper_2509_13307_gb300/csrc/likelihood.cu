@@ -125,14 +125,6 @@ struct OutF64 {
     double* p;
     __device__ __forceinline__ void put(int row, int n, int N, double v) const { p[(size_t)row * N + n] = v; }
 };
-struct OutSlices {
-    __half* p;
-    long long stride;
-    int pitch;
-    __device__ __forceinline__ void put(int row, int n, int, double v) const {
-        tc::slice_store(v, p + (size_t)row * pitch + n, stride);
-    }
-};
 struct OutBf16 {
     __nv_bfloat16* p;
     __device__ __forceinline__ void put(int row, int n, int N, float v) const {
@@ -415,45 +407,56 @@ static Head model_head(const ns_problem* p, void* out) {
                 p->out_sigma, out};
 }
 
-// FP64 with tanh hidden layers: fixed-point slices on the tensor cores.
-static int run_emulator_slices(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, double* out) {
-    const int L = p->n_layers;
-    NS_TRY(launch_emu_input<double>(p, ws->theta_full, ws->d_nrows, grid_rows, layer_act<double>(p, 0),
-                                    OutSlices{(__half*)ws->act[0], ws->plane_stride, plane_pitch(p->dims[1])}, st));
-    int cur = 0;
-    for (int l = 1; l < L; ++l) {
-        const bool last = l == L - 1;
-        SliceEpi e;
-        e.bias = (const double*)p->d_b[l];
-        e.wscale = p->d_wscale[l];
-        if (last) {
-            e.mu = (const double*)p->d_out_mu;
-            e.sigma = p->out_sigma;
-            e.out = out;
-        } else {
-            e.tanh = 1;
-            e.slices = (__half*)ws->act[cur ^ 1];
-            e.slice_stride = ws->plane_stride;
-            e.pitch = plane_pitch(p->dims[l + 1]);
-        }
-        NS_TRY(launch_gemm_slices(&p->tmWs[l], &ws->tmXs[l], e, ws->d_nrows, grid_rows, p->dims[l + 1], p->dims[l],
-                                  ws->d_err, st));
-        cur ^= 1;
-    }
+size_t slice_input_bytes(const ns_problem* p, int cap) {
+    const size_t rows_pad = ((size_t)cap + 127) / 128 * 128;
+    return sizeof(__half) * tc::kSlices * rows_pad * plane_pitch(p->hidden_max);
+}
+
+int slice_input_maps(const ns_problem* p, int cap, SliceInput* x) {
+    const int rows_pad = ((cap + 127) / 128) * 128;
+    x->stride = (long long)rows_pad * plane_pitch(p->hidden_max);
+    x->tm.resize(p->n_layers);
+    for (int l = 1; l < p->n_layers; ++l)
+        for (int i = 0; i < 3; ++i)
+            NS_TRY(make_tensor_map_slices(&x->tm[l].m[i], x->slices, rows_pad, p->dims[l], x->stride, 16 << i));
     return NS_OK;
 }
 
-// FP64 on CUDA cores: emulators with unbounded activations (CMB).
+int launch_layer_f64(const ns_problem* p, int l, const SliceInput& xs, const double* x, double* out, const int* nrows,
+                     int grid_rows, int* err, cudaStream_t st) {
+    const bool last = l == p->n_layers - 1;
+    const int K = p->dims[l], N = p->dims[l + 1];
+    const double *mu = last ? (const double*)p->d_out_mu : nullptr, sigma = last ? p->out_sigma : 0.0;
+    if (p->tmWs.empty())
+        return launch_gemm_simt(x, (const double*)p->d_W[l], (const double*)p->d_b[l],
+                                ActDev<double>{NS_ACT_TANH, nullptr, nullptr}, mu, nullptr, sigma, out, nrows, grid_rows,
+                                N, K, last ? EPI_OUT : EPI_ACT, st);
+    NS_TRY(launch_slice_rows(x, grid_rows, K, xs.slices, xs.stride, plane_pitch(K), xs.scale, nrows, st));
+    SliceEpi e;
+    e.tanh = !last;
+    e.bias = (const double*)p->d_b[l];
+    e.wscale = p->d_wscale[l];
+    e.xscale = xs.scale;
+    e.mu = mu;
+    e.sigma = sigma;
+    e.out = out;
+    return launch_gemm_slices(&p->tmWs[l], &xs.tm[l], e, nrows, grid_rows, N, K, err, st);
+}
+
+// FP64: tanh emulators on the tensor cores, others (CMB: unbounded activations, folded
+// heads) on CUDA cores.
 static int run_emulator_f64(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, const Head& hd) {
     const int L = p->n_layers;
-    if (!p->tmWs.empty()) return run_emulator_slices(p, ws, grid_rows, st, (double*)hd.out);
     NS_TRY(launch_emu_input<double>(p, ws->theta_full, ws->d_nrows, grid_rows, layer_act<double>(p, 0),
                                     OutF64{(double*)ws->act[0]}, st));
     int cur = 0;
     for (int l = 1; l < L; ++l) {
         const int K = p->dims[l], N = p->dims[l + 1];
         const double* x = (const double*)ws->act[cur];
-        if (l == L - 1) {
+        if (!p->tmWs.empty()) {
+            NS_TRY(launch_layer_f64(p, l, ws->xs, x, l == L - 1 ? (double*)hd.out : (double*)ws->act[cur ^ 1],
+                                    ws->d_nrows, grid_rows, ws->d_err, st));
+        } else if (l == L - 1) {
             NS_TRY(launch_gemm_simt(x, (const double*)hd.W, (const double*)hd.bias, ActDev<double>{0, nullptr, nullptr},
                                     (const double*)hd.mu, (const double*)hd.sig_vec, hd.sigma, (double*)hd.out,
                                     ws->d_nrows, grid_rows, hd.n_out ? hd.n_out : N, K, EPI_OUT, st));

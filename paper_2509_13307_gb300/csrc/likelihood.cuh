@@ -63,6 +63,14 @@ struct SliceMapX {
     CUtensorMap m[3];
 };
 
+// A layer's input as fixed-point slices (gemm_slices.cu): one buffer for all layers.
+struct SliceInput {
+    __half* slices = nullptr;        // kSlices x rows_pad x plane_pitch(hidden_max)
+    long long stride = 0;            // elements between slices
+    double* scale = nullptr;         // per row
+    std::vector<SliceMapX> tm;       // per layer >= 1
+};
+
 struct Workspace {
     int cap = 0;
     int* d_nrows = nullptr;       // device row count used by every stage
@@ -78,10 +86,10 @@ struct Workspace {
     double* logL = nullptr;       // cap
     // tcgen05 tensor maps (BF16 precision): A operand of layer l >= 1 and its output
     std::vector<CUtensorMap> tmA;
-    std::vector<SliceMapX> tmXs;   // FP64 tanh emulators: layer l's input slices (plane_stride apart)
+    SliceInput xs;                 // FP64 tanh emulators
     // k_gemm_planes: layer l's input planes (FP32: three; the FP32 head of a BF16 CMB problem: one)
     std::vector<PlaneMapX> tmXp;
-    long long plane_stride = 0;   // FP32, FP64 slices: elements between the planes of an activation buffer
+    long long plane_stride = 0;   // FP32: elements between the planes of an activation buffer
     CUtensorMap tmX_out{};        // the last layer's activations in kSwapRows-row boxes
     CUtensorMap tmF_out{};        // fused emulator stack: its output activations in 64-row boxes of two k-blocks
     std::vector<void*> owned;
@@ -310,23 +318,27 @@ inline int plane_pitch(int K) { return (K + 7) & ~7; }   // rows of 16-byte mult
 int make_tensor_map_planes(CUtensorMap* tm, const void* base, int rows, int K, long long stride, int planes,
                            int box_rows);
 int make_plane_maps_x(PlaneMapX* m, const void* base, int rows, int K, long long stride, int planes);
-// FP64 GEMMs on the fp16 tensor path (gemm_slices.cu): operands |v| <= 1 as six
-// fixed-point slices.  tanh: slices of tanh(acc + bias); else out = mu + sigma (acc + bias).
+// FP64 GEMMs on the fp16 tensor path (gemm_slices.cu): rows of both operands as six
+// fixed-point slices and a scale.  out (rows x N) = tanh(acc + bias), else mu + sigma (acc + bias).
 struct SliceEpi {
     int tanh = 0;
     const double* bias = nullptr;
     const double* wscale = nullptr;   // per feature: the power of two taken out of the row of W
+    const double* xscale = nullptr;   // per row of X
     const double* mu = nullptr;
     double sigma = 0;
-    double* out = nullptr;            // rows x N (tanh: the activations in FP64, if wanted)
-    __half* slices = nullptr;         // row pitch `pitch`
-    long long slice_stride = 0;
-    int pitch = 0;
+    double* out = nullptr;
 };
 int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const SliceEpi& e, const int* nrows,
                        int grid_rows, int N, int K, int* err, cudaStream_t st);
-int launch_slice_rows(const double* W, int rows, int K, __half* out, long long stride, int pitch, double* scale,
-                      cudaStream_t st);
+int launch_slice_rows(const double* in, int rows, int K, __half* out, long long stride, int pitch, double* scale,
+                      const int* nrows, cudaStream_t st);
+size_t slice_input_bytes(const ns_problem* p, int cap);
+int slice_input_maps(const ns_problem* p, int cap, SliceInput* x);   // slices and scale are set
+// Layer l >= 1 of a tanh emulator in FP64, x (rows x dims[l]) -> out (rows x dims[l + 1]):
+// slices on the tensor cores where the problem has them, FP64 FMAs else.
+int launch_layer_f64(const ns_problem* p, int l, const SliceInput& xs, const double* x, double* out, const int* nrows,
+                     int grid_rows, int* err, cudaStream_t st);
 int make_tensor_map_slices(CUtensorMap* tm, const void* base, int rows, int K, long long stride, int box_rows);
 // Dense FP64 set-up kernels (dense_linalg.cu): C (device, overwritten by L) ->
 // L^-1 (new device buffer) and sum ln L_aa; NS_EINVAL if C is not SPD.

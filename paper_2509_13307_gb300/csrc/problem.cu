@@ -98,12 +98,16 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
     c.want(&ws->logL, sizeof(double) * (size_t)cap);
     const bool gauss = p->kind == NS_KIND_GAUSS, cmb = p->kind == NS_KIND_CMB;
     const bool f64 = p->precision == NS_PREC_FP64, slices = !p->tmWs.empty();
-    // activations: FP64 (tanh: six fp16 slices), bf16, or FP32 as three bf16 planes
-    const int elt = slices ? 12 : f64 ? 8 : (p->precision == NS_PREC_FP32 ? 6 : 2), tab_elt = f64 ? 8 : 4;
+    // activations: FP64, bf16, or FP32 as three bf16 planes
+    const int elt = f64 ? 8 : (p->precision == NS_PREC_FP32 ? 6 : 2), tab_elt = f64 ? 8 : 4;
     const int rows_pad = ((cap + 127) / 128) * 128;
     const size_t act_bytes = (size_t)elt * rows_pad * plane_pitch(p->hidden_max);
     if (!gauss)
         for (int i = 0; i < 2; ++i) c.want(&ws->act[i], act_bytes);
+    if (slices) {
+        c.want(&ws->xs.slices, slice_input_bytes(p, cap));
+        c.want(&ws->xs.scale, sizeof(double) * (size_t)cap);
+    }
     if (cmb) {
         c.want(&ws->table, (size_t)tab_elt * cap * std::max(p->D, p->dims.back()));
         if (p->cmb_solve == NS_SOLVE_LITERAL && p->cmb_form == NS_CMB_GAUSS)
@@ -121,12 +125,8 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
     if (gauss) return NS_OK;
     for (int i = 0; i < 2; ++i) NS_CUDA_TRY(cudaMemset(ws->act[i], 0, act_bytes));
     if (slices) {
-        ws->plane_stride = (long long)rows_pad * plane_pitch(p->hidden_max);
-        ws->tmXs.resize(p->n_layers);
-        for (int l = 1; l < p->n_layers; ++l)
-            for (int i = 0; i < 3; ++i)
-                NS_TRY(make_tensor_map_slices(&ws->tmXs[l].m[i], ws->act[(l - 1) & 1], rows_pad, p->dims[l],
-                                              ws->plane_stride, 16 << i));
+        NS_CUDA_TRY(cudaMemset(ws->xs.slices, 0, slice_input_bytes(p, cap)));
+        NS_TRY(slice_input_maps(p, cap, &ws->xs));
     }
     if (p->precision == NS_PREC_FP32) {
         ws->plane_stride = (long long)rows_pad * plane_pitch(p->hidden_max);
@@ -596,7 +596,8 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
                 void *v, *sc;
                 if ((s = dalloc(sizeof(uint16_t) * 6 * (size_t)stride, &v, p->owned)) ||
                     (s = dalloc(sizeof(double) * N, &sc, p->owned)) ||
-                    (s = launch_slice_rows(w, N, K, (__half*)v, stride, pitch, (double*)sc, nullptr)))
+                    (s = launch_slice_rows(w, N, K, (__half*)v, stride, pitch, (double*)sc, nullptr,
+                                           nullptr)))
                     return fail(s);
                 p->tmWs.resize(e.n_layers);
                 p->d_wscale.resize(e.n_layers);

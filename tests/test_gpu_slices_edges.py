@@ -89,3 +89,32 @@ def test_slices_near_their_largest_values(width):
     assert err < 2.0 ** -49, float(err)
     for n in (1, 16, 17, 33, 64, 100):
         assert torch.equal(p.emulator(theta[:n]), whole[:n])
+
+
+@pytest.mark.parametrize("width", [1024, 200])
+@pytest.mark.parametrize("order", [1.0, 1e-3, 1e-6])
+def test_small_activations_keep_fp64(width, order):
+    """An output layer fed by activations of a given order: rows are scaled by their
+    own power of two, so small activations keep their bits.
+
+    Bound 2^-51 of sum |w| |h|: the digits' own error is below 2^-54 of it (K >= 200,
+    normal weights and activations), tanh and the seven-term input sums of both sides
+    2^-52 of each h (h's rms times 2^-52 sqrt(K) in the sum), the output 2^-53.  FP64 FMA
+    chains stay near 2^-52; digits held against 1 were off by 2^-41 at order 1e-6."""
+    inp = _inputs((width,))
+    inp["emu_W"][0] *= order
+    inp["emu_b"][0] *= order
+    inp["emu_b"][1][:] = 0.0
+    inp["emu_out_mu"][:] = 0.0
+    rows = 40
+    p = _problem(inp, rows)
+    full = free_theta(inp, random_cube(rows, p.d, 3))
+    got = p.emulator(torch.tensor(full, device="cuda")).cpu().numpy()
+    ld = np.longdouble
+    x = (full[:, inp["emu_inputs"]].astype(ld) - inp["emu_in_center"]) / inp["emu_in_scale"]
+    h = np.tanh(x @ inp["emu_W"][0].T.astype(ld) + inp["emu_b"][0])
+    W = inp["emu_W"][1].astype(ld)
+    ref, mag = inp["emu_out_sigma"] * (h @ W.T), inp["emu_out_sigma"] * (np.abs(h) @ np.abs(W).T)
+    err = float(np.max(np.abs(got - ref) / mag))
+    print(f"width {width}, order {order}: {err:.2e}")
+    assert err < 2.0 ** -51
