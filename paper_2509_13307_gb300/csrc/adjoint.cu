@@ -322,7 +322,7 @@ static int grad_state_create(const ns_problem* p, GradState* g) {
         for (int l = 1; l < L; ++l)
             part = std::max(part, (size_t)adj::back_shares(p->dims[l], p->dims[l + 1]) * p->dims[l]);
         NS_TRY(grad_alloc(g, 8 * part * cap, (void**)&g->part));
-        if (!p->tmWs.empty()) {
+        if (takes_slices(p)) {
             const size_t n = slice_input_bytes(p, cap);
             NS_TRY(grad_alloc(g, n, (void**)&g->xs.slices));
             NS_CUDA_TRY(cudaMemsetAsync(g->xs.slices, 0, n, nullptr));

@@ -20,6 +20,8 @@
 // the activations' scale order 1e-6 gave 7.7e-12; without the pairs of i + j = 6 (2^-54 of the
 // scale each) K = 64 1.5e-16 where the chain has 5.5e-17.
 //
+// Layers whose weights do not suit that (k_unfit_rows) keep the FP64 FMA kernel.
+//
 // The ranks of a cluster take whole groups of 64 k, so that every group is added
 // alike in every split: a row's bits do not depend on its batch.
 //
@@ -274,6 +276,31 @@ __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ W
     if (threadIdx.x == 0) scale[blockIdx.x] = scalbn(1.0, ex);
 }
 
+// Whether a row's largest |w| is infinite, beyond the exponents that the scales are made
+// for, or more than sqrt(K) / 2 times the row's mean |w|.  The digits' error is near
+// 0.45 max |w| / mean |w| max |h| / mean |h| / sqrt(K) of an FMA chain's (emulated for K = 64
+// to 2048), so that with the activations of a normal distribution, max |h| near 4 mean |h|, it
+// stays below the chain's up to here; a weight of 10^6 times the others against a tiny
+// activation made it 10^5 times as large.  Normal weights reach 4 to 5 times their mean: K of
+// some hundred and more takes the slices.  A NaN does not count: it marks its sums.
+__global__ void __launch_bounds__(256) k_unfit_rows(const double* __restrict__ W, int K, int* __restrict__ unfit) {
+    __shared__ double red[2][8];
+    const double* w = W + (size_t)blockIdx.x * K;
+    double m = 0, s = 0;
+    for (int k = threadIdx.x; k < K; k += 256) {
+        const double a = fmax(0.0, fabs(w[k]));
+        m = fmax(m, a);
+        s += a;
+    }
+    m = warp_max(m);
+    s = warp_sum(s);
+    if ((threadIdx.x & 31) == 0) { red[0][threadIdx.x >> 5] = m; red[1][threadIdx.x >> 5] = s; }
+    __syncthreads();
+    if (threadIdx.x) return;
+    for (int i = 1; i < 8; ++i) { m = fmax(m, red[0][i]); s += red[1][i]; }
+    if (m > 0 && !(m > 0x1p-400 && m < 0x1p400 && m * sqrt((double)K) <= 0.5 * s)) atomicOr(unfit, 1);
+}
+
 }  // namespace slc
 
 template <int BR>
@@ -331,6 +358,18 @@ int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const Slice
         case 32: return launch_slices_t<32>(tmW, &tmX->m[1], e, nrows, grid_rows, N, K, best_s, err, st);
         default: return launch_slices_t<64>(tmW, &tmX->m[2], e, nrows, grid_rows, N, K, best_s, err, st);
     }
+}
+
+int slices_fit(const double* W, int rows, int K, int* d_flag, bool* fit) {
+    int unfit = K > 65536;                       // 64-bit sums hold K < 2^17
+    if (!unfit) {
+        NS_CUDA_TRY(cudaMemset(d_flag, 0, sizeof(int)));
+        slc::k_unfit_rows<<<rows, 256>>>(W, K, d_flag);
+        NS_CUDA_TRY(cudaGetLastError());
+        NS_CUDA_TRY(cudaMemcpy(&unfit, d_flag, sizeof(int), cudaMemcpyDeviceToHost));
+    }
+    *fit = !unfit;
+    return NS_OK;
 }
 
 int launch_slice_rows(const double* in, int rows, int K, __half* out, long long stride, int pitch, double* scale,

@@ -407,6 +407,10 @@ static Head model_head(const ns_problem* p, void* out) {
                 p->out_sigma, out};
 }
 
+bool takes_slices(const ns_problem* p) {
+    return std::any_of(p->d_wscale.begin(), p->d_wscale.end(), [](const double* s) { return s != nullptr; });
+}
+
 size_t slice_input_bytes(const ns_problem* p, int cap) {
     const size_t rows_pad = ((size_t)cap + 127) / 128 * 128;
     return sizeof(__half) * tc::kSlices * rows_pad * plane_pitch(p->hidden_max);
@@ -427,7 +431,7 @@ int launch_layer_f64(const ns_problem* p, int l, const SliceInput& xs, const dou
     const bool last = l == p->n_layers - 1;
     const int K = p->dims[l], N = p->dims[l + 1];
     const double *mu = last ? (const double*)p->d_out_mu : nullptr, sigma = last ? p->out_sigma : 0.0;
-    if (p->tmWs.empty())
+    if (l >= (int)p->d_wscale.size() || !p->d_wscale[l])
         return launch_gemm_simt(x, (const double*)p->d_W[l], (const double*)p->d_b[l],
                                 ActDev<double>{NS_ACT_TANH, nullptr, nullptr}, mu, nullptr, sigma, out, nrows, grid_rows,
                                 N, K, last ? EPI_OUT : EPI_ACT, st);
@@ -443,7 +447,7 @@ int launch_layer_f64(const ns_problem* p, int l, const SliceInput& xs, const dou
     return launch_gemm_slices(&p->tmWs[l], &xs.tm[l], e, nrows, grid_rows, N, K, err, st);
 }
 
-// FP64: tanh emulators on the tensor cores, others (CMB: unbounded activations, folded
+// FP64: tanh emulators mostly on the tensor cores, others (CMB: unbounded activations, folded
 // heads) on CUDA cores.
 static int run_emulator_f64(const ns_problem* p, Workspace* ws, int grid_rows, cudaStream_t st, const Head& hd) {
     const int L = p->n_layers;
@@ -453,7 +457,7 @@ static int run_emulator_f64(const ns_problem* p, Workspace* ws, int grid_rows, c
     for (int l = 1; l < L; ++l) {
         const int K = p->dims[l], N = p->dims[l + 1];
         const double* x = (const double*)ws->act[cur];
-        if (!p->tmWs.empty()) {
+        if (!p->d_wscale.empty()) {
             NS_TRY(launch_layer_f64(p, l, ws->xs, x, l == L - 1 ? (double*)hd.out : (double*)ws->act[cur ^ 1],
                                     ws->d_nrows, grid_rows, ws->d_err, st));
         } else if (l == L - 1) {

@@ -114,8 +114,10 @@ struct ns_problem {
     std::vector<int> dims;
     std::vector<void*> d_W;          // per layer, compute dtype (layer 0: FP64 or FP32)
     std::vector<void*> d_b;          // per layer, FP64 (FP64 mode) else FP32
-    std::vector<CUtensorMap> tmWs;   // FP64 tanh emulators, layers >= 1: the weights as fixed-point slices
-    std::vector<double*> d_wscale;   // and their rows' scales
+    // FP64 tanh emulators (else empty), layers >= 1: the weights as fixed-point slices and
+    // their rows' scales (null: the layer takes FP64 FMAs)
+    std::vector<CUtensorMap> tmWs;
+    std::vector<double*> d_wscale;
     std::vector<__nv_bfloat16*> d_Wp;   // and the planes themselves (row pitch plane_pitch(K))
     std::vector<CUtensorMap> tmWp;   // FP32 layers >= 1 (and a BF16 CMB head): the weights as three bf16 planes
     std::vector<CUtensorMap> tmB;    // BF16: weight tensor maps for layers >= 1
@@ -333,10 +335,12 @@ int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const Slice
                        int grid_rows, int N, int K, int* err, cudaStream_t st);
 int launch_slice_rows(const double* in, int rows, int K, __half* out, long long stride, int pitch, double* scale,
                       const int* nrows, cudaStream_t st);
+int slices_fit(const double* W, int rows, int K, int* d_flag, bool* fit);   // synchronises
+bool takes_slices(const ns_problem* p);                // some layer does
 size_t slice_input_bytes(const ns_problem* p, int cap);
 int slice_input_maps(const ns_problem* p, int cap, SliceInput* x);   // slices and scale are set
 // Layer l >= 1 of a tanh emulator in FP64, x (rows x dims[l]) -> out (rows x dims[l + 1]):
-// slices on the tensor cores where the problem has them, FP64 FMAs else.
+// slices on the tensor cores where the layer has them, FP64 FMAs else.
 int launch_layer_f64(const ns_problem* p, int l, const SliceInput& xs, const double* x, double* out, const int* nrows,
                      int grid_rows, int* err, cudaStream_t st);
 int make_tensor_map_slices(CUtensorMap* tm, const void* base, int rows, int K, long long stride, int box_rows);

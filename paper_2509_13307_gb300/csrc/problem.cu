@@ -97,7 +97,7 @@ int workspace_create(const ns_problem* p, int cap, Workspace* ws) {
     c.want(&ws->theta_full, sizeof(double) * (size_t)cap * p->P);
     c.want(&ws->logL, sizeof(double) * (size_t)cap);
     const bool gauss = p->kind == NS_KIND_GAUSS, cmb = p->kind == NS_KIND_CMB;
-    const bool f64 = p->precision == NS_PREC_FP64, slices = !p->tmWs.empty();
+    const bool f64 = p->precision == NS_PREC_FP64, slices = takes_slices(p);
     // activations: FP64, bf16, or FP32 as three bf16 planes
     const int elt = f64 ? 8 : (p->precision == NS_PREC_FP32 ? 6 : 2), tab_elt = f64 ? 8 : 4;
     const int rows_pad = ((cap + 127) / 128) * 128;
@@ -577,6 +577,7 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
     p->d_W.assign(e.n_layers, nullptr);
     p->d_b.assign(e.n_layers, nullptr);
     Staging staging;
+    void* flag = nullptr;
     if (!f64) {
         p->tmWp.resize(e.n_layers);
         p->d_Wp.assign(e.n_layers, nullptr);
@@ -593,14 +594,18 @@ extern "C" int ns_problem_create(const ns_problem_desc* desc, ns_problem** out) 
             if (l >= 1 && !cmb && e.activation == NS_ACT_TANH && !e.out_sigma_vec) {
                 const int N = p->dims[l + 1], K = p->dims[l], pitch = plane_pitch(K);
                 const long long stride = (long long)N * pitch;
+                p->tmWs.resize(e.n_layers);
+                p->d_wscale.resize(e.n_layers);
+                bool fit = false;
+                if (!flag && (s = dalloc(sizeof(int), &flag, p->owned))) return fail(s);
+                if ((s = slices_fit(w, N, K, (int*)flag, &fit))) return fail(s);
+                if (!fit) continue;
                 void *v, *sc;
                 if ((s = dalloc(sizeof(uint16_t) * 6 * (size_t)stride, &v, p->owned)) ||
                     (s = dalloc(sizeof(double) * N, &sc, p->owned)) ||
                     (s = launch_slice_rows(w, N, K, (__half*)v, stride, pitch, (double*)sc, nullptr,
                                            nullptr)))
                     return fail(s);
-                p->tmWs.resize(e.n_layers);
-                p->d_wscale.resize(e.n_layers);
                 p->d_wscale[l] = (double*)sc;
                 if ((s = make_tensor_map_slices(&p->tmWs[l], v, N, K, stride, 128))) return fail(s);
             }

@@ -118,3 +118,42 @@ def test_small_activations_keep_fp64(width, order):
     err = float(np.max(np.abs(got - ref) / mag))
     print(f"width {width}, order {order}: {err:.2e}")
     assert err < 2.0 ** -51
+
+
+def test_infinite_weights_act_as_in_fp64():
+    """Infinite weights saturate tanh and make infinite outputs of the FP64 sums' signs."""
+    inp = _inputs((256, 256))
+    inp["emu_W"][1][17, 40] = np.inf
+    inp["emu_W"][1][99, 3] = -np.inf
+    inp["emu_W"][2][5, 7] = np.inf
+    p = _problem(inp, 9)
+    full = free_theta(inp, random_cube(9, p.d, 5))
+    got = p.emulator(torch.tensor(full, device="cuda")).cpu().numpy()
+    ref = _emulator(inp, full)
+    assert p.device_status() == 0 and np.isinf(ref[:, 5]).all()
+    assert np.allclose(got, ref, rtol=1e-11, atol=1e-11)
+
+
+@pytest.mark.parametrize("large", [1e6, 1e150])
+def test_outlying_weight_keeps_fp64(large):
+    """One weight far above the others of its row, against an activation as far below
+    its own: the other products keep their bits.  Bound 2^-49 of sum |w| |h|: sixteen
+    rounding units, where an FP64 FMA chain of 1024 terms stays within three; digits held
+    against the large weight are off by 2^-38 and more."""
+    inp = _inputs((1024,))
+    inp["emu_W"][1][:, 300] *= large
+    inp["emu_W"][0][300] /= large
+    inp["emu_b"][0][300] /= large
+    inp["emu_b"][1][:] = 0.0
+    inp["emu_out_mu"][:] = 0.0
+    p = _problem(inp, 20)
+    full = free_theta(inp, random_cube(20, p.d, 4))
+    got = p.emulator(torch.tensor(full, device="cuda")).cpu().numpy()
+    ld = np.longdouble
+    x = (full[:, inp["emu_inputs"]].astype(ld) - inp["emu_in_center"]) / inp["emu_in_scale"]
+    h = np.tanh(x @ inp["emu_W"][0].T.astype(ld) + inp["emu_b"][0])
+    W = inp["emu_W"][1].astype(ld)
+    ref, mag = inp["emu_out_sigma"] * (h @ W.T), inp["emu_out_sigma"] * (np.abs(h) @ np.abs(W).T)
+    err = float(np.max(np.abs(got - ref) / mag))
+    print(f"large {large}: {err:.2e}")
+    assert err < 2.0 ** -49
