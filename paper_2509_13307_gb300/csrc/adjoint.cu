@@ -227,11 +227,11 @@ static int back_layer(const double* A, const double* W, const double* h, double*
 
 }  // namespace adj
 
-// One problem's gradient state.
+// One problem's gradient state.  Its kernels report to the problem's status word
+// (Workspace::d_err), which ns_problem_status reads.
 struct GradState {
     const ns_problem* p = nullptr;
     int* d_nrows = nullptr;
-    int* d_err = nullptr;
     double* theta_full = nullptr;
     void* table = nullptr;     // cap x n_out (emulator output)
     void* table_fine = nullptr;
@@ -293,8 +293,6 @@ static int grad_state_create(const ns_problem* p, GradState* g) {
     g->p = p;
     NS_TRY(g->graphs.create(g->owned));
     NS_TRY(grad_alloc(g, sizeof(int), (void**)&g->d_nrows));
-    NS_TRY(grad_alloc(g, sizeof(int), (void**)&g->d_err));
-    NS_CUDA_TRY(cudaMemset(g->d_err, 0, sizeof(int)));
     NS_TRY(grad_alloc(g, sizeof(double) * (size_t)cap * p->P, (void**)&g->theta_full));
     NS_TRY(grad_alloc(g, sizeof(double) * (size_t)cap * p->P, (void**)&g->gfull));
     NS_TRY(grad_alloc(g, T * (size_t)cap * n_out, &g->table));
@@ -395,7 +393,7 @@ static int run_grad_f64(const ns_problem* p, GradState* g, int B, OutPtr logL, O
     NS_CUDA_TRY(cudaGetLastError());
     for (int l = 1; l < L; ++l)
         NS_TRY(launch_layer_f64(p, l, g->xs, g->H[l], l == L - 1 ? (double*)g->table : g->H[l + 1], g->d_nrows, B,
-                                g->d_err, st));
+                                p->ws.d_err, st));
     const double* tab = (const double*)g->table;
     const bool coarse = p->n_z_emu != sp.n_z;
     if (coarse) {
@@ -403,7 +401,7 @@ static int run_grad_f64(const ns_problem* p, GradState* g, int B, OutPtr logL, O
         tab = (const double*)g->table_fine;
     }
     NS_TRY(launch_projection_adj<double>(sp, &g->proj, g->theta_full, tab, p->d_LinvT64, (const double*)g->Linv, p->c0,
-                                         TableGrad{g->gtab}, g->gfull, logL, g->d_nrows, B, g->d_err, st));
+                                         TableGrad{g->gtab}, g->gfull, logL, g->d_nrows, B, p->ws.d_err, st));
     // table adjoint -> emulator output adjoint (transpose of the z interpolation) -> g_pre_L
     const double* gt = (const double*)g->gtab;
     if (coarse) {
@@ -452,7 +450,7 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, OutPtr logL
         }
         // BF16: no K split, so that every activation has the bits of the one chain
         NS_TRY(launch_gemm_planes(px, pw, &g->tmW[l], &g->tmH[l], e, g->d_nrows, B, p->dims[l + 1], p->dims[l],
-                                  pw == 1 ? 1 : 0, g->d_err, st));
+                                  pw == 1 ? 1 : 0, p->ws.d_err, st));
     }
     const float* tab = (const float*)g->table;
     const bool coarse = p->n_z_emu != sp.n_z;
@@ -472,7 +470,7 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, OutPtr logL
         tg.scale = (float)p->out_sigma;
     }
     NS_TRY(launch_projection_adj<float>(sp, &g->proj, g->theta_full, tab, p->d_LinvT32, (const float*)g->Linv, p->c0, tg,
-                                        g->gfull, logL, g->d_nrows, B, g->d_err, st));
+                                        g->gfull, logL, g->d_nrows, B, p->ws.d_err, st));
     if (coarse) {
         const dim3 gz((n_out + 255) / 256, B);
         adj::k_zinterp_adj<float><<<gz, 256, 0, st>>>((const float*)g->gtab, sp.n_z, p->d_zi_row, p->d_zi_w,
@@ -491,7 +489,7 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, OutPtr logL
         if (l == 1) e.out = g->G1;
         else planes_out(e, g->Gp[(L - l) & 1], p->dims[l]);
         NS_TRY(launch_gemm_planes(px, pw, &g->tmWT[l], &g->tmG[l], e, g->d_nrows, B, p->dims[l], p->dims[l + 1], 0,
-                                  g->d_err, st));
+                                  p->ws.d_err, st));
     }
     return launch_finish_grad<float>(p, g, g->G1, B, grad, st);
 }
