@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(128)
 k_window_nodes(const ShearParams sp, const double* __restrict__ theta_full, T* __restrict__ nodes,
                const int* __restrict__ nrows) {
     using M = Math<T, false>;
-    const int row = blockIdx.y, n = blockIdx.x * 128 + threadIdx.x, N = sp.N;
+    const int row = blockIdx.x, n = blockIdx.y * 128 + threadIdx.x, N = sp.N;   // rows on x: no 65535 limit
     if (row >= *nrows || n >= N) return;
     const double* t = theta_full + (size_t)row * sp.n_params;
     const T h = (T)t[2];
@@ -1065,7 +1065,7 @@ static int windows_nb(const ShearParams& sp, const double* theta_full, T* win, c
     }
     if constexpr (sizeof(T) == 8) {
         if (!nodes) return NS_EINVAL;
-        k_window_nodes<T, NB><<<dim3((sp.N + 127) / 128, grid_rows), 128, 0, st>>>(sp, theta_full, nodes, nrows);
+        k_window_nodes<T, NB><<<dim3(grid_rows, (sp.N + 127) / 128), 128, 0, st>>>(sp, theta_full, nodes, nrows);
         NS_CUDA_TRY(cudaGetLastError());
     }
     k_windows<T, NB, FAST><<<grid_rows, kProjThreads, smem, st>>>(sp, theta_full, win, nrows, nodes);
