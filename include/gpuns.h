@@ -55,11 +55,13 @@ extern "C" {
 /* ---- enums -------------------------------------------------------------- */
 enum ns_kind { NS_KIND_GAUSS = 0, NS_KIND_SHEAR = 1, NS_KIND_CMB = 2 };
 /* Arithmetic of the likelihood.  FP64: every stage in double (the GEMMs of a
- * tanh emulator as exact sums of fixed-point fp16 slices on the tensor cores).
+ * tanh emulator as sums of fixed-point fp16 slices on the tensor cores, at
+ * least as accurate as sums of doubles where the weights suit it, else as those).
  * FP32: every stage in float (GEMMs as sums of three bf16 planes per operand,
- * FP32 accumulation), the constant and the final log L in double.  BF16: emulator hidden/output GEMMs as tcgen05 BF16 x BF16 -> FP32
- * tensor-core MMAs, all other stages FP32.  BF16_F64CHI2: as BF16 but the
- * whitening solve and chi^2 in FP64. */
+ * FP32 accumulation; an infinite weight or activation gives NaN), the constant
+ * and the final log L in double.  BF16: emulator hidden/output GEMMs as tcgen05
+ * BF16 x BF16 -> FP32 tensor-core MMAs, all other stages FP32.  BF16_F64CHI2:
+ * as BF16 but the whitening solve and chi^2 in FP64. */
 enum ns_precision { NS_PREC_FP64 = 0, NS_PREC_FP32 = 1, NS_PREC_BF16 = 2, NS_PREC_BF16_F64CHI2 = 3 };
 enum ns_prior_kind { NS_PRIOR_UNIFORM = 0, NS_PRIOR_GAUSS = 1, NS_PRIOR_FIXED = 2 };
 /* Hidden-layer activation: tanh, or CosmoPower's "sigmoid-linear"

@@ -154,16 +154,28 @@ __device__ __forceinline__ float ld_cluster_f32(uint32_t cluster_addr) {
     return v;
 }
 
-// v as P bf16 planes `stride` elements apart: the leading plane rounds v, each
-// further one the remainder (exact in FP32); three hold every FP32 value.
+// The leading bf16 plane of v, which is left as the remainder (exact in FP32).  Values
+// above the largest bf16 (3.39e38), which would round to infinity, are cut instead;
+// nothing follows an infinity.
+__device__ __forceinline__ __nv_bfloat16 plane_take(float& v) {
+    __nv_bfloat16 q = __float2bfloat16_rn(v);
+    if (fabsf(v) > 3.38953138925153547590e38f) {
+        if (isinf(v)) {
+            v = 0.f;
+            return q;
+        }
+        q = __float2bfloat16_rz(v);
+    }
+    v -= __bfloat162float(q);
+    return q;
+}
+
+// v as P bf16 planes `stride` elements apart, each of the remainder of those before;
+// three hold every FP32 value.
 template <int P>
 __device__ __forceinline__ void plane_store(float v, __nv_bfloat16* out, long long stride) {
 #pragma unroll
-    for (int p = 0; p < P; ++p) {
-        const __nv_bfloat16 q = __float2bfloat16_rn(v);
-        out[p * stride] = q;
-        v -= __bfloat162float(q);
-    }
+    for (int p = 0; p < P; ++p) out[p * stride] = plane_take(v);
 }
 
 // v in [-1, 1] as kSlices fixed-point slices `stride` elements apart:
