@@ -303,7 +303,10 @@ int ns_problem_status(ns_problem* p, int* bits, int clear);
  * Table 1 prior's physical parameters); the paper's pipeline is
  * auto-differentiable (Sec. 2.2, Sec. 4.2) and its HMC comparison runs use
  * these gradients (Sec. 3.2).  Shear kind; closed form for the Gaussian test
- * kind; NS_ENOTSUP for the CMB kind.  B <= max_batch, else NS_EINVAL. */
+ * kind; NS_ENOTSUP for the CMB kind.  B <= max_batch, else NS_EINVAL.  Calls
+ * repeat bit for bit; a row's log L has the same bits in every batch, its
+ * gradient in batches of the same size up to 16 or the same 16 rows above
+ * (sums are split by the rows of a call). */
 int loglike_grad_batch(const ns_problem* p, const double* theta_dev, int B,
                        double* logL_dev, double* grad_dev, void* stream);
 

@@ -90,8 +90,9 @@ __global__ void k_back_sum(const double* __restrict__ part, int cap, int shares,
 }
 
 // Shares of a backward contraction: enough for one block per SM at one row tile,
-// at least 64 terms each.  By shape only: a row's gradient does not depend on
-// its batch.
+// at least 64 terms each, by shape only.  (The table gradient's partial sums go by the
+// rows of a call, projection_adj.cu, as do the K splits of the backward plane GEMMs: a
+// gradient has the same bits in every call of its row bucket, log L in every call.)
 static int back_shares(int N, int K) {
     const int tiles = (N + kBackN - 1) / kBackN;
     return std::max(1, std::min((K + 63) / 64, 152 / tiles));
@@ -448,9 +449,10 @@ static int run_grad_planes(const ns_problem* p, GradState* g, int B, OutPtr logL
         } else {
             planes_out(e, g->Hp[l + 1], p->dims[l + 1]);
         }
-        // BF16: no K split, so that every activation has the bits of the one chain
+        // by shape alone, so that log L does not depend on the batch; BF16: no K split, so
+        // that every activation has the bits of the one chain
         NS_TRY(launch_gemm_planes(px, pw, &g->tmW[l], &g->tmH[l], e, g->d_nrows, B, p->dims[l + 1], p->dims[l],
-                                  pw == 1 ? 1 : 0, p->ws.d_err, st));
+                                  pw == 1 ? 1 : plane_split(p->dims[l + 1], p->dims[l]), p->ws.d_err, st));
     }
     const float* tab = (const float*)g->table;
     const bool coarse = p->n_z_emu != sp.n_z;

@@ -74,13 +74,14 @@ __device__ __forceinline__ float p10(float v) { return exp2f(v * 3.3219280948873
 constexpr int kChiThreads = 960, kChiSeg = 16;
 template <typename T> constexpr int kChiV = 16 / sizeof(T);
 
-// shares of the reduction range: what the threads allow, four for many rows
-__host__ __device__ inline int chi2_adj_parts(int D, int v, int rb) {
+// Shares of the reduction range: what the threads allow, whatever the rows per block, so
+// that a row's sums have one order in every batch.
+__host__ __device__ inline int chi2_adj_parts(int D, int v) {
     const int p = kChiThreads / ((D + v - 1) / v);
-    return p < 1 ? 1 : (rb > 1 && p > 4) ? 4 : p;
+    return p < 1 ? 1 : p;
 }
 __host__ __device__ inline size_t chi2_adj_elems(int D, int v, int nb, int np, int nt, int rb) {
-    return (size_t)rb * ((2 + chi2_adj_parts(D, v, rb)) * (size_t)((D + v - 1) / v * v) + nb + np + kChiSeg * (size_t)nt);
+    return (size_t)rb * ((2 + chi2_adj_parts(D, v)) * (size_t)((D + v - 1) / v * v) + nb + np + kChiSeg * (size_t)nt);
 }
 
 template <typename T, int RB>
@@ -94,14 +95,13 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int V = kChiV<T>;
     const int D = sp.D, P = sp.n_params, nb = sp.nb, n_ell = sp.n_ell, nt = sp.n_tmpl, np = sp.n_pairs;
-    const int groups = (D + V - 1) / V, Dv = groups * V, parts = chi2_adj_parts(D, V, RB);
+    const int groups = (D + V - 1) / V, Dv = groups * V, parts = chi2_adj_parts(D, V);
     T* r = reinterpret_cast<T*>(smem_raw);     // Dv x RB, later g_m
     T* y = r + Dv * RB;                        // Dv x RB
     T* part = y + Dv * RB;                     // parts x Dv x RB
     T* th = part + (size_t)parts * Dv * RB;    // RB x nb: 1 + m_i
     T* S = th + RB * nb;                       // np x RB: sum_ell g_m C
     T* tp = S + np * RB;                       // kChiSeg x RB x nt partial template sums
-    __shared__ T wsum[(kChiThreads / 32) * RB];
     __shared__ int pi[16], pj[16];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     if (tid < np) { pi[tid] = sp.pi[tid]; pj[tid] = sp.pj[tid]; }
@@ -151,21 +151,14 @@ k_chi2_adj(const ShearParams sp, const double* __restrict__ theta_full, const T*
         return s;
     };
     columns(LinvT, r, true);
-    T sq = T(0);                               // kChiThreads is a multiple of RB: a thread keeps its row
-    static_assert(kChiThreads % RB == 0, "rows of a thread");
-    for (int i = tid; i < D * RB; i += kChiThreads) {
-        y[i] = join(i);
-        sq = fma(y[i], y[i], sq);
-    }
-    // row sums: lanes of equal row (stride RB), then over warps
-#pragma unroll
-    for (int o = 16; o >= RB; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-    if (lane < RB) wsum[wid * RB + lane] = sq;
+    for (int i = tid; i < D * RB; i += kChiThreads) y[i] = join(i);
     __syncthreads();
-    if (tid < RB && r0 + tid < M) {
-        T s = T(0);
-        for (int w = 0; w < kChiThreads / 32; ++w) s += wsum[w * RB + tid];
-        logL.get()[r0 + tid] = c0 - 0.5 * (double)s;
+    static_assert(kChiThreads / 32 >= RB, "a warp per row");
+    if (wid < RB && r0 + wid < M) {            // chi^2 of a row by one warp
+        T sq = T(0);
+        for (int a = lane; a < D; a += 32) sq = fma(y[a * RB + wid], y[a * RB + wid], sq);
+        sq = warp_sum(sq);
+        if (lane == 0) logL.get()[r0 + wid] = c0 - 0.5 * (double)sq;
     }
     // g_m = L^-T y: (g_m)_a = sum_{b >= a} (L^-1)[b][a] y_b
     columns(Linv, y, false);
