@@ -5,8 +5,7 @@
 //
 // An FP32 value is the exact sum of three bf16 values (8 significant bits
 // each): hi = bf16(v), mid = bf16(v - hi), lo = v - hi - mid.  (An infinite operand makes
-// NaN, not the infinity of an FP32 sum: it also multiplies the other operand's lower
-// planes, zeros and either sign among them.)  X comes in PX
+// NaN, not the infinity of an FP32 sum.)  X comes in PX
 // planes and W in PW planes (3: an FP32 operand, 2: the leading 16 bits, 1: a
 // bf16 operand), and the products of plane pairs with p + q <= 2 are summed;
 // the three pairs left out of 3 x 3 are below 2^-25 of the full product.
@@ -242,7 +241,7 @@ k_gemm_planes(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
                 return;
             }
         }
-        plane_store<PX>(v, e.planes + (size_t)row * e.pitch + f, e.plane_stride);
+        if constexpr (PX > 1) plane_store<PX>(v, e.planes + (size_t)row * e.pitch + f, e.plane_stride);
     };
     __syncthreads();                                 // the ring's last copies have landed
     const bool failed = s_fail != 0;
@@ -359,7 +358,7 @@ __global__ void __launch_bounds__(256) k_split_planes(const float* __restrict__ 
         for (int p = 0; p < P; ++p) {
             __align__(8) __nv_bfloat16 q[V];
 #pragma unroll
-            for (int j = 0; j < V; ++j) q[j] = plane_take(v[j]);
+            for (int j = 0; j < V; ++j) q[j] = plane_take(p, v[j]);
             if constexpr (V == 4) *reinterpret_cast<uint2*>(o + p * stride) = *reinterpret_cast<const uint2*>(q);
             else o[p * stride] = q[0];
         }
