@@ -28,7 +28,9 @@
  *   - `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *     stream).  Calls are asynchronous on that stream unless stated.
  *   - One problem or run must not be used from two streams at once: each owns
- *     scratch buffers that consecutive calls reuse.
+ *     scratch buffers that consecutive calls reuse.  (Gradient calls of a
+ *     problem may come from several threads and streams: each call, unless it
+ *     is being captured into a graph of the caller's, follows the one before.)
  */
 #ifndef GPUNS_H
 #define GPUNS_H

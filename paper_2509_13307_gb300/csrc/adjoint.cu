@@ -269,6 +269,7 @@ int CallGraphs::create(std::vector<void*>& owned) {
     if (cudaMalloc(&v, 2 * sizeof(double*)) != cudaSuccess) return NS_ENOMEM;
     owned.push_back(v);
     d_out = (double**)v;
+    NS_CUDA_TRY(cudaEventCreateWithFlags(&done, cudaEventDisableTiming));
     return NS_OK;
 }
 
@@ -277,7 +278,9 @@ void CallGraphs::release() {
         if (e.exec) cudaGraphExecDestroy(e.exec);
     entries.clear();
     if (cap) cudaStreamDestroy(cap);
+    if (done) cudaEventDestroy(done);
     cap = nullptr;
+    done = nullptr;
 }
 
 static int grad_alloc(GradState* g, size_t bytes, void** out) {
@@ -546,12 +549,14 @@ extern "C" int loglike_grad_batch(const ns_problem* p, const double* theta_dev, 
         }
     }
     double** out = gs->graphs.d_out;
-    NS_TRY(launch_free_to_full(p, theta_dev, B, gs->theta_full, gs->d_nrows, out, logL_dev, grad_dev, st));
     const int rows = call_rows(B, p->max_batch);
-    return gs->graphs.run(rows, st, [&](cudaStream_t s) {
-        return p->precision == NS_PREC_FP64 ? run_grad_f64(p, gs, rows, OutPtr{out}, OutPtr{out + 1}, s)
-                                            : run_grad_planes(p, gs, rows, OutPtr{out}, OutPtr{out + 1}, s);
-    });
+    return gs->graphs.call(
+        rows, st,
+        [&] { return launch_free_to_full(p, theta_dev, B, gs->theta_full, gs->d_nrows, out, logL_dev, grad_dev, st); },
+        [&](cudaStream_t s) {
+            return p->precision == NS_PREC_FP64 ? run_grad_f64(p, gs, rows, OutPtr{out}, OutPtr{out + 1}, s)
+                                                : run_grad_planes(p, gs, rows, OutPtr{out}, OutPtr{out + 1}, s);
+        });
 }
 
 // Called by ns_problem_free: release the gradient state of a problem.

@@ -23,12 +23,20 @@ struct OutPtr {
 struct CallGraphs {
     static constexpr int kMost = 8;
     struct Entry { int rows, seen; cudaGraphExec_t exec; };
-    std::mutex mu;                // a graph is launched by one thread at a time
+    // Held by a call from its set-up kernel to its last launch: the launches read the row
+    // count, the parameters and the result slots that this kernel writes.  Calls on
+    // different streams follow one another by `done` (1 us of host time), so that none of
+    // them can write through the slots of another, whose buffers may be gone.
+    std::mutex mu;
+    cudaEvent_t done = nullptr;
     std::vector<Entry> entries;
     cudaStream_t cap = nullptr;
     double** d_out = nullptr;     // device slots: log L, gradient
     int create(std::vector<void*>& owned);
     void release();
+    // set-up, then the launches of `body`, alone or as a graph (mu is taken)
+    template <typename S, typename F>
+    int call(int rows, cudaStream_t st, S&& setup, F&& body);
     template <typename F>
     int run(int rows, cudaStream_t st, F&& body);
 };
@@ -40,11 +48,23 @@ inline int call_rows(int B, int max_batch) {
     return r < max_batch ? r : max_batch;
 }
 
+template <typename S, typename F>
+int CallGraphs::call(int rows, cudaStream_t st, S&& setup, F&& body) {
+    std::lock_guard<std::mutex> lk(mu);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        NS_TRY(setup());                          // the caller orders the replays of its own graph
+        return body(st);
+    }
+    NS_CUDA_TRY(cudaStreamWaitEvent(st, done, 0));
+    NS_TRY(setup());
+    const int s = run(rows, st, body);
+    NS_CUDA_TRY(cudaEventRecord(done, st));       // after a failed launch too: what was queued still runs
+    return s;
+}
+
 template <typename F>
 int CallGraphs::run(int rows, cudaStream_t st, F&& body) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return body(st);
-    std::lock_guard<std::mutex> lk(mu);
     Entry* e = nullptr;
     for (Entry& x : entries)
         if (x.rows == rows) e = &x;
