@@ -36,14 +36,15 @@
 // the 39-d emulator, 42 us at the measured peak) for many rows, the copies and
 // the fixed cost of a launch for few.  Against the FP32 FMA GEMM it replaced
 // (128 x 128 tiles, 32 CTAs per hidden layer at 500 rows): log-likelihoods of
-// 500 rows of the 39-d problem 2082 -> 247 us, of 250 rows of the dense CMB
-// problem 814 -> 65 us, of 333 rows of its TT form with BF16 hidden layers
-// 200 -> 54 us; gradients of 129 rows in FP32 4128 -> 781 us (with the
-// projection's 540 us unchanged), and of 64 rows in BF16 775 -> 608 us against
-// one-CTA tiles that walked all of K = 10000.  Sending the tile through shared
-// memory to one rolled epilogue loop, instead of an epilogue unrolled over the
-// registers, took the 500-row call from 275 to 247 us.  Error of the 39-d emulator's table against FP64 over 500
-// rows: rms 8.90e-8 dex, largest 4.8e-7 (FMA chain: 9.01e-8 and 5.2e-7).
+// 500 rows of the 39-d problem 2082 -> 247 us (221 with the stages around the
+// layers of today), of 250 rows of the dense CMB problem 814 -> 65 us, of 333
+// rows of its TT form with BF16 hidden layers 200 -> 48 us.  500 FP32 rows: a
+// hidden layer 17 us, the output layer 87 us with the tensor pipe active 44 % of
+// its cycles; 4096 rows of a BF16 gradient: 43 and 280 us forward, 57 and 191
+// backward.  Sending the tile through shared memory to one rolled epilogue loop,
+// instead of an epilogue unrolled over the registers, took the 500-row call from
+// 275 to 247 us.  Error of the 39-d emulator's table against FP64 over 500 rows:
+// rms 8.90e-8 dex, largest 4.8e-7 (FMA chain: 9.01e-8 and 5.2e-7).
 #include <algorithm>
 
 #include "likelihood.cuh"

@@ -31,9 +31,12 @@
 // whose integer partial tiles are added exactly through cluster shared memory.
 // A NaN operand (its leading slice is NaN) and a timeout give NaN.
 //
-// Measured on the 39-d emulator: 64 rows 5.80 ms of FP64 FMA tiles -> 0.35 ms
-// (the call 6367 -> 1070 us); error of its table against 113-bit arithmetic
-// rms 1.17e-16, largest 4.1e-16 (FMA chain 1.18e-16 and 4.8e-16).
+// Measured on the 39-d emulator: 64 rows 5.80 ms of FP64 FMA tiles -> 0.22 ms (a
+// hidden layer 27 us, its slices 7, the output layer 107), beside the windows' 130; the call
+// 6367 -> 571 us.  With 21 pairs, 128 k per sum and activations sliced in the epilogues,
+// which lost bits, it took 559.  Error of its standardised outputs against 113-bit
+// arithmetic rms 2.34e-15, largest 9.2e-15 (FMA chain 2.41e-15 and 1.04e-14: the mean
+// table's own rounding is most of both).
 //
 // Warps 0-7 (0-15 for 64 rows): drain and epilogue; then one warp for the copies
 // and one for TMEM and MMAs.  Waits are bounded as in gemm_planes.cu.
@@ -252,8 +255,9 @@ k_gemm_slices(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ C
 }
 
 // Slices and power-of-two scale of every row of a matrix (rows x K): the weights once, the
-// activations before each layer (64 rows of 1024: beside the windows, off the call's
-// longest path).
+// activations before each layer.  A block per row, bound by its two dependent passes (64
+// rows of 1024: 7 us); the row's maximum takes all of a layer's CTAs, so that the layer's
+// epilogue cannot slice.
 __global__ void __launch_bounds__(256) k_slice_rows(const double* __restrict__ W, int K, __half* __restrict__ out,
                                                     long long stride, int pitch, double* __restrict__ scale,
                                                     const int* __restrict__ nrows) {

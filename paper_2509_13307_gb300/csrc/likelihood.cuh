@@ -118,8 +118,8 @@ struct ns_problem {
     // their rows' scales (null: the layer takes FP64 FMAs)
     std::vector<CUtensorMap> tmWs;
     std::vector<double*> d_wscale;
-    std::vector<__nv_bfloat16*> d_Wp;   // and the planes themselves (row pitch plane_pitch(K))
     std::vector<CUtensorMap> tmWp;   // FP32 layers >= 1 (and a BF16 CMB head): the weights as three bf16 planes
+    std::vector<__nv_bfloat16*> d_Wp;   // and the planes themselves (row pitch plane_pitch(K))
     std::vector<CUtensorMap> tmB;    // BF16: weight tensor maps for layers >= 1
     std::vector<int> tile_n;         // BF16: N tile per layer (hidden layers autotuned at creation)
     std::vector<CUtensorMap> tmB64;  // BF16, autotuned hidden layers: weight maps of 64-wide tiles (many rows)

@@ -25,8 +25,8 @@
 // SM).  The one-kernel form it replaced kept 250 KB of intermediates per evaluation
 // in global memory and added 16 atomics per (node, multipole) to the table
 // gradient.  Whole BF16 gradient calls of the 39-d problem: 4096 rows 9978 -> 3290
-// us, 64 rows 608 -> 290 us.  Per 4096 evaluations (BF16 problem): k_limber_adj 714
-// us, k_limber_nodes 527, k_windows_adj 519, k_chi2_adj 157, k_table_adj 153.
+// us, 64 rows 608 -> 300 us.  Per 4096 evaluations (BF16 problem): k_limber_adj 705
+// us, k_limber_nodes 539, k_windows_adj 521, k_chi2_adj 150, k_table_adj 155.
 #include <algorithm>
 #include <vector>
 
@@ -70,7 +70,7 @@ __device__ __forceinline__ float p10(float v) { return exp2f(v * 3.3219280948873
 // RB rows per block: each entry of L^-1 read serves RB rows, whose values lie
 // beside one another in shared memory.  A thread takes V neighbouring columns (one
 // 16-byte load) of one of `parts` shares of the reduction range, a short chain of
-// L2 latencies (one thread per column: 119 us for 64 rows, D = 300).
+// L2 latencies (64 rows, D = 300: one thread per column 119 us, so 23 us with a cold L2).
 constexpr int kChiThreads = 960, kChiSeg = 16;
 template <typename T> constexpr int kChiV = 16 / sizeof(T);
 
@@ -264,7 +264,7 @@ template <typename T> struct alignas(16) Z4 {
 // multipole per lane, 20 of 32 lanes worked and each node took a warp reduction of
 // six values and the loads of its windows: 460 k warp instructions per evaluation,
 // 2560 us for 4096 evaluations of the 39-d problem; the two kernels: 66 k and
-// 155 k instructions, 527 + 714 us.
+// 140 k instructions, 539 + 705 us.
 template <typename T, int NB> constexpr int kGQuads = (NB * (NB + 1) / 2 + 1) / 2;   // pairs of g_C entries
 constexpr int kNodeThreads = 256;
 
@@ -416,8 +416,8 @@ k_limber_nodes(const ShearParams sp, const T* __restrict__ table, const T* __res
     }
 }
 
-// Table gradient of g_v.  Bound by instruction issue (155 k warp instructions per
-// evaluation, 2.5 per cycle); node constants are read where they are used, which
+// Table gradient of g_v.  Bound by instruction issue (140 k warp instructions per
+// evaluation, 2.4 per cycle); node constants are read where they are used, which
 // leaves registers for 28 warps per SM (held for four nodes at a time: 870 us against
 // 714 for 4096 evaluations).  One warp walks a contiguous range of chi nodes, one
 // multipole per lane.  Neighbouring nodes fall into the same z cell, and at most
