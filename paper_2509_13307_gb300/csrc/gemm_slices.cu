@@ -340,10 +340,12 @@ int launch_gemm_slices(const CUtensorMap* tmW, const SliceMapX* tmX, const Slice
     // Rows per tile and K split by the cycles of the SM that ends last (every group of
     // 64 k is added alike in each, so the choice does not change a bit).  A slot is 52 MMAs of ~65 cycles
     // each up to N = 64; the epilogue's FP64 runs at two operations per cycle (tanh
-    // ~75 per element, the output 6); 64-row tiles have one set of
-    // accumulators and wait for each drain; clusters of 8 (4) find room on about 96
-    // (128) SMs.  64 rows: 64-row output tiles 1 wave of 79 CTAs against two of 158
-    // (111 us); 16-row hidden tiles spread the FP64 of tanh over 128 SMs.
+    // ~75 per element, the output 6); 64-row tiles have one set of accumulators and
+    // wait for each drain; clusters of 8 (4) find room on about 96 (128) SMs.  Timed
+    // against all twelve (rows per tile, split) at 1 to 256 rows of 1024 -> 1024,
+    // 1024 -> 2000 and 1024 -> 10000: the choice is the fastest or within 3 % (64 rows,
+    // whole emulator: 242 us with 16 / 4 hidden and 64 / 4 output tiles; 64 / 1 output 251,
+    // 32 / 1 267; 16 / 2 hidden 285, 64 / 4 312).
     const int nk = (K + slc::SBK - 1) / slc::SBK, mt = (N + 127) / 128;
     int best_br = 32, best_s = 1;
     double best = 1e300;
