@@ -307,8 +307,8 @@ int ns_problem_status(ns_problem* p, int* bits, int clear);
  * these gradients (Sec. 3.2).  Shear kind; closed form for the Gaussian test
  * kind; NS_ENOTSUP for the CMB kind.  B <= max_batch, else NS_EINVAL.  Calls
  * repeat bit for bit; a row's log L has the same bits in every batch, its
- * gradient in batches of the same size up to 16 or the same 16 rows above
- * (sums are split by the rows of a call). */
+ * gradient in batches of one size class (1, 2, 4, 8, 16, then every 16 rows):
+ * some of its sums are split by the rows of a call. */
 int loglike_grad_batch(const ns_problem* p, const double* theta_dev, int B,
                        double* logL_dev, double* grad_dev, void* stream);
 
